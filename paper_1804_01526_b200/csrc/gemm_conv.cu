@@ -208,7 +208,7 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
             }
         } else if (warp == CV_MMA_WARP) {
             // -------------------------------------------------------------- MMA issuer
-            if (lane == 0) {
+            if (elect_one()) {
                 constexpr uint32_t idesc = idesc_conv<N_TILE>(false), idesc_ones = idesc_conv<N_TILE>(true);
                 const uint64_t ones_desc = smem_desc_rows<C>(base + ones_off, true);
                 uint32_t s = 0, ph = 0, b = 0, bph = 0;
@@ -349,11 +349,7 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
             for (int tap = 0; tap < p.taps; ++tap) {
                 const uint32_t taddr = lane_addr + b * CV_COLS;
                 uint32_t v[2][CH];
-                {   // polled first: a warp that try_wait has put to sleep wakes up late
-                    bool hit = false;
-                    for (int i = 0; i < 2048 && !hit; ++i) hit = cv_test_wait(tfull_bar + 8 * b, bph);
-                    if (!__all_sync(0xffffffffu, hit) && !mbar_wait_warp(tfull_bar + 8 * b, bph, abort_flag, p.status, 321)) { ok = false; break; }
-                }
+                if (!mbar_wait_warp_fast(tfull_bar + 8 * b, bph, abort_flag, p.status, 321)) { ok = false; break; }
                 tc_fence_after();
                 tc_ld8(taddr, v[0]);
                 const uint32_t* tab = tables + slot * G::SLOT_WORDS + half * HALF;
@@ -380,8 +376,7 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                         } else {
                             // the whole buffer is in registers: hand it back before the last chunk's arithmetic
                             tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(tempty_bar + 8 * b);
+                            mbar_arrive_elect(tempty_bar + 8 * b);
                         }
                         const uint32_t(&x)[CH] = v[idx & 1];
 #pragma unroll

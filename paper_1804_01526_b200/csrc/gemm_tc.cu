@@ -389,7 +389,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             }
         } else if (warp == MMA_WARP) {
             // -------------------------------------------------------------- MMA issuer
-            if (lane == 0) {
+            if (elect_one()) {
                 const MmaArgs ma{full_bar, empty_bar, tfull_bar, tempty_bar, done_bar, mant_base, tmem_base, total_work, abort_flag};
                 if (sh.lng) mma_issue_loop<N_TILE, PLANES, MAGIC, true, 4, TSTORE>(p, sh, ma);
                 else if (sh.spb == 2) mma_issue_loop<N_TILE, PLANES, MAGIC, false, 2, TSTORE>(p, sh, ma);

@@ -23,6 +23,16 @@ constexpr uint32_t WAIT_HINT_NS = 200000u;              // one try_wait may slee
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of the (converged) warp. A branch on this predicate is one the compiler knows to be taken by a single
+// lane of a converged warp: the instructions that one thread issues (tcgen05.mma, tcgen05.commit) cost it far less issue
+// time than behind `lane == 0` (two MMAs, a commit and two looks at barriers: 112 against 215 cycles; a commit alone: 5
+// against 46).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -73,6 +83,29 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
                                                int32_t* status, int code) {
     const bool ok = mbar_wait(bar, parity, abort_flag, status, code);
     return __all_sync(0xffffffffu, ok);
+}
+
+// One try_wait with the default suspend time (wakes promptly, unlike a wait with the long hint above).
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Whole-warp wait on the critical path of an arithmetic warp: one straight try_wait and a vote, loops only when that
+// failed. A loop that each lane may leave by itself costs the warp some 100 cycles per wait (lanes split and join again):
+// reading and adding 128 columns takes a warp 437 cycles with such a loop and 311 with this form.
+__device__ __forceinline__ bool mbar_wait_warp_fast(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    for (int i = 0; i < 64; ++i)
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    return mbar_wait_warp(bar, parity, abort_flag, status, code);
+}
+// Arrival of one lane of a converged warp, on a barrier of this CTA or (a cluster address) of any CTA of the cluster.
+__device__ __forceinline__ void mbar_arrive_elect(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster_elect(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\t@p mbarrier.arrive.shared::cluster.b64 _, [%0];\n\t}" ::"r"(bar) : "memory");
 }
 
 // Same copy with an L2 eviction-priority hint (a createpolicy-style 64-bit descriptor).
