@@ -358,7 +358,7 @@ HBFP_API int hbfp_gemm_block_partials(int64_t M, int64_t N, int64_t K, const hbf
 
 /* Host-only: name of the GEMM kernel that the calling thread's most recent hbfp_gemm, hbfp_gemm_q,
  * hbfp_gemm_static or hbfp_gemm_block_partials call launched ("gemm_tc2_kernel": two SMs per 256 x 256
- * tile; "gemm_tc_kernel": one SM per tile; "gemm_simt_kernel"; "conv_fwd_kernel" after hbfp_conv_forward),
+ * tile; "gemm_tc_kernel": one SM per tile, and the floating-point operand forms; "gemm_simt_kernel"; "conv_fwd_kernel" after hbfp_conv_forward),
  * "" before the first launch. For
  * measurement scripts that must name the kernel they timed (the paper has no counterpart). The
  * string is static storage. */

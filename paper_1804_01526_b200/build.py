@@ -13,13 +13,14 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhbfp.so")
-SOURCES = ["api.cu", "quantize.cu", "gemm_simt.cu", "gemm_small.cu", "gemm_tc.cu", "gemm_tc2.cu", "gemm_conv.cu", "gemm_static.cu"]
+SOURCES = ["api.cu", "quantize.cu", "gemm_simt.cu", "gemm_small.cu", "gemm_tc.cu", "gemm_tc2.cu", "gemm_fp.cu", "gemm_conv.cu", "gemm_static.cu"]
 # (object name, source, extra flags): quantize.cu is compiled a second time for the full-tile kernel of small tiles
 EXTRA_OBJECTS = [("quantize_tiles_small.o", "quantize.cu", ["-DHBFP_QUANT_PART=2", "-Xptxas", "-O1"])]
 # Per-file additions. The paired-SM GEMM is built with ptxas -O1: measured in SM cycles per launch (16384^3, b = 128)
 # 8.57 M against 8.86 M at the default level, and 12 % / 9 % fewer cycles for blocks of 64 / 32; the other files were
 # measured too and are a toss-up kernel by kernel (single-SM GEMM: 8-bit + 9 %, 12-bit - 6 %), so they keep the default.
 EXTRA_FLAGS = {"gemm_tc2.cu": ["-Xptxas", "-O1"],
+               "gemm_fp.cu": ["-Xptxas", "-O1"],
                "gemm_conv.cu": ["-Xptxas", "-O1"]}      # 128-channel forward 16.0 -> 15.0 us, 64-channel unchanged
 
 NVCC_FLAGS = [

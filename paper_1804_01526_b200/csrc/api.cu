@@ -34,7 +34,26 @@ struct GemmPlan {
     Layout la, lb;
     size_t off_am, off_ae, off_bm, off_be, off_partial, total;
     TensorPlan tp;
+    // the floating-point operand forms (gemm_fp.cu) lie behind the packed operands: A, then B
+    FpPlan fp;
+    size_t off_fa, off_fb, total_fp;
 };
+
+size_t fp_plane_bytes(const Layout& L) { return align_up(2 * (size_t)(L.rows * L.kst), 1024); }
+size_t fp_bytes(const Layout& L, const FpPlan& f, bool is_b) {
+    return (is_b ? f.planes_b : 1) * fp_plane_bytes(L) + (f.form ? align_up(4 * (size_t)(L.nkb * L.rs), 1024) : 0);
+}
+FpOperand fp_operand(const Layout& L, const FpPlan& f, bool is_b, char* at) {
+    FpOperand o{};
+    const int planes = is_b ? f.planes_b : 1;
+    o.p0 = at;
+    o.p1 = planes > 1 ? at + fp_plane_bytes(L) : nullptr;
+    o.scales = f.form ? reinterpret_cast<float*>(at + planes * fp_plane_bytes(L)) : nullptr;
+    o.rows = L.rows;
+    o.kst = L.kst;
+    o.rs = L.rs;
+    return o;
+}
 
 int check_operand(const hbfp_operand* o) {
     if (!o || o->struct_size != sizeof(hbfp_operand)) return HBFP_ERR_INVALID_ARG;
@@ -60,8 +79,13 @@ int make_plan(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     g->off_be = off; if (b->kind == HBFP_OPERAND_FP32) off += align_up((size_t)g->lb.exp_bytes, 1024);
     g->tp = plan_gemm_tensor(M, N, K, g->la, g->lb, a->fmt.mant_bits, b->fmt.mant_bits);
     g->off_partial = off;
-    off += align_up(g->tp.partial_bytes, 1024);
-    g->total = off;
+    g->total = off + align_up(g->tp.partial_bytes, 1024);
+    g->fp = plan_gemm_fp(M, N, g->la, g->lb);
+    g->off_fa = off;
+    if (g->fp.use) off += fp_bytes(g->la, g->fp, false);
+    g->off_fb = off;
+    if (g->fp.use) off += fp_bytes(g->lb, g->fp, true);
+    g->total_fp = off;
     return HBFP_OK;
 }
 
@@ -123,6 +147,9 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         if (!workspace || ws_bytes < g.total) return HBFP_ERR_WORKSPACE;
         if (reinterpret_cast<uintptr_t>(workspace) & 255) return HBFP_ERR_ALIGNMENT;
     }
+    // A caller whose workspace holds the packed operands only (hbfp_gemm_static) gets the integer kernels.
+    const bool use_fp = g.fp.use && !P && workspace && ws_bytes >= g.total_fp && (reinterpret_cast<uintptr_t>(workspace) & 255) == 0 &&
+                        (flags == HBFP_GEMM_AUTO || flags == HBFP_GEMM_FORCE_TENSOR) && (reinterpret_cast<uintptr_t>(C) & 3) == 0;
     char* ws = static_cast<char*>(workspace);
     Packed pa, pb;
     rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, st);
@@ -136,6 +163,15 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         return launch_gemm_small(M, N, pa, pb, C, ldc, st);
     }
     if (flags == HBFP_GEMM_FORCE_SMALL) return HBFP_ERR_UNSUPPORTED;
+    if (use_fp) {
+        const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
+        rc = launch_expand(pa, g.fp, false, fa, st);
+        if (rc) return rc;
+        rc = launch_expand(pb, g.fp, true, fb, st);
+        if (rc) return rc;
+        t_last_gemm_kernel = "gemm_tc_kernel";      // one SM per tile, like its integer sibling
+        return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, C, ldc, st);
+    }
     const bool quad_rows = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (ldc % 4) == 0;
     const bool want_tensor = flags != HBFP_GEMM_FORCE_SIMT && g.tp.supported &&
                              (reinterpret_cast<uintptr_t>(C) & 3) == 0;
@@ -159,6 +195,19 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
 }
 
 }  // namespace
+
+int gemm_least_workspace(int transA, int transB, int64_t M, int64_t N, int64_t K, const hbfp_format* fmtA, const hbfp_format* fmtB, size_t* bytes) {
+    if (!fmtA || !fmtB) return HBFP_ERR_INVALID_ARG;
+    hbfp_operand a, b;
+    fill_operand(&a, nullptr, 0, transA, fmtA);
+    fill_operand(&b, nullptr, 0, transB, fmtB);
+    GemmPlan g;
+    int rc = make_plan(M, N, K, &a, &b, &g);
+    if (rc) return rc;
+    *bytes = g.total;
+    return HBFP_OK;
+}
+
 }  // namespace hbfp
 
 using namespace hbfp;
@@ -384,7 +433,7 @@ int hbfp_gemm_q_workspace(int64_t M, int64_t N, int64_t K, const hbfp_operand* a
     GemmPlan g;
     int rc = make_plan(M, N, K, a, b, &g);
     if (rc) return rc;
-    *bytes = g.total;
+    *bytes = g.total_fp > g.total ? g.total_fp : g.total;
     return HBFP_OK;
 }
 

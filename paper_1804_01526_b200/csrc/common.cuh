@@ -96,6 +96,10 @@ int launch_gemm_simt(int64_t M, int64_t N, int64_t K, const Packed& a, const Pac
 bool small_gemm_eligible(int64_t M, int64_t N, const Packed& a, const Packed& b, bool any_size);
 int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, float* C, int64_t ldc, cudaStream_t st);
 
+// Workspace of the integer kernels alone (hbfp_gemm_workspace may ask for more).
+int gemm_least_workspace(int transA, int transB, int64_t M, int64_t N, int64_t K, const hbfp_format* fmtA,
+                         const hbfp_format* fmtB, size_t* bytes);
+
 struct TensorPlan {
     int supported;      // 0: this case has no tensor-core kernel
     int n_tile;         // 64, 128 or 256
@@ -114,6 +118,22 @@ int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const P
 bool pair_gemm_eligible(int64_t M, int64_t N, const Packed& a, const Packed& b, const TensorPlan& plan);
 int launch_gemm_tensor_pair(int64_t M, int64_t N, const Packed& a, const Packed& b, float* C, int64_t ldc,
                             const TensorPlan& plan, void* partial, cudaStream_t st);
+
+// Floating-point operand forms (gemm_fp.cu): short blocks of 8-bit mantissas, and 9 to 12 bits.
+struct FpOperand {          // device buffers, rows x kst elements of two bytes
+    void* p0;               // form S: bfloat16 q * 2^s; form W: binary16 q (A) or its upper part (B)
+    void* p1;               // form W, B: binary16 lower part
+    float* scales;          // form W: 2^s [nkb][rs]
+    int64_t rows, kst, rs;
+};
+struct FpPlan {
+    int use;                // 0: the integer kernels
+    int form, pair, ncol, splits, kb_per_split, planes_b;
+};
+FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb);
+int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const FpOperand& out, cudaStream_t st);
+int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, float* C,
+                   int64_t ldc, cudaStream_t st);
 
 // Convolution forward as an implicit GEMM over the packed pixels (gemm_conv.cu).
 int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw,

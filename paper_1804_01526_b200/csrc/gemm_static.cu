@@ -41,7 +41,8 @@ extern "C" int hbfp_gemm_static(int transA, int transB, int64_t M, int64_t N, in
                                 int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc,
                                 const hbfp_format* fmtA, const hbfp_format* fmtB, uint32_t flags, void* stream) {
     size_t need = 0;
-    int rc = hbfp_gemm_workspace(transA, transB, M, N, K, fmtA, fmtB, &need);
+    // what the kernels that need least ask for; hbfp_gemm takes the faster ones where the array holds their scratch too
+    int rc = hbfp::gemm_least_workspace(transA, transB, M, N, K, fmtA, fmtB, &need);
     if (rc) return rc;
     if (need > (size_t)HBFP_STATIC_WORKSPACE_BYTES) return HBFP_ERR_STATIC_LIMIT;
     void* ws = nullptr;

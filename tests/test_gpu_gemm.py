@@ -406,3 +406,37 @@ def test_last_gemm_cycles_reports_the_paired_kernel_length(hb):
     assert 32 * 4 * 300 < cycles < 32 * 4 * 20000
     assert 500 < mhz < 2200
     assert hb.device_status() == 0
+
+
+# The floating-point operand forms (gemm_fp.cu): short blocks of 8-bit mantissas, 9 to 12 bits; one SM or a pair per tile.
+# Edges of tiles in M and N, a last K stage with a single block, padded blocks, an output pitch that TMA cannot store.
+FP_FORM_CASES = [
+    # m, block, M, N, K, law
+    (8, 32, 2304, 2176, 1760, "lognormal"),
+    (8, 24, 2305, 2051, 1751, "lognormal"),
+    (8, 64, 2304, 2310, 1664, "normal"),
+    (6, 48, 2433, 2177, 1700, "lognormal"),
+    (12, 32, 2176, 2050, 1888, "outliers"),
+    (12, 64, 2433, 2303, 1600, "lognormal"),
+    (10, 40, 2177, 2052, 1990, "normal"),
+]
+
+
+@pytest.mark.parametrize("m,b,M,N,K,law", FP_FORM_CASES)
+def test_floating_point_operand_forms_are_bit_equal_to_the_sequential_definition(hb, m, b, M, N, K, law):
+    """Block sums are exact in every form and blocks are added in ascending order with one rounding each, so without
+    split-K the result is the reference kernel's (gemm_simt, itself bit-equal to the oracle's c_seq) bit for bit;
+    the largest mantissas everywhere give the largest block sums."""
+    import torch
+    fa, fb = hb.Format(m, b, rounding=1, seed=3), hb.Format(m, b, rounding=1, seed=3, stream_id=1)
+    A, B = to_dev(wl.draw(law, (M, K), seed=91)), to_dev(wl.draw(law, (K, N), seed=92))
+    for X, Y in ((A, B), (torch.full_like(A, 1.999), torch.full_like(B, -1.999))):
+        pa, pb = hb.quantize(X, 1, fa), hb.quantize(Y, 0, fb)
+        want = hb.gemm_q(M, N, K, pa, pb, flags=hb.GEMM_FORCE_SIMT)
+        buf = torch.full((M, N + 3), 7.0, device="cuda")
+        for out in (None, buf[:, 1:1 + N]):
+            got = hb.gemm(0, 0, X, Y, fa, fb, out=out)
+            assert hb.last_gemm_kernel() == "gemm_tc_kernel" and hb.device_status() == 0
+            assert torch.equal(got, want)
+            assert torch.equal(hb.gemm_q(M, N, K, pa, pb, out=out), want)
+        assert bool((buf[:, 0] == 7).all()) and bool((buf[:, N + 1:] == 7).all())
