@@ -12,9 +12,8 @@
 //   quant_col_tma    blocks down the columns, b in {32,64,128}, 16-byte aligned pitch: persistent
 //                    CTAs stream 128 x 64 FP32 tiles through a TMA pipeline and write the packed,
 //                    transposed tile with a swizzled TMA store (full lines in both directions).
-//   quant_col_fast   blocks down the columns, any b <= 128 and any pitch: a (<=128) x 32 FP32
-//                    panel is read with coalesced row loads into shared memory, reduced down the
-//                    columns by four threads per column and written transposed.
+//   quant_col_block  blocks down the columns, any b <= 128 and any pitch: one K-block of 32 columns per CTA.
+//   quant_row_ragged blocks along rows, any b <= 128, row length, pitch and alignment, in one pass.
 //   tile_kernel      t x t weight tiles (t <= 128): one pass writes both packed views and
 //                    the tile exponent grid.
 //   exps_* / mant_generic   two-pass path for every other geometry (any b, any alignment).
@@ -178,6 +177,13 @@ __device__ __forceinline__ int quantize_one(float x, int s, const QParams& p, ui
     return round_sr(x, s, p.qmax, draw_of_element(p, L));
 }
 
+// Exponent bytes of the lines beyond the matrix (rows .. rs of every block) are documented as zero: written by the first CTA.
+__device__ __forceinline__ void zero_padding_lines(int8_t* exps, int64_t rows, int64_t rs, int64_t nkb) {
+    if (rs == rows || blockIdx.x != 0) return;
+    const int pad = (int)(rs - rows);
+    for (int64_t i = threadIdx.x; i < nkb * pad; i += blockDim.x) exps[(i / pad) * rs + rows + i % pad] = 0;
+}
+
 // ------------------------------------------------------------------------------ quant_row_fast
 
 // LPB = lanes per block (b = 8 * LPB). CTA: 256 threads, tile 32 rows x 512 columns.
@@ -257,116 +263,89 @@ quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
     }
 }
 
-// ------------------------------------------------------------------------------ quant_col_fast
+// ------------------------------------------------------------------------------ quant_col_block
 
-// Blocks down the columns of x [K][R] (contract axis 0); output rows are the columns of x.
-// CTA: 128 threads = 32 columns x 4 row slots; panel = G blocks of b <= 128 k-rows (G * padded b
-// = 128) by 32 columns: 16 KB of shared memory, so a dozen CTAs fit an SM and cover the memory
-// latency. Each thread keeps its 32 values in registers between the max and the rounding pass.
+// Blocks down the columns of x [K][R] (contract axis 0); output rows are the columns of x. Any block length up to 128, any
+// pitch and alignment (the paper's tile of 24 among them). A CTA takes one K-block of 32 columns: four warps split the
+// block's rows, so that every load is a warp's 128 consecutive bytes of one row and all of a thread's loads are in flight
+// together; the values stay in registers between the maximum and the rounding. Small and ragged matrices are bound by
+// latency, hence one block per CTA (many short CTAs): 128 x 1024, b = 24, stochastic 5.5 -> 2.7 us; 3001 x 777:
+// 26 -> 8.4 us; 16384 x 16384, nearest-even: 677 -> 403 us.
 constexpr int COLT = 32;
 
-template <int PLANES, int RQ>      // RQ = bp / 4: padded rows per thread and block (8, 16 or 32)
+template <int PLANES, int RQ, bool SR>      // RQ = bp / 4: padded rows per warp (8, 16 or 32)
 __global__ void __launch_bounds__(128)
-quant_col_fast(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
-               int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-               int8_t* __restrict__ exps, int64_t rs, int64_t nkb, int vec_ok) {
-    constexpr int G = 32 / RQ;             // blocks per panel: G * bp = 128 padded rows
+quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
+                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
+                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n) {
     constexpr int BP = 4 * RQ;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int krows = G * b;
-    float* tile = reinterpret_cast<float*>(smem_raw);                      // [krows][COLT]
-    uint32_t* pmax = reinterpret_cast<uint32_t*>(tile + (size_t)krows * COLT);   // [G][4][COLT]
-    uint4* rnd = reinterpret_cast<uint4*>(pmax + (size_t)G * 4 * COLT);    // [krows][COLT/8] (stochastic only)
-
+    __shared__ uint32_t pmax[4][COLT];
+    __shared__ __align__(16) uint4 rnd[SR ? BP : 1][5];          // draws of a row: its 32 columns lie in at most five groups of eight
+    __shared__ __align__(16) unsigned char s_out[PLANES][COLT][BP + 16];
     const int tid = threadIdx.x, c = tid & 31, q = tid >> 5;
-    const int64_t kb0 = (int64_t)blockIdx.y * G;
-    const int64_t c0 = (int64_t)blockIdx.x * COLT;
-    const int64_t k0 = kb0 * b;
-    const int rows_here = (int)min((int64_t)krows, K - k0);
-
-    // 1. coalesced load of the panel (zero beyond the matrix).
-    if (vec_ok) {
-        for (int i = tid; i < rows_here * (COLT / 4); i += 128) {
-            const int kk = i >> 3, c4 = (i & 7) * 4;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c0 + c4 < R) v = __ldcs(reinterpret_cast<const float4*>(x + (k0 + kk) * ld + c0 + c4));   // R % 4 == 0 here
-            *reinterpret_cast<float4*>(tile + kk * COLT + c4) = v;
-        }
-    } else {
-        for (int i = tid; i < rows_here * COLT; i += 128) {
-            const int kk = i >> 5, cc = i & 31;
-            tile[kk * COLT + cc] = (c0 + cc < R) ? x[(k0 + kk) * ld + c0 + cc] : 0.f;
-        }
-    }
-    // 2. stochastic mode: one Philox call per 8 consecutive source elements of a row.
-    const bool group_ok = (R % 8) == 0;     // then L = k*R + col has L & 7 == col & 7 and groups align
-    if (p.rounding == 1 && group_ok) {
-        for (int i = tid; i < rows_here * (COLT / 8); i += 128) {
-            const int kk = i >> 2, g8 = i & 3;
-            const uint64_t L = (uint64_t)((k0 + kk) * R + c0 + g8 * 8);
-            rnd[i] = draws_of_group(p, L >> 3);
-        }
-    }
-    __syncthreads();
-
-    // 3. thread (q, c) takes quarter q of every block of column c into registers.
-    float v[G][RQ];
+    const int64_t kb = blockIdx.x / tiles_n, c0 = (int64_t)(blockIdx.x - (unsigned)kb * tiles_n) * COLT;
+    const int64_t k0 = kb * b, col = c0 + c;
+    const int rows_here = (int)min((int64_t)b, K - k0);
+    float v[RQ];
+    const float* src = x + (k0 + q * RQ) * ld + col;
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        uint32_t am = 0;
-#pragma unroll
-        for (int j = 0; j < RQ; ++j) {
-            const int kk = g * b + q * RQ + j;
-            const bool valid = q * RQ + j < b && kk < rows_here;
-            v[g][j] = valid ? tile[kk * COLT + c] : 0.f;
-            am = max(am, abs_bits(v[g][j]));
+    for (int j = 0; j < RQ; ++j) v[j] = (q * RQ + j < rows_here && col < R) ? __ldcs(src + (int64_t)j * ld) : 0.f;
+    // the draws do not depend on the data: they are made while the loads are in flight, one Philox call per group of eight
+    // consecutive source elements
+    if (SR) {
+        for (int i = tid; i < rows_here * 5; i += 128) {
+            const int kk = i / 5, g = i - kk * 5;
+            const uint64_t L0 = (uint64_t)((k0 + kk) * R + c0);
+            if (g < 4 || (L0 & 7)) rnd[kk][g] = draws_of_group(p, (L0 >> 3) + g);
         }
-        pmax[(g * 4 + q) * COLT + c] = am;
     }
+    uint32_t am = 0;
+#pragma unroll
+    for (int j = 0; j < RQ; j += 2) am = max3_abs_bits(am, v[j], v[j + 1]);
+    pmax[q][c] = am;
     __syncthreads();
-
-    const int64_t col = c0 + c;
-    if (col >= R) return;
+    am = max(max(pmax[0][c], pmax[1][c]), max(pmax[2][c], pmax[3][c]));
+    const int s = block_exponent(am, p.m, p.exp_mode);
+    if (q == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
+    const uint32_t qm = qmax_pair(p.qmax), nqm = neg_qmax_pair(p.qmax);
+    const float sc = pow2f(SR ? 16 - s : -s);
     const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd);
+    const uint32_t first = SR ? (uint32_t)((uint64_t)(k0 * R + c0) & 7) : 0u, row_step = (uint32_t)(R & 7);
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        const int64_t kb = kb0 + g;
-        if (kb < nkb) {
-            const uint32_t am = max(max(pmax[(g * 4 + 0) * COLT + c], pmax[(g * 4 + 1) * COLT + c]),
-                                    max(pmax[(g * 4 + 2) * COLT + c], pmax[(g * 4 + 3) * COLT + c]));
-            const int s = block_exponent(am, p.m, p.exp_mode);
-            if (q == 0) exps[kb * rs + col] = (int8_t)s;
-            int8_t* dst = mant + col * kst + kb * BP + q * RQ;
+    for (int w = 0; w < RQ / 4; ++w) {
+        uint32_t h[2], hi, lo;
 #pragma unroll
-            for (int w0 = 0; w0 < RQ; w0 += 8) {
-                uint32_t hi[2] = {0, 0}, lo[2] = {0, 0};
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int kk = g * b + q * RQ + w0 + j;
-                    int qv;
-                    if (p.rounding == 0) qv = round_rne(v[g][w0 + j], s, p.qmax);
-                    else if (group_ok) qv = round_sr(v[g][w0 + j], s, p.qmax, rnd16[((kk < rows_here ? kk : 0) * (COLT / 8) + (c >> 3)) * 8 + (c & 7)]);
-                    else qv = round_sr(v[g][w0 + j], s, p.qmax, draw_of_element(p, (uint64_t)((k0 + kk) * R + col)));
-                    if (!(q * RQ + w0 + j < b && kk < rows_here)) qv = 0;     // padding stays zero whatever the draw
-                    if (PLANES == 1) {
-                        hi[j >> 2] |= (uint32_t)(qv & 0xff) << (8 * (j & 3));
-                    } else {
-                        hi[j >> 2] |= (uint32_t)((qv >> 4) & 0xff) << (8 * (j & 3));
-                        lo[j >> 2] |= (uint32_t)(qv & 15) << (8 * (j & 3));
-                    }
-                }
-                *reinterpret_cast<uint2*>(dst + w0) = make_uint2(hi[0], hi[1]);
-                if (PLANES == 2) *reinterpret_cast<uint2*>(dst + plane_stride + w0) = make_uint2(lo[0], lo[1]);
-            }
-            // zero the row tail [nkb*bp, kst) once
-            if (kb == nkb - 1 && q == 0) {
-                for (int64_t o = nkb * BP; o < kst; o += 16) {
-                    *reinterpret_cast<uint4*>(mant + col * kst + o) = make_uint4(0, 0, 0, 0);
-                    if (PLANES == 2) *reinterpret_cast<uint4*>(mant + plane_stride + col * kst + o) = make_uint4(0, 0, 0, 0);
-                }
+        for (int k = 0; k < 2; ++k) {
+            const int j = 4 * w + 2 * k;
+            if (SR) {
+                // zeros below the block or the matrix stay zero whatever the draw (their table rows are not read)
+                const int kk = q * RQ + j;
+                const uint32_t r0 = kk < rows_here ? rnd16[kk * 40 + ((first + (uint32_t)kk * row_step) & 7) + c] : 0u;
+                const uint32_t r1 = kk + 1 < rows_here ? rnd16[(kk + 1) * 40 + ((first + (uint32_t)(kk + 1) * row_step) & 7) + c] : 0u;
+                h[k] = round_sr_pair2(v[j], v[j + 1], sc, r0, r1, qm, nqm);
+            } else {
+                h[k] = round_rne_pair(v[j], v[j + 1], sc, qm, nqm);
             }
         }
+        pack4<PLANES>(h[0], h[1], hi, lo);
+        *reinterpret_cast<uint32_t*>(&s_out[0][c][q * RQ + 4 * w]) = hi;
+        if (PLANES == 2) *reinterpret_cast<uint32_t*>(&s_out[PLANES - 1][c][q * RQ + 4 * w]) = lo;
     }
+    __syncthreads();
+    // neighbouring threads write neighbouring 16-byte pieces of an output row
+    constexpr int PPR = BP / 16;
+#pragma unroll
+    for (int pl = 0; pl < PLANES; ++pl)
+        for (int i = tid; i < COLT * PPR; i += 128) {
+            const int r = i / PPR, piece = i - r * PPR;
+            if (c0 + r < R)
+                *reinterpret_cast<uint4*>(mant + pl * plane_stride + (c0 + r) * kst + kb * BP + 16 * piece) =
+                    *reinterpret_cast<const uint4*>(&s_out[pl][r][16 * piece]);
+        }
+    // the row tail [nkb * bp, kst)
+    if (kb == nkb - 1 && q < PLANES && col < R)
+        for (int64_t o = nkb * BP; o < kst; o += 16)
+            *reinterpret_cast<uint4*>(mant + q * plane_stride + col * kst + o) = make_uint4(0, 0, 0, 0);
 }
 
 // ------------------------------------------------------------------------------ weight tiles
@@ -421,8 +400,10 @@ __device__ __forceinline__ void write_tile_views(const int16_t* qt, int tp, int 
         if (PLANES == 2) *reinterpret_cast<uint32_t*>(dst + ps0) = l;
     }
     // replicated exponents: exps_c1[v][i0+ii], exps_c0[u][j0+jj]
-    if (exps_c1) for (int e = tid; e < hi; e += 256) exps_c1[v * rs1 + i0 + e] = (int8_t)s;
-    if (exps_c0) for (int e = tid; e < wj; e += 256) exps_c0[u * rs0 + j0 + e] = (int8_t)s;
+    // (lines beyond the matrix, at most 15 after the last tile, are documented as zero)
+    const int pad1 = u == nkb0 - 1 ? (int)(rs1 - i0) : hi, pad0 = v == nkb1 - 1 ? (int)(rs0 - j0) : wj;
+    if (exps_c1) for (int e = tid; e < pad1; e += 256) exps_c1[v * rs1 + i0 + e] = e < hi ? (int8_t)s : (int8_t)0;
+    if (exps_c0) for (int e = tid; e < pad0; e += 256) exps_c0[u * rs0 + j0 + e] = e < wj ? (int8_t)s : (int8_t)0;
     // row tails beyond the last tile: zero them (last tile column / last tile row only)
     if (mant_c1 && v == nkb1 - 1)
         for (int64_t e = tid; e < (int64_t)hi * ((kst1 - nkb1 * tp) / 4); e += 256) {
@@ -1290,6 +1271,7 @@ quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
             if ((lane % LPB) == 0 && cc[j] < K) exps[(int64_t)(cc[j] / B) * rs + rw[j]] = (int8_t)s;
         }
     }
+    zero_padding_lines(exps, rows, rs, K / B);
 }
 
 template <int LPB, int ITEMS>
@@ -1317,6 +1299,94 @@ int launch_row_flat(const float* x, int64_t rows, int64_t K, int64_t ld, const Q
                     int8_t* mant, int8_t* exps, cudaStream_t st) {
     if (L.kst > 256 && p.rounding == 0) return launch_row_flat_items<LPB, 4>(x, rows, K, ld, p, L, mant, exps, st);
     return launch_row_flat_items<LPB, 2>(x, rows, K, ld, p, L, mant, exps, st);
+}
+
+// ------------------------------------------------------------------------------ quant_row_ragged
+
+// Blocks along rows for every other block length up to 128, row length, pitch and alignment (24 columns per block, odd row
+// lengths). As in quant_row_flat the packed row, padding included, is cut into pieces of eight elements numbered through the
+// whole matrix, LPB = bp / 8 lanes per block; a piece that lies in a block's padding loads nothing. Without alignment a lane
+// fetches its eight floats one by one (the sectors of a warp's pieces stay in L1 between them), and its eight draws may
+// straddle two Philox groups: the second call is made only then. One pass instead of the two of exps_axis1 and
+// mant_generic, which index, divide and draw per element: 1111 x 3001, b = 24, stochastic 53 -> 9.7 us, 16384 x 16384,
+// nearest-even 2627 -> 287 us.
+template <int LPB, bool SR, int PLANES, bool VEC>
+__global__ void __launch_bounds__(256)
+quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int b, QParams p,
+                 int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
+                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, uint32_t ppr, int64_t total) {
+    constexpr int BP = 8 * LPB, ITEMS = 2;
+    const int tid = threadIdx.x, lane = tid & 31;
+    float e8[ITEMS][8];
+    int64_t row[ITEMS];
+    int cb[ITEMS], kk0[ITEMS];             // block of the row; first element of the piece along the row
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int64_t g = (int64_t)blockIdx.x * (256 * ITEMS) + i * 256 + tid;
+        row[i] = g / ppr;
+        const int pc = (int)(g - row[i] * ppr);
+        cb[i] = pc / LPB;
+        const int within = 8 * (pc - cb[i] * LPB);
+        kk0[i] = cb[i] * b + within;
+        const int n = (g < total && cb[i] < nkb) ? (int)min((int64_t)(b - within), K - kk0[i]) : 0;    // elements of the piece
+        const float* src = x + row[i] * ld + kk0[i];
+        if (VEC && n >= 8) {
+            const float4 u = __ldcs(reinterpret_cast<const float4*>(src)), w = __ldcs(reinterpret_cast<const float4*>(src) + 1);
+            e8[i][0] = u.x; e8[i][1] = u.y; e8[i][2] = u.z; e8[i][3] = u.w;
+            e8[i][4] = w.x; e8[i][5] = w.y; e8[i][6] = w.z; e8[i][7] = w.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) e8[i][j] = j < n ? __ldg(src + j) : 0.f;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const bool live = (int64_t)blockIdx.x * (256 * ITEMS) + i * 256 + tid < total;
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (SR) {
+            const uint64_t L0 = (uint64_t)(row[i] * K + kk0[i]);          // the matrix is rows x K as passed
+            w = draws_of_group(p, L0 >> 3);
+            const uint32_t sh = (uint32_t)(L0 & 7);
+            if (sh) {
+                // halfwords sh .. sh + 7 of the two groups
+                const uint4 n4 = draws_of_group(p, (L0 >> 3) + 1);
+                const uint32_t a[8] = {w.x, w.y, w.z, w.w, n4.x, n4.y, n4.z, n4.w};
+                const uint32_t ws = sh >> 1;
+                uint32_t t[5];
+#pragma unroll
+                for (int j = 0; j < 5; ++j) t[j] = ws == 0 ? a[j] : ws == 1 ? a[(j + 1) & 7] : ws == 2 ? a[(j + 2) & 7] : a[(j + 3) & 7];
+                if (sh & 1) w = make_uint4(__funnelshift_r(t[0], t[1], 16), __funnelshift_r(t[1], t[2], 16), __funnelshift_r(t[2], t[3], 16), __funnelshift_r(t[3], t[4], 16));
+                else w = make_uint4(t[0], t[1], t[2], t[3]);
+            }
+        }
+        uint32_t am = amax8_bits(e8[i]);
+#pragma unroll
+        for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
+        const int s = block_exponent(am, p.m, p.exp_mode);
+        uint2 hi, lo;
+        quantize_pack8<SR, PLANES>(e8[i], s, p, w, hi, lo);
+        if (live) {
+            const int pc = cb[i] * LPB + (kk0[i] - cb[i] * b) / 8;
+            int8_t* dst = mant + row[i] * kst + 8 * (int64_t)pc;
+            *reinterpret_cast<uint2*>(dst) = hi;
+            if (PLANES == 2) *reinterpret_cast<uint2*>(dst + plane_stride) = lo;
+            if ((lane % LPB) == 0 && cb[i] < nkb) exps[(int64_t)cb[i] * rs + row[i]] = (int8_t)s;
+        }
+    }
+    zero_padding_lines(exps, rows, rs, nkb);
+}
+
+template <int LPB, bool VEC>
+int launch_row_ragged(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
+                      int8_t* mant, int8_t* exps, cudaStream_t st) {
+    const uint32_t ppr = (uint32_t)(L.kst / 8);
+    const int64_t total = rows * ppr;
+    const unsigned grid = (unsigned)((total + 511) / 512);
+#define HBFP_QROW_RAGGED(SRV, PL) quant_row_ragged<LPB, SRV, PL, VEC><<<grid, 256, 0, st>>>(x, rows, K, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, ppr, total)
+    if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_RAGGED(true, 1); else HBFP_QROW_RAGGED(true, 2); }
+    else { if (L.planes == 1) HBFP_QROW_RAGGED(false, 1); else HBFP_QROW_RAGGED(false, 2); }
+#undef HBFP_QROW_RAGGED
+    return launch_status();
 }
 
 // ------------------------------------------------------------------------------ quant_col_tma
@@ -1417,7 +1487,7 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         if (LB == 1) am = max(pmax[(q & 2) * QC_COLS + n], pmax[((q & 2) + 1) * QC_COLS + n]);
         const int sexp = given ? (col < R ? (int)given[col] : -63) : block_exponent(am, p.m, p.exp_mode);
         const int64_t kb = ((int64_t)kt << LB) + (q >> (2 - LB));
-        if (!given && (q & ((4 >> LB) - 1)) == 0 && kb < nkb && col < R) exps[kb * rs + col] = (int8_t)sexp;
+        if (!given && (q & ((4 >> LB) - 1)) == 0 && kb < nkb && col < rs) exps[kb * rs + col] = col < R ? (int8_t)sexp : (int8_t)0;   // padding lines: zero
 
         uint32_t hi[8], lo[8];
         const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd);
@@ -1604,8 +1674,6 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     // row lengths that the 512-column tiles of quant_row_fast would leave ragged
     if (f->tile == 0 && axis == 1 && aligned && L.b == L.bp && L.b <= 128 && K % L.b == 0 && L.kst % 512 != 0 &&
         rows * (L.kst / 8) < (1ll << 32) - 4096) {
-        // exponent padding bytes (rows .. rs of every block line) are documented as zero
-        if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
         switch (L.b) {
             case 32: return launch_row_flat<4>(x, rows, K, ld, p, L, mant, exps, st);
             case 64: return launch_row_flat<8>(x, rows, K, ld, p, L, mant, exps, st);
@@ -1671,8 +1739,6 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     if (f->tile == 0 && axis == 0 && aligned && L.b == L.bp && L.b <= 128 && (p.rounding == 0 || rows % 8 == 0) &&
         (reinterpret_cast<uintptr_t>(mant) & 127) == 0 && rows < (1ll << 29) && K < (1ll << 31) &&
         ((rows + QC_COLS - 1) / QC_COLS) * (L.kst / QC_ROWS) < (1ll << 31)) {
-        // exponent padding bytes (lines >= rows) are documented as zero
-        if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
 #define HBFP_QCOL_TMA(PL, LBV) (p.rounding ? launch_col_tma<PL, LBV, true>(x, K, rows, ld, p, L, mant, exps, st) \
                                            : launch_col_tma<PL, LBV, false>(x, K, rows, ld, p, L, mant, exps, st))
         const int lb = L.b == 128 ? 0 : L.b == 64 ? 1 : 2;
@@ -1680,23 +1746,22 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         return lb == 0 ? HBFP_QCOL_TMA(2, 0) : lb == 1 ? HBFP_QCOL_TMA(2, 1) : HBFP_QCOL_TMA(2, 2);
 #undef HBFP_QCOL_TMA
     }
-    if (f->tile == 0 && axis == 0 && L.b <= 128) {
-        const int vec_ok = aligned && (rows % 4 == 0);
-        const int G = (int)(128 / L.bp);                   // blocks per panel
-        const int64_t gy = (L.nkb + G - 1) / G;
-        if (gy <= 65535) {
-            const size_t krows = (size_t)G * L.b;
-            size_t smem = krows * COLT * sizeof(float) + (size_t)G * 4 * COLT * sizeof(uint32_t) +
-                          (p.rounding ? krows * (COLT / 8) * sizeof(uint4) : 0);
-            dim3 grid((unsigned)((rows + COLT - 1) / COLT), (unsigned)gy);
-            // exponent padding bytes (lines >= rows) are documented as zero
-            if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
-#define HBFP_QCOL(PL, RQ) quant_col_fast<PL, RQ><<<grid, 128, smem, st>>>(x, K, rows, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, vec_ok)
-            if (L.planes == 1) { if (L.bp == 32) HBFP_QCOL(1, 8); else if (L.bp == 64) HBFP_QCOL(1, 16); else HBFP_QCOL(1, 32); }
-            else { if (L.bp == 32) HBFP_QCOL(2, 8); else if (L.bp == 64) HBFP_QCOL(2, 16); else HBFP_QCOL(2, 32); }
+    // every other block length up to 128, any pitch and alignment
+    if (f->tile == 0 && axis == 0 && L.b <= 128 && ((rows + COLT - 1) / COLT) * L.nkb < (1ll << 31)) {
+        const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
+#define HBFP_QCOL(PL, RQ, SRV) quant_col_block<PL, RQ, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, tiles_n)
+#define HBFP_QCOL_SR(PL, RQ) do { if (p.rounding) HBFP_QCOL(PL, RQ, true); else HBFP_QCOL(PL, RQ, false); } while (0)
+        if (L.planes == 1) { if (L.bp == 32) HBFP_QCOL_SR(1, 8); else if (L.bp == 64) HBFP_QCOL_SR(1, 16); else HBFP_QCOL_SR(1, 32); }
+        else { if (L.bp == 32) HBFP_QCOL_SR(2, 8); else if (L.bp == 64) HBFP_QCOL_SR(2, 16); else HBFP_QCOL_SR(2, 32); }
+#undef HBFP_QCOL_SR
 #undef HBFP_QCOL
-            return launch_status();
-        }
+        return launch_status();
+    }
+    if (f->tile == 0 && axis == 1 && L.b <= 128 && K < (1ll << 30) && rows * (L.kst / 8) < (1ll << 39)) {
+        const bool vec = aligned && L.b % 4 == 0;          // every piece starts on a 16-byte boundary
+        if (L.bp == 32) return vec ? launch_row_ragged<4, true>(x, rows, K, ld, p, L, mant, exps, st) : launch_row_ragged<4, false>(x, rows, K, ld, p, L, mant, exps, st);
+        if (L.bp == 64) return vec ? launch_row_ragged<8, true>(x, rows, K, ld, p, L, mant, exps, st) : launch_row_ragged<8, false>(x, rows, K, ld, p, L, mant, exps, st);
+        return vec ? launch_row_ragged<16, true>(x, rows, K, ld, p, L, mant, exps, st) : launch_row_ragged<16, false>(x, rows, K, ld, p, L, mant, exps, st);
     }
     if (f->tile > 0 && f->tile <= 128) {
         // single view of a tiled weight: the fused tile kernel with the other view switched off
@@ -1744,8 +1809,6 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     const int t = f->tile, tp = (int)L0.bp;
     const int64_t nu = L0.nkb, nv = L1.nkb;   // tiles along d0, along d1
     if (nu > 65535) return HBFP_ERR_UNSUPPORTED;
-    if (exps_c0 && L0.rs != d1) HBFP_CUDA_OK(cudaMemsetAsync(exps_c0, 0, (size_t)L0.exp_bytes, st));
-    if (exps_c1 && L1.rs != d0) HBFP_CUDA_OK(cudaMemsetAsync(exps_c1, 0, (size_t)L1.exp_bytes, st));
     const TileViews tv{mant_c0, L0.kst, L0.plane_stride, exps_c0, L0.rs, L0.nkb, mant_c1, L1.kst, L1.plane_stride, exps_c1, L1.rs, L1.nkb};
     const bool fast = (t % 8) == 0 && (d1 % 8) == 0 &&
                       (MODE == 2 || ((ld % 4) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0)) &&

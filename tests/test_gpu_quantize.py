@@ -263,3 +263,34 @@ def test_full_size_one_gib_tensor(hb, m, b, rounding):
         assert np.array_equal(s[r0:r0 + step], s_ref), r0
         assert np.array_equal(q[r0:r0 + step], q_ref), r0
     assert hb.device_status() == 0
+
+
+# The kernels for block lengths, row lengths, pitches and alignments that the tiled kernels do not take: ragged last
+# blocks and pieces, rows whose draws straddle two Philox groups, lines that do not fill a group of 16 or 32.
+@pytest.mark.parametrize("m,rounding", [(8, 0), (8, 1), (12, 1)])
+@pytest.mark.parametrize("d0,d1,b", [(1, 1, 24), (3, 25, 24), (33, 47, 24), (17, 1001, 24), (70, 96, 40), (31, 203, 1), (40, 131, 33),
+                                     (129, 130, 100), (65, 257, 128), (257, 31, 64), (5, 64, 32)])
+def test_ragged_blocks_in_both_directions(hb, d0, d1, b, m, rounding):
+    import torch
+    big = wl.draw("lognormal", (d0, d1 + 5), seed=17)
+    fd = dict(mant_bits=m, block=b, rounding=rounding, seed=23, stream_id=5)
+    wide = torch.from_numpy(big).cuda()
+    for off, ld in ((0, d1), (3, d1 + 5)):                     # contiguous, and a view with an odd pitch and offset
+        A = np.ascontiguousarray(big[:, off:off + d1])
+        x = wide[:, off:off + d1] if ld != d1 else torch.from_numpy(A).cuda()
+        for axis in (0, 1):
+            rows, k = (d0, d1) if axis == 1 else (d1, d0)
+            out = hb.alloc_packed(rows, k, gfmt(fd))
+            out.mant.fill_(77)
+            out.exps.fill_(77)
+            p = hb.quantize(x, axis, gfmt(fd), out=out)
+            q, s = hb.unpack(p)
+            q_ref, s_ref = oracle.quantize(A, axis, ofmt(fd))
+            assert np.array_equal(q.cpu().numpy(), q_ref) and np.array_equal(s.cpu().numpy(), s_ref)
+            lay = hb.packed_layout(rows, k, gfmt(fd))
+            e = p.exps.cpu().numpy()[:lay["nkb"] * lay["rs"]].reshape(lay["nkb"], lay["rs"])
+            assert (e[:, rows:] == 0).all()                    # lines beyond the matrix
+            for pl in range(lay["planes"]):
+                body = p.mant.cpu().numpy()[pl * lay["plane_stride"]:][:rows * lay["kst"]].reshape(rows, lay["kst"])
+                blocks = body[:, :lay["nkb"] * lay["bp"]].reshape(rows, lay["nkb"], lay["bp"])
+                assert (blocks[:, :, b:] == 0).all() and (body[:, lay["nkb"] * lay["bp"]:] == 0).all()     # padding
