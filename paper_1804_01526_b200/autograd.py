@@ -32,24 +32,17 @@ class _HbfpLinearFn(torch.autograd.Function):
     def forward(ctx, x, weight, bias, layer):
         ctx.layer = layer
         ctx.save_for_backward(x)
-        batch = x.shape[0]
-        y = hb.gemm_q(batch, layer.fout, layer.fin, x.contiguous(), layer.views[0], fmtA=layer.fmt_act(0))
-        return y + bias if bias is not None else y
+        return hb._got(hb.host().linear_forward(x.contiguous(), layer.views[0], layer.fmt_act(0), layer.fin, layer.fout, bias), "hbfp_gemm_q")
 
     @staticmethod
     def backward(ctx, dy):
         layer = ctx.layer
         (x,) = ctx.saved_tensors
-        dy = dy.contiguous()
-        batch = x.shape[0]
-        dx = dw = db = None
-        if ctx.needs_input_grad[0]:
-            dx = hb.gemm_q(batch, layer.fin, layer.fout, dy, layer.views[1], fmtA=layer.fmt_act(2))
-        if ctx.needs_input_grad[1]:
-            # contraction over the batch axis: 1-D blocks down the columns of X and dY
-            dw = hb.gemm(1, 0, x.contiguous(), dy, layer.fmt_act(0, batch_axis=True), layer.fmt_act(2, batch_axis=True))
-        if ctx.needs_input_grad[2]:
-            db = dy.sum(dim=0)
+        need_dx, need_dw, need_db, _ = ctx.needs_input_grad
+        # backward-data on the shared weight view, backward-weight with 1-D blocks down the columns of X and dY (the
+        # contraction over the batch axis), the bias gradient
+        dx, dw, db = hb._got(hb.host().linear_backward(dy.contiguous(), x.contiguous(), layer.views[1], layer.fmt_act(2), layer.fmt_act(0, batch_axis=True),
+                                                       layer.fmt_act(2, batch_axis=True), layer.fin, layer.fout, need_dx, need_dw, need_db), "hbfp_gemm_q")
         return dx, dw, db, None
 
 

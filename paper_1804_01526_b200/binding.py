@@ -1,4 +1,5 @@
-"""ctypes binding of ``libhbfp.so`` (the C ABI declared in ``include/hbfp.h``).
+"""Binding of ``libhbfp.so`` (the C ABI declared in ``include/hbfp.h``): ctypes, and for the calls of a
+training or serving loop the compiled ``_host`` (``csrc/host.cpp``).
 
 Argument marshalling only: every step of the path runs in the CUDA kernels of the library.
 PyTorch supplies device memory and the current stream. There is no fallback: if the shared
@@ -74,6 +75,7 @@ class Format:
 
 
 _lib = None
+_native = None
 
 
 def lib() -> ctypes.CDLL:
@@ -117,6 +119,32 @@ def lib() -> ctypes.CDLL:
                 getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
+
+
+# Entry points that _host calls, in the order it takes them (csrc/host.cpp, struct Api).
+_HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q", "hbfp_gemm_q_workspace", "hbfp_wide_update", "hbfp_wide_dequantize",
+                      "hbfp_conv_forward", "hbfp_conv_dgrad_filters", "hbfp_im2col_packed_t")
+
+
+def host():
+    """The compiled host side of this binding, bound to the library that ``lib()`` has loaded."""
+    global _native
+    if _native is None:
+        L = lib()
+        try:
+            from . import _host
+        except ImportError as e:
+            raise ImportError("_host.so is missing: build it with `python -m paper_1804_01526_b200.build` (there is no fallback path)") from e
+        _host.bind(*(ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in _HOST_ENTRY_POINTS))
+        _native = _host
+    return _native
+
+
+def _got(result, where: str):
+    """What a function of ``_host`` returned: its result, or the status code of the call that failed."""
+    if type(result) is int:
+        raise HbfpError(result, where)
+    return result
 
 
 def status_string(code: int) -> str:
@@ -182,15 +210,12 @@ def _ld(x: torch.Tensor) -> int:
 
 def quantize(x: torch.Tensor, contract_axis: int, fmt: Format, out: Optional[Packed] = None) -> Packed:
     """hbfp_quantize: blocks along ``contract_axis`` of the 2-D float32 CUDA tensor ``x``."""
-    _check_f32(x, "x")
+    m, e = _got((_native or host()).quantize(x, contract_axis, fmt, out.mant if out is not None else None, out.exps if out is not None else None), "hbfp_quantize")
+    if out is not None:
+        return out
     d0, d1 = x.shape
     rows, k = (d0, d1) if contract_axis == 1 else (d1, d0)
-    if out is None:
-        out = alloc_packed(rows, k, fmt, x.device)
-    cf = fmt.c()
-    _check(lib().hbfp_quantize(_dptr(x), d0, d1, _ld(x), contract_axis, ctypes.byref(cf), _dptr(out.mant),
-                               _dptr(out.exps), _stream()), "hbfp_quantize")
-    return out
+    return Packed(m, e, rows, k, fmt)
 
 
 def quantize_tiles(w: torch.Tensor, fmt: Format, out: Optional[Tuple[Packed, Packed]] = None,
@@ -250,14 +275,12 @@ def wide_update(wide: Wide, delta: torch.Tensor, fmt: Format, views: Optional[Tu
                 want_views: bool = True):
     """hbfp_wide_update: ``wide <- Q16(float32(wide + delta))`` in place; returns the narrow views."""
     _check_f32(delta, "delta")
-    d0, d1 = wide.mant.shape
-    if tuple(delta.shape) != (d0, d1):
+    if delta.shape != wide.mant.shape:
         raise ValueError("delta must have the shape of the weights")
     if views is None and want_views:
-        views = _alloc_views(d0, d1, fmt, delta.device)
-    f = fmt.c()
-    _check(lib().hbfp_wide_update(_dptr(wide.mant), _dptr(wide.exps), _dptr(delta), d0, d1, _ld(delta), ctypes.byref(f),
-                                  *_view_args(views), _stream()), "hbfp_wide_update")
+        views = _alloc_views(*wide.mant.shape, fmt, delta.device)
+    c0, c1 = views if views is not None else (None, None)
+    _check((_native or host()).wide_update(wide.mant, wide.exps, delta, fmt, c0, c1), "hbfp_wide_update")
     return views
 
 
@@ -274,13 +297,7 @@ def wide_narrow(wide: Wide, fmt: Format, views: Optional[Tuple[Packed, Packed]] 
 
 def wide_dequantize(wide: Wide, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """hbfp_wide_dequantize: the FP32 value ``mant * 2^exps`` of the wide copy (exact)."""
-    d0, d1 = wide.mant.shape
-    if out is None:
-        out = torch.empty((d0, d1), dtype=torch.float32, device=wide.mant.device)
-    _check_f32(out, "out")
-    _check(lib().hbfp_wide_dequantize(_dptr(wide.mant), _dptr(wide.exps), d0, d1, wide.tile, _dptr(out), _ld(out),
-                                      _stream()), "hbfp_wide_dequantize")
-    return out
+    return _got((_native or host()).wide_dequantize(wide.mant, wide.exps, wide.tile, out), "hbfp_wide_dequantize")
 
 
 def selftest_bounded_wait(limit_cycles: int = 20000, code: int = 777) -> int:
@@ -323,12 +340,9 @@ def quantize_conv_weights(w: torch.Tensor, taps: int, fmt: Format, want_grid: bo
 def conv_dgrad_filters(c1: Packed, kh: int, kw: int, c_in: int, c_out: int, out: Optional[Packed] = None) -> Packed:
     """hbfp_conv_dgrad_filters: the filter operand of the backward-data convolution (rows = c_in, k = kh*kw*c_out)
     from view ``c1`` of ``quantize_conv_weights``: the forward pass's mantissas and tile exponents, taps reversed."""
-    if out is None:
-        out = alloc_packed(c_in, kh * kw * c_out, c1.fmt, c1.mant.device)
-    f = c1.fmt.c()
-    _check(lib().hbfp_conv_dgrad_filters(_dptr(c1.mant), _dptr(c1.exps), kh, kw, c_in, c_out, ctypes.byref(f), _dptr(out.mant),
-                                         _dptr(out.exps), _stream()), "hbfp_conv_dgrad_filters")
-    return out
+    m, e = _got((_native or host()).conv_dgrad_filters(c1, kh, kw, c_in, c_out, out.mant if out is not None else None, out.exps if out is not None else None),
+                "hbfp_conv_dgrad_filters")
+    return out if out is not None else Packed(m, e, c_in, kh * kw * c_out, c1.fmt)
 
 
 def conv_forward(px: Packed, filters: Packed, n: int, h: int, w: int, c: int, kh: int, kw: int, pad: int,
@@ -336,29 +350,18 @@ def conv_forward(px: Packed, filters: Packed, n: int, h: int, w: int, c: int, kh
     """hbfp_conv_forward: the convolution ``[n*h*w][filters]`` of packed pixels ``px`` (block = c) with the
     packed filters ``filters`` (rows = filters, k = kh*kw*c) as one implicit GEMM. Raises ``HbfpError``
     (ERR_UNSUPPORTED) for shapes the kernel does not cover."""
-    nf = filters.rows
-    if out is None:
-        out = torch.empty((n * h * w, nf), dtype=torch.float32, device=px.mant.device)
-    _check_f32(out, "out")
-    fx = px.fmt.c()
-    op = filters.operand()
-    _check(lib().hbfp_conv_forward(_dptr(px.mant), _dptr(px.exps), n, h, w, c, kh, kw, pad, ctypes.byref(fx), ctypes.byref(op),
-                                   nf, _dptr(out), _ld(out), _stream()), "hbfp_conv_forward")
-    return out
+    return _got((_native or host()).conv_forward(px, filters, n, h, w, c, kh, kw, pad, filters.rows, out), "hbfp_conv_forward")
 
 
 def im2col_packed_t(x: torch.Tensor, kh: int, kw: int, pad: int, fmt: Format, out: Optional[Packed] = None) -> Packed:
     """hbfp_im2col_packed_t: the packed backward-weight operand ``[kh*kw*c][n*h*w]`` (blocks of
     ``fmt.block`` consecutive output pixels) straight from FP32 activations ``x [n][h][w][c]``."""
-    if not (x.is_cuda and x.dtype == torch.float32 and x.dim() == 4 and x.is_contiguous()):
-        raise ValueError("x must be a contiguous float32 CUDA tensor [n][h][w][c]")
+    m, e = _got((_native or host()).im2col_packed_t(x, kh, kw, pad, fmt, out.mant if out is not None else None, out.exps if out is not None else None),
+                "hbfp_im2col_packed_t")
+    if out is not None:
+        return out
     n, h, w, c = x.shape
-    if out is None:
-        out = alloc_packed(kh * kw * c, n * h * w, fmt, x.device)
-    f = fmt.c()
-    _check(lib().hbfp_im2col_packed_t(_dptr(x), n, h, w, c, kh, kw, pad, ctypes.byref(f), _dptr(out.mant),
-                                      _dptr(out.exps), _stream()), "hbfp_im2col_packed_t")
-    return out
+    return Packed(m, e, kh * kw * c, n * h * w, fmt)
 
 
 def unpack(p: Packed) -> Tuple[torch.Tensor, torch.Tensor]:
@@ -400,19 +403,7 @@ def gemm(transA: int, transB: int, A: torch.Tensor, B: torch.Tensor, fmtA: Forma
          out: Optional[torch.Tensor] = None, workspace: Optional[torch.Tensor] = None,
          flags: int = GEMM_AUTO) -> torch.Tensor:
     """hbfp_gemm: ``C = op(A) op(B)`` with both FP32 operands quantised by the call."""
-    _check_f32(A, "A")
-    _check_f32(B, "B")
-    M, N, K = _gemm_dims(transA, transB, A, B)
-    if out is None:
-        out = torch.empty((M, N), dtype=torch.float32, device=A.device)
-    if workspace is None:
-        workspace = torch.empty(max(gemm_workspace(transA, transB, M, N, K, fmtA, fmtB), 1), dtype=torch.int8,
-                                device=A.device)
-    fa, fb = fmtA.c(), fmtB.c()
-    _check(lib().hbfp_gemm(transA, transB, M, N, K, _dptr(A), _ld(A), _dptr(B), _ld(B), _dptr(out), _ld(out),
-                           ctypes.byref(fa), ctypes.byref(fb), _dptr(workspace), workspace.numel(), flags,
-                           _stream()), "hbfp_gemm")
-    return out
+    return _got((_native or host()).gemm(transA, transB, A, B, fmtA, fmtB, out, workspace, flags), "hbfp_gemm")
 
 
 def gemm_static(transA: int, transB: int, A: torch.Tensor, B: torch.Tensor, fmtA: Format, fmtB: Format,
@@ -451,16 +442,7 @@ def gemm_q(M: int, N: int, K: int, a, b, transA: int = 0, transB: int = 0, fmtA:
            fmtB: Optional[Format] = None, out: Optional[torch.Tensor] = None,
            workspace: Optional[torch.Tensor] = None, flags: int = GEMM_AUTO) -> torch.Tensor:
     """hbfp_gemm_q: each operand is an FP32 tensor (with its trans flag and format) or a ``Packed``."""
-    oa, ob = _as_operand(a, transA, fmtA), _as_operand(b, transB, fmtB)
-    dev = a.mant.device if isinstance(a, Packed) else a.device
-    if out is None:
-        out = torch.empty((M, N), dtype=torch.float32, device=dev)
-    if workspace is None:
-        workspace = torch.empty(max(gemm_q_workspace(M, N, K, a, b, transA, transB, fmtA, fmtB), 1),
-                                dtype=torch.int8, device=dev)
-    _check(lib().hbfp_gemm_q(M, N, K, ctypes.byref(oa), ctypes.byref(ob), _dptr(out), _ld(out), _dptr(workspace),
-                             workspace.numel(), flags, _stream()), "hbfp_gemm_q")
-    return out
+    return _got((_native or host()).gemm_q(M, N, K, a, b, transA, transB, fmtA, fmtB, out, workspace, flags), "hbfp_gemm_q")
 
 
 def gemm_block_partials(a: Packed, b: Packed, impl: int = GEMM_FORCE_SIMT) -> torch.Tensor:

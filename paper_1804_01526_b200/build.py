@@ -6,6 +6,7 @@ file (``libhbfp.so``) so that it travels with the source tree.
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 
@@ -13,6 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhbfp.so")
+HOST = os.path.join(HERE, "_host.so")      # host side of the Python binding (csrc/host.cpp)
 SOURCES = ["api.cu", "quantize.cu", "gemm_simt.cu", "gemm_small.cu", "gemm_tc.cu", "gemm_tc2.cu", "gemm_fp.cu", "gemm_conv.cu", "gemm_static.cu"]
 # (object name, source, extra flags): quantize.cu is compiled a second time for the full-tile kernel of small tiles
 EXTRA_OBJECTS = [("quantize_tiles_small.o", "quantize.cu", ["-DHBFP_QUANT_PART=2", "-Xptxas", "-O1"])]
@@ -33,11 +35,24 @@ NVCC_FLAGS = [
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(HOST)):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(HOST))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "hbfp.h")]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def _host_command(out: str) -> list:
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    inc, libs = os.path.join(root, "include"), os.path.join(root, "lib")
+    cuda = os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"))
+    return ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-fvisibility=hidden", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+            "-I", os.path.join(ROOT, "include"), "-isystem", inc, "-isystem", os.path.join(inc, "torch", "csrc", "api", "include"),
+            "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), os.path.join(CSRC, "host.cpp"),
+            "-o", out, "-L", libs, f"-Wl,-rpath,{libs}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -59,6 +74,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objs.append(obj)
         cmd = ["nvcc", *NVCC_FLAGS, *flags, "-c", os.path.join(CSRC, src), "-o", obj]
         procs.append((obj_name, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    host_tmp = HOST + f".tmp{os.getpid()}"
+    procs.append(("host.cpp", subprocess.Popen(_host_command(host_tmp), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
     failed = False
     for src, p in procs:
         out, _ = p.communicate()
@@ -71,6 +88,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.run(["nvcc", "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a",
                     "-cudart", "static"], check=True)
     os.replace(tmp, LIB)
+    os.replace(host_tmp, HOST)
     return LIB
 
 

@@ -3,13 +3,22 @@
 
 #include <string.h>
 
+#include <atomic>
+
 namespace hbfp {
 
 __device__ int32_t g_device_status;
 
+// The address belongs to the device and never changes: asked for once per device (threads that race store the same value).
 int32_t* device_status_word() {
-    int32_t* p = nullptr;
-    if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_device_status) != cudaSuccess) return nullptr;
+    static std::atomic<int32_t*> known[64];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    int32_t* p = known[dev].load(std::memory_order_acquire);
+    if (!p) {
+        if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_device_status) != cudaSuccess) return nullptr;
+        known[dev].store(p, std::memory_order_release);
+    }
     return p;
 }
 
