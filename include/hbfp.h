@@ -341,8 +341,8 @@ HBFP_API int hbfp_gemm_q(int64_t M, int64_t N, int64_t K, const hbfp_operand* a,
  * the packed pixels (one 4-D TMA box per tap and 128 output pixels; positions outside the image read as
  * zero mantissas): the packed im2col operand of hbfp_im2col_packed is never formed. The result equals
  * hbfp_gemm_q on that operand bit for bit (taps accumulated in ascending order, one FP32 rounding each).
- * Y: FP32, 16-byte aligned, row stride ldy >= filters, ldy % 4 == 0. Supported: c in {64, 128}, mantissas
- * up to 8 bits, w in {16, 32, 64, 128}, h a multiple of 128 / w, up to 256 filters, kh * kw <= 25; any
+ * Y: FP32, 16-byte aligned, row stride ldy >= filters, ldy % 4 == 0. Supported: blocks of 64 or 128
+ * channels (c itself, or c = 2 to 4 whole blocks, then K-blocks run tap by tap, block by block), mantissas up to 8 bits, w in {16, 32, 64, 128}, h a multiple of 128 / w, up to 256 filters, at most 36 K-blocks; any
  * other case returns HBFP_ERR_UNSUPPORTED and leaves Y untouched (use hbfp_im2col_packed + hbfp_gemm_q).
  * Exponent range as for the paired-SM GEMM (hbfp_gemm). Asynchronous on `stream`, allocates nothing. */
 HBFP_API int hbfp_conv_forward(const void* mant_x, const int8_t* exps_x, int64_t n, int64_t h, int64_t w, int64_t c,

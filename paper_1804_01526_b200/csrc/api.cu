@@ -362,7 +362,7 @@ int hbfp_conv_forward(const void* mant_x, const int8_t* exps_x, int64_t n, int64
     if (filters_op->struct_size != sizeof(hbfp_operand) || filters_op->kind != HBFP_OPERAND_PACKED || !filters_op->data ||
         !filters_op->exps)
         return HBFP_ERR_INVALID_ARG;
-    if (fmt_x->block != c || fmt_x->tile != 0 || filters_op->fmt.block != c) return HBFP_ERR_UNSUPPORTED;
+    if (fmt_x->block <= 0 || c % fmt_x->block != 0 || fmt_x->tile != 0 || filters_op->fmt.block != fmt_x->block) return HBFP_ERR_UNSUPPORTED;
     if ((reinterpret_cast<uintptr_t>(mant_x) & 255) || (reinterpret_cast<uintptr_t>(filters_op->data) & 255)) return HBFP_ERR_ALIGNMENT;
     Packed px, pw;
     int rc = make_layout(n * h * w, c, fmt_x, &px.L);

@@ -1,9 +1,9 @@
 // Convolution forward pass as an implicit BFP GEMM for sm_100a (Sec. 5.1: convolutions run through the
 // same BFP dot products; Eq. 2 per filter tap, taps accumulated in FP32).
 //
-// The activations were converted once per pixel (one block of c channels, one exponent, per pixel),
-// the filters once per (tap, filter) block. Row p of the GEMM is output pixel p, K-block t is filter
-// tap t = (dy, dx), and the operand of (p, t) is the packed channel vector of input pixel
+// The activations were converted once per pixel (one block of c channels, one exponent, or up to four such blocks),
+// the filters once per (tap, channel block, filter). Row p of the GEMM is output pixel p, K-block t is filter
+// tap t = (dy, dx) (with several channel blocks: tap by tap, block by block within it), and the operand of (p, t) is the packed channel vector of input pixel
 // (y + dy - pad, x + dx - pad): nothing has to be gathered into an im2col operand first. The producer
 // warp issues, per tap, one 4-D TMA box per 128 output pixels straight from the packed pixels
 // [n][h][w][c]; coordinates outside the image are filled with zero mantissas by the copy engine, which
@@ -12,7 +12,7 @@
 // One CTA per SM, persistent over "super tiles" of RT x 128 output pixels x all filters (RT = 256 /
 // N_TILE row tiles share one hand-over per tap, so that a hand-over always covers 128 x 256
 // accumulator words). Roles as in the other tensor-core kernels: warp 0 producer, warp 1 MMA issuer and
-// tensor-memory owner, warp 2 scale-table builder (it also gathers the pixel exponents of the taps),
+// tensor-memory owner, warps 2 and 3 scale-table builders (they also gather the pixel exponents of the taps),
 // warps 4-11 rescale. Block sums: every tap starts with an MMA step of two constant all-255 operands
 // taken as unsigned bytes, which overwrites the accumulator with OFFSET = 32 * 255 * 255; the tap's own
 // steps land on top, a word read back is the positive pattern OFFSET + P, as binary32 the subnormal
@@ -27,7 +27,7 @@ namespace hbfp {
 namespace {
 
 constexpr int CV_RESCALE_WARPS = 8, CV_CONTROL_WARPS = 4;
-constexpr int CV_PRODUCER_WARP = 0, CV_MMA_WARP = 1, CV_TABLE_WARP = 2;
+constexpr int CV_PRODUCER_WARP = 0, CV_MMA_WARP = 1, CV_TABLE_WARP = 2;      // two table builders: warps 2 and 3
 constexpr int CV_THREADS = 32 * (CV_CONTROL_WARPS + CV_RESCALE_WARPS);
 constexpr int CV_REGS_RESCALE = 216, CV_REGS_CONTROL = 72;      // totals stay inside 384 threads x 168 registers
 constexpr int CV_OFFSET = 32 * 255 * 255;
@@ -35,7 +35,7 @@ constexpr int CV_SHIFT = 86;
 constexpr int CV_COLS = 256;          // accumulator columns per buffer: RT row tiles of N_TILE columns
 constexpr int CV_BUFS = TMEM_COLS / CV_COLS;
 constexpr int CV_TSLOTS = 2 * CV_BUFS;
-constexpr int CV_MAX_TAPS = 25, CV_MAX_PAD = 2;
+constexpr int CV_MAX_STEPS = 36, CV_MAX_CBS = 4, CV_MAX_PAD = 2;      // K-blocks (taps x channel blocks), channel blocks per pixel
 constexpr int CV_GRID_BYTES = 832;    // (R + 2 pad) rows of w + 32 pixel exponents of one row tile (data from column 16), pad <= 2
 
 template <int C, int N_TILE>
@@ -48,8 +48,9 @@ struct ConvCfg {
     static constexpr int ONES_BYTES = 1024;
     static constexpr int SLOT_WORDS = N_TILE + RT * TILE_M;
     static constexpr int TABLE_BYTES = 4 * CV_TSLOTS * SLOT_WORDS;
-    static constexpr int GRID_BYTES = RT * CV_GRID_BYTES;
-    static constexpr int WEXP_BYTES = CV_MAX_TAPS * N_TILE;
+    static constexpr int GRID_ONE = CV_MAX_CBS * RT * CV_GRID_BYTES;        // [channel block][row tile]
+    static constexpr int GRID_BYTES = 2 * GRID_ONE;                         // one grid per table builder
+    static constexpr int WEXP_BYTES = CV_MAX_STEPS * N_TILE;
     static constexpr int FIXED = 1024 /*align*/ + ONES_BYTES + TABLE_BYTES + GRID_BYTES + WEXP_BYTES + 1024 /*barriers*/;
     static constexpr int STAGES_RAW = (232448 - FIXED) / STAGE;
     static constexpr int STAGES = STAGES_RAW > 4 ? 4 : STAGES_RAW;
@@ -61,13 +62,15 @@ struct ConvCfg {
 
 struct ConvProblem {
     int n, h, w, kh, kw, pad, taps;
+    int cbs, steps;             // channel blocks per pixel; K-blocks = taps x cbs
     int rows_per_tile;          // R = 128 / w image rows per row tile
     int tiles_per_image;        // h / R
     int row_tiles;              // n * h / R
     int super_tiles;
     int filters;
-    const int8_t* exps_x;       // [n*h*w] pixel exponents
-    const int8_t* exps_w;       // [taps][rs_w] filter exponents
+    const int8_t* exps_x;       // [cbs][rs_x] pixel exponents
+    int64_t rs_x;
+    const int8_t* exps_w;       // [steps][rs_w] filter exponents
     int64_t rs_w;
     float* Y;
     int64_t ldy;
@@ -96,15 +99,10 @@ __device__ __forceinline__ constexpr uint32_t idesc_conv(bool unsigned_ops) {
     return (2u << 4) | (unsigned_ops ? 0u : ((1u << 7) | (1u << 10))) | ((uint32_t)(N_TILE >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
 }
 
-__device__ __forceinline__ bool cv_test_wait(uint32_t bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    return done != 0;
-}
-// Poll first (a thread that try_wait has put to sleep wakes up late), then the bounded suspending wait.
-__device__ __forceinline__ bool cv_wait_polled(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code) {
-    for (int i = 0; i < 4096; ++i)
-        if (cv_test_wait(bar, parity)) return true;
+// Bounded wait of a single thread: prompt tries first (a wait with the long suspend hint wakes late).
+__device__ __forceinline__ bool cv_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status, int code) {
+    for (int i = 0; i < 256; ++i)
+        if (mbar_try(bar, parity)) return true;
     return mbar_wait(bar, parity, abort_flag, status, code);
 }
 
@@ -133,8 +131,8 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     const uint32_t wexp_off = grid_off + G::GRID_BYTES;
     const uint32_t bar_off = (wexp_off + G::WEXP_BYTES + 15u) & ~15u;
     uint32_t* tables = reinterpret_cast<uint32_t*>(base_ptr + table_off);     // [slot][N_TILE column scales | RT*128 row scales]
-    int8_t* grid = reinterpret_cast<int8_t*>(base_ptr + grid_off);            // [row tile][(R + 2 pad) x (w + 2 pad)]
-    int8_t* wexp = reinterpret_cast<int8_t*>(base_ptr + wexp_off);            // [tap][N_TILE]
+    int8_t* grid = reinterpret_cast<int8_t*>(base_ptr + grid_off);            // [builder][channel block][row tile][(R + 2 pad) x (w + 32)]
+    int8_t* wexp = reinterpret_cast<int8_t*>(base_ptr + wexp_off);            // [K-block][N_TILE]
     const uint32_t bars = base + bar_off;
     const uint32_t full_bar = bars;                          // stage landed
     const uint32_t empty_bar = full_bar + 8 * STAGES;        // stage consumed (MMA commit)
@@ -161,10 +159,12 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     }
     // constant operand of the offset step, and the filter exponents (the same for every tile)
     for (int i = threadIdx.x; i < G::ONES_BYTES / 4; i += CV_THREADS) reinterpret_cast<uint32_t*>(base_ptr + ones_off)[i] = 0xFFFFFFFFu;
-    for (int i = threadIdx.x; i < p.taps * N_TILE; i += CV_THREADS) {
+    for (int i = threadIdx.x; i < p.steps * N_TILE; i += CV_THREADS) {
         const int t = i / N_TILE, j = i - t * N_TILE;
         wexp[i] = j < p.filters ? p.exps_w[(int64_t)t * p.rs_w + j] : (int8_t)0;
     }
+    // 127 marks a position outside the image (the columns next to the data stay marked for good)
+    for (int i = threadIdx.x; i < G::GRID_BYTES / 4; i += CV_THREADS) reinterpret_cast<uint32_t*>(base_ptr + grid_off)[i] = 0x7f7f7f7fu;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (warp == CV_MMA_WARP) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
@@ -179,24 +179,36 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(CV_REGS_CONTROL));
         if (warp == CV_PRODUCER_WARP) {
             // -------------------------------------------------------------- TMA producer
-            if (lane == 0) {
+            // The coordinates are kept in registers and counted on: with a division by a run-time value per copy, behind a
+            // lane == 0 branch, issuing the copies of one K-block took 1 600 cycles, half as much again as everything else
+            // a K-block needs (64 -> 64 channels at 32 x 32, batch 128: 25.9 -> 24.5 us).
+            if (elect_one()) {
                 uint32_t s = 0, ph = 0, it = 0;
                 bool ok = true;
                 for (int st = blockIdx.x; ok && st < p.super_tiles; st += gridDim.x) {
-                    for (int tap = 0; tap < p.taps; ++tap, ++it) {
-                        if (!mbar_wait(empty_bar + 8 * s, ph ^ 1, abort_flag, p.status, 121)) { ok = false; break; }
+                    // row tiles past the end lie in image n >= p.n: filled with zeros like any coordinate outside
+                    int img[RT], y0[RT];
+                    img[0] = st * RT / p.tiles_per_image;
+                    y0[0] = (st * RT - img[0] * p.tiles_per_image) * p.rows_per_tile;
+#pragma unroll
+                    for (int r = 1; r < RT; ++r) {
+                        const bool wrap = y0[r - 1] + p.rows_per_tile == p.h;
+                        img[r] = img[r - 1] + (wrap ? 1 : 0);
+                        y0[r] = wrap ? 0 : y0[r - 1] + p.rows_per_tile;
+                    }
+                    int dx = -p.pad, dy = -p.pad, cb = 0;
+                    for (int step = 0; step < p.steps; ++step, ++it) {
+                        if (!cv_wait(empty_bar + 8 * s, ph ^ 1, abort_flag, p.status, 121)) { ok = false; break; }
                         const uint32_t fb = full_bar + 8 * s;
                         mbar_expect_tx(fb, (uint32_t)G::STAGE);
                         const uint32_t dst = stage_base + s * G::STAGE;
-                        const int dy = tap / p.kw, dx = tap - dy * p.kw;
 #pragma unroll
-                        for (int r = 0; r < RT; ++r) {
-                            // row tiles past the end lie in image n >= p.n: filled with zeros like any coordinate outside
-                            const int rt = st * RT + r;
-                            const int img = rt / p.tiles_per_image, y0 = (rt - img * p.tiles_per_image) * p.rows_per_tile;
-                            tma_load_4d(dst + r * G::A_TILE, &mapX, 0, dx - p.pad, y0 + dy - p.pad, img, fb);
+                        for (int r = 0; r < RT; ++r) tma_load_4d(dst + r * G::A_TILE, &mapX, cb * C, dx, y0[r] + dy, img[r], fb);
+                        tma_load_2d(dst + G::A_BYTES, &mapW, step * C, 0, fb);
+                        if (++cb == p.cbs) {
+                            cb = 0;
+                            if (++dx == p.kw - p.pad) { dx = -p.pad; ++dy; }
                         }
-                        tma_load_2d(dst + G::A_BYTES, &mapW, tap * C, 0, fb);
                         cv_ring_next<STAGES>(s, ph);
                     }
                 }
@@ -214,9 +226,11 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 uint32_t s = 0, ph = 0, b = 0, bph = 0;
                 bool ok = true;
                 for (int st = blockIdx.x; ok && st < p.super_tiles; st += gridDim.x) {
-                    for (int tap = 0; tap < p.taps; ++tap) {
-                        if (!mbar_wait(full_bar + 8 * s, ph, abort_flag, p.status, 221)) { ok = false; break; }
-                        if (!cv_wait_polled(tempty_bar + 8 * b, bph, abort_flag, p.status, 222)) { ok = false; break; }
+                    for (int step = 0; step < p.steps; ++step) {
+                        // both first looks are under way before either answer is needed
+                        const bool landed = mbar_try(full_bar + 8 * s, ph), is_free = mbar_try(tempty_bar + 8 * b, bph);
+                        if (!landed && !cv_wait(full_bar + 8 * s, ph, abort_flag, p.status, 221)) { ok = false; break; }
+                        if (!is_free && !cv_wait(tempty_bar + 8 * b, bph, abort_flag, p.status, 222)) { ok = false; break; }
                         tc_fence_after();
                         const uint32_t src = stage_base + s * G::STAGE;
                         const uint64_t b_desc = smem_desc_rows<C>(src + G::A_BYTES);
@@ -237,25 +251,26 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                 tc_commit(done_bar);
                 mbar_wait(done_bar, 0, abort_flag, p.status, 223, false);
             }
-        } else if (warp == CV_TABLE_WARP) {
-            // -------------------------------------------------------------- scale-table builder
-            // Per super tile it first lays out, for each row tile, the exponents of the input pixels that the
-            // taps touch (the tile's image rows plus `pad` rows and columns around them; 127 marks a position
-            // outside the image). The table of step k (tap by tap, across tiles) goes to slot k % 4 and its
-            // arrival counts on tfull[k % 2]; it is written once the phase of step k - 2 on that barrier is
-            // complete (see gemm_tc2.cu for why the slot's last readers are done by then).
-            // Grid row gy holds image row y0 + gy - pad; its pixel x sits in column 16 + x, so that 16-byte pieces
-            // of the exponent array land aligned; the columns next to the data stay at the mark for good.
+        } else {
+            // -------------------------------------------------------------- scale-table builders (warps 2 and 3)
+            // Warp 2 builds the tables of the even K-blocks (buffer 0), warp 3 those of the odd ones. Per super tile each lays
+            // out, in a grid of its own, for each channel block and row tile, the exponents of the input pixels that the taps touch (the tile's image rows
+            // plus `pad` rows around them). The table of step k (across tiles) goes to slot k % 4 and its arrival counts on
+            // tfull[k % 2]; it is written once the phase of step k - 2 on that barrier is complete (see gemm_tc2.cu for why the
+            // slot's last readers are done by then). Four exponents of a row go through packed byte operations together.
+            // Grid row gy holds image row y0 + gy - pad; its pixel x sits in column 16 + x, so that 16-byte pieces of the
+            // exponent array land aligned.
+            const uint32_t me = (uint32_t)(warp - CV_TABLE_WARP);
+            int8_t* const my_grid = grid + me * G::GRID_ONE;
             const int gw = p.w + 32, gh = p.rows_per_tile + 2 * p.pad;
             const int lw = 31 - __clz(p.w);                           // w is a power of two
             const int cpr = p.w >> 4;                                 // 16-byte pieces per image row
-            for (int i = lane; i < RT * CV_GRID_BYTES; i += 32) grid[i] = (int8_t)127;
-            __syncwarp();
-            uint32_t b = 0, bph = 0, slot = 0;
+            const int pieces = p.cbs * RT * gh * cpr;
+            uint32_t ph = 0, slot = me, k = 0;                        // k: step number across tiles
             bool ok = true, out_of_range = false;
             for (int st = blockIdx.x; ok && st < p.super_tiles; st += gridDim.x) {
-                // all the loads of a super tile are issued together: one trip to L2, not one per piece
-                for (int i0 = 0; i0 < RT * gh * cpr; i0 += 64) {
+                // the loads of a super tile are issued together: one trip to L2, not one per piece
+                for (int i0 = 0; i0 < pieces; i0 += 64) {
                     uint4 val[2];
                     int dst[2];
 #pragma unroll
@@ -263,46 +278,49 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                         const int i = i0 + 32 * u + lane;
                         dst[u] = -1;
                         val[u] = make_uint4(0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu);
-                        if (i < RT * gh * cpr) {
-                            const int r = i / (gh * cpr), j = i - r * (gh * cpr);
+                        if (i < pieces) {
+                            const int r = i / (gh * cpr), j = i - r * (gh * cpr);          // r = channel block * RT + row tile
                             const int gy = j / cpr, xc = j - gy * cpr;
-                            const int rt = st * RT + r;
+                            const int cb = r / RT, rt = st * RT + (r - cb * RT);
                             const int img = rt / p.tiles_per_image, y0 = (rt - img * p.tiles_per_image) * p.rows_per_tile;
                             const int yy = y0 + gy - p.pad;
                             dst[u] = r * CV_GRID_BYTES + gy * gw + 16 + 16 * xc;
                             if (img < p.n && yy >= 0 && yy < p.h)
-                                val[u] = *reinterpret_cast<const uint4*>(p.exps_x + (((int64_t)img * p.h + yy) << lw) + 16 * xc);
+                                val[u] = *reinterpret_cast<const uint4*>(p.exps_x + (int64_t)cb * p.rs_x + (((int64_t)img * p.h + yy) << lw) + 16 * xc);
                         }
                     }
 #pragma unroll
                     for (int u = 0; u < 2; ++u)
-                        if (dst[u] >= 0) *reinterpret_cast<uint4*>(grid + dst[u]) = val[u];
+                        if (dst[u] >= 0) *reinterpret_cast<uint4*>(my_grid + dst[u]) = val[u];
                 }
                 __syncwarp();
-                for (int tap = 0; ok && tap < p.taps; ++tap) {
-                    const int dy = tap / p.kw, dx = tap - dy * p.kw;
-                    // this lane's 4 rows of every row tile and its N_TILE / 32 columns
-                    int ea[RT][4];
-                    int a_lo = 127, a_hi = -128;
+                // this lane's four rows of every row tile are four neighbouring pixels of one image row
+                const int yl = (4 * lane) >> lw, xl = (4 * lane) & (p.w - 1);
+                for (int step = 0; step < p.steps; ++step, ++k) {
+                    if ((k & 1u) != me) continue;
+                    const int tap = step / p.cbs, cb = step - tap * p.cbs, dy = tap / p.kw, dx = tap - dy * p.kw;
+                    const int at = cb * RT * CV_GRID_BYTES + (yl + dy) * gw + 16 + xl + dx - p.pad;
+                    const int word = at & ~3, shift = 8 * (at & 3);
+                    uint32_t ea[RT], lo4 = 0x7f7f7f7fu, hi4 = 0x80808080u;
 #pragma unroll
-                    for (int r = 0; r < RT; ++r)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int row = 4 * lane + k;
-                            const int yl = row >> lw, xl = row & (p.w - 1);
-                            const int e = grid[r * CV_GRID_BYTES + (yl + dy) * gw + 16 + xl + dx - p.pad];
-                            ea[r][k] = e;
-                            if (e != 127) { a_lo = min(a_lo, e); a_hi = max(a_hi, e); }
-                        }
+                    for (int r = 0; r < RT; ++r) {
+                        const uint32_t* g4 = reinterpret_cast<const uint32_t*>(my_grid + word + r * CV_GRID_BYTES);
+                        ea[r] = __funnelshift_r(g4[0], g4[1], shift);
+                        lo4 = __vmins4(lo4, ea[r]);                       // the mark is the largest byte: neutral here ...
+                        const uint32_t out = __vcmpeq4(ea[r], 0x7f7f7f7fu);
+                        hi4 = __vmaxs4(hi4, (ea[r] & ~out) | (0x80808080u & out));     // ... and replaced there
+                    }
+                    lo4 = __vmins4(lo4, lo4 >> 16); lo4 = __vmins4(lo4, lo4 >> 8);
+                    hi4 = __vmaxs4(hi4, hi4 >> 16); hi4 = __vmaxs4(hi4, hi4 >> 8);
+                    int a_lo = __reduce_min_sync(0xffffffffu, (int)(int8_t)lo4), a_hi = __reduce_max_sync(0xffffffffu, (int)(int8_t)hi4);
                     constexpr int CPL = N_TILE / 32;
                     int eb[CPL];
                     int b_lo = 127, b_hi = -128;
 #pragma unroll
-                    for (int k = 0; k < CPL; ++k) {
-                        eb[k] = wexp[tap * N_TILE + CPL * lane + k];
-                        b_lo = min(b_lo, eb[k]); b_hi = max(b_hi, eb[k]);
+                    for (int j = 0; j < CPL; ++j) {
+                        eb[j] = wexp[step * N_TILE + CPL * lane + j];
+                        b_lo = min(b_lo, eb[j]); b_hi = max(b_hi, eb[j]);
                     }
-                    a_lo = __reduce_min_sync(0xffffffffu, a_lo); a_hi = __reduce_max_sync(0xffffffffu, a_hi);
                     b_lo = __reduce_min_sync(0xffffffffu, b_lo); b_hi = __reduce_max_sync(0xffffffffu, b_hi);
                     if (a_lo > a_hi) a_lo = a_hi = 0;                 // every position of the tap lies outside the image
                     // split of the scale 2^(sA + sB) = 2^(sA + c) * 2^(sB + 149 - c): every factor and every
@@ -310,19 +328,23 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
                     const int c_lo = max(23 - a_lo, 22 + b_hi), c_hi = min(127 - a_hi, 275 + b_lo);
                     out_of_range |= c_lo > c_hi;
                     const int c = min(max(CV_SHIFT, c_lo), c_hi);
-                    if (!mbar_wait_warp(tfull_bar + 8 * b, bph ^ 1, abort_flag, p.status, 421)) { ok = false; break; }
+                    if (!mbar_wait_warp_fast(tfull_bar + 8 * me, ph ^ 1, abort_flag, p.status, 421)) { ok = false; break; }
                     uint32_t* tb = tables + slot * G::SLOT_WORDS;
 #pragma unroll
-                    for (int k = 0; k < CPL; ++k) tb[CPL * lane + k] = cv_scale_bits(eb[k], 149 - c);
+                    for (int j = 0; j < CPL; ++j) tb[CPL * lane + j] = cv_scale_bits(eb[j], 149 - c);
+                    const uint32_t inside = (uint32_t)(a_lo & 0xff) * 0x01010101u;
 #pragma unroll
-                    for (int r = 0; r < RT; ++r)
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)      // outside the image the mantissas are zero: any finite scale gives +0
-                            tb[N_TILE + r * TILE_M + 4 * lane + k] = cv_scale_bits(ea[r][k] == 127 ? a_lo : ea[r][k], c);
+                    for (int r = 0; r < RT; ++r) {
+                        // outside the image the mantissas are zero: any finite scale gives +0
+                        const uint32_t out = __vcmpeq4(ea[r], 0x7f7f7f7fu), e = (ea[r] & ~out) | (inside & out);
+                        *reinterpret_cast<uint4*>(tb + N_TILE + r * TILE_M + 4 * lane) =
+                            make_uint4(cv_scale_bits((int)(int8_t)e, c), cv_scale_bits((int)(int8_t)(e >> 8), c),
+                                       cv_scale_bits((int)(int8_t)(e >> 16), c), cv_scale_bits((int)(int8_t)(e >> 24), c));
+                    }
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(tfull_bar + 8 * b);
-                    cv_ring_next<CV_BUFS>(b, bph);
-                    slot = (slot + 1) & (CV_TSLOTS - 1);
+                    mbar_arrive_elect(tfull_bar + 8 * me);
+                    ph ^= 1u;
+                    slot = (slot + 2) & (CV_TSLOTS - 1);
                 }
                 __syncwarp();
             }
@@ -346,7 +368,7 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
             for (int r = 0; r < RT; ++r)
 #pragma unroll
                 for (int k = 0; k < HALF / 2; ++k) acc2[r][k] = 0ull;
-            for (int tap = 0; tap < p.taps; ++tap) {
+            for (int step = 0; step < p.steps; ++step) {
                 const uint32_t taddr = lane_addr + b * CV_COLS;
                 uint32_t v[2][CH];
                 if (!mbar_wait_warp_fast(tfull_bar + 8 * b, bph, abort_flag, p.status, 321)) { ok = false; break; }
@@ -432,12 +454,12 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     }
 }
 
-// 4-D byte tensor of the packed pixels: [n][h][w][pitch bytes], of which the first c bytes of every pixel
-// are copied; box = c bytes x w pixels x R image rows x 1 image.
-int make_map_pixels(CUtensorMap* m, const void* ptr, int c, uint64_t pitch, int w, int h, int n, int rows_per_tile) {
+// 4-D byte tensor of the packed pixels: [n][h][w][pitch bytes], of which the first `channels` bytes of every pixel count;
+// box = one block of c bytes x w pixels x R image rows x 1 image.
+int make_map_pixels(CUtensorMap* m, const void* ptr, int channels, int c, uint64_t pitch, int w, int h, int n, int rows_per_tile) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return HBFP_ERR_CUDA;
-    cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
+    cuuint64_t dims[4] = {(cuuint64_t)channels, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)n};
     cuuint64_t strides[3] = {pitch, pitch * (uint64_t)w, pitch * (uint64_t)w * (uint64_t)h};
     cuuint32_t box[4] = {(cuuint32_t)c, (cuuint32_t)w, (cuuint32_t)rows_per_tile, 1};
     cuuint32_t estr[4] = {1, 1, 1, 1};
@@ -478,13 +500,16 @@ int launch_conv_cfg(const CUtensorMap& mX, const CUtensorMap& mW, const ConvProb
 
 }  // namespace
 
-// x: packed pixels (rows = n*h*w, k = c, one block); wt: packed filters (rows = filters, k = kh*kw*c, blocks of c).
-int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw,
+// x: packed pixels (rows = n*h*w, k = channels, whole blocks of c = 64 or 128); wt: packed filters (rows = filters, k =
+// kh*kw*channels, blocks of c).
+int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h, int64_t w, int64_t channels, int kh, int kw,
                         int pad, int64_t filters, float* Y, int64_t ldy, cudaStream_t st) {
+    const int64_t c = x.L.b;
     // what the kernel covers; everything else is the caller's gather + GEMM path
     if (c != 64 && c != 128) return HBFP_ERR_UNSUPPORTED;
-    if (x.L.planes != 1 || wt.L.planes != 1 || x.L.bp != c || wt.L.bp != c || x.L.nkb != 1) return HBFP_ERR_UNSUPPORTED;
-    if (kh * kw > CV_MAX_TAPS || pad > CV_MAX_PAD || 2 * pad != kh - 1 || 2 * pad != kw - 1) return HBFP_ERR_UNSUPPORTED;
+    if (x.L.planes != 1 || wt.L.planes != 1 || x.L.bp != c || wt.L.bp != c || wt.L.b != c || channels % c != 0) return HBFP_ERR_UNSUPPORTED;
+    const int64_t cbs = channels / c;
+    if (cbs > CV_MAX_CBS || kh * kw * cbs > CV_MAX_STEPS || pad > CV_MAX_PAD || 2 * pad != kh - 1 || 2 * pad != kw - 1) return HBFP_ERR_UNSUPPORTED;
     if (w < 16 || w > 128 || (128 % w) != 0 || (h % (128 / w)) != 0) return HBFP_ERR_UNSUPPORTED;
     if (reinterpret_cast<uintptr_t>(x.exps) & 15) return HBFP_ERR_UNSUPPORTED;
     if (filters < 1 || filters > 256 || n * h * w > (1ll << 30)) return HBFP_ERR_UNSUPPORTED;
@@ -494,6 +519,8 @@ int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h,
     const int n_tile = filters <= 64 ? 64 : filters <= 128 ? 128 : 256;
     ConvProblem p{};
     p.n = (int)n; p.h = (int)h; p.w = (int)w; p.kh = kh; p.kw = kw; p.pad = pad; p.taps = kh * kw;
+    p.cbs = (int)cbs;
+    p.steps = p.taps * p.cbs;
     p.rows_per_tile = 128 / (int)w;
     p.tiles_per_image = (int)h / p.rows_per_tile;
     p.row_tiles = (int)n * p.tiles_per_image;
@@ -501,6 +528,7 @@ int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h,
     p.super_tiles = (p.row_tiles + rt - 1) / rt;
     p.filters = (int)filters;
     p.exps_x = x.exps;
+    p.rs_x = x.L.rs;
     p.exps_w = wt.exps;
     p.rs_w = wt.L.rs;
     p.Y = Y;
@@ -509,7 +537,7 @@ int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h,
     if (!p.status) return HBFP_ERR_CUDA;
     if (p.super_tiles == 0) return HBFP_OK;
     CUtensorMap mX, mW;
-    int rc = make_map_pixels(&mX, x.mant, (int)c, (uint64_t)x.L.kst, (int)w, (int)h, (int)n, p.rows_per_tile);
+    int rc = make_map_pixels(&mX, x.mant, (int)channels, (int)c, (uint64_t)x.L.kst, (int)w, (int)h, (int)n, p.rows_per_tile);
     if (rc) return rc;
     rc = make_map_filters(&mW, wt.mant, (uint64_t)wt.L.kst, (uint64_t)wt.L.rows, (int)c, n_tile);
     if (rc) return rc;

@@ -303,3 +303,24 @@ def test_backward_data_filter_operand_says_what_it_does_not_cover(hb):
     with pytest.raises(hb.HbfpError) as e:
         hb.conv_dgrad_filters(c1, 3, 3, 24, 40)
     assert e.value.code == hb.ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("n,h,w_,channels,t,f,k,pad", [(2, 32, 32, 128, 64, 64, 3, 1), (3, 16, 16, 256, 64, 128, 3, 1), (1, 16, 16, 256, 128, 200, 3, 1),
+                                                       (1, 8, 16, 512, 128, 64, 3, 1), (5, 8, 64, 256, 128, 12, 1, 0)])
+def test_implicit_convolution_with_several_channel_blocks_per_pixel(hb, n, h, w_, channels, t, f, k, pad):
+    """Pixels of `channels` maps in blocks of t: K-blocks run tap by tap, block by block; bit for bit the oracle's
+    sequential GEMM on the gathered blocks (a super tile that is only partly there, partial filter tiles, borders)."""
+    taps = k * k
+    x = wl.draw("lognormal", (n * h * w_, channels), seed=103)
+    wt = wl.draw("he_weight", (taps * channels, f), seed=104, fan_in=taps * channels)
+    fx = dict(mant_bits=8, block=t, rounding=1, seed=3, stream_id=4)
+    fw = dict(mant_bits=8, block=t, stream_id=1)
+    px = hb.quantize(to_dev(x), 1, gfmt(fx))
+    pw = hb.quantize(to_dev(wt), 0, gfmt(fw))
+    Y = hb.conv_forward(px, pw, n, h, w_, channels, k, k, pad).cpu().numpy()
+    assert hb.device_status() == 0 and hb.last_gemm_kernel() == "conv_fwd_kernel"
+    qp, sp = oracle.quantize(x, 1, ofmt(fx))
+    qa = oracle.im2col(qp.reshape(n, h, w_, channels), k, k, pad)
+    sa = oracle.im2col(sp.reshape(n, h, w_, channels // t), k, k, pad)
+    qb, sb = oracle.quantize(wt, 0, ofmt(fw))
+    assert np.array_equal(Y, oracle.gemm(qa, sa, qb, sb, t)["c_seq"])
