@@ -324,3 +324,21 @@ def test_implicit_convolution_with_several_channel_blocks_per_pixel(hb, n, h, w_
     sa = oracle.im2col(sp.reshape(n, h, w_, channels // t), k, k, pad)
     qb, sb = oracle.quantize(wt, 0, ofmt(fw))
     assert np.array_equal(Y, oracle.gemm(qa, sa, qb, sb, t)["c_seq"])
+
+
+@pytest.mark.parametrize("n,h,w,c,kh,m,rounding", [(1, 8, 8, 4, 3, 8, 0), (3, 16, 8, 40, 3, 8, 1), (2, 4, 16, 36, 3, 12, 0), (1, 8, 16, 200, 3, 8, 1),
+                                                   (1, 2, 32, 64, 3, 8, 0), (2, 6, 32, 16, 3, 12, 1), (1, 1, 64, 72, 3, 8, 0), (1, 3, 64, 8, 3, 4, 1)])
+def test_backward_weight_operand_for_three_wide_filters(hb, n, h, w, c, kh, m, rounding):
+    """Every image width of the kernel for 3 x 3 filters and blocks of 64 pixels, image borders in every block, channel counts
+    around its CTA size; under stochastic rounding each entry takes its activation's draw."""
+    x = wl.draw("lognormal", (n * h * w, c), seed=107).reshape(n, h, w, c)
+    fd = dict(mant_bits=m, block=64, rounding=rounding, seed=29, stream_id=2)
+    pa = hb.im2col_packed_t(to_dev(x), kh, 3, 1, gfmt(fd))
+    assert hb.device_status() == 0
+    cols = oracle.im2col(x, kh, 3, 1)
+    if rounding:
+        q_ref, s_ref = oracle.quantize_indexed(cols, 0, ofmt(fd), oracle.im2col_index(n, h, w, c, kh, 3, 1))
+    else:
+        q_ref, s_ref = oracle.quantize(cols, 0, ofmt(fd))
+    q, s = decode_packed(pa, hb.packed_layout(pa.rows, pa.k, pa.fmt))
+    assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
