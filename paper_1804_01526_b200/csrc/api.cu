@@ -89,7 +89,9 @@ int make_plan(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     g->tp = plan_gemm_tensor(M, N, K, g->la, g->lb, a->fmt.mant_bits, b->fmt.mant_bits);
     g->off_partial = off;
     g->total = off + align_up(g->tp.partial_bytes, 1024);
-    g->fp = plan_gemm_fp(M, N, g->la, g->lb);
+    // operands that need a pass of their own to take the form
+    const int passes = (a->kind != HBFP_OPERAND_FP32 || a->fmt.tile != 0) + (b->kind != HBFP_OPERAND_FP32 || b->fmt.tile != 0);
+    g->fp = plan_gemm_fp(M, N, g->la, g->lb, passes);
     g->off_fa = off;
     if (g->fp.use) off += fp_bytes(g->la, g->fp, false);
     g->off_fb = off;
@@ -108,6 +110,15 @@ void fill_operand(hbfp_operand* o, const float* data, int64_t ld, int trans, con
     if (f) o->fmt = *f;
 }
 
+// How an FP32 operand is stored. A: trans 0 = [rows][K] (blocks along rows), trans 1 = [K][rows]; B: trans 0 = [K][rows]
+// (blocks down columns), trans 1 = [rows][K].
+bool k_contiguous(const hbfp_operand* o, bool is_a) { return is_a ? o->trans == 0 : o->trans != 0; }
+
+int check_fp32(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K) {
+    if (!o->data && rows * K > 0) return HBFP_ERR_INVALID_ARG;
+    return o->ld < (k_contiguous(o, is_a) ? K : rows) ? HBFP_ERR_INVALID_ARG : HBFP_OK;
+}
+
 // Quantises an FP32 operand into the workspace (or takes a packed one as is).
 int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const Layout& L,
                     char* ws, size_t off_m, size_t off_e, Packed* out, cudaStream_t st) {
@@ -121,21 +132,31 @@ int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, c
         out->exps = o->exps;
         return HBFP_OK;
     }
-    if (!o->data && rows * K > 0) return HBFP_ERR_INVALID_ARG;
+    const int rc = check_fp32(o, is_a, rows, K);
+    if (rc) return rc;
     int8_t* m = reinterpret_cast<int8_t*>(ws + off_m);
     int8_t* e = reinterpret_cast<int8_t*>(ws + off_e);
     out->mant = m;
     out->exps = e;
     const float* x = static_cast<const float*>(o->data);
-    // A: trans 0 = stored [rows][K] (blocks along rows); trans 1 = stored [K][rows].
-    // B: trans 0 = stored [K][rows] (blocks down columns); trans 1 = stored [rows][K].
-    const bool k_contiguous = is_a ? (o->trans == 0) : (o->trans != 0);
-    if (k_contiguous) {
-        if (o->ld < K) return HBFP_ERR_INVALID_ARG;
-        return launch_quantize(x, rows, K, o->ld, 1, &o->fmt, m, e, st);
+    return k_contiguous(o, is_a) ? launch_quantize(x, rows, K, o->ld, 1, &o->fmt, m, e, st) : launch_quantize(x, K, rows, o->ld, 0, &o->fmt, m, e, st);
+}
+
+// An operand in the floating-point form at `f`: converted straight to it where it is an FP32 matrix without weight tiles,
+// otherwise packed (or taken packed) and expanded.
+int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const GemmPlan& g, char* ws, const FpOperand& f, cudaStream_t st) {
+    if (o->kind == HBFP_OPERAND_FP32) {
+        const int rc = check_fp32(o, is_a, rows, K);
+        if (rc) return rc;
+        const float* x = static_cast<const float*>(o->data);
+        const int done = k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, f, st)
+                                               : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, f, st);
+        if (done != HBFP_ERR_UNSUPPORTED) return done;
     }
-    if (o->ld < rows) return HBFP_ERR_INVALID_ARG;
-    return launch_quantize(x, K, rows, o->ld, 0, &o->fmt, m, e, st);
+    Packed p;
+    const int rc = is_a ? resolve_operand(o, true, rows, K, g.la, ws, g.off_am, g.off_ae, &p, st) : resolve_operand(o, false, rows, K, g.lb, ws, g.off_bm, g.off_be, &p, st);
+    if (rc) return rc;
+    return launch_expand(p, g.fp, !is_a, f, st);
 }
 
 int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp_operand* b, float* C,
@@ -160,26 +181,26 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     const bool use_fp = g.fp.use && !P && workspace && ws_bytes >= g.total_fp && (reinterpret_cast<uintptr_t>(workspace) & 255) == 0 &&
                         (flags == HBFP_GEMM_AUTO || flags == HBFP_GEMM_FORCE_TENSOR) && (reinterpret_cast<uintptr_t>(C) & 3) == 0;
     char* ws = static_cast<char*>(workspace);
-    Packed pa, pb;
+    Packed pa{nullptr, nullptr, g.la, a->fmt.mant_bits}, pb{nullptr, nullptr, g.lb, b->fmt.mant_bits};
+    // a problem of a few hundred MOPs is over before a tensor-core kernel has filled its pipeline
+    const bool small = !P && (flags == HBFP_GEMM_AUTO || flags == HBFP_GEMM_FORCE_SMALL) && small_gemm_eligible(M, N, pa, pb, flags == HBFP_GEMM_FORCE_SMALL);
+    if (flags == HBFP_GEMM_FORCE_SMALL && !small) return HBFP_ERR_UNSUPPORTED;
+    if (use_fp && !small) {
+        const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
+        rc = resolve_form(a, true, M, K, g, ws, fa, st);
+        if (rc) return rc;
+        rc = resolve_form(b, false, N, K, g, ws, fb, st);
+        if (rc) return rc;
+        t_last_gemm_kernel = "gemm_tc_kernel";      // one SM per tile, like its integer sibling
+        return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, C, ldc, st);
+    }
     rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, st);
     if (rc) return rc;
     rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, st);
     if (rc) return rc;
-    // a problem of a few hundred MOPs is over before a tensor-core kernel has filled its pipeline
-    if (!P && (flags == HBFP_GEMM_AUTO || flags == HBFP_GEMM_FORCE_SMALL) &&
-        small_gemm_eligible(M, N, pa, pb, flags == HBFP_GEMM_FORCE_SMALL)) {
+    if (small) {
         t_last_gemm_kernel = "gemm_small_kernel";
         return launch_gemm_small(M, N, pa, pb, C, ldc, st);
-    }
-    if (flags == HBFP_GEMM_FORCE_SMALL) return HBFP_ERR_UNSUPPORTED;
-    if (use_fp) {
-        const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
-        rc = launch_expand(pa, g.fp, false, fa, st);
-        if (rc) return rc;
-        rc = launch_expand(pb, g.fp, true, fb, st);
-        if (rc) return rc;
-        t_last_gemm_kernel = "gemm_tc_kernel";      // one SM per tile, like its integer sibling
-        return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, C, ldc, st);
     }
     const bool quad_rows = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (ldc % 4) == 0;
     const bool want_tensor = flags != HBFP_GEMM_FORCE_SIMT && g.tp.supported &&

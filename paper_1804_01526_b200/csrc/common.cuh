@@ -130,8 +130,11 @@ struct FpPlan {
     int use;                // 0: the integer kernels
     int form, pair, ncol, splits, kb_per_split, planes_b;
 };
-FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb);
+FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, int passes);
 int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const FpOperand& out, cudaStream_t st);
+// Converts an FP32 operand straight to a form (quantize.cu); HBFP_ERR_UNSUPPORTED for weight tiles.
+int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int contract_axis, const hbfp_format* f, int wide, bool is_b,
+                         const FpOperand& out, cudaStream_t st);
 int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, float* C,
                    int64_t ldc, cudaStream_t st);
 

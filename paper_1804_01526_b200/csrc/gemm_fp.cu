@@ -698,17 +698,18 @@ inline int log2_of(int64_t v) { int l = 0; while ((1ll << l) < v) ++l; return l;
 
 }  // namespace
 
-FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb) {
+FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, int passes) {
     FpPlan f{};
     if (M <= 0 || N <= 0 || la.nkb <= 0 || la.planes != lb.planes || la.bp != lb.bp || la.nkb != lb.nkb || la.b != lb.b) return f;
     const bool w = la.planes == 2;
     // blocks of 128: the integer kernels are as fast (8 bits) or faster (12 bits, 4096 cube: 230 against 310 us)
     if (la.bp > 64) return f;
     if (M > (1ll << 28) || N > (1ll << 28) || la.kst > (1ll << 29)) return f;
-    // The forms cost a pass over both operands. It pays where every element is used often enough and the product is large
-    // (all with that pass): 2048 cube 34 against 51 us (8 bits, b = 32), 27 against 31 (b = 64), 48 against 58 (12 bits, b = 64),
-    // 4096 cube 186 / 290, 123 / 159, 261 / 368; but 1024 x 1024 x 2048 20 / 20, 18 / 14 and 24 / 18 us.
-    if (M * N < 600 * (M + N) || (double)M * (double)N * (double)(la.nkb * la.b) < 8.0e9) return f;
+    // Packed operands cost a pass each to take the form. It pays where every element is used often enough and the product is
+    // large (all with both passes): 2048 cube 34 against 51 us (8 bits, b = 32), 27 against 31 (b = 64), 48 against 58 (12 bits,
+    // b = 64), 4096 cube 186 / 290, 123 / 159, 261 / 368; but 1024 x 1024 x 2048 20 / 20, 18 / 14 and 24 / 18 us.
+    // FP32 operands are converted straight to the form, which pays at (nearly) every size: see below.
+    if (passes > 0 && (M * N < 600 * (M + N) || (double)M * (double)N * (double)(la.nkb * la.b) < 8.0e9)) return f;
     f.form = w ? FORM_W : FORM_S;
     const int64_t SMS = 148;                       // planning constant: the target part
     const int64_t nst = (la.nkb * la.bp + FP_STAGE_ELEMS - 1) / FP_STAGE_ELEMS;
@@ -724,6 +725,14 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb) {
             const double t = waves * ((double)((nst + sp - 1) / sp) * cost + 4.0 + (sp > 1 ? 3.0 : 0.0));
             if (t < best * 0.999) { best = t; f.ncol = ncol; f.splits = (int)sp; }
         }
+    }
+    // A few tiles with a long contraction want more splits than a cluster has CTAs: the integer kernels (split-K over the whole
+    // chip, a second launch adds the parts) take them, 64 x 64 x 16384 19 against 25 us, 576 x 64 x 32768 39 against 58. Otherwise
+    // from FP32 operands (b = 32): 128 x 10 x 1024 12 against 24 us, 512 x 512 x 1024 13 / 18, 1111 x 777 x 3001 41 / 47, 8192 x 256 x 256
+    // 13 / 15, 4096 cube 197 / 329.
+    {
+        const int64_t nout = w ? f.ncol / 2 : f.ncol, ctas = ((M + 127) / 128) * ((N + nout - 1) / nout) * f.splits;
+        if (ctas < 74 && nst / f.splits > 24) return FpPlan{};
     }
     // Blocks of 64 feed the tensor cores twice as fast as blocks of 32, and one SM's shared memory cannot deliver it: a stage
     // costs 48 KB written and 48 KB read (768 cycles) for 512 cycles of MMAs. A pair of SMs stages and reads a third less each

@@ -134,6 +134,86 @@ __device__ __forceinline__ void quantize_pack8(const float (&e8)[8], int s, cons
     pack4<PLANES>(h[2], h[3], hi.y, lo.y);
 }
 
+// ---- Output kinds. 1 and 2: the packed layout with one or two mantissa planes. The others are the operand forms of gemm_fp.cu,
+// rows of kst two-byte elements: FORM_SCALED bfloat16 q * 2^s, FORM_WIDE_A binary16 q, FORM_WIDE_B binary16 h and l with
+// q = 64 h + l (two planes plane_stride elements apart); the wide forms keep 2^s as floats in place of the exponents.
+// Writing the form here instead of expanding packed operands saves a pass over both: 1024 x 4096 x 4096 backward-weight, b = 32,
+// 94 -> 77 us; 4096 cube with 12 bits 354 -> 326 us; 1111 x 777 x 3001, b = 24, 65 -> 56 us.
+constexpr int FORM_SCALED = 3, FORM_WIDE_A = 4, FORM_WIDE_B = 5;
+__host__ __device__ constexpr bool is_form(int out) { return out >= FORM_SCALED; }
+// what the row and column kernels need beside the packed case
+struct FormArgs {
+    int32_t* status;      // FORM_WIDE_A: exponents beyond the GEMM's exact range are reported here
+};
+
+// Two rounded values (packed signed halfwords) as the form's elements: a (and for FORM_WIDE_B b) hold two elements each.
+template <int OUT>
+__device__ __forceinline__ void form_pair(uint32_t h, float two_s, uint32_t& a, uint32_t& b) {
+    // halfword + 2^15 in the low bits of 2^23: no integer-to-float conversion
+    const uint32_t u = h ^ 0x80008000u;
+    float f0 = __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7610)) - 8421376.0f;
+    float f1 = __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7632)) - 8421376.0f;
+    if (OUT == FORM_SCALED) {
+        a = __byte_perm(__float_as_uint(f0 * two_s), __float_as_uint(f1 * two_s), 0x7632);      // exact: the low halves are zero
+        b = 0;
+    } else {
+        float l0 = 0.f, l1 = 0.f;
+        if (OUT == FORM_WIDE_B) {
+            const float h0 = __fmaf_rn(f0, 0.015625f, 12582912.0f) - 12582912.0f, h1 = __fmaf_rn(f1, 0.015625f, 12582912.0f) - 12582912.0f;
+            l0 = __fmaf_rn(-64.0f, h0, f0);                                                       // in [-32, 32]
+            l1 = __fmaf_rn(-64.0f, h1, f1);
+            f0 = h0; f1 = h1;
+        }
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(a) : "f"(f1), "f"(f0));
+        if (OUT == FORM_WIDE_B) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(b) : "f"(l1), "f"(l0));
+        else b = 0;
+    }
+}
+// Eight consecutive values with the exponent s: sixteen bytes of the form (two planes for FORM_WIDE_B).
+template <bool SR, int OUT>
+__device__ __forceinline__ void quantize_form8(const float (&e8)[8], int s, const QParams& p, uint4 w, uint4& a, uint4& b) {
+    const uint32_t qm = qmax_pair(p.qmax), nqm = neg_qmax_pair(p.qmax);
+    const float sc = pow2f(SR ? 16 - s : -s), two_s = pow2f(s);
+    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+    uint32_t ra[4], rb[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const uint32_t h = SR ? round_sr_pair(e8[2 * j], e8[2 * j + 1], sc, ww[j], qm, nqm) : round_rne_pair(e8[2 * j], e8[2 * j + 1], sc, qm, nqm);
+        form_pair<OUT>(h, two_s, ra[j], rb[j]);
+    }
+    a = make_uint4(ra[0], ra[1], ra[2], ra[3]);
+    b = make_uint4(rb[0], rb[1], rb[2], rb[3]);
+}
+// The exponent (packed), nothing (FORM_SCALED) or the scale of a block.
+template <int OUT>
+__device__ __forceinline__ void store_exponent(int8_t* exps, int64_t at, int s) {
+    if (!is_form(OUT)) exps[at] = (int8_t)s;
+    else if (OUT != FORM_SCALED) reinterpret_cast<float*>(exps)[at] = pow2f(s);
+}
+// Eight consecutive elements at element offset `at` of the row-major result.
+template <bool SR, int OUT>
+__device__ __forceinline__ void round_and_store8(const float (&e8)[8], int s, const QParams& p, uint4 w, int8_t* mant, int64_t at, int64_t plane_stride, bool store) {
+    if constexpr (is_form(OUT)) {
+        uint4 a, b;
+        quantize_form8<SR, OUT>(e8, s, p, w, a, b);
+        if (store) {
+            *reinterpret_cast<uint4*>(mant + 2 * at) = a;
+            if (OUT == FORM_WIDE_B) *reinterpret_cast<uint4*>(mant + 2 * (at + plane_stride)) = b;
+        }
+    } else {
+        uint2 hi, lo;
+        quantize_pack8<SR, OUT>(e8, s, p, w, hi, lo);
+        if (store) {
+            *reinterpret_cast<uint2*>(mant + at) = hi;
+            if (OUT == 2) *reinterpret_cast<uint2*>(mant + plane_stride + at) = lo;
+        }
+    }
+}
+template <int OUT>
+__device__ __forceinline__ void check_exponent(int s, const FormArgs& fa) {
+    if (OUT == FORM_WIDE_A && s > 96) atomicCAS(fa.status, 0, STATUS_EXPONENT_RANGE);
+}
+
 // round-half-even( x * 2^-s ), saturated
 __device__ __forceinline__ int round_rne(float x, int s, int qmax) {
     float y = __fmul_rn(x, pow2f(-s));           // s >= -63 and s <= 126 for finite input, m >= 3
@@ -199,7 +279,7 @@ template <int LPB, bool SR, int PLANES>
 __global__ void __launch_bounds__(256)
 quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-               int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const int8_t* __restrict__ given = nullptr) {
+               int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const int8_t* __restrict__ given = nullptr, const FormArgs fa = FormArgs{}) {
     // given != nullptr: one exponent per row for the whole axis, computed beforehand (a block longer than the
     // tile); the kernel then only rounds and packs
     constexpr int B = 8 * LPB;
@@ -248,26 +328,26 @@ quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
             for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
             const int s = given ? (r < rows ? (int)given[r] : -63) : block_exponent(am, p.m, p.exp_mode);
             const uint4 w = wd[i];
-            uint2 hi, lo;
-            quantize_pack8<SR, PLANES>(e8, s, p, w, hi, lo);
-            if (r < rows && col < kst) {
-                *reinterpret_cast<uint2*>(mant + r * kst + col) = hi;
-                if (PLANES == 2) *reinterpret_cast<uint2*>(mant + plane_stride + r * kst + col) = lo;
-            }
+            round_and_store8<SR, PLANES>(e8, s, p, w, mant, r * kst + col, plane_stride, r < rows && col < kst);
+            check_exponent<PLANES>(s, fa);
             if ((lane % LPB) == 0 && r < rows && col < K)
                 s_exps[span * KB_PER_SPAN + lane / LPB][warp * 4 + i] = (int8_t)s;
         }
     }
     __syncthreads();
-    if (given) return;
+    if (given || PLANES == FORM_SCALED) return;
     // exponents: [kb][row], 32 rows of one block are 32 contiguous bytes.
     const int64_t kb0 = c0 / B;
     for (int i = tid; i < KB_PER_TILE * 8; i += 256) {
         const int kbl = i >> 3, part = i & 7;
         const int64_t kb = kb0 + kbl, r = r0 + part * 4;
-        if (kb < nkb && r < rs)
-            *reinterpret_cast<uint32_t*>(exps + kb * rs + r) =
-                *reinterpret_cast<const uint32_t*>(&s_exps[kbl][part * 4]);
+        if (kb < nkb && r < rs) {
+            const uint32_t e4 = *reinterpret_cast<const uint32_t*>(&s_exps[kbl][part * 4]);
+            if (is_form(PLANES))
+                *reinterpret_cast<float4*>(reinterpret_cast<float*>(exps) + kb * rs + r) =
+                    make_float4(pow2f((int8_t)e4), pow2f((int8_t)(e4 >> 8)), pow2f((int8_t)(e4 >> 16)), pow2f((int8_t)(e4 >> 24)));
+            else *reinterpret_cast<uint32_t*>(exps + kb * rs + r) = e4;
+        }
     }
 }
 
@@ -285,11 +365,11 @@ template <int PLANES, int RQ, bool SR>      // RQ = bp / 4: padded rows per warp
 __global__ void __launch_bounds__(128)
 quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
                 int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n) {
-    constexpr int BP = 4 * RQ;
+                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa) {
+    constexpr int BP = 4 * RQ, BYTE_PLANES = is_form(PLANES) ? 1 : PLANES;
     __shared__ uint32_t pmax[4][COLT];
     __shared__ __align__(16) uint4 rnd[SR ? BP : 1][5];          // draws of a row: its 32 columns lie in at most five groups of eight
-    __shared__ __align__(16) unsigned char s_out[PLANES][COLT][BP + 16];
+    __shared__ __align__(16) unsigned char s_out[BYTE_PLANES][is_form(PLANES) ? 1 : COLT][BP + 16];
     const int tid = threadIdx.x, c = tid & 31, q = tid >> 5;
     const int64_t kb = blockIdx.x / tiles_n, c0 = (int64_t)(blockIdx.x - (unsigned)kb * tiles_n) * COLT;
     const int64_t k0 = kb * b, col = c0 + c;
@@ -314,11 +394,14 @@ quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
     __syncthreads();
     am = max(max(pmax[0][c], pmax[1][c]), max(pmax[2][c], pmax[3][c]));
     const int s = block_exponent(am, p.m, p.exp_mode);
-    if (q == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
+    check_exponent<PLANES>(s, fa);
+    if constexpr (is_form(PLANES)) { if (q == 0 && col < R) store_exponent<PLANES>(exps, kb * rs + col, s); }
+    else if (q == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
     const uint32_t qm = qmax_pair(p.qmax), nqm = neg_qmax_pair(p.qmax);
     const float sc = pow2f(SR ? 16 - s : -s);
     const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd);
     const uint32_t first = SR ? (uint32_t)((uint64_t)(k0 * R + c0) & 7) : 0u, row_step = (uint32_t)(R & 7);
+    uint32_t fo[is_form(PLANES) ? 2 : 1][RQ / 2];               // the form's elements of this thread, pair by pair
 #pragma unroll
     for (int w = 0; w < RQ / 4; ++w) {
         uint32_t h[2], hi, lo;
@@ -335,15 +418,32 @@ quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
                 h[k] = round_rne_pair(v[j], v[j + 1], sc, qm, nqm);
             }
         }
-        pack4<PLANES>(h[0], h[1], hi, lo);
-        *reinterpret_cast<uint32_t*>(&s_out[0][c][q * RQ + 4 * w]) = hi;
-        if (PLANES == 2) *reinterpret_cast<uint32_t*>(&s_out[PLANES - 1][c][q * RQ + 4 * w]) = lo;
+        if constexpr (is_form(PLANES)) {
+            form_pair<PLANES>(h[0], pow2f(s), fo[0][2 * w], fo[1][2 * w]);
+            form_pair<PLANES>(h[1], pow2f(s), fo[0][2 * w + 1], fo[1][2 * w + 1]);
+        } else {
+            pack4<BYTE_PLANES>(h[0], h[1], hi, lo);
+            *reinterpret_cast<uint32_t*>(&s_out[0][c][q * RQ + 4 * w]) = hi;
+            if (PLANES == 2) *reinterpret_cast<uint32_t*>(&s_out[BYTE_PLANES - 1][c][q * RQ + 4 * w]) = lo;
+        }
+    }
+    if constexpr (is_form(PLANES)) {
+        if (col >= R) return;
+#pragma unroll
+        for (int pl = 0; pl < (PLANES == FORM_WIDE_B ? 2 : 1); ++pl) {
+            uint4* dst = reinterpret_cast<uint4*>(mant + 2 * (pl * plane_stride + col * kst + kb * BP + q * RQ));
+#pragma unroll
+            for (int i = 0; i < RQ / 8; ++i) dst[i] = make_uint4(fo[pl][4 * i], fo[pl][4 * i + 1], fo[pl][4 * i + 2], fo[pl][4 * i + 3]);
+            if (kb == nkb - 1 && q == 0)                          // the row tail [nkb * bp, kst)
+                for (int64_t o = nkb * BP; o < kst; o += 8) *reinterpret_cast<uint4*>(mant + 2 * (pl * plane_stride + col * kst + o)) = make_uint4(0, 0, 0, 0);
+        }
+        return;
     }
     __syncthreads();
     // neighbouring threads write neighbouring 16-byte pieces of an output row
     constexpr int PPR = BP / 16;
 #pragma unroll
-    for (int pl = 0; pl < PLANES; ++pl)
+    for (int pl = 0; pl < BYTE_PLANES; ++pl)
         for (int i = tid; i < COLT * PPR; i += 128) {
             const int r = i / PPR, piece = i - r * PPR;
             if (c0 + r < R)
@@ -351,7 +451,7 @@ quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
                     *reinterpret_cast<const uint4*>(&s_out[pl][r][16 * piece]);
         }
     // the row tail [nkb * bp, kst)
-    if (kb == nkb - 1 && q < PLANES && col < R)
+    if (kb == nkb - 1 && q < BYTE_PLANES && col < R)
         for (int64_t o = nkb * BP; o < kst; o += 16)
             *reinterpret_cast<uint4*>(mant + q * plane_stride + col * kst + o) = make_uint4(0, 0, 0, 0);
 }
@@ -1316,7 +1416,7 @@ template <int LPB, bool SR, int PLANES, int ITEMS>
 __global__ void __launch_bounds__(256)
 quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-               int8_t* __restrict__ exps, int64_t rs, uint32_t gpr, uint32_t total_groups) {
+               int8_t* __restrict__ exps, int64_t rs, uint32_t gpr, uint32_t total_groups, const FormArgs fa) {
     constexpr int B = 8 * LPB;
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t g0 = blockIdx.x * (256u * ITEMS) + tid;
@@ -1358,31 +1458,25 @@ quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
         for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
         const int s = block_exponent(am, p.m, p.exp_mode);
         const uint4 w = wd[j];
-        uint2 hi, lo;
-        quantize_pack8<SR, PLANES>(e8, s, p, w, hi, lo);
-        if (live) {
-            int8_t* dst = mant + (int64_t)rw[j] * kst + cc[j];
-            *reinterpret_cast<uint2*>(dst) = hi;
-            if (PLANES == 2) *reinterpret_cast<uint2*>(dst + plane_stride) = lo;
-            // blocks that lie in the padding beyond K have no exponent
-            if ((lane % LPB) == 0 && cc[j] < K) exps[(int64_t)(cc[j] / B) * rs + rw[j]] = (int8_t)s;
-        }
+        round_and_store8<SR, PLANES>(e8, s, p, w, mant, (int64_t)rw[j] * kst + cc[j], plane_stride, live);
+        check_exponent<PLANES>(s, fa);
+        // blocks that lie in the padding beyond K have no exponent
+        if (live && (lane % LPB) == 0 && cc[j] < K) store_exponent<PLANES>(exps, (int64_t)(cc[j] / B) * rs + rw[j], s);
     }
-    zero_padding_lines(exps, rows, rs, K / B);
+    if (!is_form(PLANES)) zero_padding_lines(exps, rows, rs, K / B);
 }
 
-template <int LPB, int ITEMS>
+// FORM: 0 for the packed layout (its planes as L says), else the form to write.
+template <int LPB, int ITEMS, int FORM>
 int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
-                          int8_t* mant, int8_t* exps, cudaStream_t st) {
+                          int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa) {
     const uint32_t gpr = (uint32_t)(L.kst / 8), total = (uint32_t)(rows * (L.kst / 8));
     const unsigned grid = (total + 256u * ITEMS - 1u) / (256u * ITEMS);
-    if (p.rounding == 1) {
-        if (L.planes == 1) quant_row_flat<LPB, true, 1, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total);
-        else quant_row_flat<LPB, true, 2, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total);
-    } else {
-        if (L.planes == 1) quant_row_flat<LPB, false, 1, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total);
-        else quant_row_flat<LPB, false, 2, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total);
-    }
+#define HBFP_QFLAT(SRV, OUT) quant_row_flat<LPB, SRV, OUT, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
+    if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QFLAT(true, FORM); else HBFP_QFLAT(false, FORM); }
+    else if (p.rounding == 1) { if (L.planes == 1) HBFP_QFLAT(true, 1); else HBFP_QFLAT(true, 2); }
+    else { if (L.planes == 1) HBFP_QFLAT(false, 1); else HBFP_QFLAT(false, 2); }
+#undef HBFP_QFLAT
     return launch_status();
 }
 
@@ -1391,11 +1485,11 @@ int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, c
 // nearest-even rounding; 91 / 84 / 82 us with stochastic rounding (the Philox state of every group in flight
 // is live). Narrow rows (one or two 128-byte units, e.g. one block of 64 channels per pixel, half of whose
 // groups are padding that loads nothing) do best with two.
-template <int LPB>
+template <int LPB, int FORM = 0>
 int launch_row_flat(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
-                    int8_t* mant, int8_t* exps, cudaStream_t st) {
-    if (L.kst > 256 && p.rounding == 0) return launch_row_flat_items<LPB, 4>(x, rows, K, ld, p, L, mant, exps, st);
-    return launch_row_flat_items<LPB, 2>(x, rows, K, ld, p, L, mant, exps, st);
+                    int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa = FormArgs{}) {
+    if (L.kst > 256 && p.rounding == 0) return launch_row_flat_items<LPB, 4, FORM>(x, rows, K, ld, p, L, mant, exps, st, fa);
+    return launch_row_flat_items<LPB, 2, FORM>(x, rows, K, ld, p, L, mant, exps, st, fa);
 }
 
 // ------------------------------------------------------------------------------ quant_row_ragged
@@ -1411,7 +1505,7 @@ template <int LPB, bool SR, int PLANES, bool VEC>
 __global__ void __launch_bounds__(256)
 quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int b, QParams p,
                  int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, uint32_t ppr, int64_t total) {
+                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, uint32_t ppr, int64_t total, const FormArgs fa) {
     constexpr int ITEMS = 2;
     const int tid = threadIdx.x, lane = tid & 31;
     float e8[ITEMS][8];
@@ -1460,27 +1554,23 @@ quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t l
 #pragma unroll
         for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
         const int s = block_exponent(am, p.m, p.exp_mode);
-        uint2 hi, lo;
-        quantize_pack8<SR, PLANES>(e8[i], s, p, w, hi, lo);
-        if (live) {
-            const int pc = cb[i] * LPB + (kk0[i] - cb[i] * b) / 8;
-            int8_t* dst = mant + row[i] * kst + 8 * (int64_t)pc;
-            *reinterpret_cast<uint2*>(dst) = hi;
-            if (PLANES == 2) *reinterpret_cast<uint2*>(dst + plane_stride) = lo;
-            if ((lane % LPB) == 0 && cb[i] < nkb) exps[(int64_t)cb[i] * rs + row[i]] = (int8_t)s;
-        }
+        const int pc = cb[i] * LPB + (kk0[i] - cb[i] * b) / 8;
+        round_and_store8<SR, PLANES>(e8[i], s, p, w, mant, row[i] * kst + 8 * (int64_t)pc, plane_stride, live);
+        check_exponent<PLANES>(s, fa);
+        if (live && (lane % LPB) == 0 && cb[i] < nkb) store_exponent<PLANES>(exps, (int64_t)cb[i] * rs + row[i], s);
     }
-    zero_padding_lines(exps, rows, rs, nkb);
+    if (!is_form(PLANES)) zero_padding_lines(exps, rows, rs, nkb);
 }
 
-template <int LPB, bool VEC>
+template <int LPB, bool VEC, int FORM = 0>
 int launch_row_ragged(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
-                      int8_t* mant, int8_t* exps, cudaStream_t st) {
+                      int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa = FormArgs{}) {
     const uint32_t ppr = (uint32_t)(L.kst / 8);
     const int64_t total = rows * ppr;
     const unsigned grid = (unsigned)((total + 511) / 512);
-#define HBFP_QROW_RAGGED(SRV, PL) quant_row_ragged<LPB, SRV, PL, VEC><<<grid, 256, 0, st>>>(x, rows, K, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, ppr, total)
-    if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_RAGGED(true, 1); else HBFP_QROW_RAGGED(true, 2); }
+#define HBFP_QROW_RAGGED(SRV, PL) quant_row_ragged<LPB, SRV, PL, VEC><<<grid, 256, 0, st>>>(x, rows, K, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, ppr, total, fa)
+    if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QROW_RAGGED(true, FORM); else HBFP_QROW_RAGGED(false, FORM); }
+    else if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_RAGGED(true, 1); else HBFP_QROW_RAGGED(true, 2); }
     else { if (L.planes == 1) HBFP_QROW_RAGGED(false, 1); else HBFP_QROW_RAGGED(false, 2); }
 #undef HBFP_QROW_RAGGED
     return launch_status();
@@ -1508,14 +1598,15 @@ __global__ void __launch_bounds__(QC_THREADS)
 quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapM0,
               const __grid_constant__ CUtensorMap mapM1, QParams p, int8_t* __restrict__ exps, int64_t rs,
               int64_t nkb, int64_t K, int64_t R, int tiles_n, int total_tiles, int32_t* status,
-              const int8_t* __restrict__ given) {
+              const int8_t* __restrict__ given, int8_t* __restrict__ form_out, int64_t kst, int64_t plane_stride) {
     // given != nullptr: one exponent per column for the whole axis, computed beforehand (blocks longer than a
     // tile); the kernel then only rounds and packs
     extern __shared__ unsigned char smem_dyn[];
     const uint32_t base = (smem_u32(smem_dyn) + 1023u) & ~1023u;
     unsigned char* base_ptr = smem_dyn + (base - smem_u32(smem_dyn));
     // [out planes | in stages | draws (stochastic) | block maxima | barriers]
-    constexpr int OFF_IN = PLANES * QC_OUT_BYTES;
+    // forms leave from registers: a thread's 32 consecutive k are two whole sectors of its output row
+    constexpr int OFF_IN = is_form(PLANES) ? 0 : PLANES * QC_OUT_BYTES;
     constexpr int OFF_RND = OFF_IN + QC_STAGES * QC_IN_BYTES;
     constexpr int OFF_PMAX = OFF_RND + (SR ? QC_ROWS * QC_COLS * 2 : 0);
     constexpr int OFF_BAR = OFF_PMAX + 4 * QC_COLS * 4;
@@ -1584,9 +1675,15 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
         if (LB == 1) am = max(pmax[(q & 2) * QC_COLS + n], pmax[((q & 2) + 1) * QC_COLS + n]);
         const int sexp = given ? (col < R ? (int)given[col] : -63) : block_exponent(am, p.m, p.exp_mode);
         const int64_t kb = ((int64_t)kt << LB) + (q >> (2 - LB));
-        if (!given && (q & ((4 >> LB) - 1)) == 0 && kb < nkb && col < rs) exps[kb * rs + col] = col < R ? (int8_t)sexp : (int8_t)0;   // padding lines: zero
+        if constexpr (is_form(PLANES)) {
+            check_exponent<PLANES>(sexp, FormArgs{status});
+            if ((q & ((4 >> LB) - 1)) == 0 && kb < nkb && col < R) store_exponent<PLANES>(exps, kb * rs + col, sexp);
+        } else if (!given && (q & ((4 >> LB) - 1)) == 0 && kb < nkb && col < rs) {
+            exps[kb * rs + col] = col < R ? (int8_t)sexp : (int8_t)0;   // padding lines: zero
+        }
 
         uint32_t hi[8], lo[8];
+        uint32_t fo[is_form(PLANES) ? 2 : 1][16];
         const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd);
         const uint32_t qm = qmax_pair(p.qmax), nqm = neg_qmax_pair(p.qmax);
         const float sc = pow2f(SR ? 16 - sexp : -sexp);
@@ -1603,7 +1700,25 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
                     h[k] = round_rne_pair(v[j], v[j + 1], sc, qm, nqm);
                 }
             }
-            pack4<PLANES>(h[0], h[1], hi[w], lo[w]);
+            if constexpr (is_form(PLANES)) {
+                form_pair<PLANES>(h[0], pow2f(sexp), fo[0][2 * w], fo[1][2 * w]);
+                form_pair<PLANES>(h[1], pow2f(sexp), fo[0][2 * w + 1], fo[1][2 * w + 1]);
+            } else {
+                pack4<PLANES>(h[0], h[1], hi[w], lo[w]);
+            }
+        }
+        if constexpr (is_form(PLANES)) {
+            if (col < R) {
+#pragma unroll
+                for (int pl = 0; pl < (PLANES == FORM_WIDE_B ? 2 : 1); ++pl) {
+                    int8_t* dst = form_out + 2 * (pl * plane_stride + col * kst + (int64_t)kt * QC_ROWS + 32 * q);
+                    store_sector(dst, &fo[pl][0]);
+                    store_sector(dst + 32, &fo[pl][8]);
+                }
+            }
+            if (SR) __syncthreads();                             // the table of draws is rewritten by the next tile
+            if (++s == QC_STAGES) { s = 0; ph ^= 1u; }
+            continue;
         }
         // 128B swizzle of the store tile: 16-byte chunk c of row n sits at chunk position c ^ (n % 8)
         unsigned char* orow = base_ptr + (n >> 3) * 1024 + (n & 7) * 128;
@@ -1653,14 +1768,17 @@ int launch_col_tma(const float* x, int64_t K, int64_t rows, int64_t ld, const QP
     CUtensorMap mX, mM0, mM1;
     int rc = make_map(&mX, x, (uint64_t)rows * 4, (uint64_t)K, (uint64_t)ld * 4, QC_COLS * 4, QC_ROWS, false);
     if (rc) return rc;
-    rc = make_map(&mM0, mant, (uint64_t)L.kst, (uint64_t)rows, (uint64_t)L.kst, QC_ROWS, QC_COLS, true);
-    if (rc) return rc;
+    mM0 = mX;
+    if (!is_form(PLANES)) {
+        rc = make_map(&mM0, mant, (uint64_t)L.kst, (uint64_t)rows, (uint64_t)L.kst, QC_ROWS, QC_COLS, true);
+        if (rc) return rc;
+    }
     mM1 = mM0;
     if (PLANES == 2) {
         rc = make_map(&mM1, mant + L.plane_stride, (uint64_t)L.kst, (uint64_t)rows, (uint64_t)L.kst, QC_ROWS, QC_COLS, true);
         if (rc) return rc;
     }
-    constexpr int smem = 1024 + PLANES * QC_OUT_BYTES + QC_STAGES * QC_IN_BYTES + (SR ? QC_ROWS * QC_COLS * 2 : 0) +
+    constexpr int smem = 1024 + (is_form(PLANES) ? 0 : PLANES * QC_OUT_BYTES) + QC_STAGES * QC_IN_BYTES + (SR ? QC_ROWS * QC_COLS * 2 : 0) +
                          4 * QC_COLS * 4 + 64;
     // attribute and occupancy belong to the device: cached per device ordinal
     static int ctas_per_sm_dev[MAX_DEVICES] = {};
@@ -1680,7 +1798,7 @@ int launch_col_tma(const float* x, int64_t K, int64_t rows, int64_t ld, const QP
     const int64_t cap = (int64_t)sm_count() * ctas_per_sm;
     const int grid = (int)(total < cap ? total : cap);
     quant_col_tma<PLANES, LB, SR><<<grid, QC_THREADS, smem, st>>>(mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
-                                                              (int)total, status, given);
+                                                              (int)total, status, given, mant, L.kst, L.plane_stride);
     return launch_status();
 }
 
@@ -1846,7 +1964,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     // every other block length up to 128, any pitch and alignment
     if (f->tile == 0 && axis == 0 && L.b <= 128 && ((rows + COLT - 1) / COLT) * L.nkb < (1ll << 31)) {
         const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
-#define HBFP_QCOL(PL, RQ, SRV) quant_col_block<PL, RQ, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, tiles_n)
+#define HBFP_QCOL(PL, RQ, SRV) quant_col_block<PL, RQ, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, tiles_n, FormArgs{})
 #define HBFP_QCOL_SR(PL, RQ) do { if (p.rounding) HBFP_QCOL(PL, RQ, true); else HBFP_QCOL(PL, RQ, false); } while (0)
         if (L.planes == 1) { if (L.bp == 32) HBFP_QCOL_SR(1, 8); else if (L.bp == 64) HBFP_QCOL_SR(1, 16); else HBFP_QCOL_SR(1, 32); }
         else { if (L.bp == 32) HBFP_QCOL_SR(2, 8); else if (L.bp == 64) HBFP_QCOL_SR(2, 16); else HBFP_QCOL_SR(2, 32); }
@@ -1887,6 +2005,64 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     else
         mant_generic<2><<<blocks_for(rows * (L.kst / 4), 256), 256, 0, st>>>(x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     return launch_status();
+}
+
+namespace {
+
+template <int FORM>
+int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows, int64_t K, const QParams& p, const Layout& L, int8_t* out, int8_t* scales,
+                  const FormArgs& fa, cudaStream_t st) {
+    const bool aligned = ((reinterpret_cast<uintptr_t>(x) & 15) == 0) && (ld % 4 == 0);
+    if (axis == 1) {
+        if (aligned && L.b == L.bp && K % L.b == 0 && L.kst % 512 != 0 && rows * (L.kst / 8) < (1ll << 32) - 4096)
+            return L.b == 32 ? launch_row_flat<4, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_flat<8, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
+        if (aligned && d1 % 8 == 0 && L.b == L.bp && rows <= 32ll * 65535) {
+            const dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
+#define HBFP_QFAST(LPB, SRV) quant_row_fast<LPB, SRV, FORM><<<grid, 256, 0, st>>>(x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
+            if (L.b == 32) { if (p.rounding) HBFP_QFAST(4, true); else HBFP_QFAST(4, false); }
+            else { if (p.rounding) HBFP_QFAST(8, true); else HBFP_QFAST(8, false); }
+#undef HBFP_QFAST
+            return launch_status();
+        }
+        if (K >= (1ll << 30) || rows * (L.kst / 8) >= (1ll << 39)) return HBFP_ERR_UNSUPPORTED;
+        const bool vec = aligned && L.b % 4 == 0;
+        if (L.bp == 32) return vec ? launch_row_ragged<4, true, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_ragged<4, false, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
+        return vec ? launch_row_ragged<8, true, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_ragged<8, false, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
+    }
+    if (aligned && L.b == L.bp && (p.rounding == 0 || rows % 8 == 0) && rows < (1ll << 29) && K < (1ll << 31) &&
+        ((rows + QC_COLS - 1) / QC_COLS) * (L.kst / QC_ROWS) < (1ll << 31)) {
+        if (L.b == 64) return p.rounding ? launch_col_tma<FORM, 1, true>(x, K, rows, ld, p, L, out, scales, st) : launch_col_tma<FORM, 1, false>(x, K, rows, ld, p, L, out, scales, st);
+        return p.rounding ? launch_col_tma<FORM, 2, true>(x, K, rows, ld, p, L, out, scales, st) : launch_col_tma<FORM, 2, false>(x, K, rows, ld, p, L, out, scales, st);
+    }
+    if (((rows + COLT - 1) / COLT) * L.nkb >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
+    const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
+#define HBFP_QCOL(RQ, SRV) quant_col_block<FORM, RQ, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, (int)L.b, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, tiles_n, fa)
+    if (L.bp == 32) { if (p.rounding) HBFP_QCOL(8, true); else HBFP_QCOL(8, false); }
+    else { if (p.rounding) HBFP_QCOL(16, true); else HBFP_QCOL(16, false); }
+#undef HBFP_QCOL
+    return launch_status();
+}
+
+}  // namespace
+
+// Converts an FP32 operand straight to a floating-point operand form: blocks of at most 64, no weight tiles, elements
+// aligned to 32 bytes (HBFP_ERR_UNSUPPORTED otherwise; the caller converts to the packed layout and expands that).
+int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f, int wide, bool is_b, const FpOperand& o,
+                         cudaStream_t st) {
+    const int64_t K = axis == 1 ? d1 : d0, rows = axis == 1 ? d0 : d1;
+    Layout L;
+    int rc = make_layout(rows, K, f, &L);
+    if (rc) return rc;
+    if (f->tile != 0 || L.bp > 64 || rows == 0 || K == 0 || (L.planes == 2) != (wide != 0)) return HBFP_ERR_UNSUPPORTED;
+    const QParams p = make_params(f);
+    const FormArgs fa{device_status_word()};
+    if (!fa.status) return HBFP_ERR_CUDA;
+    int8_t* out = static_cast<int8_t*>(o.p0);
+    int8_t* scales = reinterpret_cast<int8_t*>(o.scales);
+    if (is_b && wide) L.plane_stride = (static_cast<int8_t*>(o.p1) - out) / 2;        // in elements
+    if (!wide) return quantize_form<FORM_SCALED>(x, d1, ld, axis, rows, K, p, L, out, scales, fa, st);
+    return is_b ? quantize_form<FORM_WIDE_B>(x, d1, ld, axis, rows, K, p, L, out, scales, fa, st)
+                : quantize_form<FORM_WIDE_A>(x, d1, ld, axis, rows, K, p, L, out, scales, fa, st);
 }
 
 namespace {

@@ -440,3 +440,20 @@ def test_floating_point_operand_forms_are_bit_equal_to_the_sequential_definition
             assert torch.equal(got, want)
             assert torch.equal(hb.gemm_q(M, N, K, pa, pb, out=out), want)
         assert bool((buf[:, 0] == 7).all()) and bool((buf[:, N + 1:] == 7).all())
+
+
+@pytest.mark.parametrize("m,b,M,N,K,rounding", [(8, 24, 1, 1, 100, 1), (8, 32, 130, 70, 1024, 0), (8, 64, 16, 4096, 4096, 1), (12, 64, 129, 65, 2048, 1),
+                                                (12, 24, 257, 10, 700, 0), (8, 32, 640, 500, 33, 1), (5, 40, 1000, 260, 900, 0)])
+@pytest.mark.parametrize("tA,tB", [(0, 0), (1, 1)])
+def test_small_products_of_fp32_operands_converted_straight_to_the_form(hb, m, b, M, N, K, rounding, tA, tB):
+    """FP32 operands of both storage orders, few tiles, K split over the CTAs of a cluster: within 1e-6 of the accumulator
+    magnitude of the product of the packed operands."""
+    import torch
+    A = to_dev(wl.draw("outliers", (K, M) if tA else (M, K), seed=95))
+    B = to_dev(wl.draw("normal", (N, K) if tB else (K, N), seed=96))
+    fa, fb = hb.Format(m, b, rounding=rounding, seed=6), hb.Format(m, b, rounding=rounding, seed=6, stream_id=1)
+    C = hb.gemm(tA, tB, A, B, fa, fb, flags=hb.GEMM_FORCE_TENSOR)
+    pa, pb = hb.quantize(A, 0 if tA else 1, fa), hb.quantize(B, 1 if tB else 0, fb)
+    da, db = hb.dequantize(pa).double(), hb.dequantize(pb).double()
+    assert hb.device_status() == 0
+    assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
