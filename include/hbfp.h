@@ -183,6 +183,8 @@ HBFP_API int hbfp_conv_dgrad_filters(const void* mant_c1, const int8_t* exps_c1,
  *   hbfp_wide_update    wide <- 16-bit quantisation of fl32(wide * 2^s16 + delta) with fresh tile
  *                       exponents, in place; delta: FP32 [d0][d1], pitch ldd >= d1 (the update the
  *                       optimiser computed in FP32, Sec. 5.1) (+ narrow views of the new weights)
+ *   hbfp_wide_update_value  the same, and the FP32 value of the new weights (what hbfp_wide_dequantize gives) to
+ *                       `value` (device, [d0][d1], pitch ldv >= d1) in the same pass; NULL skips it
  *   hbfp_wide_narrow    wide storage -> narrow views only (reads 2 bytes per weight)
  * One launch, one CTA per tile; asynchronous on `stream`. Errors: HBFP_ERR_INVALID_ARG (null or
  * inconsistent arguments, tile != block), HBFP_ERR_UNSUPPORTED (tile > 128, m outside 3..12),
@@ -193,6 +195,9 @@ HBFP_API int hbfp_wide_quantize(const float* w, int64_t d0, int64_t d1, int64_t 
 HBFP_API int hbfp_wide_update(int16_t* wide, int8_t* wide_exps, const float* delta, int64_t d0, int64_t d1,
                               int64_t ldd, const hbfp_format* fmt, void* mant_c0, int8_t* exps_c0,
                               void* mant_c1, int8_t* exps_c1, void* stream);
+HBFP_API int hbfp_wide_update_value(int16_t* wide, int8_t* wide_exps, const float* delta, int64_t d0, int64_t d1,
+                                    int64_t ldd, const hbfp_format* fmt, void* mant_c0, int8_t* exps_c0,
+                                    void* mant_c1, int8_t* exps_c1, float* value, int64_t ldv, void* stream);
 HBFP_API int hbfp_wide_narrow(const int16_t* wide, const int8_t* wide_exps, int64_t d0, int64_t d1,
                               const hbfp_format* fmt, void* mant_c0, int8_t* exps_c0, void* mant_c1,
                               int8_t* exps_c1, void* stream);

@@ -11,7 +11,7 @@ no arithmetic of its own:
 * forward and backward-data read those views (``hbfp_gemm_q``), so the backward pass converts no
   weights; activations and gradients are converted by the GEMM call with 1-D blocks along the
   contraction axis; backward-weight is ``hbfp_gemm`` with ``transA = 1``;
-* ``apply_update(delta)`` hands the optimiser's FP32 update to ``hbfp_wide_update`` and refreshes the
+* ``apply_update(delta)`` hands the optimiser's FP32 update to ``hbfp_wide_update_value`` and refreshes the
   views in the same launch.
 
 Stochastic rounding draws are keyed by (seed + step, stream id, element index): a layer takes three
@@ -79,10 +79,9 @@ class HbfpLinear(torch.nn.Module):
         self.weight.data = hb.wide_dequantize(self.wide)
 
     def apply_update(self, delta: torch.Tensor) -> None:
-        """``W <- Q16(float32(W + delta))`` in wide storage, views refreshed by the same launch."""
+        """``W <- Q16(float32(W + delta))`` in wide storage, views and the FP32 copy refreshed by the same launch."""
         self.steps += 1
-        hb.wide_update(self.wide, delta.contiguous(), self.fmt_weight(), views=self.views)
-        self._refresh_fp32_copy()
+        self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         return _HbfpLinearFn.apply(x, self.weight, self.bias, self)
@@ -171,8 +170,7 @@ class HbfpConv3x3(torch.nn.Module):
         self.weight.data = hb.wide_dequantize(self.wide)
 
     def apply_update(self, delta: torch.Tensor) -> None:
-        hb.wide_update(self.wide, delta.contiguous(), self.fmt_weight(), views=self.views)
-        self._refresh_fp32_copy()
+        self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         return _HbfpConv3x3Fn.apply(x, self.weight, self)

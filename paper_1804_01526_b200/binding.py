@@ -28,7 +28,7 @@ EXPORTS = [
     "hbfp_status_string", "hbfp_packed_layout", "hbfp_packed_sizes", "hbfp_quantize",
     "hbfp_quantize_tiles", "hbfp_unpack", "hbfp_dequantize", "hbfp_gemm_workspace",
     "hbfp_gemm_q_workspace", "hbfp_gemm", "hbfp_gemm_q", "hbfp_gemm_block_partials",
-    "hbfp_device_status", "hbfp_gemm_static", "hbfp_wide_quantize", "hbfp_wide_update", "hbfp_wide_narrow",
+    "hbfp_device_status", "hbfp_gemm_static", "hbfp_wide_quantize", "hbfp_wide_update", "hbfp_wide_update_value", "hbfp_wide_narrow",
     "hbfp_im2col_packed", "hbfp_im2col_packed_t", "hbfp_wide_dequantize", "hbfp_selftest_bounded_wait", "hbfp_last_gemm_kernel", "hbfp_last_gemm_cycles", "hbfp_conv_forward", "hbfp_quantize_conv_weights", "hbfp_conv_dgrad_filters",
 ]
 
@@ -94,6 +94,7 @@ def lib() -> ctypes.CDLL:
         L.hbfp_quantize_tiles.argtypes = [p, i64, i64, i64, p, p, p, p, p, p, p]
         L.hbfp_wide_quantize.argtypes = [p, i64, i64, i64, p, p, p, p, p, p, p, p]
         L.hbfp_wide_update.argtypes = [p, p, p, i64, i64, i64, p, p, p, p, p, p]
+        L.hbfp_wide_update_value.argtypes = [p, p, p, i64, i64, i64, p, p, p, p, p, p, i64, p]
         L.hbfp_wide_narrow.argtypes = [p, p, i64, i64, p, p, p, p, p, p]
         L.hbfp_im2col_packed.argtypes = [p, p, i64, i64, i64, i64, i32, i32, i32, p, p, p, p]
         L.hbfp_im2col_packed_t.argtypes = [p, i64, i64, i64, i64, i32, i32, i32, p, p, p, p]
@@ -122,7 +123,7 @@ def lib() -> ctypes.CDLL:
 
 
 # Entry points that _host calls, in the order it takes them (csrc/host.cpp, struct Api).
-_HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q", "hbfp_gemm_q_workspace", "hbfp_wide_update", "hbfp_wide_dequantize",
+_HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q", "hbfp_gemm_q_workspace", "hbfp_wide_update_value", "hbfp_wide_dequantize",
                       "hbfp_conv_forward", "hbfp_conv_dgrad_filters", "hbfp_im2col_packed_t")
 
 
@@ -274,14 +275,16 @@ def wide_quantize(w: torch.Tensor, fmt: Format, out: Optional[Wide] = None, view
 def wide_update(wide: Wide, delta: torch.Tensor, fmt: Format, views: Optional[Tuple[Packed, Packed]] = None,
                 want_views: bool = True):
     """hbfp_wide_update: ``wide <- Q16(float32(wide + delta))`` in place; returns the narrow views."""
-    _check_f32(delta, "delta")
-    if delta.shape != wide.mant.shape:
-        raise ValueError("delta must have the shape of the weights")
     if views is None and want_views:
         views = _alloc_views(*wide.mant.shape, fmt, delta.device)
     c0, c1 = views if views is not None else (None, None)
-    _check((_native or host()).wide_update(wide.mant, wide.exps, delta, fmt, c0, c1), "hbfp_wide_update")
+    _check((_native or host()).wide_update(wide.mant, wide.exps, delta, fmt, c0, c1, False), "hbfp_wide_update")
     return views
+
+
+def wide_update_value(wide: Wide, delta: torch.Tensor, fmt: Format, views: Tuple[Packed, Packed]) -> torch.Tensor:
+    """hbfp_wide_update_value: ``wide_update`` that also returns the FP32 value of the new weights (a new tensor)."""
+    return _got((_native or host()).wide_update(wide.mant, wide.exps, delta, fmt, *views, True), "hbfp_wide_update_value")
 
 
 def wide_narrow(wide: Wide, fmt: Format, views: Optional[Tuple[Packed, Packed]] = None) -> Tuple[Packed, Packed]:

@@ -332,17 +332,23 @@ int hbfp_wide_quantize(const float* w, int64_t d0, int64_t d1, int64_t ld, const
     int rc = wide_views_ok(mant_c0, exps_c0, mant_c1, exps_c1);
     if (rc) return rc;
     return launch_wide(0, w, ld, d0, d1, fmt, wide, wide_exps, static_cast<int8_t*>(mant_c0), exps_c0,
-                       static_cast<int8_t*>(mant_c1), exps_c1, static_cast<cudaStream_t>(stream));
+                       static_cast<int8_t*>(mant_c1), exps_c1, nullptr, 0, static_cast<cudaStream_t>(stream));
 }
 
 int hbfp_wide_update(int16_t* wide, int8_t* wide_exps, const float* delta, int64_t d0, int64_t d1, int64_t ldd,
                      const hbfp_format* fmt, void* mant_c0, int8_t* exps_c0, void* mant_c1, int8_t* exps_c1, void* stream) {
-    if (d0 < 0 || d1 < 0 || ldd < d1 || !fmt) return HBFP_ERR_INVALID_ARG;
+    return hbfp_wide_update_value(wide, wide_exps, delta, d0, d1, ldd, fmt, mant_c0, exps_c0, mant_c1, exps_c1, nullptr, 0, stream);
+}
+
+int hbfp_wide_update_value(int16_t* wide, int8_t* wide_exps, const float* delta, int64_t d0, int64_t d1, int64_t ldd,
+                           const hbfp_format* fmt, void* mant_c0, int8_t* exps_c0, void* mant_c1, int8_t* exps_c1,
+                           float* value, int64_t ldv, void* stream) {
+    if (d0 < 0 || d1 < 0 || ldd < d1 || (value && ldv < d1) || !fmt) return HBFP_ERR_INVALID_ARG;
     if (d0 * d1 > 0 && (!delta || !wide || !wide_exps)) return HBFP_ERR_INVALID_ARG;
     int rc = wide_views_ok(mant_c0, exps_c0, mant_c1, exps_c1);
     if (rc) return rc;
     return launch_wide(1, delta, ldd, d0, d1, fmt, wide, wide_exps, static_cast<int8_t*>(mant_c0), exps_c0,
-                       static_cast<int8_t*>(mant_c1), exps_c1, static_cast<cudaStream_t>(stream));
+                       static_cast<int8_t*>(mant_c1), exps_c1, value, ldv, static_cast<cudaStream_t>(stream));
 }
 
 int hbfp_wide_narrow(const int16_t* wide, const int8_t* wide_exps, int64_t d0, int64_t d1, const hbfp_format* fmt,
@@ -352,7 +358,7 @@ int hbfp_wide_narrow(const int16_t* wide, const int8_t* wide_exps, int64_t d0, i
     int rc = wide_views_ok(mant_c0, exps_c0, mant_c1, exps_c1);
     if (rc) return rc;
     return launch_wide(2, nullptr, d1, d0, d1, fmt, const_cast<int16_t*>(wide), const_cast<int8_t*>(wide_exps),
-                       static_cast<int8_t*>(mant_c0), exps_c0, static_cast<int8_t*>(mant_c1), exps_c1,
+                       static_cast<int8_t*>(mant_c0), exps_c0, static_cast<int8_t*>(mant_c1), exps_c1, nullptr, 0,
                        static_cast<cudaStream_t>(stream));
 }
 

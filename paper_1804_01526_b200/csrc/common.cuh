@@ -73,10 +73,10 @@ int launch_quantize_conv_weights(const float* w, int64_t taps, int64_t c_in, int
                                  const hbfp_format* f, int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1,
                                  int8_t* tile_exps, cudaStream_t st);
 // Wide weight storage: mode 0 quantise FP32 weights, 1 apply an FP32 update in place, 2 read only; in every
-// mode the packed narrow views are written when their pointers are given.
+// mode the packed narrow views are written when their pointers are given, in mode 1 also the FP32 values.
 int launch_wide(int mode, const float* src, int64_t ld, int64_t d0, int64_t d1, const hbfp_format* f,
                 int16_t* wide, int8_t* wide_exps, int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1,
-                cudaStream_t st);
+                float* value, int64_t ldv, cudaStream_t st);
 int launch_wide_dequantize(const int16_t* wide, const int8_t* exps, int64_t d0, int64_t d1, int tile, float* out,
                            int64_t ldo, cudaStream_t st);
 // Packed convolution operand gathered from the packed per-pixel operand.

@@ -22,7 +22,7 @@ struct Api {
     decltype(&hbfp_quantize) quantize;
     decltype(&hbfp_gemm_q) gemm_q;
     decltype(&hbfp_gemm_q_workspace) gemm_q_workspace;
-    decltype(&hbfp_wide_update) wide_update;
+    decltype(&hbfp_wide_update_value) wide_update;
     decltype(&hbfp_wide_dequantize) wide_dequantize;
     decltype(&hbfp_conv_forward) conv_forward;
     decltype(&hbfp_conv_dgrad_filters) conv_dgrad_filters;
@@ -221,7 +221,8 @@ PyObject* gemm_q(PyObject*, PyObject* const* a, Py_ssize_t n) {
     });
 }
 
-// wide_update(mant, exps, delta, fmt, c0 or None, c1 or None) -> None; c0, c1: objects with mant and exps
+// wide_update(mant, exps, delta, fmt, c0 or None, c1 or None, whether the FP32 value is wanted) -> None or the value;
+// c0, c1: objects with mant and exps
 struct ViewPtrs { void* m0 = nullptr; int8_t* e0 = nullptr; void* m1 = nullptr; int8_t* e1 = nullptr; };
 void view_of(PyObject* v, void** m, int8_t** e) {
     PyObject* pm = attr(v, n_mant);
@@ -233,14 +234,18 @@ void view_of(PyObject* v, void** m, int8_t** e) {
     if (!ok) { PyErr_SetString(PyExc_TypeError, "a view holds tensors"); throw Fail{}; }
 }
 PyObject* wide_update(PyObject*, PyObject* const* a, Py_ssize_t n) {
-    if (!want(n, 6)) return nullptr;
+    if (!want(n, 7)) return nullptr;
     return guarded([&]() -> PyObject* {
         const at::Tensor m = tensor_of(a[0], "mantissas"), e = tensor_of(a[1], "exponents"), d = tensor_of(a[2], "delta");
+        check_f32(d, "delta");
+        if (d.dim() != 2 || d.size(0) != m.size(0) || d.size(1) != m.size(1)) value_error("%s must have the shape of the weights", "delta");
         const hbfp_format f = format_of(a[3]);
         ViewPtrs v;
         if (a[4] != Py_None) { view_of(a[4], &v.m0, &v.e0); view_of(a[5], &v.m1, &v.e1); }
-        return code(api.wide_update((int16_t*)m.data_ptr(), (int8_t*)e.data_ptr(), (const float*)d.data_ptr(), m.size(0), m.size(1), ld_of(d), &f,
-                                    v.m0, v.e0, v.m1, v.e1, stream()));
+        const at::Tensor value = a[6] == Py_True ? empty_f32({m.size(0), m.size(1)}, m) : at::Tensor();
+        const int rc = api.wide_update((int16_t*)m.data_ptr(), (int8_t*)e.data_ptr(), (const float*)d.data_ptr(), m.size(0), m.size(1), ld_of(d), &f,
+                                       v.m0, v.e0, v.m1, v.e1, value.defined() ? (float*)value.data_ptr() : nullptr, m.size(1), stream());
+        return !rc && value.defined() ? THPVariable_Wrap(value) : code(rc);
     });
 }
 

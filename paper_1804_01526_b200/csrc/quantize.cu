@@ -464,7 +464,22 @@ quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
 struct TileViews {
     int8_t* mant_c0; int64_t kst0, ps0; int8_t* exps_c0; int64_t rs0, nkb0;
     int8_t* mant_c1; int64_t kst1, ps1; int8_t* exps_c1; int64_t rs1, nkb1;
+    float* value; int64_t ldv;      // FP32 value of the wide words (modes that write them), or null
 };
+
+// 2^e for every stored exponent: below -126 the power itself is subnormal, and its product with a mantissa is exact.
+__device__ __forceinline__ float pow2f_stored(int e) {
+    return __uint_as_float(e >= -126 ? (uint32_t)(e + 127) << 23 : 0x00400000u >> (-127 - e));
+}
+// The values of two packed 16-bit mantissas.
+__device__ __forceinline__ float2 wide_values(uint32_t q2, float scale) {
+    return make_float2(__fmul_rn((float)(int16_t)(q2 & 0xFFFFu), scale), __fmul_rn((float)((int32_t)q2 >> 16), scale));
+}
+__device__ __forceinline__ void store_wide_values(float* dst, const uint32_t h[4], float scale) {
+    const float2 a = wide_values(h[0], scale), b = wide_values(h[1], scale), c = wide_values(h[2], scale), d = wide_values(h[3], scale);
+    reinterpret_cast<float4*>(dst)[0] = make_float4(a.x, a.y, b.x, b.y);
+    reinterpret_cast<float4*>(dst)[1] = make_float4(c.x, c.y, d.x, d.y);
+}
 
 // qt rows have a pitch of tp + 2 halfwords, so that the column reads of view c0 spread over the banks.
 // sh: the views take the top bits of the words in qt (an arithmetic shift by sh bits); for wide storage qt
@@ -541,6 +556,9 @@ __device__ __forceinline__ int round_sr_wide(float x, int s, uint32_t r) {
 //   MODE 0  quantise FP32 weights src to wide storage: int16 mantissas `wide` (row-major, pitch d1) and
 //           one exponent per tile in grid [tiles along d0][tiles along d1]
 //   MODE 1  update: w = fl32(wide * 2^s + src) with src the FP32 update, re-quantised to 16 bits in place
+//   MODE 4  the same, and the FP32 value of the new words to tv.value (a mode of its own: a runtime test in mode 1
+//           cost the plain update of 8192 x 8192 weights 1.5 us of 110); 4 bytes per weight more instead of a second
+//           pass that reads the words again, 12.1 -> 13.1 us against 12.1 + 5.5 for 1024 x 4096 weights
 //   MODE 2  read wide storage only
 // In every mode, when view pointers are given, the tile goes to the two packed views
 //   c1: rows = d0, contraction along d1 (the stored orientation);  c0: rows = d1, contraction along d0
@@ -565,6 +583,7 @@ tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, i
     const int64_t i0 = u * t, j0 = v * t;
     const int hi = (int)min((int64_t)t, d0 - i0), wj = (int)min((int64_t)t, d1 - j0);
     const int G = wj >> 3;                              // FAST: groups of eight per tile row
+    constexpr bool UPDATE = MODE == 1 || MODE == 4;
     const int wbits = MODE == 3 ? p.m : 16, wqmax = MODE == 3 ? p.qmax : 32767;
     // Wide modes: qt holds the stored word the views are cut from: the mantissa plus half a narrow unit,
     // held inside the range whose top bits stay within +-qmax (so the shift alone rounds to nearest and
@@ -593,14 +612,14 @@ tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, i
                 for (int jj = lane; jj < wj; jj += 32) qt[ii * qp + jj] = (int16_t)stored_one(wide[(i0 + ii) * d1 + j0 + jj]);
         }
     } else {
-        const float old_scale = MODE == 1 ? pow2f(grid[u * grid_ld + v]) : 0.f;
+        const float old_scale = UPDATE ? pow2f(grid[u * grid_ld + v]) : 0.f;
         uint32_t am = 0;
         if (FAST) {
             for (int item = tid; item < hi * G; item += 256) {
                 const int ii = item / G, gj = item - ii * G;
                 const float4* sp = reinterpret_cast<const float4*>(src + (i0 + ii) * ld + j0 + 8 * gj);
                 float4 a = __ldcs(sp), b = __ldcs(sp + 1);
-                if (MODE == 1) {
+                if (UPDATE) {
                     const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
                     a.x = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x & 0xFFFFu), old_scale), a.x);
                     a.y = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x >> 16), old_scale), a.y);
@@ -620,7 +639,7 @@ tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, i
             for (int ii = wrow; ii < hi; ii += 8)
                 for (int jj = lane; jj < wj; jj += 32) {
                     float val = src[(i0 + ii) * ld + j0 + jj];
-                    if (MODE == 1) val = __fadd_rn(__fmul_rn((float)wide[(i0 + ii) * d1 + j0 + jj], old_scale), val);
+                    if (UPDATE) val = __fadd_rn(__fmul_rn((float)wide[(i0 + ii) * d1 + j0 + jj], old_scale), val);
                     tile[ii * fp + jj] = val;
                     am = max(am, abs_bits(val));
                 }
@@ -671,6 +690,7 @@ tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, i
                 uint32_t* dst = reinterpret_cast<uint32_t*>(qt + ii * qp + 8 * gj);
                 dst[0] = stored_pair(h[0]); dst[1] = stored_pair(h[1]); dst[2] = stored_pair(h[2]); dst[3] = stored_pair(h[3]);
                 if (MODE != 3) *reinterpret_cast<uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) = make_uint4(h[0], h[1], h[2], h[3]);
+                if (MODE == 4) store_wide_values(tv.value + (i0 + ii) * tv.ldv + j0 + 8 * gj, h, pow2f_stored(s));
             }
         } else {
             for (int ii = wrow; ii < hi; ii += 8)
@@ -683,6 +703,7 @@ tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, i
                     else q = round_sr_wide(val, s, draw_of_element(p, L));
                     qt[ii * qp + jj] = (int16_t)stored_one(q);
                     if (MODE != 3) wide[(i0 + ii) * d1 + j0 + jj] = (int16_t)q;
+                    if (MODE == 4) tv.value[(i0 + ii) * tv.ldv + j0 + jj] = __fmul_rn((float)q, pow2f_stored(s));
                 }
         }
     }
@@ -711,6 +732,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
     const int tid = threadIdx.x, lane = tid & 31, wrow = tid >> 5;
     const int64_t u = blockIdx.y, v = blockIdx.x;
     const int64_t i0 = u * TP, j0 = v * TP;
+    constexpr bool UPDATE = MODE == 1 || MODE == 4;
     const int wbits = MODE == 3 ? p.m : 16, wqmax = MODE == 3 ? p.qmax : 32767;
     const int sh = MODE == 3 ? 0 : 16 - p.m;
     const int half = sh > 0 ? 1 << (sh - 1) : 0;
@@ -731,7 +753,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
             }
         }
     } else {
-        const float old_scale = MODE == 1 ? pow2f(grid[u * grid_ld + v]) : 0.f;
+        const float old_scale = UPDATE ? pow2f(grid[u * grid_ld + v]) : 0.f;
         // the FP32 groups of the tile are requested before anything waits for them; for an update the wide
         // words follow, combined as fl32(wide * 2^s + delta) with one rounding
         float4 a[ITEMS], b[ITEMS];
@@ -748,7 +770,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
                 b[k] = __ldcs(sp + 1);
             }
         }
-        if (MODE == 1) {
+        if (UPDATE) {
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
                 const int item = tid + 256 * k;
@@ -815,6 +837,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
                 }
                 *reinterpret_cast<uint4*>(qt + ii * QP + 8 * gj) = make_uint4(stored_pair(h[0]), stored_pair(h[1]), stored_pair(h[2]), stored_pair(h[3]));
                 if (MODE != 3) *reinterpret_cast<uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) = make_uint4(h[0], h[1], h[2], h[3]);
+                if (MODE == 4) store_wide_values(tv.value + (i0 + ii) * tv.ldv + j0 + 8 * gj, h, pow2f_stored(s));
             }
         }
     }
@@ -1860,6 +1883,7 @@ int launch_tile_full_small(int mode, int planes, int t, unsigned gx, unsigned gy
     else if (mode == 1) HBFP_TILE_FULL_MODE(1);
     else if (mode == 2) HBFP_TILE_FULL_MODE(2);
     else if (mode == 3) HBFP_TILE_FULL_MODE(3);
+    else if (mode == 4) HBFP_TILE_FULL_MODE(4);
     else return HBFP_ERR_INVALID_ARG;
 #undef HBFP_TILE_FULL_MODE
 #undef HBFP_TILE_FULL_SMALL
@@ -2069,7 +2093,8 @@ namespace {
 
 template <int MODE>
 int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbfp_format* f, int16_t* wide,
-                 int8_t* grid, int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1, cudaStream_t st) {
+                 int8_t* grid, int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1, float* value, int64_t ldv,
+                 cudaStream_t st) {
     if (f->tile <= 0 || f->tile != f->block) return HBFP_ERR_INVALID_ARG;
     if (f->tile > 128) return HBFP_ERR_UNSUPPORTED;
     Layout L0, L1;
@@ -2082,10 +2107,11 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     const int t = f->tile, tp = (int)L0.bp;
     const int64_t nu = L0.nkb, nv = L1.nkb;   // tiles along d0, along d1
     if (nu > 65535) return HBFP_ERR_UNSUPPORTED;
-    const TileViews tv{mant_c0, L0.kst, L0.plane_stride, exps_c0, L0.rs, L0.nkb, mant_c1, L1.kst, L1.plane_stride, exps_c1, L1.rs, L1.nkb};
+    const TileViews tv{mant_c0, L0.kst, L0.plane_stride, exps_c0, L0.rs, L0.nkb, mant_c1, L1.kst, L1.plane_stride, exps_c1, L1.rs, L1.nkb, value, ldv};
     const bool fast = (t % 8) == 0 && (d1 % 8) == 0 &&
                       (MODE == 2 || ((ld % 4) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0)) &&
-                      (MODE == 3 || (reinterpret_cast<uintptr_t>(wide) & 15) == 0);
+                      (MODE == 3 || (reinterpret_cast<uintptr_t>(wide) & 15) == 0) &&
+                      (!value || ((ldv % 4) == 0 && (reinterpret_cast<uintptr_t>(value) & 15) == 0));
     const size_t smem = (size_t)t * (t + 4) * sizeof(float) + (size_t)tp * (tp + 2) * sizeof(int16_t);
     const dim3 grid_dim((unsigned)nv, (unsigned)nu);
     // full tiles of 32 / 64 / 128, both views or none, narrow bits cut by 32-bit shifts (see tile_kernel_full)
@@ -2119,7 +2145,7 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
 int launch_quantize_tiles(const float* w, int64_t d0, int64_t d1, int64_t ld, const hbfp_format* f,
                           int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1,
                           int8_t* tile_exps, cudaStream_t st) {
-    return launch_tiles<3>(w, ld, d0, d1, f, nullptr, tile_exps, mant_c0, exps_c0, mant_c1, exps_c1, st);
+    return launch_tiles<3>(w, ld, d0, d1, f, nullptr, tile_exps, mant_c0, exps_c0, mant_c1, exps_c1, nullptr, 0, st);
 }
 
 // Convolution weights w [taps * c_in][c_out] with one exponent per (t input maps) x (t output maps) tile over
@@ -2175,10 +2201,11 @@ int launch_quantize_conv_weights(const float* w, int64_t taps, int64_t c_in, int
 
 int launch_wide(int mode, const float* src, int64_t ld, int64_t d0, int64_t d1, const hbfp_format* f,
                 int16_t* wide, int8_t* wide_exps, int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1,
-                cudaStream_t st) {
-    if (mode == 0) return launch_tiles<0>(src, ld, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, st);
-    if (mode == 1) return launch_tiles<1>(src, ld, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, st);
-    return launch_tiles<2>(nullptr, d1, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, st);
+                float* value, int64_t ldv, cudaStream_t st) {
+    if (mode == 0) return launch_tiles<0>(src, ld, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, nullptr, 0, st);
+    if (mode == 1 && value) return launch_tiles<4>(src, ld, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, value, ldv, st);
+    if (mode == 1) return launch_tiles<1>(src, ld, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, nullptr, 0, st);
+    return launch_tiles<2>(nullptr, d1, d0, d1, f, wide, wide_exps, mant_c0, exps_c0, mant_c1, exps_c1, nullptr, 0, st);
 }
 
 int launch_im2col_packed(const int8_t* xm, const int8_t* xe, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw,
@@ -2285,13 +2312,41 @@ int launch_unpack(const Packed& p, int16_t* q, int8_t* s, cudaStream_t st) {
 }
 
 // Value of wide weight storage, Eq. 1: out[i][j] = q16[i][j] * 2^s16[i/t][j/t] (exact in binary32: 16-bit mantissas).
-__global__ void wide_dequant_kernel(const int16_t* __restrict__ wide, const int8_t* __restrict__ exps, int64_t d0,
-                                    int64_t d1, int t, int64_t tiles1, float* __restrict__ out, int64_t ldo) {
-    const int64_t n = d0 * d1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / d1, c = i - r * d1;
-        const int e = exps[(r / t) * tiles1 + c / t];
-        out[r * ldo + c] = ldexpf((float)wide[i], e);
+// Bound by its 6 bytes per weight. V = 4 weights of a row per access and four rows in flight per thread where the
+// tile, the pitches and the bases are multiples of four (then the four share an exponent); one weight per access
+// otherwise. A CTA covers 4 rows x (256 V) columns, so that no thread divides a linear index by the row length.
+// One weight per thread with a 64-bit division each took 28.4 us for 1024 x 4096 weights (0.9 TB/s), this form 5.5 us; 437 and 63 us
+// (6.4 TB/s) for 8192 x 8192.
+template <int V>
+__global__ void __launch_bounds__(256)
+wide_dequant_kernel(const int16_t* __restrict__ wide, const int8_t* __restrict__ exps, int64_t d0, int64_t d1, int t,
+                    int64_t tiles1, float* __restrict__ out, int64_t ldo) {
+    constexpr int ROWS = 4;
+    const int64_t c = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V;
+    if (c >= d1) return;
+    const int64_t tc = d1 < (1ll << 31) ? (int64_t)((uint32_t)c / (uint32_t)t) : c / t;
+    for (int64_t r0 = (int64_t)blockIdx.y * ROWS; r0 < d0; r0 += (int64_t)gridDim.y * ROWS) {
+        const int64_t tr = r0 / t;
+        const int r_in = (int)(r0 - tr * t);
+        uint2 q[ROWS] = {};
+        int e[ROWS] = {};
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i)
+            if (r0 + i < d0) {
+                const int16_t* at = wide + (r0 + i) * d1 + c;
+                if (V == 4) q[i] = *reinterpret_cast<const uint2*>(at);
+                else q[i].x = (uint16_t)*at;
+                e[i] = exps[(tr + (uint32_t)(r_in + i) / (uint32_t)t) * tiles1 + tc];
+            }
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i)
+            if (r0 + i < d0) {
+                const float sc = pow2f_stored(e[i]);
+                float* to = out + (r0 + i) * ldo + c;
+                const float2 a = wide_values(q[i].x, sc), b = wide_values(q[i].y, sc);
+                if (V == 4) *reinterpret_cast<float4*>(to) = make_float4(a.x, a.y, b.x, b.y);
+                else *to = a.x;
+            }
     }
 }
 
@@ -2299,7 +2354,11 @@ int launch_wide_dequantize(const int16_t* wide, const int8_t* exps, int64_t d0, 
                            int64_t ldo, cudaStream_t st) {
     if (d0 * d1 == 0) return HBFP_OK;
     const int64_t tiles1 = (d1 + tile - 1) / tile;
-    wide_dequant_kernel<<<blocks_for(d0 * d1, 256), 256, 0, st>>>(wide, exps, d0, d1, tile, tiles1, out, ldo);
+    const unsigned rows = (unsigned)std::min<int64_t>((d0 + 3) / 4, 65535);
+    const bool vec = tile % 4 == 0 && d1 % 4 == 0 && ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(wide) & 7) == 0 &&
+                     (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    if (vec) wide_dequant_kernel<4><<<dim3(blocks_for(d1, 1024), rows), 256, 0, st>>>(wide, exps, d0, d1, tile, tiles1, out, ldo);
+    else wide_dequant_kernel<1><<<dim3(blocks_for(d1, 256), rows), 256, 0, st>>>(wide, exps, d0, d1, tile, tiles1, out, ldo);
     return launch_status();
 }
 

@@ -144,3 +144,20 @@ def test_wide_storage_of_an_empty_matrix(hb):
     hb.wide_update(wide, torch.empty((0, 32), device="cuda"), f, views=views)
     hb.wide_narrow(wide, f, views=views)
     assert hb.device_status() == 0
+
+
+@pytest.mark.parametrize("shape,t,rounding", [
+    ((1, 4), 4, 0), ((3, 1028), 4, 1),                  # four weights per access: one row, a part of a group of rows
+    ((130, 2056), 24, 1), ((128, 256), 64, 0),          # several column blocks; whole tiles
+    ((9, 1030), 24, 1), ((70, 36), 6, 0),               # one weight per access: ragged rows; a tile that is no multiple of 4
+])
+def test_update_also_writes_the_fp32_value(hb, shape, t, rounding):
+    fd = F(8, t, rounding, seed=3)
+    w, delta = wl.draw("normal", shape, seed=5), wl.draw("normal", shape, seed=6) * np.float32(0.01)
+    wide, views = hb.wide_quantize(to_dev(w), gfmt(fd))
+    value = hb.wide_update_value(wide, to_dev(delta), gfmt(fd), views).cpu().numpy()
+    q16, e = wide.mant.cpu().numpy(), wide.exps.cpu().numpy().astype(np.int64)
+    s16 = np.repeat(np.repeat(e, t, axis=0)[: shape[0]], t, axis=1)[:, : shape[1]]
+    exact = np.ldexp(q16.astype(np.float64), s16).astype(np.float32)      # 16-bit mantissas: exact in binary32
+    assert np.array_equal(value, exact)
+    assert np.array_equal(hb.wide_dequantize(wide).cpu().numpy(), exact)
