@@ -714,13 +714,18 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, in
     const int64_t SMS = 148;                       // planning constant: the target part
     const int64_t nst = (la.nkb * la.bp + FP_STAGE_ELEMS - 1) / FP_STAGE_ELEMS;
     f.splits = 1;
-    // the time of a block grows with the tile's columns but not in proportion; K is split only where one wave of CTAs results
+    // The time of a block grows with the tile's columns but not in proportion. K is split only where all clusters run at once:
+    // a cluster's CTAs share a GPU processing cluster, so that of 148 SMs only this many clusters of one CTA per SM are resident
+    // (cudaOccupancyMaxActiveClusters). 36 clusters of four took two rounds: 1111 x 777 x 3001 with b = 24 51.4 us with its
+    // conversions, 63 clusters of two 41.2; 1500 x 600 x 3000, b = 64: 38.4 against 30.9; 128 x 4000 x 2000, b = 32: 37.7 against 27.0.
+    static constexpr int resident[9] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
     double best = 1e30;
     for (int ncol = 256; ncol >= (w ? 128 : 64); ncol /= 2) {
         const int64_t nout = w ? ncol / 2 : ncol, tiles = ((M + 127) / 128) * ((N + nout - 1) / nout);
         const double cost = ncol == 256 ? 1.0 : ncol == 128 ? 0.55 : 0.45;
-        for (int64_t sp = 1; sp <= 8; sp *= 2) {
-            if (sp > 1 && (tiles * sp > SMS || nst < 4 * sp)) break;
+        for (int64_t sp = 1; sp <= 8; ++sp) {
+            if (sp > 1 && (tiles > resident[sp] || nst < 4 * sp)) continue;
+            if ((nst + (nst + sp - 1) / sp - 1) / ((nst + sp - 1) / sp) != sp) continue;       // a split would be empty
             const double waves = (double)((tiles * sp + SMS - 1) / SMS);
             const double t = waves * ((double)((nst + sp - 1) / sp) * cost + 4.0 + (sp > 1 ? 3.0 : 0.0));
             if (t < best * 0.999) { best = t; f.ncol = ncol; f.splits = (int)sp; }

@@ -457,3 +457,15 @@ def test_small_products_of_fp32_operands_converted_straight_to_the_form(hb, m, b
     da, db = hb.dequantize(pa).double(), hb.dequantize(pb).double()
     assert hb.device_status() == 0
     assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
+
+
+@pytest.mark.parametrize("m,b,M,N,K", [(8, 24, 600, 520, 1700), (8, 24, 1111, 777, 3001), (8, 32, 640, 1280, 2048), (8, 64, 900, 500, 1300), (12, 24, 600, 520, 1700),
+                                       (12, 24, 1000, 600, 1000), (8, 32, 650, 330, 900), (8, 32, 640, 500, 2600), (8, 64, 511, 385, 3300)])
+def test_contraction_split_over_clusters_of_any_size(hb, m, b, M, N, K):
+    """K split over clusters of 2 to 7 CTAs, last parts shorter than the others: within 1e-6 of the accumulator magnitude."""
+    A, B = to_dev(wl.draw("outliers", (M, K), seed=97)), to_dev(wl.draw("lognormal", (K, N), seed=98))
+    fa, fb = hb.Format(m, b), hb.Format(m, b, stream_id=1)
+    C = hb.gemm(0, 0, A, B, fa, fb)
+    da, db = (hb.dequantize(hb.quantize(x, ax, f)).double() for x, ax, f in ((A, 1, fa), (B, 0, fb)))
+    assert hb.device_status() == 0 and hb.last_gemm_kernel() == "gemm_tc_kernel"
+    assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
