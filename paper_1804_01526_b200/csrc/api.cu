@@ -185,6 +185,15 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     // a problem of a few hundred MOPs is over before a tensor-core kernel has filled its pipeline
     const bool small = !P && (flags == HBFP_GEMM_AUTO || flags == HBFP_GEMM_FORCE_SMALL) && small_gemm_eligible(M, N, pa, pb, flags == HBFP_GEMM_FORCE_SMALL);
     if (flags == HBFP_GEMM_FORCE_SMALL && !small) return HBFP_ERR_UNSUPPORTED;
+    if (!P && flags == HBFP_GEMM_AUTO && a->kind == HBFP_OPERAND_FP32 && a->trans == 0 && a->fmt.tile == 0 &&
+        b->kind == HBFP_OPERAND_PACKED && skinny_gemm_eligible(M, N, g.la, g.lb, a->fmt.mant_bits, b->fmt.mant_bits)) {
+        rc = check_fp32(a, true, M, K);
+        if (rc) return rc;
+        rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, st);
+        if (rc) return rc;
+        t_last_gemm_kernel = "gemm_skinny_kernel";
+        return launch_gemm_skinny(M, N, K, static_cast<const float*>(a->data), a->ld, &a->fmt, pb, C, ldc, st);
+    }
     if (use_fp && !small) {
         const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
         rc = resolve_form(a, true, M, K, g, ws, fa, st);

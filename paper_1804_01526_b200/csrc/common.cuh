@@ -96,6 +96,11 @@ int launch_gemm_simt(int64_t M, int64_t N, int64_t K, const Packed& a, const Pac
 bool small_gemm_eligible(int64_t M, int64_t N, const Packed& a, const Packed& b, bool any_size);
 int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, float* C, int64_t ldc, cudaStream_t st);
 
+// A few rows of FP32 activations against packed weights, conversion included (gemm_skinny.cu): one launch, no scratch.
+bool skinny_gemm_eligible(int64_t M, int64_t N, const Layout& la, const Layout& lb, int bits_a, int bits_b);
+int launch_gemm_skinny(int64_t M, int64_t N, int64_t K, const float* x, int64_t ld, const hbfp_format* fx, const Packed& w, float* C,
+                       int64_t ldc, cudaStream_t st);
+
 // Workspace of the integer kernels alone (hbfp_gemm_workspace may ask for more).
 int gemm_least_workspace(int transA, int transB, int64_t M, int64_t N, int64_t K, const hbfp_format* fmtA,
                          const hbfp_format* fmtB, size_t* bytes);

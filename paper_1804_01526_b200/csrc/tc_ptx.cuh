@@ -248,6 +248,14 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 EncodeTiledFn encode_fn() {
     static EncodeTiledFn fn = nullptr;
+    // The driver call wants the thread's context current, which a thread's first runtime call that needs one makes it (a
+    // backward pass runs on a thread of its own, and encoding a map may be the first thing it does).
+    static thread_local bool bound = false;
+    if (!bound) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return nullptr;
+        bound = true;
+    }
     if (!fn) {
         void* ptr = nullptr;
         cudaDriverEntryPointQueryResult q;

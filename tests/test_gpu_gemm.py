@@ -469,3 +469,40 @@ def test_contraction_split_over_clusters_of_any_size(hb, m, b, M, N, K):
     da, db = (hb.dequantize(hb.quantize(x, ax, f)).double() for x, ax, f in ((A, 1, fa), (B, 0, fb)))
     assert hb.device_status() == 0 and hb.last_gemm_kernel() == "gemm_tc_kernel"
     assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
+
+
+@pytest.mark.parametrize("M,N,K,m,t,rounding", [(1, 1, 1, 8, 32, 0), (16, 4096, 4096, 8, 64, 0), (17, 129, 128, 8, 128, 1), (5, 1000, 777, 8, 24, 1), (32, 127, 3001, 8, 48, 1),
+                                                (33, 640, 513, 4, 32, 0), (64, 300, 8192, 8, 128, 1), (128, 10, 1024, 8, 24, 1), (100, 900, 1000, 6, 40, 0), (16, 256, 11000, 8, 32, 0)])
+def test_few_rows_against_packed_weights_in_one_launch(hb, M, N, K, m, t, rounding):
+    """Conversion, product and sum over K in one kernel: edges of the 128 weight rows and of the 16, 32 and 64 activation rows,
+    blocks with padding, odd row lengths, more blocks than tensor memory holds, an output that starts at an odd column. Within
+    1e-6 of the accumulator magnitude of the product of what hbfp_quantize makes of the same operand."""
+    import torch
+    X, W = to_dev(wl.draw("outliers", (M, K), seed=71)), to_dev(wl.draw("he_weight", (K, N), seed=72, fan_in=K))
+    fx = hb.Format(mant_bits=m, block=t, rounding=rounding, seed=3)
+    c0 = hb.quantize_tiles(W, hb.Format(mant_bits=m, block=t, tile=t, rounding=rounding, seed=3, stream_id=1), want_grid=False)[0]
+    dx, dw = hb.dequantize(hb.quantize(X, 1, fx)).double(), hb.dequantize(c0).double()
+    want, mag = dx @ dw.t(), dx.abs() @ dw.abs().t()
+    buf = torch.full((M, N + 3), 7.0, device="cuda")
+    for out in (None, buf[:, 1:1 + N]):
+        got = hb.gemm_q(M, N, K, X, c0, fmtA=fx, out=out)
+        assert hb.last_gemm_kernel() in ("gemm_skinny_kernel", "gemm_small_kernel") and hb.device_status() == 0
+        assert bool(((got.double() - want).abs() <= TOL * mag + 1e-30).all())
+    assert bool((buf[:, 0] == 7).all()) and bool((buf[:, N + 1:] == 7).all())
+
+
+def test_few_rows_kernel_reports_weights_beyond_its_exact_range(hb):
+    """P * 2^sB leaves binary32 above sB = 104: the oracle's values or the status, nothing else."""
+    M, N, K, t = 4, 160, 1024, 64
+    X, W = wl.draw("normal", (M, K), seed=73), wl.draw("normal", (K, N), seed=74)
+    fx, fw = hb.Format(8, t), hb.Format(8, t, tile=t, stream_id=1)
+    for scale_x, scale_w in ((2.0 ** -60, 2.0 ** 100), (2.0 ** 100, 2.0 ** -60), (2.0 ** -100, 2.0 ** 118)):
+        x, w = to_dev(X * np.float32(scale_x)), to_dev(W * np.float32(scale_w))
+        c0 = hb.quantize_tiles(w, fw, want_grid=False)[0]
+        got = hb.gemm_q(M, N, K, x, c0, fmtA=fx)
+        assert hb.last_gemm_kernel() == "gemm_skinny_kernel"
+        want = hb.dequantize(hb.quantize(x, 1, fx)).double() @ hb.dequantize(c0).double().t()
+        if hb.device_status() == 0:
+            assert bool(((got.double() - want).abs() <= 1e-5 * want.abs().max()).all())
+        else:
+            assert scale_w > 2.0 ** 110
