@@ -4,7 +4,7 @@ The paper simulates HBFP by redefining PyTorch's linear module with ``autograd.F
 forward product ``Y = X W``, the backward-data product ``dX = dY W^T`` and the backward-weight
 product ``dW = X^T dY`` take BFP operands, every other operation (bias, activations, loss, the
 optimiser's arithmetic) stays FP32. This module is that wrapper over the library's calls; it holds
-no arithmetic of its own:
+no arithmetic of its own, and the passes themselves are autograd nodes in compiled code (``csrc/host.cpp``):
 
 * the weights live in wide storage (16-bit mantissas per tile, ``hbfp_wide_quantize``); the two
   packed narrow views the GEMMs read are the top ``mant_bits`` bits (Sec. 4.2);
@@ -25,25 +25,6 @@ from __future__ import annotations
 import torch
 
 from . import binding as hb
-
-
-class _HbfpLinearFn(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, x, weight, bias, layer):
-        ctx.layer = layer
-        ctx.save_for_backward(x)
-        return hb._got(hb.host().linear_forward(x.contiguous(), layer.views[0], layer.fmt_act(0), layer.fin, layer.fout, bias), "hbfp_gemm_q")
-
-    @staticmethod
-    def backward(ctx, dy):
-        layer = ctx.layer
-        (x,) = ctx.saved_tensors
-        need_dx, need_dw, need_db, _ = ctx.needs_input_grad
-        # backward-data on the shared weight view, backward-weight with 1-D blocks down the columns of X and dY (the
-        # contraction over the batch axis), the bias gradient
-        dx, dw, db = hb._got(hb.host().linear_backward(dy.contiguous(), x.contiguous(), layer.views[1], layer.fmt_act(2), layer.fmt_act(0, batch_axis=True),
-                                                       layer.fmt_act(2, batch_axis=True), layer.fin, layer.fout, need_dx, need_dw, need_db), "hbfp_gemm_q")
-        return dx, dw, db, None
 
 
 class HbfpLinear(torch.nn.Module):
@@ -84,59 +65,8 @@ class HbfpLinear(torch.nn.Module):
         self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        return _HbfpLinearFn.apply(x, self.weight, self.bias, self)
-
-
-class _HbfpConv3x3Fn(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, x, weight, layer):
-        n, h, w, c = x.shape
-        ctx.layer = layer
-        ctx.save_for_backward(x)
-        x = x.contiguous()
-        px = hb.quantize(x.view(n * h * w, c), 1, layer.fmt_pixels(0))
-        try:
-            # the implicit GEMM reads the taps straight from the packed pixels
-            y = hb.conv_forward(px, layer.views[0], n, h, w, c, 3, 3, 1)
-        except hb.HbfpError as e:
-            if e.code != hb.ERR_UNSUPPORTED:
-                raise
-            # shapes it does not cover: gather the packed operand, then the ordinary GEMM (same product)
-            pa = hb.im2col_packed(px, n, h, w, c, 3, 3, 1)
-            y = hb.gemm_q(n * h * w, layer.fout, 9 * c, pa, layer.views[0])
-        return y.view(n, h, w, layer.fout)
-
-    @staticmethod
-    def backward(ctx, dy):
-        layer = ctx.layer
-        (x,) = ctx.saved_tensors
-        n, h, w, c = x.shape
-        f = layer.fout
-        dy2 = dy.contiguous().view(n * h * w, f)
-        dx = dw = None
-        if ctx.needs_input_grad[0]:
-            try:
-                # the convolution of the packed output gradient with the forward weights regrouped (taps turned by
-                # 180 degrees, feature-map roles swapped) yields dX itself
-                pg = hb.quantize(dy2, 1, layer.fmt_pixels(2))
-                turned = hb.conv_dgrad_filters(layer.views[1], 3, 3, c, f)
-                dx = hb.conv_forward(pg, turned, n, h, w, f, 3, 3, 1).view(n, h, w, c)
-            except hb.HbfpError as e:
-                if e.code != hb.ERR_UNSUPPORTED:
-                    raise
-        if ctx.needs_input_grad[0] and dx is None:
-            # shapes that route does not cover: gradient of the im2col matrix, then its scatter back onto the
-            # pixels (an FP32 operation)
-            dcols = hb.gemm_q(n * h * w, 9 * c, f, dy2, layer.views[1], fmtA=layer.fmt_pixels(2)).view(n, h, w, 3, 3, c)
-            dxp = torch.zeros((n, h + 2, w + 2, c), device=x.device)
-            for i in range(3):
-                for j in range(3):
-                    dxp[:, i:i + h, j:j + w, :] += dcols[:, :, :, i, j, :]
-            dx = dxp[:, 1:h + 1, 1:w + 1, :].contiguous()
-        if ctx.needs_input_grad[1]:
-            pa_t = hb.im2col_packed_t(x.contiguous(), 3, 3, 1, layer.fmt_batch(0))
-            dw = hb.gemm_q(9 * c, f, n * h * w, pa_t, dy2, fmtB=layer.fmt_batch(2))
-        return dx, dw, None
+        return hb.host().linear(x, self.weight, self.bias, self.views[0], self.views[1], self.mant_bits, self.tile, self.batch_block,
+                                self.rounding, self.seed + self.steps, self.stream_id)
 
 
 class HbfpConv3x3(torch.nn.Module):
@@ -173,4 +103,4 @@ class HbfpConv3x3(torch.nn.Module):
         self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        return _HbfpConv3x3Fn.apply(x, self.weight, self)
+        return hb.host().conv3x3(x, self.weight, self.views[0], self.views[1], self.mant_bits, self.pixel_block, self.c, self.fout)

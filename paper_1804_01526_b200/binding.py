@@ -124,7 +124,7 @@ def lib() -> ctypes.CDLL:
 
 # Entry points that _host calls, in the order it takes them (csrc/host.cpp, struct Api).
 _HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q", "hbfp_gemm_q_workspace", "hbfp_wide_update_value", "hbfp_wide_dequantize",
-                      "hbfp_conv_forward", "hbfp_conv_dgrad_filters", "hbfp_im2col_packed_t")
+                      "hbfp_conv_forward", "hbfp_conv_dgrad_filters", "hbfp_im2col_packed_t", "hbfp_im2col_packed")
 
 
 def host():
@@ -136,7 +136,7 @@ def host():
             from . import _host
         except ImportError as e:
             raise ImportError("_host.so is missing: build it with `python -m paper_1804_01526_b200.build` (there is no fallback path)") from e
-        _host.bind(*(ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in _HOST_ENTRY_POINTS))
+        _host.bind(HbfpError, *(ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in _HOST_ENTRY_POINTS))
         _native = _host
     return _native
 

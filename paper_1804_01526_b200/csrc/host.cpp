@@ -5,7 +5,11 @@
 // that whichever build of it the binding has loaded is the one that runs.
 //
 // Every function returns its result, or the library's status code as a Python int (the binding raises it).
+#include <torch/csrc/Exceptions.h>
+#include <torch/csrc/autograd/function.h>
+#include <torch/csrc/autograd/functions/utils.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/autograd/saved_variable.h>
 #include <ATen/ATen.h>
 #include <ATen/core/LegacyTypeDispatch.h>
 #include <ATen/cuda/CUDAContext.h>
@@ -27,6 +31,7 @@ struct Api {
     decltype(&hbfp_conv_forward) conv_forward;
     decltype(&hbfp_conv_dgrad_filters) conv_dgrad_filters;
     decltype(&hbfp_im2col_packed_t) im2col_packed_t;
+    decltype(&hbfp_im2col_packed) im2col_packed;
 } api;
 
 // ------------------------------------------------------------------------------ arguments
@@ -79,9 +84,13 @@ void check_f32(const at::Tensor& x, const char* name) {
     if (!(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 2 && (x.size(1) <= 1 || x.stride(1) == 1)))
         value_error("%s must be a 2-D float32 CUDA tensor with contiguous rows", name);
 }
+void check_f32_cpp(const at::Tensor& x) {
+    TORCH_CHECK_VALUE(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 2 && (x.size(1) <= 1 || x.stride(1) == 1),
+                      "operand must be a 2-D float32 CUDA tensor with contiguous rows");
+}
 int64_t ld_of(const at::Tensor& x) { return x.size(0) > 1 ? x.stride(0) : std::max<int64_t>(x.size(1), 1); }
 
-void* stream() { return at::cuda::getCurrentCUDAStream().stream(); }
+void* cur_stream() { return at::cuda::getCurrentCUDAStream().stream(); }
 
 at::Tensor empty_f32(at::IntArrayRef sizes, const at::Tensor& like) { return at::empty(sizes, like.options().dtype(at::kFloat).requires_grad(false)); }
 at::Tensor empty_i8(int64_t n, const at::Tensor& like) { return at::empty({n}, like.options().dtype(at::kChar).requires_grad(false)); }
@@ -124,13 +133,13 @@ Operand operand_of(PyObject* x, long long trans, PyObject* fmt) {
 
 // hbfp_gemm_q with the workspace from the caching allocator (stream-ordered, as a temporary tensor's memory is).
 int run_gemm(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_operand& b, const at::Tensor& out, const at::Tensor* ws, uint32_t flags) {
-    if (ws) return api.gemm_q(M, N, K, &a, &b, (float*)out.data_ptr(), ld_of(out), ws->data_ptr(), (size_t)ws->numel(), flags, stream());
+    if (ws) return api.gemm_q(M, N, K, &a, &b, (float*)out.data_ptr(), ld_of(out), ws->data_ptr(), (size_t)ws->numel(), flags, cur_stream());
     size_t bytes = 0;
     const int rc = api.gemm_q_workspace(M, N, K, &a, &b, &bytes);
     if (rc) return rc;
     c10::DataPtr mem;
     if (bytes) mem = c10::cuda::CUDACachingAllocator::get()->allocate(bytes);
-    return api.gemm_q(M, N, K, &a, &b, (float*)out.data_ptr(), ld_of(out), mem.get(), bytes, flags, stream());
+    return api.gemm_q(M, N, K, &a, &b, (float*)out.data_ptr(), ld_of(out), mem.get(), bytes, flags, cur_stream());
 }
 
 template <class F>
@@ -139,6 +148,24 @@ PyObject* guarded(F f) {
         at::AutoDispatchBelowADInplaceOrView below;          // plain tensors: nothing here is recorded for autograd
         return f();
     } catch (const Fail&) {
+        return nullptr;
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+// A layer's forward pass: it records its own node, so nothing is switched off around it; a library error is already a Python one.
+template <class F>
+PyObject* layer_call(F f) {
+    try {
+        return f();
+    } catch (const Fail&) {
+        return nullptr;
+    } catch (python_error& e) {
+        e.restore();
+        return nullptr;
+    } catch (const c10::ValueError& e) {
+        PyErr_SetString(PyExc_ValueError, e.what_without_backtrace());
         return nullptr;
     } catch (const std::exception& e) {
         PyErr_SetString(PyExc_RuntimeError, e.what());
@@ -174,7 +201,7 @@ PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
             m = tensor_of(a[3], "mantissas");
             e = tensor_of(a[4], "exponents");
         }
-        const int rc = api.quantize((const float*)x.data_ptr(), x.size(0), x.size(1), ld_of(x), axis, &f, m.data_ptr(), (int8_t*)e.data_ptr(), stream());
+        const int rc = api.quantize((const float*)x.data_ptr(), x.size(0), x.size(1), ld_of(x), axis, &f, m.data_ptr(), (int8_t*)e.data_ptr(), cur_stream());
         if (rc) return code(rc);
         return Py_BuildValue("(NN)", a[3] == Py_None ? THPVariable_Wrap(m) : same(a[3]), a[3] == Py_None ? THPVariable_Wrap(e) : same(a[4]));
     });
@@ -244,7 +271,7 @@ PyObject* wide_update(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (a[4] != Py_None) { view_of(a[4], &v.m0, &v.e0); view_of(a[5], &v.m1, &v.e1); }
         const at::Tensor value = a[6] == Py_True ? empty_f32({m.size(0), m.size(1)}, m) : at::Tensor();
         const int rc = api.wide_update((int16_t*)m.data_ptr(), (int8_t*)e.data_ptr(), (const float*)d.data_ptr(), m.size(0), m.size(1), ld_of(d), &f,
-                                       v.m0, v.e0, v.m1, v.e1, value.defined() ? (float*)value.data_ptr() : nullptr, m.size(1), stream());
+                                       v.m0, v.e0, v.m1, v.e1, value.defined() ? (float*)value.data_ptr() : nullptr, m.size(1), cur_stream());
         return !rc && value.defined() ? THPVariable_Wrap(value) : code(rc);
     });
 }
@@ -258,7 +285,7 @@ PyObject* wide_dequantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor out = fresh ? empty_f32({m.size(0), m.size(1)}, m) : tensor_of(a[3], "out");
         check_f32(out, "out");
         const int rc = api.wide_dequantize((const int16_t*)m.data_ptr(), (const int8_t*)e.data_ptr(), m.size(0), m.size(1), (int32_t)as_ll(a[2]),
-                                           (float*)out.data_ptr(), ld_of(out), stream());
+                                           (float*)out.data_ptr(), ld_of(out), cur_stream());
         if (rc) return code(rc);
         return fresh ? THPVariable_Wrap(out) : same(a[3]);
     });
@@ -274,7 +301,7 @@ PyObject* conv_forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor out = fresh ? empty_f32({nn * h * w, nf}, px.data) : tensor_of(a[10], "out");
         check_f32(out, "out");
         const int rc = api.conv_forward(px.o.data, px.o.exps, nn, h, w, as_ll(a[5]), (int)as_ll(a[6]), (int)as_ll(a[7]), (int)as_ll(a[8]), &px.o.fmt, &fl.o,
-                                        nf, (float*)out.data_ptr(), ld_of(out), stream());
+                                        nf, (float*)out.data_ptr(), ld_of(out), cur_stream());
         if (rc) return code(rc);
         return fresh ? THPVariable_Wrap(out) : same(a[10]);
     });
@@ -298,7 +325,7 @@ PyObject* conv_dgrad_filters(PyObject*, PyObject* const* a, Py_ssize_t n) {
             m = tensor_of(a[5], "mantissas");
             e = tensor_of(a[6], "exponents");
         }
-        const int rc = api.conv_dgrad_filters(c1.o.data, c1.o.exps, kh, kw, ci, co, &c1.o.fmt, m.data_ptr(), (int8_t*)e.data_ptr(), stream());
+        const int rc = api.conv_dgrad_filters(c1.o.data, c1.o.exps, kh, kw, ci, co, &c1.o.fmt, m.data_ptr(), (int8_t*)e.data_ptr(), cur_stream());
         if (rc) return code(rc);
         return Py_BuildValue("(NN)", THPVariable_Wrap(m), THPVariable_Wrap(e));
     });
@@ -325,58 +352,272 @@ PyObject* im2col_packed_t(PyObject*, PyObject* const* a, Py_ssize_t n) {
             e = tensor_of(a[6], "exponents");
         }
         const int rc = api.im2col_packed_t((const float*)x.data_ptr(), x.size(0), x.size(1), x.size(2), x.size(3), kh, kw, (int)as_ll(a[3]), &f, m.data_ptr(),
-                                           (int8_t*)e.data_ptr(), stream());
+                                           (int8_t*)e.data_ptr(), cur_stream());
         if (rc) return code(rc);
         return Py_BuildValue("(NN)", THPVariable_Wrap(m), THPVariable_Wrap(e));
     });
 }
 
-// linear_forward(x, c0, fmt, fin, fout, bias or None) -> y
-PyObject* linear_forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
-    if (!want(n, 6)) return nullptr;
-    return guarded([&]() -> PyObject* {
-        const Operand x = operand_of(a[0], 0, a[2]), w = operand_of(a[1], 0, Py_None);
-        const int64_t batch = x.data.size(0), fin = as_ll(a[3]), fout = as_ll(a[4]);
-        at::Tensor y = empty_f32({batch, fout}, x.data);
-        const int rc = run_gemm(batch, fout, fin, x.o, w.o, y, nullptr, HBFP_GEMM_AUTO);
-        if (rc) return code(rc);
-        if (a[5] != Py_None) y.add_(tensor_of(a[5], "bias"));
+// ------------------------------------------------------------------------------ layers
+
+// The two layers as autograd nodes of their own. As Python functions their forward and backward passes spent most of a
+// training step in the interpreter: argument marshalling, packed-operand and format objects, one call into the library per
+// product and the hand-over between the autograd engine and Python for every layer. A node runs its whole pass here, on the
+// engine's thread, without the interpreter.
+
+PyObject* error_type = nullptr;              // HbfpError(code, where)
+
+// Raises HbfpError from code that may hold no interpreter lock.
+[[noreturn]] void raise_status(int rc, const char* where) {
+    pybind11::gil_scoped_acquire gil;
+    PyObject* e = PyObject_CallFunction(error_type, "is", rc, where);
+    if (e) {
+        PyErr_SetObject(error_type, e);
+        Py_DECREF(e);
+    }
+    python_error err;
+    err.persist();
+    throw err;
+}
+void ok_or_raise(int rc, const char* where) {
+    if (rc) raise_status(rc, where);
+}
+
+struct PackedTensor {
+    at::Tensor mant, exps;
+    hbfp_format fmt{};
+    hbfp_operand operand() const {
+        hbfp_operand o{};
+        o.struct_size = sizeof(o);
+        o.kind = HBFP_OPERAND_PACKED;
+        o.data = mant.data_ptr();
+        o.exps = (const int8_t*)exps.data_ptr();
+        o.fmt = fmt;
+        return o;
+    }
+};
+PackedTensor packed_of(PyObject* x) {
+    const Operand o = operand_of(x, 0, Py_None);
+    if (o.o.kind != HBFP_OPERAND_PACKED) {
+        PyErr_SetString(PyExc_TypeError, "a packed operand is expected");
+        throw Fail{};
+    }
+    return {o.data, o.exps, o.o.fmt};
+}
+hbfp_operand fp32_operand(const at::Tensor& x, int trans, const hbfp_format& f) {
+    check_f32_cpp(x);
+    hbfp_operand o{};
+    o.struct_size = sizeof(o);
+    o.kind = HBFP_OPERAND_FP32;
+    o.data = x.data_ptr();
+    o.ld = ld_of(x);
+    o.trans = trans;
+    o.fmt = f;
+    return o;
+}
+hbfp_format make_format(int mant_bits, int block, int rounding, uint64_t seed, uint32_t stream_id) {
+    hbfp_format f{};
+    f.struct_size = sizeof(f);
+    f.mant_bits = mant_bits;
+    f.block = block;
+    f.rounding = rounding;
+    f.seed = seed;
+    f.stream_id = stream_id;
+    return f;
+}
+PackedTensor alloc_packed(int64_t rows, int64_t k, const hbfp_format& f, const at::Tensor& like, const char* where) {
+    hbfp_layout L;
+    ok_or_raise(api.packed_layout(rows, k, &f, &L), where);
+    return {empty_i8(L.mant_bytes, like), empty_i8(L.exp_bytes, like), f};
+}
+at::Tensor product(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_operand& b, const at::Tensor& like) {
+    at::Tensor out = empty_f32({M, N}, like);
+    ok_or_raise(run_gemm(M, N, K, a, b, out, nullptr, HBFP_GEMM_AUTO), "hbfp_gemm_q");
+    return out;
+}
+// Everything a pass computes lies below autograd; gradients come out as plain tensors.
+struct Below {
+    at::AutoDispatchBelowADInplaceOrView below;
+    c10::AutoGradMode off{false};
+};
+using torch::autograd::SavedVariable;
+using torch::autograd::variable_list;
+
+struct LinearNode : public torch::autograd::Node {
+    SavedVariable x_;
+    PackedTensor c1;
+    int mant_bits, tile, batch_block, rounding;
+    uint64_t seed;
+    uint32_t stream_id;
+    int64_t fin, fout;
+    // X (which = 0) or dY (which = 2) in blocks along a feature axis or along the batch axis
+    hbfp_format act(int which, bool batch_axis) const { return make_format(mant_bits, batch_axis ? batch_block : tile, rounding, seed, stream_id + which); }
+    std::string name() const override { return "HbfpLinearBackward"; }
+    void release_variables() override { x_.reset_data(); }
+    variable_list apply(variable_list&& grads) override {
+        variable_list out(3);
+        if (!grads[0].defined()) return out;
+        const at::Tensor x0 = x_.unpack(shared_from_this());
+        Below guard;
+        const at::Tensor dy = grads[0].contiguous(), x = x0.contiguous();
+        const int64_t batch = x.size(0);
+        // backward-data on the shared weight view; backward-weight with blocks down the columns of X and dY
+        if (task_should_compute_output(0)) out[0] = product(batch, fin, fout, fp32_operand(dy, 0, act(2, false)), c1.operand(), dy);
+        if (task_should_compute_output(1)) out[1] = product(fin, fout, batch, fp32_operand(x, 1, act(0, true)), fp32_operand(dy, 0, act(2, true)), dy);
+        if (task_should_compute_output(2)) out[2] = dy.sum(0);
+        return out;
+    }
+};
+
+// linear(x, weight, bias or None, c0, c1, mant_bits, tile, batch_block, rounding, seed, stream_id) -> y
+PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!want(n, 11)) return nullptr;
+    return layer_call([&]() -> PyObject* {
+        const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
+        const at::Tensor bias = a[2] != Py_None ? tensor_of(a[2], "bias") : at::Tensor();
+        const PackedTensor c0 = packed_of(a[3]);
+        LinearNode proto;
+        proto.mant_bits = (int)as_ll(a[5]); proto.tile = (int)as_ll(a[6]); proto.batch_block = (int)as_ll(a[7]); proto.rounding = (int)as_ll(a[8]);
+        proto.seed = PyLong_AsUnsignedLongLongMask(a[9]);
+        proto.stream_id = (uint32_t)PyLong_AsUnsignedLongLongMask(a[10]);
+        if (PyErr_Occurred()) throw Fail{};
+        proto.fin = w.size(0);
+        proto.fout = w.size(1);
+        at::Tensor y;
+        {
+            Below guard;
+            const at::Tensor xc = x.contiguous();
+            y = product(xc.size(0), proto.fout, proto.fin, fp32_operand(xc, 0, proto.act(0, false)), c0.operand(), xc);
+            if (bias.defined()) y.add_(bias);
+        }
+        if (torch::autograd::compute_requires_grad(x, w, bias)) {
+            auto node = std::shared_ptr<LinearNode>(new LinearNode(), torch::autograd::deleteNode);
+            node->set_next_edges(torch::autograd::collect_next_edges(x, w, bias));
+            node->x_ = SavedVariable(x, false);
+            node->c1 = packed_of(a[4]);
+            node->mant_bits = proto.mant_bits; node->tile = proto.tile; node->batch_block = proto.batch_block; node->rounding = proto.rounding;
+            node->seed = proto.seed; node->stream_id = proto.stream_id; node->fin = proto.fin; node->fout = proto.fout;
+            torch::autograd::set_history(y, node);
+        }
         return THPVariable_Wrap(y);
     });
 }
 
-// linear_backward(dy, x, c1, fmt of dy, batch-axis fmts of x and dy, fin, fout, need dx, need dw, need db) -> (dx, dw, db)
-PyObject* linear_backward(PyObject*, PyObject* const* a, Py_ssize_t n) {
-    if (!want(n, 11)) return nullptr;
-    return guarded([&]() -> PyObject* {
-        const at::Tensor dy = tensor_of(a[0], "dy"), x = tensor_of(a[1], "x");
-        check_f32(dy, "dy");
-        check_f32(x, "x");
-        const int64_t batch = x.size(0), fin = as_ll(a[6]), fout = as_ll(a[7]);
-        at::Tensor dx, dw, db;
-        if (PyObject_IsTrue(a[8])) {
-            const Operand g = operand_of(a[0], 0, a[3]), w = operand_of(a[2], 0, Py_None);
-            dx = empty_f32({batch, fin}, dy);
-            const int rc = run_gemm(batch, fin, fout, g.o, w.o, dx, nullptr, HBFP_GEMM_AUTO);
-            if (rc) return code(rc);
+struct ConvNode : public torch::autograd::Node {
+    SavedVariable x_;
+    PackedTensor c1;
+    int mant_bits, pixel_block;
+    int64_t c, f;
+    hbfp_format pixels(int which) const { return make_format(mant_bits, (int)c, 0, 0, which); }           // blocks of c channels of a pixel
+    hbfp_format batch(int which) const { return make_format(mant_bits, pixel_block, 0, 0, which); }       // blocks of consecutive pixels
+    std::string name() const override { return "HbfpConv3x3Backward"; }
+    void release_variables() override { x_.reset_data(); }
+    static PackedTensor convert(const at::Tensor& x2, const hbfp_format& fmt) {
+        PackedTensor p = alloc_packed(x2.size(0), x2.size(1), fmt, x2, "hbfp_quantize");
+        ok_or_raise(api.quantize((const float*)x2.data_ptr(), x2.size(0), x2.size(1), ld_of(x2), 1, &fmt, p.mant.data_ptr(), (int8_t*)p.exps.data_ptr(), cur_stream()),
+                    "hbfp_quantize");
+        return p;
+    }
+    // 3 x 3 taps, one pixel of padding, as an implicit GEMM: HBFP_ERR_UNSUPPORTED for shapes the kernel does not cover
+    static int implicit(const PackedTensor& px, const PackedTensor& filters, int64_t n, int64_t h, int64_t w, int64_t ch, const at::Tensor& y) {
+        const hbfp_operand fo = filters.operand();
+        const int64_t nf = y.size(-1);
+        return api.conv_forward(px.mant.data_ptr(), (const int8_t*)px.exps.data_ptr(), n, h, w, ch, 3, 3, 1, &px.fmt, &fo, nf, (float*)y.data_ptr(), nf, cur_stream());
+    }
+    at::Tensor forward(const at::Tensor& x, const PackedTensor& c0) const {
+        const int64_t n = x.size(0), h = x.size(1), w = x.size(2), px = n * h * w;
+        const PackedTensor q = convert(x.view({px, c}), pixels(0));
+        at::Tensor y = empty_f32({n, h, w, f}, x);
+        const int rc = implicit(q, c0, n, h, w, c, y);
+        if (rc != HBFP_ERR_UNSUPPORTED) {
+            ok_or_raise(rc, "hbfp_conv_forward");
+            return y;
         }
-        if (PyObject_IsTrue(a[9])) {
-            // contraction over the batch axis: blocks down the columns of X and dY
-            const Operand xt = operand_of(a[1], 1, a[4]), g = operand_of(a[0], 0, a[5]);
-            dw = empty_f32({fin, fout}, dy);
-            const int rc = run_gemm(fin, fout, batch, xt.o, g.o, dw, nullptr, HBFP_GEMM_AUTO);
-            if (rc) return code(rc);
+        // gather the packed operand, then the ordinary GEMM (same product)
+        const PackedTensor cols = alloc_packed(px, 9 * c, q.fmt, x, "hbfp_im2col_packed");
+        ok_or_raise(api.im2col_packed(q.mant.data_ptr(), (const int8_t*)q.exps.data_ptr(), n, h, w, c, 3, 3, 1, &q.fmt, cols.mant.data_ptr(),
+                                      (int8_t*)cols.exps.data_ptr(), cur_stream()), "hbfp_im2col_packed");
+        ok_or_raise(run_gemm(px, f, 9 * c, cols.operand(), c0.operand(), y.view({px, f}), nullptr, HBFP_GEMM_AUTO), "hbfp_gemm_q");
+        return y;
+    }
+    at::Tensor data_gradient(const at::Tensor& dy2, int64_t n, int64_t h, int64_t w) const {
+        // the convolution of the packed output gradient with the forward weights regrouped (taps turned by 180 degrees,
+        // feature-map roles swapped) yields dX itself
+        hbfp_layout L;
+        int rc = api.packed_layout(c, 9 * f, &c1.fmt, &L);
+        if (!rc) {
+            const PackedTensor turned{empty_i8(L.mant_bytes, dy2), empty_i8(L.exp_bytes, dy2), c1.fmt};
+            rc = api.conv_dgrad_filters(c1.mant.data_ptr(), (const int8_t*)c1.exps.data_ptr(), 3, 3, c, f, &c1.fmt, turned.mant.data_ptr(),
+                                        (int8_t*)turned.exps.data_ptr(), cur_stream());
+            if (!rc) {
+                const PackedTensor g = convert(dy2, pixels(2));
+                at::Tensor dx = empty_f32({n, h, w, c}, dy2);
+                rc = implicit(g, turned, n, h, w, f, dx);
+                if (!rc) return dx;
+            }
         }
-        if (PyObject_IsTrue(a[10])) db = dy.sum(0);
-        auto wrap = [](const at::Tensor& t) { return t.defined() ? THPVariable_Wrap(t) : same(Py_None); };
-        return Py_BuildValue("(NNN)", wrap(dx), wrap(dw), wrap(db));
+        if (rc != HBFP_ERR_UNSUPPORTED) raise_status(rc, "hbfp_conv_forward");
+        // shapes that route does not cover: gradient of the im2col matrix, then its scatter back onto the pixels (FP32)
+        const at::Tensor dcols = product(n * h * w, 9 * c, f, fp32_operand(dy2, 0, pixels(2)), c1.operand(), dy2).view({n, h, w, 3, 3, c});
+        at::Tensor dxp = at::zeros({n, h + 2, w + 2, c}, dy2.options());
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) dxp.slice(1, i, i + h).slice(2, j, j + w).add_(dcols.select(4, j).select(3, i));
+        return dxp.slice(1, 1, h + 1).slice(2, 1, w + 1).contiguous();
+    }
+    variable_list apply(variable_list&& grads) override {
+        variable_list out(2);
+        if (!grads[0].defined()) return out;
+        const at::Tensor x0 = x_.unpack(shared_from_this());
+        Below guard;
+        const at::Tensor x = x0.contiguous();
+        const int64_t n = x.size(0), h = x.size(1), w = x.size(2), px = n * h * w;
+        const at::Tensor dy2 = grads[0].contiguous().view({px, f});
+        if (task_should_compute_output(0)) out[0] = data_gradient(dy2, n, h, w);
+        if (task_should_compute_output(1)) {
+            const hbfp_format fx = batch(0);
+            const PackedTensor xt = alloc_packed(9 * c, px, fx, x, "hbfp_im2col_packed_t");
+            ok_or_raise(api.im2col_packed_t((const float*)x.data_ptr(), n, h, w, c, 3, 3, 1, &fx, xt.mant.data_ptr(), (int8_t*)xt.exps.data_ptr(), cur_stream()),
+                        "hbfp_im2col_packed_t");
+            out[1] = product(9 * c, f, px, xt.operand(), fp32_operand(dy2, 0, batch(2)), dy2);
+        }
+        return out;
+    }
+};
+
+// conv3x3(x, weight, c0, c1, mant_bits, pixel_block, c, f) -> y
+PyObject* conv3x3(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!want(n, 8)) return nullptr;
+    return layer_call([&]() -> PyObject* {
+        const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
+        if (!(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 4)) value_error("%s must be a float32 CUDA tensor [n][h][w][c]", "x");
+        auto node = std::shared_ptr<ConvNode>(new ConvNode(), torch::autograd::deleteNode);
+        node->mant_bits = (int)as_ll(a[4]);
+        node->pixel_block = (int)as_ll(a[5]);
+        node->c = as_ll(a[6]);
+        node->f = as_ll(a[7]);
+        const PackedTensor c0 = packed_of(a[2]);
+        at::Tensor y;
+        {
+            Below guard;
+            y = node->forward(x.contiguous(), c0);
+        }
+        if (torch::autograd::compute_requires_grad(x, w)) {
+            node->set_next_edges(torch::autograd::collect_next_edges(x, w));
+            node->x_ = SavedVariable(x, false);
+            node->c1 = packed_of(a[3]);
+            torch::autograd::set_history(y, node);
+        }
+        return THPVariable_Wrap(y);
     });
 }
 
-// bind(addresses in the order of Api)
+// bind(type of the error to raise, addresses in the order of Api)
 PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
     constexpr Py_ssize_t N = sizeof(Api) / sizeof(void*);
-    if (!want(n, N)) return nullptr;
+    if (!want(n, N + 1)) return nullptr;
+    Py_INCREF(a[0]);
+    Py_XSETREF(error_type, a[0]);
+    ++a;
     void* p[N];
     for (Py_ssize_t i = 0; i < N; ++i) {
         p[i] = PyLong_AsVoidPtr(a[i]);
@@ -393,7 +634,7 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
 #define HBFP_METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {HBFP_METHOD(bind), HBFP_METHOD(quantize), HBFP_METHOD(gemm), HBFP_METHOD(gemm_q), HBFP_METHOD(wide_update),
                          HBFP_METHOD(wide_dequantize), HBFP_METHOD(conv_forward), HBFP_METHOD(conv_dgrad_filters),
-                         HBFP_METHOD(im2col_packed_t), HBFP_METHOD(linear_forward), HBFP_METHOD(linear_backward),
+                         HBFP_METHOD(im2col_packed_t), HBFP_METHOD(linear), HBFP_METHOD(conv3x3),
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 

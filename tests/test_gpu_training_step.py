@@ -156,3 +156,52 @@ def test_convolution_layer_products_match_the_oracle_and_fp32(env):
     y32 = torch.nn.functional.conv2d(x.detach().permute(0, 3, 1, 2), w4, padding=1).permute(0, 2, 3, 1)
     rel = (y.detach() - y32).norm() / y32.norm()
     assert float(rel) < 2e-2
+
+
+@pytest.mark.parametrize("c,f", [(24, 40), (64, 40), (32, 96)])
+def test_convolution_layer_on_shapes_without_an_implicit_route(env, c, f):
+    """Feature-map counts that the implicit GEMM or the regrouped filters do not cover take the gathered operand and the scatter:
+    the same products as the library's calls one by one (the scatter's FP32 sums to rounding: nine terms, 9 * 2^-24)."""
+    torch, hbfp_nn, hb = env
+    torch.manual_seed(4)
+    n, hw = 2, 8
+    px = n * hw * hw
+    layer = hbfp_nn.HbfpConv3x3(c, f)
+    x = torch.randn(n, hw, hw, c, device="cuda").requires_grad_(True)
+    dy = torch.randn(n, hw, hw, f, device="cuda")
+    y = layer(x)
+    y.backward(dy)
+    q = hb.quantize(x.detach().view(px, c), 1, layer.fmt_pixels(0))
+    want = hb.gemm_q(px, f, 9 * c, hb.im2col_packed(q, n, hw, hw, c, 3, 3, 1), layer.views[0])
+    assert torch.allclose(y.detach().view(px, f), want, rtol=1e-6, atol=1e-6 * float(want.abs().max()))
+    dcols = hb.gemm_q(px, 9 * c, f, dy.view(px, f), layer.views[1], fmtA=layer.fmt_pixels(2)).view(n, hw, hw, 3, 3, c)
+    dxp = torch.zeros((n, hw + 2, hw + 2, c), device="cuda")
+    for i in range(3):
+        for j in range(3):
+            dxp[:, i:i + hw, j:j + hw, :] += dcols[:, :, :, i, j, :]
+    want = dxp[:, 1:hw + 1, 1:hw + 1, :]
+    assert torch.allclose(x.grad, want, rtol=1e-5, atol=9 * 2.0 ** -24 * float(dcols.abs().max()) * 9)
+    assert layer.weight.grad.shape == (9 * c, f) and hb.device_status() == 0
+
+
+def test_layer_nodes_follow_autograd(env):
+    """Gradients only for what asks for one, none recorded under no_grad, the library's error out of a backward pass."""
+    torch, hbfp_nn, hb = env
+    layer = hbfp_nn.HbfpLinear(48, 24)
+    x = torch.randn(32, 48, device="cuda")
+    layer(x).sum().backward()
+    assert x.grad is None and layer.weight.grad.shape == (48, 24) and layer.bias.grad.shape == (24,)
+    with torch.no_grad():
+        assert layer(x).grad_fn is None
+    layer.requires_grad_(False)
+    assert not layer(x).requires_grad
+    xg = x.clone().requires_grad_(True)
+    layer(xg).sum().backward()
+    assert xg.grad.shape == x.shape
+    wide = hbfp_nn.HbfpLinear(48, 24, mant_bits=12, batch_block=600)      # block sums of 600 products of 12 bits exceed int32
+    y = wide(x)
+    with pytest.raises(hb.HbfpError) as e:
+        y.sum().backward()
+    assert e.value.code == hb.ERR_UNSUPPORTED
+    with pytest.raises(ValueError):
+        layer(x.half())
