@@ -336,6 +336,16 @@ HBFP_API int hbfp_gemm_q(int64_t M, int64_t N, int64_t K, const hbfp_operand* a,
                          const hbfp_operand* b, float* C, int64_t ldc, void* workspace,
                          size_t workspace_bytes, uint32_t flags, void* stream);
 
+/* hbfp_gemm_q followed by the FP32 addition of bias[N] to every row of C (NULL: none), in the product's own store
+ * where its kernel allows it: the same values as adding afterwards, without another pass over C. */
+HBFP_API int hbfp_gemm_q_bias(int64_t M, int64_t N, int64_t K, const hbfp_operand* a,
+                              const hbfp_operand* b, const float* bias, float* C, int64_t ldc, void* workspace,
+                              size_t workspace_bytes, uint32_t flags, void* stream);
+
+/* out[j] = sum over i of x[i][j] in FP32, x [rows][cols] with pitch ld: the bias gradient. The order of the additions
+ * depends on the extents alone. */
+HBFP_API int hbfp_column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, void* stream);
+
 /* Convolution forward pass as one implicit GEMM (Sec. 5.1: convolutions run through the same BFP dot
  * products): Y [n*h*w][filters] = conv(x, filters), stride 1, `pad` zeros around the image, an output as
  * large as the input (2 pad == kh - 1 == kw - 1). x: the activations [n][h][w][c] converted once per

@@ -159,8 +159,10 @@ int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, cons
     return launch_expand(p, g.fp, !is_a, f, st);
 }
 
-int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp_operand* b, float* C,
+// bias (may be null) is added in the kernel's own store where it can; *bias_done says so, otherwise the caller adds it.
+int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp_operand* b, const float* bias, bool* bias_done, float* C,
               int64_t ldc, void* workspace, size_t ws_bytes, uint32_t flags, int32_t* P, cudaStream_t st) {
+    *bias_done = false;
     GemmPlan g;
     int rc = make_plan(M, N, K, a, b, &g);
     if (rc) return rc;
@@ -192,7 +194,8 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, st);
         if (rc) return rc;
         t_last_gemm_kernel = "gemm_skinny_kernel";
-        return launch_gemm_skinny(M, N, K, static_cast<const float*>(a->data), a->ld, &a->fmt, pb, C, ldc, st);
+        *bias_done = true;
+        return launch_gemm_skinny(M, N, K, static_cast<const float*>(a->data), a->ld, &a->fmt, pb, bias, C, ldc, st);
     }
     if (use_fp && !small) {
         const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
@@ -201,7 +204,8 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         rc = resolve_form(b, false, N, K, g, ws, fb, st);
         if (rc) return rc;
         t_last_gemm_kernel = "gemm_tc_kernel";      // one SM per tile, like its integer sibling
-        return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, C, ldc, st);
+        *bias_done = true;
+        return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, bias, C, ldc, st);
     }
     rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, st);
     if (rc) return rc;
@@ -493,9 +497,21 @@ int hbfp_gemm_workspace(int transA, int transB, int64_t M, int64_t N, int64_t K,
 
 int hbfp_gemm_q(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp_operand* b, float* C,
                 int64_t ldc, void* workspace, size_t workspace_bytes, uint32_t flags, void* stream) {
+    return hbfp_gemm_q_bias(M, N, K, a, b, nullptr, C, ldc, workspace, workspace_bytes, flags, stream);
+}
+
+int hbfp_gemm_q_bias(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp_operand* b, const float* bias, float* C,
+                     int64_t ldc, void* workspace, size_t workspace_bytes, uint32_t flags, void* stream) {
     if (!C && M * N > 0) return HBFP_ERR_INVALID_ARG;
-    return gemm_impl(M, N, K, a, b, C, ldc, workspace, workspace_bytes, flags, nullptr,
-                     static_cast<cudaStream_t>(stream));
+    bool bias_done = false;
+    const int rc = gemm_impl(M, N, K, a, b, bias, &bias_done, C, ldc, workspace, workspace_bytes, flags, nullptr, static_cast<cudaStream_t>(stream));
+    if (rc || !bias || bias_done || M == 0 || N == 0) return rc;
+    return launch_add_bias(C, M, N, ldc, bias, static_cast<cudaStream_t>(stream));
+}
+
+int hbfp_column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, void* stream) {
+    if (rows < 0 || cols < 0 || ld < cols || (cols > 0 && (!out || (rows > 0 && !x)))) return HBFP_ERR_INVALID_ARG;
+    return launch_column_sums(x, rows, cols, ld, out, static_cast<cudaStream_t>(stream));
 }
 
 int hbfp_gemm(int transA, int transB, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
@@ -513,7 +529,8 @@ int hbfp_gemm_block_partials(int64_t M, int64_t N, int64_t K, const hbfp_operand
     if (!P || !a || !b) return HBFP_ERR_INVALID_ARG;
     if (a->kind != HBFP_OPERAND_PACKED || b->kind != HBFP_OPERAND_PACKED) return HBFP_ERR_INVALID_ARG;
     if (impl != HBFP_GEMM_FORCE_SIMT && impl != HBFP_GEMM_FORCE_TENSOR) return HBFP_ERR_INVALID_ARG;
-    return gemm_impl(M, N, K, a, b, nullptr, N, nullptr, 0, impl, P, static_cast<cudaStream_t>(stream));
+    bool bias_done;
+    return gemm_impl(M, N, K, a, b, nullptr, &bias_done, nullptr, N, nullptr, 0, impl, P, static_cast<cudaStream_t>(stream));
 }
 
 int hbfp_selftest_bounded_wait(int64_t limit_cycles, int32_t code, int32_t* outcome, void* stream) {

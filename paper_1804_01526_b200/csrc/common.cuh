@@ -98,7 +98,7 @@ int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, fl
 
 // A few rows of FP32 activations against packed weights, conversion included (gemm_skinny.cu): one launch, no scratch.
 bool skinny_gemm_eligible(int64_t M, int64_t N, const Layout& la, const Layout& lb, int bits_a, int bits_b);
-int launch_gemm_skinny(int64_t M, int64_t N, int64_t K, const float* x, int64_t ld, const hbfp_format* fx, const Packed& w, float* C,
+int launch_gemm_skinny(int64_t M, int64_t N, int64_t K, const float* x, int64_t ld, const hbfp_format* fx, const Packed& w, const float* bias, float* C,
                        int64_t ldc, cudaStream_t st);
 
 // Workspace of the integer kernels alone (hbfp_gemm_workspace may ask for more).
@@ -140,8 +140,12 @@ int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const FpOperan
 // Converts an FP32 operand straight to a form (quantize.cu); HBFP_ERR_UNSUPPORTED for weight tiles.
 int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int contract_axis, const hbfp_format* f, int wide, bool is_b,
                          const FpOperand& out, cudaStream_t st);
-int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, float* C,
+int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, const float* bias, float* C,
                    int64_t ldc, cudaStream_t st);
+
+// FP32 parts of a layer (layer.cu): the bias added to a stored product, the column sums that are its gradient.
+int launch_add_bias(float* C, int64_t M, int64_t N, int64_t ldc, const float* bias, cudaStream_t st);
+int launch_column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, cudaStream_t st);
 
 // Convolution forward as an implicit GEMM over the packed pixels (gemm_conv.cu).
 int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw,

@@ -67,6 +67,7 @@ struct FpProblem {
     int tiles_m, tiles_n;
     int splits, kb_per_split;     // splits > 1: the CTAs of a cluster share a tile
     int tma_out;                  // C leaves through TMA stores (16-byte aligned, pitch of whole quads)
+    const float* bias;            // may be null
     float* C;
     int64_t ldc;
     int32_t* status;
@@ -250,10 +251,26 @@ __device__ __forceinline__ void fp_store_rows(const uint64_t (&acc2)[NC / 2], co
     }
 }
 
+// The bias of the columns [gj0, gj0 + NC): one more addition per output, after the last block. One load per 32 columns and
+// shuffles: a load per column held up the end of every tile by 2400 cycles.
+template <int NC>
+__device__ __forceinline__ void fp_add_bias(uint64_t (&acc2)[NC / 2], const FpProblem& p, int gj0) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < NC; h += 32) {
+        const int gj = gj0 + h + lane;
+        const float mine = gj < p.N ? __ldg(p.bias + gj) : 0.f;
+#pragma unroll
+        for (int c = 0; c < 32; c += 2)
+            acc2[(h + c) / 2] = fadd2(acc2[(h + c) / 2], pack2(__float_as_uint(__shfl_sync(0xffffffffu, mine, c)), __float_as_uint(__shfl_sync(0xffffffffu, mine, c + 1))));
+    }
+}
+
 // Split-K parts of a tile, one per CTA of the cluster: every part goes to its CTA's shared memory (rows padded so that
 // eight lanes' 16-byte stores hit all banks), then each CTA adds up a share of the rows over the cluster in ascending
 // order of K. Runs in the rescale warps; called whether or not their waits succeeded, so that every barrier is met.
-template <int NOUT, int NC>
+template <int NOUT, int NC, bool BIAS>
 __device__ __forceinline__ void fp_split_sum(const uint64_t (&acc2)[NC / 2], const FpProblem& p, uint32_t base, unsigned char* base_ptr,
                                              const FpWork& w, int rank, int row, int col0) {
     constexpr int NT = 32 * FP_RW;
@@ -280,6 +297,10 @@ __device__ __forceinline__ void fp_split_sum(const uint64_t (&acc2)[NC / 2], con
 #pragma unroll
             for (int e = 0; e < 4; ++e) x[e] = sp == 0 ? y[e] : __fadd_rn(x[e], y[e]);
         }
+        if constexpr (BIAS)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (gj + e < p.N) x[e] = __fadd_rn(x[e], __ldg(p.bias + gj + e));
         float* dst = p.C + (int64_t)gi * p.ldc + gj;
         if (quad && gj + 3 < p.N) *reinterpret_cast<float4*>(dst) = make_float4(x[0], x[1], x[2], x[3]);
         else
@@ -291,7 +312,8 @@ __device__ __forceinline__ void fp_split_sum(const uint64_t (&acc2)[NC / 2], con
 
 // ------------------------------------------------------------------------------ kernel
 
-template <int FORM, int NCOL, int BP, bool PAIR>
+// BIAS is a parameter of the kernel and not a run-time branch: the branch alone cost the 12-bit kernel 4 % (222 -> 232 us, 4096 cube).
+template <int FORM, int NCOL, int BP, bool PAIR, bool BIAS>
 __global__ void __launch_bounds__(FP_THREADS, 1)
 gemm_fp_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapB1,
                const __grid_constant__ CUtensorMap mapSA, const __grid_constant__ CUtensorMap mapSB,
@@ -464,10 +486,11 @@ gemm_fp_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             const bool ok = fp_blocks<FORM, NCOL, BP, PAIR>(acc2, p, ra, nblk, col0, ring);
             if constexpr (!PAIR) if (split) {
                 __syncwarp();
-                fp_split_sum<C::NOUT, NC>(acc2, p, base, base_ptr, w, rank, quarter * 32 + lane, col0);
+                fp_split_sum<C::NOUT, NC, BIAS>(acc2, p, base, base_ptr, w, rank, quarter * 32 + lane, col0);
                 break;
             }
             if (!ok) break;
+            if constexpr (BIAS) fp_add_bias<NC>(acc2, p, w.n0 + col0);
             const int gi0 = w.m0 + (PAIR ? rank * TILE_M : 0) + quarter * 32;
             if constexpr (FORM == FORM_W) { fp_store_rows<NC>(acc2, p, gi0 + lane, w.n0 + col0); continue; }
 #pragma unroll
@@ -610,14 +633,14 @@ int make_map_f32(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t outer
 }
 
 // Shared-memory attribute and, for pairs, the number of clusters the device holds: they belong to the device.
-template <int FORM, int NCOL, int BP, bool PAIR>
+template <int FORM, int NCOL, int BP, bool PAIR, bool BIAS>
 int fp_device_setup(int* clusters) {
     using C = FpCfg<FORM, NCOL, BP, PAIR>;
     static int ready[MAX_DEVICES] = {};        // 0: not yet, else 1 + clusters
     const int dev = current_device();
     if (dev < 0) return HBFP_ERR_CUDA;
     if (!ready[dev]) {
-        HBFP_CUDA_OK(cudaFuncSetAttribute(gemm_fp_kernel<FORM, NCOL, BP, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+        HBFP_CUDA_OK(cudaFuncSetAttribute(gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
         int n = 0;
         if (PAIR) {
             cudaLaunchConfig_t cfg = {};
@@ -629,7 +652,7 @@ int fp_device_setup(int* clusters) {
             cfg.dynamicSmemBytes = C::SMEM;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&n, gemm_fp_kernel<FORM, NCOL, BP, PAIR>, &cfg) != cudaSuccess || n < 1) {
+            if (cudaOccupancyMaxActiveClusters(&n, gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, &cfg) != cudaSuccess || n < 1) {
                 cudaGetLastError();
                 return HBFP_ERR_CUDA;
             }
@@ -640,14 +663,14 @@ int fp_device_setup(int* clusters) {
     return HBFP_OK;
 }
 
-template <int FORM, int NCOL, int BP, bool PAIR>
+template <int FORM, int NCOL, int BP, bool PAIR, bool BIAS>
 int fp_launch(FpProblem p, const FpOperand& a, const FpOperand& b, cudaStream_t st) {
     using C = FpCfg<FORM, NCOL, BP, PAIR>;
     constexpr int TM = PAIR ? 2 * TILE_M : TILE_M;
     p.tiles_m = (p.M + TM - 1) / TM;
     p.tiles_n = (p.N + C::NOUT - 1) / C::NOUT;
     int clusters = 0;
-    int rc = fp_device_setup<FORM, NCOL, BP, PAIR>(&clusters);
+    int rc = fp_device_setup<FORM, NCOL, BP, PAIR, BIAS>(&clusters);
     if (rc) return rc;
     CUtensorMap mA, mB, mB1, mSA, mSB, mC;
     rc = make_map(&mA, a.p0, 2 * a.kst, a.rows, 2 * a.kst, 128, TILE_M, true);
@@ -681,17 +704,21 @@ int fp_launch(FpProblem p, const FpOperand& a, const FpOperand& b, cudaStream_t 
     at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = csize > 1 ? 1 : 0;
-    HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_fp_kernel<FORM, NCOL, BP, PAIR>, mA, mB, mB1, mSA, mSB, mC, p));
+    HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, mA, mB, mB1, mSA, mSB, mC, p));
     return HBFP_OK;
 }
 
-template <int FORM, int BP>
+template <int FORM, int BP, bool BIAS>
 int fp_launch_bp(const FpProblem& p, const FpPlan& plan, const FpOperand& a, const FpOperand& b, cudaStream_t st) {
-    if (plan.pair) return fp_launch<FORM, 256, BP, true>(p, a, b, st);
-    if (plan.ncol == 256) return fp_launch<FORM, 256, BP, false>(p, a, b, st);
-    if (plan.ncol == 128) return fp_launch<FORM, 128, BP, false>(p, a, b, st);
-    if constexpr (FORM == FORM_S) return fp_launch<FORM, 64, BP, false>(p, a, b, st);
+    if (plan.pair) return fp_launch<FORM, 256, BP, true, BIAS>(p, a, b, st);
+    if (plan.ncol == 256) return fp_launch<FORM, 256, BP, false, BIAS>(p, a, b, st);
+    if (plan.ncol == 128) return fp_launch<FORM, 128, BP, false, BIAS>(p, a, b, st);
+    if constexpr (FORM == FORM_S) return fp_launch<FORM, 64, BP, false, BIAS>(p, a, b, st);
     return HBFP_ERR_UNSUPPORTED;
+}
+template <int FORM, int BP>
+int fp_launch_bias(const FpProblem& p, const FpPlan& plan, const FpOperand& a, const FpOperand& b, cudaStream_t st) {
+    return p.bias ? fp_launch_bp<FORM, BP, true>(p, plan, a, b, st) : fp_launch_bp<FORM, BP, false>(p, plan, a, b, st);
 }
 
 inline int log2_of(int64_t v) { int l = 0; while ((1ll << l) < v) ++l; return l; }
@@ -772,19 +799,20 @@ int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const FpOperan
     return launch_status();
 }
 
-int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, float* Cout, int64_t ldc, cudaStream_t st) {
+int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, const float* bias, float* Cout, int64_t ldc, cudaStream_t st) {
     FpProblem p{};
     p.M = (int)M;
     p.N = (int)N;
     p.nkb = (int)la.nkb;
     p.splits = plan.splits;
     p.kb_per_split = plan.kb_per_split;
+    p.bias = bias;
     p.C = Cout;
     p.ldc = ldc;
     p.status = device_status_word();
     if (!p.status) return HBFP_ERR_CUDA;
-    if (plan.form == FORM_S) return la.bp == 32 ? fp_launch_bp<FORM_S, 32>(p, plan, a, b, st) : fp_launch_bp<FORM_S, 64>(p, plan, a, b, st);
-    return la.bp == 32 ? fp_launch_bp<FORM_W, 32>(p, plan, a, b, st) : fp_launch_bp<FORM_W, 64>(p, plan, a, b, st);
+    if (plan.form == FORM_S) return la.bp == 32 ? fp_launch_bias<FORM_S, 32>(p, plan, a, b, st) : fp_launch_bias<FORM_S, 64>(p, plan, a, b, st);
+    return la.bp == 32 ? fp_launch_bias<FORM_W, 32>(p, plan, a, b, st) : fp_launch_bias<FORM_W, 64>(p, plan, a, b, st);
 }
 
 }  // namespace hbfp

@@ -31,6 +31,7 @@ struct SkinnyProblem {
     int tmem_cols;
     int off_x, off_xs, off_we, off_bar;   // shared memory
     int vec;                        // pieces of eight activations are 16-byte aligned
+    const float* bias;              // may be null
     float* C;
     int64_t ldc;
     int32_t* status;
@@ -266,6 +267,10 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap mapW, const SkinnyProblem
 #pragma unroll
                 for (int e = 0; e < 4; ++e) y[e] = sp == 0 ? v[e] : __fadd_rn(y[e], v[e]);
             }
+            if (p.bias)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (gj + e < p.N) y[e] = __fadd_rn(y[e], __ldg(p.bias + gj + e));
             float* dst = p.C + (int64_t)gi * p.ldc + gj;
             if (quad && gj + 3 < p.N) *reinterpret_cast<float4*>(dst) = make_float4(y[0], y[1], y[2], y[3]);
             else
@@ -387,8 +392,8 @@ bool skinny_gemm_eligible(int64_t M, int64_t N, const Layout& la, const Layout& 
     return sk_plan(M, N, lb, &plan);
 }
 
-int launch_gemm_skinny(int64_t M, int64_t N, int64_t K, const float* x, int64_t ld, const hbfp_format* fx, const Packed& w, float* C, int64_t ldc,
-                       cudaStream_t st) {
+int launch_gemm_skinny(int64_t M, int64_t N, int64_t K, const float* x, int64_t ld, const hbfp_format* fx, const Packed& w, const float* bias, float* C,
+                       int64_t ldc, cudaStream_t st) {
     SkinnyPlan plan;
     if (!sk_plan(M, N, w.L, &plan)) return HBFP_ERR_UNSUPPORTED;
     const int bp = (int)w.L.bp;
@@ -408,6 +413,7 @@ int launch_gemm_skinny(int64_t M, int64_t N, int64_t K, const float* x, int64_t 
     p.tmem_cols = plan.tmem_cols;
     sk_smem(plan.rows, bp, plan.segs_per_cta, plan.tmem_cols, &p);
     p.vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0 && (ld & 3) == 0 && (p.b & 3) == 0;
+    p.bias = bias;
     p.C = C;
     p.ldc = ldc;
     p.status = device_status_word();

@@ -32,6 +32,8 @@ struct Api {
     decltype(&hbfp_conv_dgrad_filters) conv_dgrad_filters;
     decltype(&hbfp_im2col_packed_t) im2col_packed_t;
     decltype(&hbfp_im2col_packed) im2col_packed;
+    decltype(&hbfp_gemm_q_bias) gemm_q_bias;
+    decltype(&hbfp_column_sums) column_sums;
 } api;
 
 // ------------------------------------------------------------------------------ arguments
@@ -132,14 +134,15 @@ Operand operand_of(PyObject* x, long long trans, PyObject* fmt) {
 }
 
 // hbfp_gemm_q with the workspace from the caching allocator (stream-ordered, as a temporary tensor's memory is).
-int run_gemm(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_operand& b, const at::Tensor& out, const at::Tensor* ws, uint32_t flags) {
-    if (ws) return api.gemm_q(M, N, K, &a, &b, (float*)out.data_ptr(), ld_of(out), ws->data_ptr(), (size_t)ws->numel(), flags, cur_stream());
+int run_gemm(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_operand& b, const at::Tensor& out, const at::Tensor* ws, uint32_t flags,
+             const float* bias = nullptr) {
+    if (ws) return api.gemm_q_bias(M, N, K, &a, &b, bias, (float*)out.data_ptr(), ld_of(out), ws->data_ptr(), (size_t)ws->numel(), flags, cur_stream());
     size_t bytes = 0;
     const int rc = api.gemm_q_workspace(M, N, K, &a, &b, &bytes);
     if (rc) return rc;
     c10::DataPtr mem;
     if (bytes) mem = c10::cuda::CUDACachingAllocator::get()->allocate(bytes);
-    return api.gemm_q(M, N, K, &a, &b, (float*)out.data_ptr(), ld_of(out), mem.get(), bytes, flags, cur_stream());
+    return api.gemm_q_bias(M, N, K, &a, &b, bias, (float*)out.data_ptr(), ld_of(out), mem.get(), bytes, flags, cur_stream());
 }
 
 template <class F>
@@ -430,9 +433,9 @@ PackedTensor alloc_packed(int64_t rows, int64_t k, const hbfp_format& f, const a
     ok_or_raise(api.packed_layout(rows, k, &f, &L), where);
     return {empty_i8(L.mant_bytes, like), empty_i8(L.exp_bytes, like), f};
 }
-at::Tensor product(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_operand& b, const at::Tensor& like) {
+at::Tensor product(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_operand& b, const at::Tensor& like, const float* bias = nullptr) {
     at::Tensor out = empty_f32({M, N}, like);
-    ok_or_raise(run_gemm(M, N, K, a, b, out, nullptr, HBFP_GEMM_AUTO), "hbfp_gemm_q");
+    ok_or_raise(run_gemm(M, N, K, a, b, out, nullptr, HBFP_GEMM_AUTO, bias), "hbfp_gemm_q");
     return out;
 }
 // Everything a pass computes lies below autograd; gradients come out as plain tensors.
@@ -460,11 +463,15 @@ struct LinearNode : public torch::autograd::Node {
         const at::Tensor x0 = x_.unpack(shared_from_this());
         Below guard;
         const at::Tensor dy = grads[0].contiguous(), x = x0.contiguous();
+        check_f32_cpp(dy);
         const int64_t batch = x.size(0);
         // backward-data on the shared weight view; backward-weight with blocks down the columns of X and dY
         if (task_should_compute_output(0)) out[0] = product(batch, fin, fout, fp32_operand(dy, 0, act(2, false)), c1.operand(), dy);
         if (task_should_compute_output(1)) out[1] = product(fin, fout, batch, fp32_operand(x, 1, act(0, true)), fp32_operand(dy, 0, act(2, true)), dy);
-        if (task_should_compute_output(2)) out[2] = dy.sum(0);
+        if (task_should_compute_output(2)) {
+            out[2] = empty_f32({fout}, dy);
+            ok_or_raise(api.column_sums((const float*)dy.data_ptr(), batch, fout, ld_of(dy), (float*)out[2].data_ptr(), cur_stream()), "hbfp_column_sums");
+        }
         return out;
     }
 };
@@ -487,8 +494,9 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
         {
             Below guard;
             const at::Tensor xc = x.contiguous();
-            y = product(xc.size(0), proto.fout, proto.fin, fp32_operand(xc, 0, proto.act(0, false)), c0.operand(), xc);
-            if (bias.defined()) y.add_(bias);
+            const at::Tensor bc = bias.defined() ? bias.contiguous() : bias;
+            if (bc.defined()) TORCH_CHECK_VALUE(bc.is_cuda() && bc.scalar_type() == at::kFloat && bc.numel() == proto.fout, "bias must hold a float32 value per output on the GPU");
+            y = product(xc.size(0), proto.fout, proto.fin, fp32_operand(xc, 0, proto.act(0, false)), c0.operand(), xc, bc.defined() ? (const float*)bc.data_ptr() : nullptr);
         }
         if (torch::autograd::compute_requires_grad(x, w, bias)) {
             auto node = std::shared_ptr<LinearNode>(new LinearNode(), torch::autograd::deleteNode);

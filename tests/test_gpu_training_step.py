@@ -205,3 +205,24 @@ def test_layer_nodes_follow_autograd(env):
     assert e.value.code == hb.ERR_UNSUPPORTED
     with pytest.raises(ValueError):
         layer(x.half())
+
+
+@pytest.mark.parametrize("batch,fin,fout,m,t", [(16, 300, 130, 8, 64), (128, 784, 1024, 8, 24), (300, 256, 128, 8, 128), (256, 40, 33, 8, 32), (2304, 1024, 2048, 12, 64),
+                                                (640, 2048, 1280, 8, 32), (2048, 2048, 2560, 8, 128), (300, 4096, 100, 8, 64), (130, 500, 131, 12, 24)])
+def test_bias_added_by_the_product_and_its_gradient(env, batch, fin, fout, m, t):
+    """Whichever kernel the product takes, adding the bias in its store gives the bits of adding it afterwards; the column sums
+    of dY against binary64 (a chain of at most batch / 64 + 22 additions of like magnitude)."""
+    torch, hbfp_nn, hb = env
+    torch.manual_seed(6)
+    layer = hbfp_nn.HbfpLinear(fin, fout, mant_bits=m, tile=t, seed=2)
+    x, bias = torch.randn(batch, fin, device="cuda"), torch.randn(fout, device="cuda")
+    with torch.no_grad():
+        plain = layer(x)                     # the bias starts as zeros
+        layer.bias.copy_(bias)
+        assert torch.equal(layer(x), plain + bias)
+    dy = torch.randn(batch, fout, device="cuda")
+    layer.weight.requires_grad_(False)
+    layer(x).backward(dy)
+    d = dy.double()
+    bound = (batch / 64 + 22) * 2.0 ** -24 * d.abs().sum(0)
+    assert bool(((layer.bias.grad.double() - d.sum(0)).abs() <= bound).all()) and hb.device_status() == 0
