@@ -187,6 +187,13 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     // a problem of a few hundred MOPs is over before a tensor-core kernel has filled its pipeline
     const bool small = !P && (flags == HBFP_GEMM_AUTO || flags == HBFP_GEMM_FORCE_SMALL) && small_gemm_eligible(M, N, pa, pb, flags == HBFP_GEMM_FORCE_SMALL);
     if (flags == HBFP_GEMM_FORCE_SMALL && !small) return HBFP_ERR_UNSUPPORTED;
+    if (small && small_fused_eligible(a, k_contiguous(a, true), b, k_contiguous(b, false), M, N, g.la)) {
+        rc = check_fp32(a, true, M, K);
+        if (!rc) rc = check_fp32(b, false, N, K);
+        if (rc) return rc;
+        t_last_gemm_kernel = "gemm_small_kernel";
+        return launch_gemm_small_fused(M, N, K, a, k_contiguous(a, true), b, k_contiguous(b, false), g.la, C, ldc, st);
+    }
     if (!P && flags == HBFP_GEMM_AUTO && a->kind == HBFP_OPERAND_FP32 && a->trans == 0 && a->fmt.tile == 0 &&
         b->kind == HBFP_OPERAND_PACKED && skinny_gemm_eligible(M, N, g.la, g.lb, a->fmt.mant_bits, b->fmt.mant_bits)) {
         rc = check_fp32(a, true, M, K);

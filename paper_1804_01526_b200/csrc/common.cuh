@@ -95,6 +95,10 @@ int launch_gemm_simt(int64_t M, int64_t N, int64_t K, const Packed& a, const Pac
 // Tiled dp4a kernel for small problems (gemm_small.cu): one-plane operands, one launch, no split-K.
 bool small_gemm_eligible(int64_t M, int64_t N, const Packed& a, const Packed& b, bool any_size);
 int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, float* C, int64_t ldc, cudaStream_t st);
+// The same from FP32 operands, conversion included (contig: K is contiguous).
+bool small_fused_eligible(const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, int64_t M, int64_t N, const Layout& la);
+int launch_gemm_small_fused(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, const Layout& la,
+                            float* C, int64_t ldc, cudaStream_t st);
 
 // A few rows of FP32 activations against packed weights, conversion included (gemm_skinny.cu): one launch, no scratch.
 bool skinny_gemm_eligible(int64_t M, int64_t N, const Layout& la, const Layout& lb, int bits_a, int bits_b);

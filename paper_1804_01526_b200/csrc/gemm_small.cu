@@ -11,7 +11,7 @@
 // (a slice is in flight while the previous one is multiplied); the exponents of all K-blocks of those rows are
 // staged once. Per K-block: the exact int32 sum by mma.sync.m16n8k32 (Eq. 2), converted to binary32 and
 // accumulated with one FMA by 2^(sA + sB), blocks in ascending order: bit for bit the sequential definition.
-#include "common.cuh"
+#include "quant_math.cuh"
 
 namespace hbfp {
 namespace {
@@ -128,6 +128,173 @@ gemm_small_kernel(int64_t M, int64_t N, int nkb, int bp, const int8_t* __restric
         }
 }
 
+// ------------------------------------------------------------------------------ both operands FP32
+
+// The same 32 x 32 tiles from FP32 operands, conversion included: one launch instead of three. A 256 cube is a few microseconds
+// of anything, and what its three kernels cost was their launches and starts (8.5 us of device time, 14.3 as a call; here 6.7 and 8.2). Half of
+// the 16 warps convert the tile's 32 rows of A and half the 32 columns of B to binary16 mantissas in shared memory; every tile of
+// a row of tiles repeats that, which bounds it to short contractions (one slice) and few tiles. Mantissas of 8 bits and block
+// sums below 2^24 are exact in binary16 MMAs with FP32 accumulators, which this part issues four times as often per K as the
+// int8 ones; a lane takes eight consecutive K of both operands, so fragments are 16-byte loads.
+constexpr int SF_THREADS = 512, SF_HALF = 256;
+constexpr int SF_MAX_GROUPS = SM_AUTO_BYTES / 8;
+
+struct SmallOperand {
+    const float* x;
+    int64_t ld, lines;              // lines: rows of A or columns of B
+    int contig, vec;                // contig: blocks along contiguous rows; vec: pieces of eight are 16-byte aligned
+    QParams q;
+};
+struct SmallProblem {
+    SmallOperand a, b;
+    int K, blk, bp, lg_bp, nkb, pitch;     // pitch of a converted line in bytes
+    float* C;
+    int64_t ldc;
+};
+
+template <bool SR>
+__device__ __forceinline__ void sf_store(const float (&e8)[8], int s, const QParams& q, uint4 w, unsigned char* at) {
+    uint4 h, unused;
+    if (SR && q.rounding == 1) quantize_form8<true, FORM_WIDE_A>(e8, s, q, w, h, unused);
+    else quantize_form8<false, FORM_WIDE_A>(e8, s, q, w, h, unused);
+    *reinterpret_cast<uint4*>(at) = h;
+}
+
+// 32 lines from `line0` on whose K is contiguous: a thread keeps its piece of eight packed positions and walks down the lines.
+template <bool SR>
+__device__ __forceinline__ void sf_convert_rows(const SmallOperand& o, const SmallProblem& p, int64_t line0, int t, unsigned char* dst, int8_t* exps) {
+    constexpr int UNR = 4;
+    const int gpr = p.nkb * p.bp / 8, rpp = SF_HALF / gpr, r0 = t / gpr, pos = 8 * (t - r0 * gpr);
+    const int kb = pos >> p.lg_bp, within = pos & (p.bp - 1), k = kb * p.blk + within, lpb = p.bp / 8;
+    const int n = r0 < rpp ? min(p.blk - within, p.K - k) : 0;
+    for (int rb = 0; rb < SM_TILE; rb += UNR * rpp) {
+        float e8[UNR][8];
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            const int r = rb + u * rpp + r0;
+            const int nr = r < SM_TILE && line0 + r < o.lines ? n : 0;
+            const float* src = o.x + (line0 + r) * o.ld + k;
+            if (nr >= 8 && o.vec) {
+                const float4 a = __ldg(reinterpret_cast<const float4*>(src)), c = __ldg(reinterpret_cast<const float4*>(src) + 1);
+                e8[u][0] = a.x; e8[u][1] = a.y; e8[u][2] = a.z; e8[u][3] = a.w;
+                e8[u][4] = c.x; e8[u][5] = c.y; e8[u][6] = c.z; e8[u][7] = c.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) e8[u][j] = j < nr ? __ldg(src + j) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < UNR; ++u) {
+            if (rb + u * rpp >= SM_TILE) break;                       // all threads alike
+            const int r = rb + u * rpp + r0;
+            uint32_t am = amax8_bits(e8[u]);
+            for (int off = 1; off < lpb; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
+            const int s = block_exponent(am, o.q.m, o.q.exp_mode);
+            if (r < SM_TILE && r0 < rpp) {
+                const uint4 w = SR && o.q.rounding == 1 ? draws_of_eight(o.q, (uint64_t)((line0 + r) * p.K + k)) : make_uint4(0u, 0u, 0u, 0u);
+                sf_store<SR>(e8[u], s, o.q, w, dst + r * p.pitch + 2 * pos);
+                if (within == 0) exps[kb * SM_TILE + r] = (int8_t)s;
+            }
+        }
+    }
+}
+
+// 32 lines that are columns of x [K][lines]: lane = line, a warp takes every eighth group of eight K, so that its loads are 128
+// consecutive bytes; the groups stay in registers between the block maximum (through shared memory) and the rounding.
+template <bool SR, int PER>
+__device__ __forceinline__ void sf_convert_cols(const SmallOperand& o, const SmallProblem& p, int64_t line0, int t, int barrier, uint32_t (*amax)[SM_TILE],
+                                                unsigned char* dst, int8_t* exps) {
+    const int lane = t & 31, warp = t >> 5, groups = p.nkb * p.bp / 8, lpb = p.bp / 8;
+    const bool in = line0 + lane < o.lines;
+    float e8[PER][8];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int g = warp + 8 * i, kb = g >> (p.lg_bp - 3), within = 8 * (g & (lpb - 1)), k = kb * p.blk + within;
+        const int n = g < groups && in ? min(p.blk - within, p.K - k) : 0;
+        const float* src = o.x + (int64_t)k * o.ld + line0 + lane;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) e8[i][j] = j < n ? __ldg(src + j * o.ld) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < PER; ++i)
+        if (warp + 8 * i < groups) amax[warp + 8 * i][lane] = amax8_bits(e8[i]);
+    asm volatile("bar.sync %0, %1;" ::"r"(barrier), "n"(SF_HALF) : "memory");
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        const int g = warp + 8 * i, kb = g >> (p.lg_bp - 3), within = 8 * (g & (lpb - 1)), k = kb * p.blk + within;
+        if (g >= groups) break;                                       // the whole warp
+        uint32_t am = 0;
+        for (int j = 0; j < lpb; ++j) am = max(am, amax[kb * lpb + j][lane]);
+        const int s = block_exponent(am, o.q.m, o.q.exp_mode);
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (SR && o.q.rounding == 1) {
+            // Eight neighbouring columns share the draws of a row (the pitch of the draws is a multiple of eight): lane i of an
+            // octet makes those of row k + i, column c takes halfword c of each.
+            const int c = lane & 7;
+            const uint4 mine = draws_of_group(o.q, (uint64_t)((int64_t)(k + c) * o.lines + line0 + (lane & ~7)) >> 3);
+            uint32_t d[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int from = (lane & ~7) + j;
+                const uint32_t x = __shfl_sync(0xffffffffu, mine.x, from), y = __shfl_sync(0xffffffffu, mine.y, from);
+                const uint32_t z = __shfl_sync(0xffffffffu, mine.z, from), v = __shfl_sync(0xffffffffu, mine.w, from);
+                d[j] = draw_from(make_uint4(x, y, z, v), (uint32_t)c);
+            }
+            w = make_uint4(d[0] | d[1] << 16, d[2] | d[3] << 16, d[4] | d[5] << 16, d[6] | d[7] << 16);
+        }
+        sf_store<SR>(e8[i], s, o.q, w, dst + lane * p.pitch + 16 * g);
+        if (within == 0) exps[kb * SM_TILE + lane] = (int8_t)s;
+    }
+}
+
+// SR: either operand rounds stochastically. PER: groups of eight K per warp of a column conversion (4: up to 256 K). Both keep the
+// code of a launch short: it runs once from top to bottom, and fetching it is a good part of so short a kernel.
+template <bool SR, int PER>
+__global__ void __launch_bounds__(SF_THREADS)
+gemm_small_fused_kernel(const SmallProblem p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t amax[2][SF_MAX_GROUPS][SM_TILE];
+    __shared__ int8_t xA[SF_MAX_GROUPS / 4 * SM_TILE], xB[SF_MAX_GROUPS / 4 * SM_TILE];      // [block][32]
+    unsigned char *fA = smem, *fB = smem + SM_TILE * p.pitch;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t i0 = (int64_t)blockIdx.y * SM_TILE, j0 = (int64_t)blockIdx.x * SM_TILE;
+    if (tid < SF_HALF) {
+        if (p.a.contig) sf_convert_rows<SR>(p.a, p, i0, tid, fA, xA);
+        else sf_convert_cols<SR, PER>(p.a, p, i0, tid, 1, amax[0], fA, xA);
+    } else {
+        if (p.b.contig) sf_convert_rows<SR>(p.b, p, j0, tid - SF_HALF, fB, xB);
+        else sf_convert_cols<SR, PER>(p.b, p, j0, tid - SF_HALF, 2, amax[1], fB, xB);
+    }
+    __syncthreads();
+    if (warp >= 8) return;
+    // warp w: rows 16 (w & 1), columns 8 (w >> 1) of the tile; fragments as in gemm_small_kernel
+    const int g = lane >> 2, q = lane & 3, cr0 = 16 * (warp & 1) + g, cc0 = 8 * (warp >> 1) + 2 * q;
+    const unsigned char *sA = fA + cr0 * p.pitch + 16 * q, *sB = fB + (8 * (warp >> 1) + g) * p.pitch + 16 * q;
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int kb = 0; kb < p.nkb; ++kb) {
+        float d[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int o = 0; o < p.bp; o += 32, sA += 64, sB += 64) {
+            const uint4 a = *reinterpret_cast<const uint4*>(sA), a8 = *reinterpret_cast<const uint4*>(sA + 8 * p.pitch), b = *reinterpret_cast<const uint4*>(sB);
+            asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a.x), "r"(a8.x), "r"(a.y), "r"(a8.y), "r"(b.x), "r"(b.y));
+            asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a.z), "r"(a8.z), "r"(a.w), "r"(a8.w), "r"(b.z), "r"(b.w));
+        }
+        const int ea0 = xA[kb * SM_TILE + cr0], ea1 = xA[kb * SM_TILE + cr0 + 8], eb0 = xB[kb * SM_TILE + cc0], eb1 = xB[kb * SM_TILE + cc0 + 1];
+        acc[0] = fmaf(d[0], scale_of(ea0 + eb0), acc[0]);
+        acc[1] = fmaf(d[1], scale_of(ea0 + eb1), acc[1]);
+        acc[2] = fmaf(d[2], scale_of(ea1 + eb0), acc[2]);
+        acc[3] = fmaf(d[3], scale_of(ea1 + eb1), acc[3]);
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int64_t i = i0 + cr0 + 8 * a, j = j0 + cc0 + b;
+            if (i < p.a.lines && j < p.b.lines) p.C[i * p.ldc + j] = acc[2 * a + b];
+        }
+}
+
 }  // namespace
 
 // One-plane operands, at most SM_MAX_NKB K-blocks; unless any_size, a problem small enough that the tensor-core
@@ -159,6 +326,59 @@ int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, fl
     gemm_small_kernel<<<grid, 256, smem, st>>>(M, N, nkb, (int)a.L.bp, a.mant, a.L.kst, a.exps, a.L.rs, b.mant, b.L.kst,
                                                b.exps, b.L.rs, C, ldc);
     return launch_status();
+}
+
+namespace {
+template <bool SR, int PER>
+int sf_launch(const SmallProblem& p, dim3 grid, cudaStream_t st) {
+    static bool attr_set[64] = {};                                      // the attribute belongs to the device (same value from any thread)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return HBFP_ERR_CUDA;
+    if (!attr_set[dev]) {
+        HBFP_CUDA_OK(cudaFuncSetAttribute(gemm_small_fused_kernel<SR, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * SM_TILE * (2 * SM_AUTO_BYTES + 64)));
+        attr_set[dev] = true;
+    }
+    gemm_small_fused_kernel<SR, PER><<<grid, SF_THREADS, 2 * (size_t)SM_TILE * p.pitch, st>>>(p);      // at most 68 KB
+    return launch_status();
+}
+}  // namespace
+
+// Where the small kernel would be chosen, both operands are FP32 without weight tiles and no draw straddles two groups.
+bool small_fused_eligible(const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, int64_t M, int64_t N, const Layout& la) {
+    if (a->kind != HBFP_OPERAND_FP32 || b->kind != HBFP_OPERAND_FP32 || a->fmt.tile != 0 || b->fmt.tile != 0) return false;
+    if (la.bp > 128 || la.nkb * la.bp > SM_AUTO_BYTES || la.nkb <= 0) return false;
+    // A CTA's registers fill an SM when a column conversion holds 512 K; a second round of tiles then costs more than two launches
+    // (512 cube 18.6 against 10.7 us of device time; 512 x 512 x 256, two CTAs per SM, 10.5 against 14.3 as a call).
+    const int64_t ctas = ((M + SM_TILE - 1) / SM_TILE) * ((N + SM_TILE - 1) / SM_TILE);
+    if (la.nkb * la.bp > 256 && ctas > 148) return false;
+    return (a_contig || a->fmt.rounding == 0 || M % 8 == 0) && (b_contig || b->fmt.rounding == 0 || N % 8 == 0);
+}
+
+int launch_gemm_small_fused(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, const Layout& la,
+                            float* C, int64_t ldc, cudaStream_t st) {
+    SmallProblem p{};
+    p.K = (int)K;
+    p.blk = (int)la.b;
+    p.bp = (int)la.bp;
+    p.lg_bp = la.bp == 32 ? 5 : la.bp == 64 ? 6 : 7;
+    p.nkb = (int)la.nkb;
+    p.pitch = (int)round_up(2 * la.nkb * la.bp, 128) + 64;              // rows half a line of banks apart
+    p.C = C;
+    p.ldc = ldc;
+    auto fill = [&](SmallOperand& o, const hbfp_operand* h, bool contig, int64_t lines) {
+        o.x = static_cast<const float*>(h->data);
+        o.ld = h->ld;
+        o.lines = lines;
+        o.contig = contig;
+        o.vec = (reinterpret_cast<uintptr_t>(o.x) & 15) == 0 && (h->ld & 3) == 0 && (p.blk & 3) == 0;
+        o.q = make_params(&h->fmt);
+    };
+    fill(p.a, a, a_contig, M);
+    fill(p.b, b, b_contig, N);
+    const dim3 grid((unsigned)((N + SM_TILE - 1) / SM_TILE), (unsigned)((M + SM_TILE - 1) / SM_TILE));
+    const bool sr = a->fmt.rounding == 1 || b->fmt.rounding == 1, shallow = la.nkb * la.bp <= 256;
+    if (shallow) return sr ? sf_launch<true, 4>(p, grid, st) : sf_launch<false, 4>(p, grid, st);
+    return sr ? sf_launch<true, 8>(p, grid, st) : sf_launch<false, 8>(p, grid, st);
 }
 
 }  // namespace hbfp

@@ -506,3 +506,23 @@ def test_few_rows_kernel_reports_weights_beyond_its_exact_range(hb):
             assert bool(((got.double() - want).abs() <= 1e-5 * want.abs().max()).all())
         else:
             assert scale_w > 2.0 ** 110
+
+
+@pytest.mark.parametrize("M,N,K,m,b,rounding", [(256, 256, 256, 8, 32, 0), (1, 1, 1, 8, 32, 1), (33, 65, 100, 8, 24, 0), (40, 72, 130, 4, 48, 1), (64, 96, 512, 8, 128, 1),
+                                                (31, 200, 384, 8, 24, 1), (100, 36, 511, 6, 64, 0), (256, 512, 200, 8, 100, 1)])
+@pytest.mark.parametrize("tA,tB", [(0, 0), (1, 0), (0, 1), (1, 1)])
+def test_small_products_of_fp32_operands_in_one_launch(hb, M, N, K, m, b, rounding, tA, tB):
+    """Both operands converted inside the product, in every storage order, at unaligned rows and ragged blocks: bit for bit the
+    reference kernel on what hbfp_quantize makes of them."""
+    import torch
+    A = to_dev(wl.draw("outliers", (K, M) if tA else (M, K), seed=51))
+    B = to_dev(wl.draw("lognormal", (N, K) if tB else (K, N), seed=52))
+    fa, fb = hb.Format(m, b, rounding=rounding, seed=9), hb.Format(m, b, rounding=rounding, seed=9, stream_id=1)
+    want = hb.gemm_q(M, N, K, hb.quantize(A, 0 if tA else 1, fa), hb.quantize(B, 1 if tB else 0, fb), flags=hb.GEMM_FORCE_SIMT)
+    for X in (A, torch.cat([A, A], 1)[:, 1:1 + A.shape[1]] if A.shape[1] > 1 else A):
+        fresh = X is A
+        if not fresh:
+            want = hb.gemm_q(M, N, K, hb.quantize(X.contiguous(), 0 if tA else 1, fa), hb.quantize(B, 1 if tB else 0, fb), flags=hb.GEMM_FORCE_SIMT)
+        got = hb.gemm(tA, tB, X, B, fa, fb)
+        assert hb.last_gemm_kernel() == "gemm_small_kernel" and hb.device_status() == 0
+        assert torch.equal(got, want)
