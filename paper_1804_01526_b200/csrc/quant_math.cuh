@@ -186,6 +186,17 @@ __device__ __forceinline__ void round_and_store8(const float (&e8)[8], int s, co
         }
     }
 }
+// Eight zero elements there.
+template <int OUT>
+__device__ __forceinline__ void store_zero8(int8_t* mant, int64_t at, int64_t plane_stride) {
+    if constexpr (is_form(OUT)) {
+        *reinterpret_cast<uint4*>(mant + 2 * at) = make_uint4(0u, 0u, 0u, 0u);
+        if (OUT == FORM_WIDE_B) *reinterpret_cast<uint4*>(mant + 2 * (at + plane_stride)) = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        *reinterpret_cast<uint2*>(mant + at) = make_uint2(0u, 0u);
+        if (OUT == 2) *reinterpret_cast<uint2*>(mant + plane_stride + at) = make_uint2(0u, 0u);
+    }
+}
 template <int OUT>
 __device__ __forceinline__ void check_exponent(int s, const FormArgs& fa) {
     if (OUT == FORM_WIDE_A && s > 96) atomicCAS(fa.status, 0, STATUS_EXPONENT_RANGE);

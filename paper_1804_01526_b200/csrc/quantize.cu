@@ -1189,9 +1189,12 @@ __global__ void dequant_kernel(const int8_t* __restrict__ mant, const int8_t* __
 // ------------------------------------------------------------------------------ quant_row_flat
 
 // Blocks along contiguous rows for row lengths that are not a multiple of the 512-column tile of
-// quant_row_fast (K % b == 0, e.g. im2col matrices with K = 576 or 1152): the packed rows, padding
-// included, are cut into 8-element groups that are numbered through the whole matrix, and a warp takes
-// 32 consecutive groups wherever the row boundaries fall, so no lane idles on a ragged last tile.
+// quant_row_fast (K % b == 0, e.g. im2col matrices with K = 576 or 1152): the rows are cut into 8-element groups that are
+// numbered through the whole matrix, and a warp takes 32 consecutive groups wherever the row boundaries fall, so no lane
+// idles on a ragged last tile. The zeros between K and the packed pitch are written by the lanes of the row's first
+// groups (numbered like the others, half of the lanes of 64-channel pixels had nothing to
+// load: 131072 x 64 12.6 us, now 8.5 = 5.9 TB/s; 10^6 x 32 with stochastic rounding, three quarters idle, 125 -> 42 us; 131072 x 576
+// 64.8 -> 61.1).
 // CTA: 256 threads x ITEMS groups each (256 ITEMS consecutive groups).
 template <int LPB, bool SR, int PLANES, int ITEMS>
 __global__ void __launch_bounds__(256)
@@ -1210,7 +1213,7 @@ quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
     for (int j = 0; j < ITEMS; ++j) {
         rw[j] = row;
         cc[j] = cg * 8;
-        const bool in = g0 + j * 256u < total_groups && cc[j] < K;
+        const bool in = g0 + j * 256u < total_groups;
         if (in) {
             const float4* src = reinterpret_cast<const float4*>(x + (int64_t)row * ld + cc[j]);
             v[j][0] = __ldcs(src);
@@ -1241,8 +1244,9 @@ quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
         const uint4 w = wd[j];
         round_and_store8<SR, PLANES>(e8, s, p, w, mant, (int64_t)rw[j] * kst + cc[j], plane_stride, live);
         check_exponent<PLANES>(s, fa);
-        // blocks that lie in the padding beyond K have no exponent
-        if (live && (lane % LPB) == 0 && cc[j] < K) store_exponent<PLANES>(exps, (int64_t)(cc[j] / B) * rs + rw[j], s);
+        if (live)
+            for (uint32_t o = (uint32_t)K + cc[j]; o < kst; o += 8u * gpr) store_zero8<PLANES>(mant, (int64_t)rw[j] * kst + o, plane_stride);
+        if (live && (lane % LPB) == 0) store_exponent<PLANES>(exps, (int64_t)(cc[j] / B) * rs + rw[j], s);
     }
     if (!is_form(PLANES)) zero_padding_lines(exps, rows, rs, K / B);
 }
@@ -1251,7 +1255,7 @@ quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
 template <int LPB, int ITEMS, int FORM>
 int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
                           int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa) {
-    const uint32_t gpr = (uint32_t)(L.kst / 8), total = (uint32_t)(rows * (L.kst / 8));
+    const uint32_t gpr = (uint32_t)(K / 8), total = (uint32_t)(rows * (K / 8));
     const unsigned grid = (total + 256u * ITEMS - 1u) / (256u * ITEMS);
 #define HBFP_QFLAT(SRV, OUT) quant_row_flat<LPB, SRV, OUT, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
     if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QFLAT(true, FORM); else HBFP_QFLAT(false, FORM); }
@@ -1264,8 +1268,7 @@ int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, c
 // Groups per thread: more of them amortise the index arithmetic, fewer keep the register footprint small
 // and more loads in flight. Measured on 131072 x 576 (b = 64): eight 68 us, four 58 us, two 61 us with
 // nearest-even rounding; 91 / 84 / 82 us with stochastic rounding (the Philox state of every group in flight
-// is live). Narrow rows (one or two 128-byte units, e.g. one block of 64 channels per pixel, half of whose
-// groups are padding that loads nothing) do best with two.
+// is live). Narrow rows (one or two 128-byte units, e.g. one block of 64 channels per pixel) do as well with two.
 template <int LPB, int FORM = 0>
 int launch_row_flat(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
                     int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa = FormArgs{}) {

@@ -294,3 +294,15 @@ def test_ragged_blocks_in_both_directions(hb, d0, d1, b, m, rounding):
                 body = p.mant.cpu().numpy()[pl * lay["plane_stride"]:][:rows * lay["kst"]].reshape(rows, lay["kst"])
                 blocks = body[:, :lay["nkb"] * lay["bp"]].reshape(rows, lay["nkb"], lay["bp"])
                 assert (blocks[:, :, b:] == 0).all() and (body[:, lay["nkb"] * lay["bp"]:] == 0).all()     # padding
+
+
+@pytest.mark.parametrize("rows,K,b", [(1, 32, 32), (1000, 32, 32), (777, 64, 64), (300, 96, 32), (65, 160, 32), (33, 192, 64), (50, 640, 128), (9, 2080, 32)])
+@pytest.mark.parametrize("m,rounding", [(8, 0), (8, 1), (12, 1)])
+def test_rows_whose_packed_pitch_is_longer_than_they_are(hb, rows, K, b, m, rounding):
+    """Row lengths of whole blocks that do not fill their 128-byte units: mantissas, exponents and the zeros behind them."""
+    x = wl.draw("lognormal", (rows, K), seed=61)
+    fd = dict(mant_bits=m, block=b, rounding=rounding, seed=8, stream_id=3)
+    p = hb.quantize(to_dev(x), 1, gfmt(fd))
+    q, s = decode_packed(p, hb.packed_layout(rows, K, p.fmt))
+    q_ref, s_ref = oracle.quantize(x, 1, ofmt(fd))
+    assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
