@@ -33,8 +33,10 @@ namespace {
 // ------------------------------------------------------------------------------ quant_row_fast
 
 // LPB = lanes per block (b = 8 * LPB). CTA: 256 threads, tile 32 rows x 512 columns.
+// Three CTAs per SM with draws, four without: left to itself the compiler took 88 to 98 registers for the former and so two
+// CTAs (3186 x 12360 and 265 x 12360, b = 128, stochastic: 54.2 us, now 47.5; the 12-bit form of a 4096 x 4096 operand 22.4, now 20.6).
 template <int LPB, bool SR, int PLANES>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, SR ? 3 : 4)
 quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const int8_t* __restrict__ given = nullptr, const FormArgs fa = FormArgs{}) {
