@@ -125,7 +125,8 @@ template <int PLANES, int RQ, bool SR>      // RQ = bp / 4: padded rows per warp
 __global__ void __launch_bounds__(128)
 quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
                 int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa) {
+                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa, const int8_t* __restrict__ given = nullptr) {
+    // given != nullptr: one exponent per column for the whole axis, computed beforehand; the blocks are then pieces of it
     constexpr int BP = 4 * RQ, BYTE_PLANES = is_form(PLANES) ? 1 : PLANES;
     __shared__ uint32_t pmax[4][COLT];
     __shared__ __align__(16) uint4 rnd[SR ? BP : 1][5];          // draws of a row: its 32 columns lie in at most five groups of eight
@@ -153,10 +154,10 @@ quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
     pmax[q][c] = am;
     __syncthreads();
     am = max(max(pmax[0][c], pmax[1][c]), max(pmax[2][c], pmax[3][c]));
-    const int s = block_exponent(am, p.m, p.exp_mode);
+    const int s = given ? (col < R ? (int)given[col] : -63) : block_exponent(am, p.m, p.exp_mode);
     check_exponent<PLANES>(s, fa);
     if constexpr (is_form(PLANES)) { if (q == 0 && col < R) store_exponent<PLANES>(exps, kb * rs + col, s); }
-    else if (q == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
+    else if (!given && q == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
     const uint32_t qm = qmax_pair(p.qmax), nqm = neg_qmax_pair(p.qmax);
     const float sc = pow2f(SR ? 16 - s : -s);
     const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd);
@@ -1517,13 +1518,14 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
 }
 
 // Whole-axis blocks down the columns (one exponent per column of the stored matrix): pass 1 of 2. Each CTA takes
-// 256 columns and a band of rows, reads rows coalesced and folds its band's maxima into one word per column.
-constexpr int CMAX_ROWS = 128;
+// 256 columns and a band of rows, reads rows coalesced and folds its band's maxima into one word per column. Bands of 128 rows
+// where that makes four CTAs per SM, otherwise of 32: a thread's loads leave eight at a time.
+constexpr int CMAX_ROWS = 128, CMAX_ROWS_SHORT = 32;
 __global__ void __launch_bounds__(256)
-col_amax_kernel(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, uint32_t* __restrict__ amax) {
+col_amax_kernel(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int band, uint32_t* __restrict__ amax) {
     const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (col >= R) return;
-    const int64_t k0 = (int64_t)blockIdx.y * CMAX_ROWS, k1 = min(K, k0 + CMAX_ROWS);
+    const int64_t k0 = (int64_t)blockIdx.y * band, k1 = min(K, k0 + band);
     uint32_t am = 0;
 #pragma unroll 8
     for (int64_t k = k0; k < k1; ++k) am = max(am, abs_bits(__ldg(x + k * ld + col)));
@@ -1695,22 +1697,34 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         }
     }
     // one block per column over the whole axis: column maxima first (scratch: the head of the mantissa buffer, which
-    // the second pass overwrites), then the tile kernel with the exponents given
-    if (f->tile == 0 && axis == 0 && aligned && L.nkb == 1 && L.b == K && K % QC_ROWS == 0 && L.kst == K && K > 128 &&
-        (p.rounding == 0 || rows % 8 == 0) && (reinterpret_cast<uintptr_t>(mant) & 127) == 0 && rows < (1ll << 29) &&
-        K < (1ll << 31) && (K + CMAX_ROWS - 1) / CMAX_ROWS <= 65535 && (int64_t)rows * 4 <= (int64_t)rows * L.kst &&
-        ((rows + QC_COLS - 1) / QC_COLS) * (L.kst / QC_ROWS) < (1ll << 31)) {
+    // the second pass overwrites), then a tile kernel with the exponents given: the streaming one for whole tiles, the ragged one
+    // (pieces of 128) for every other length, pitch and alignment - 3432 x 597 170 us through the generic path (a thread per
+    // column, an index division per element), now 20.4; 8000 x 8000 1386, now 121; 777 x 333 stochastic 45.5, now 14.8
+    if (f->tile == 0 && axis == 0 && L.nkb == 1 && L.b == K && K > 128 && K < (1ll << 31) && rows < (1ll << 29) &&
+        (K + CMAX_ROWS - 1) / CMAX_ROWS <= 65535 && ((rows + COLT - 1) / COLT) * (L.kst / 128) < (1ll << 31)) {
+        const bool stream = aligned && K % QC_ROWS == 0 && L.kst == K && (p.rounding == 0 || rows % 8 == 0) &&
+                            (reinterpret_cast<uintptr_t>(mant) & 127) == 0;
         if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
         uint32_t* amax = reinterpret_cast<uint32_t*>(mant);
         HBFP_CUDA_OK(cudaMemsetAsync(amax, 0, (size_t)rows * 4, st));
-        const dim3 g1((unsigned)((rows + 255) / 256), (unsigned)((K + CMAX_ROWS - 1) / CMAX_ROWS));
-        col_amax_kernel<<<g1, 256, 0, st>>>(x, K, rows, ld, amax);
-        col_exps_kernel<<<(unsigned)((rows + 255) / 256), 256, 0, st>>>(amax, rows, p, exps);
+        const int64_t wide = (rows + 255) / 256;
+        const int band = wide * ((K + CMAX_ROWS - 1) / CMAX_ROWS) >= 4 * 148 || K > 65535ll * CMAX_ROWS_SHORT ? CMAX_ROWS : CMAX_ROWS_SHORT;
+        col_amax_kernel<<<dim3((unsigned)wide, (unsigned)((K + band - 1) / band)), 256, 0, st>>>(x, K, rows, ld, band, amax);
+        col_exps_kernel<<<(unsigned)wide, 256, 0, st>>>(amax, rows, p, exps);
         if (launch_status()) return HBFP_ERR_CUDA;
+        if (stream) {
 #define HBFP_QCOL_GIVEN(PL) (p.rounding ? launch_col_tma<PL, 0, true>(x, K, rows, ld, p, L, mant, exps, st, exps) \
                                         : launch_col_tma<PL, 0, false>(x, K, rows, ld, p, L, mant, exps, st, exps))
-        return L.planes == 1 ? HBFP_QCOL_GIVEN(1) : HBFP_QCOL_GIVEN(2);
+            return L.planes == 1 ? HBFP_QCOL_GIVEN(1) : HBFP_QCOL_GIVEN(2);
 #undef HBFP_QCOL_GIVEN
+        }
+        const int64_t pieces = L.kst / 128;
+        const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * pieces);
+#define HBFP_QCOL_GIVEN(PL, SRV) quant_col_block<PL, 32, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, 128, p, mant, L.kst, L.plane_stride, exps, L.rs, pieces, tiles_n, FormArgs{}, exps)
+        if (L.planes == 1) { if (p.rounding) HBFP_QCOL_GIVEN(1, true); else HBFP_QCOL_GIVEN(1, false); }
+        else { if (p.rounding) HBFP_QCOL_GIVEN(2, true); else HBFP_QCOL_GIVEN(2, false); }
+#undef HBFP_QCOL_GIVEN
+        return launch_status();
     }
     if (f->tile == 0 && axis == 0 && aligned && L.b == L.bp && L.b <= 128 && (p.rounding == 0 || rows % 8 == 0) &&
         (reinterpret_cast<uintptr_t>(mant) & 127) == 0 && rows < (1ll << 29) && K < (1ll << 31) &&

@@ -306,3 +306,20 @@ def test_rows_whose_packed_pitch_is_longer_than_they_are(hb, rows, K, b, m, roun
     q, s = decode_packed(p, hb.packed_layout(rows, K, p.fmt))
     q_ref, s_ref = oracle.quantize(x, 1, ofmt(fd))
     assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
+
+
+@pytest.mark.parametrize("K,cols", [(129, 1), (200, 33), (1000, 64), (3432, 597), (257, 31), (384, 40), (12801, 7)])
+@pytest.mark.parametrize("m,rounding", [(8, 0), (5, 1)])
+def test_one_exponent_per_column_of_any_length(hb, K, cols, m, rounding):
+    """Whole-axis blocks down the columns at lengths, pitches and column counts that fit no tile."""
+    import torch
+    x = wl.draw("outliers", (K, cols), seed=62)
+    fd = dict(mant_bits=m, block=0, rounding=rounding, seed=8, stream_id=3)
+    q_ref, s_ref = oracle.quantize(x, 0, ofmt(fd))
+    xd = to_dev(x)
+    for X in (xd, torch.cat([xd, xd], 1)[:, 1:1 + cols] if cols > 1 else xd):
+        if X is not xd:
+            q_ref, s_ref = oracle.quantize(X.cpu().numpy(), 0, ofmt(fd))
+        p = hb.quantize(X, 0, gfmt(fd))
+        q, s = decode_packed(p, hb.packed_layout(cols, K, p.fmt))
+        assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
