@@ -123,7 +123,7 @@ def lib() -> ctypes.CDLL:
 
 
 # Entry points that _host calls, in the order it takes them (csrc/host.cpp, struct Api).
-_HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q", "hbfp_gemm_q_workspace", "hbfp_wide_update_value", "hbfp_wide_dequantize",
+_HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q_workspace", "hbfp_wide_update_value", "hbfp_wide_dequantize",
                       "hbfp_conv_forward", "hbfp_conv_dgrad_filters", "hbfp_im2col_packed_t", "hbfp_im2col_packed", "hbfp_gemm_q_bias",
                       "hbfp_column_sums")
 

@@ -24,7 +24,6 @@ namespace {
 struct Api {
     decltype(&hbfp_packed_layout) packed_layout;
     decltype(&hbfp_quantize) quantize;
-    decltype(&hbfp_gemm_q) gemm_q;
     decltype(&hbfp_gemm_q_workspace) gemm_q_workspace;
     decltype(&hbfp_wide_update_value) wide_update;
     decltype(&hbfp_wide_dequantize) wide_dequantize;
