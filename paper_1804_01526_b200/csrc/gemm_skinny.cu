@@ -248,6 +248,15 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap mapW, const SkinnyProblem
     }
     tc_fence_before();
     __syncthreads();
+    // Tensor memory goes back before the CTA waits for its cluster, on every way through the kernel: a CTA that holds columns
+    // depends on nobody but itself, so one that blocks in tcgen05.alloc waits for work that always ends - whatever launches, of this
+    // or of other plans, on this or on other streams, share the SMs. (Held across the barriers, two clusters that each hold columns
+    // on one SM and ask for them on the other would wait for one another for good.) The library's other tensor-core kernels take an
+    // SM's registers whole and are nobody's neighbours.
+    if (warp == SK_CONV_WARPS) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
+    }
     if (p.splits > 1) sk_cluster_barrier();
     // each CTA adds up a share of the outputs, parts in ascending order of K
     constexpr int QPR = SK_NT / 4;
@@ -281,10 +290,6 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap mapW, const SkinnyProblem
     __syncwarp();
     // no neighbour still reads this CTA's part (what it read has arrived in registers, so the arrival orders nothing more)
     if (p.splits > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-    if (warp == SK_CONV_WARPS) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
-    }
 }
 
 // ------------------------------------------------------------------------------ host side
@@ -320,8 +325,9 @@ bool sk_plan(int64_t M, int64_t N, const Layout& lb, SkinnyPlan* out) {
     for (int sp = 8; sp >= 1; --sp) {
         const int per = (segs + sp - 1) / sp, blocks = per * (SK_SEG / bp);
         if ((segs + per - 1) / per != sp || per > SK_MAX_SEGS) continue;
-        // Tensor memory is asked for by every resident CTA, and CTAs of different clusters may wait for one another's: what all
-        // CTAs that fit an SM ask for together must fit its 512 columns. Shared memory sets how many fit.
+        // Every resident CTA asks for tensor memory when it starts, and one that finds too little of it waits until a neighbour is
+        // through with its MMAs: what the CTAs of a launch that fit an SM ask for together is kept within its 512 columns, by shared
+        // memory. That is a matter of time only; the kernel gives its columns back before it waits for anyone.
         int cols = 32;
         while (cols < blocks * rows && cols < 512) cols *= 2;
         if (cols / rows > SK_MAX_GROUPS) cols = SK_MAX_GROUPS * rows;

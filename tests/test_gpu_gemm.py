@@ -526,3 +526,28 @@ def test_small_products_of_fp32_operands_in_one_launch(hb, M, N, K, m, b, roundi
         got = hb.gemm(tA, tB, X, B, fa, fb)
         assert hb.last_gemm_kernel() == "gemm_small_kernel" and hb.device_status() == 0
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("first,second", [((32, 4096, 4096, 64), (16, 4096, 1024, 64)), ((64, 2048, 2048, 64), (64, 4096, 1024, 64)), ((1, 2048, 4096, 24), (1, 512, 512, 24))])
+def test_few_rows_kernels_of_different_plans_run_on_two_streams(hb, first, second):
+    """Two launches whose CTAs fit an SM by shared memory but not by tensor memory (512 and 32, 256 and 128, 512 and 64 columns), on
+    two streams at once: a CTA gives its columns back before it waits for its cluster, so both finish, with the bits of a run alone."""
+    import torch
+    work = []
+    for k, (M, N, K, t) in enumerate((first, second)):
+        X, W = to_dev(wl.draw("normal", (M, K), seed=110 + k)), to_dev(wl.draw("he_weight", (K, N), seed=120 + k, fan_in=K))
+        fx = hb.Format(8, t)
+        c0 = hb.quantize_tiles(W, hb.Format(8, t, tile=t, stream_id=1), want_grid=False)[0]
+        alone = hb.gemm_q(M, N, K, X, c0, fmtA=fx)
+        assert hb.last_gemm_kernel() == "gemm_skinny_kernel"
+        ws = torch.empty(max(hb.gemm_q_workspace(M, N, K, X, c0, fmtA=fx), 1), dtype=torch.int8, device="cuda")
+        work.append((torch.cuda.Stream(), alone, [torch.empty_like(alone) for _ in range(64)], lambda o, a=(M, N, K, X, c0), f=fx, w=ws: hb.gemm_q(*a, fmtA=f, out=o, workspace=w)))
+    torch.cuda.synchronize()
+    for i in range(64):
+        for stream, _, outs, call in work:
+            with torch.cuda.stream(stream):
+                call(outs[i])
+    torch.cuda.synchronize()
+    assert hb.device_status() == 0
+    for _, alone, outs, _ in work:
+        assert all(torch.equal(o, alone) for o in outs)
