@@ -177,12 +177,15 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap mapW, const SkinnyProblem
             }
             if (ok) issued = i + 1;
         }
-        // nothing of this CTA is in flight when it leaves (in a normal run all has completed)
+        // nothing of this CTA is in flight when it leaves (in a normal run all has completed). MMAs of a segment that was given up
+        // half way write tensor memory, which goes back below: they too are committed and waited for, abort flag or not.
         if (!ok) {
-            if (elect_one()) tc_commit(free_bar);        // MMAs of a segment given up half way: nobody waits for this barrier any more
+            if (elect_one()) tc_commit(done_bar + 8 * issued);
+            ++issued;
             for (int i = 0; i < nseg; ++i) mbar_wait(full_bar + 8 * i, 0, abort_flag, p.status, 163, false);
         }
-        for (int i = 0; i < issued; ++i) mbar_wait_warp_fast(done_bar + 8 * i, 0, abort_flag, p.status, 164);
+        for (int i = 0; i < issued; ++i)
+            if (!mbar_wait_warp_fast(done_bar + 8 * i, 0, abort_flag, p.status, 164)) mbar_wait(done_bar + 8 * i, 0, abort_flag, p.status, 164, false);
         __syncwarp();
     } else {
         constexpr int NC = ROWS / 2;                              // accumulator columns of a warp
