@@ -144,6 +144,11 @@ int run_gemm(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const hbfp_
     return api.gemm_q_bias(M, N, K, &a, &b, bias, (float*)out.data_ptr(), ld_of(out), mem.get(), bytes, flags, cur_stream());
 }
 
+// The exception in flight as torch's own binding raises it: out of memory as torch.OutOfMemoryError, a Python error as itself.
+PyObject* python_error_set() {
+    torch::translate_exception_to_python(std::current_exception());
+    return nullptr;
+}
 template <class F>
 PyObject* guarded(F f) {
     try {
@@ -151,9 +156,8 @@ PyObject* guarded(F f) {
         return f();
     } catch (const Fail&) {
         return nullptr;
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
+    } catch (...) {
+        return python_error_set();
     }
 }
 // A layer's forward pass: it records its own node, so nothing is switched off around it; a library error is already a Python one.
@@ -163,15 +167,8 @@ PyObject* layer_call(F f) {
         return f();
     } catch (const Fail&) {
         return nullptr;
-    } catch (python_error& e) {
-        e.restore();
-        return nullptr;
-    } catch (const c10::ValueError& e) {
-        PyErr_SetString(PyExc_ValueError, e.what_without_backtrace());
-        return nullptr;
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return nullptr;
+    } catch (...) {
+        return python_error_set();
     }
 }
 PyObject* code(int rc) { return PyLong_FromLong(rc); }
