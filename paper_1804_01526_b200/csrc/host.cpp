@@ -463,7 +463,8 @@ struct LinearNode : public torch::autograd::Node {
         const int64_t batch = x.size(0);
         // backward-data on the shared weight view; backward-weight with blocks down the columns of X and dY
         if (task_should_compute_output(0)) out[0] = product(batch, fin, fout, fp32_operand(dy, 0, act(2, false)), c1.operand(), dy);
-        if (task_should_compute_output(1)) out[1] = product(fin, fout, batch, fp32_operand(x, 1, act(0, true)), fp32_operand(dy, 0, act(2, true)), dy);
+        // (of all columns of X: where there are more than the weights have rows, autograd refuses the gradient's shape)
+        if (task_should_compute_output(1)) out[1] = product(x.size(1), fout, batch, fp32_operand(x, 1, act(0, true)), fp32_operand(dy, 0, act(2, true)), dy);
         if (task_should_compute_output(2)) {
             out[2] = empty_f32({fout}, dy);
             ok_or_raise(api.column_sums((const float*)dy.data_ptr(), batch, fout, ld_of(dy), (float*)out[2].data_ptr(), cur_stream()), "hbfp_column_sums");

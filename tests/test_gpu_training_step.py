@@ -247,3 +247,16 @@ def test_out_of_memory_keeps_its_type(env):
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
     assert layer(x).shape == (60000, 6000)
+
+
+def test_inputs_of_the_wrong_width_do_not_train(env):
+    """More columns than the weights have rows: no gradient of the right shape from the first columns alone. Fewer: refused at once."""
+    torch, hbfp_nn, hb = env
+    layer = hbfp_nn.HbfpLinear(96, 48, rounding=0)
+    for requires_grad in (False, True):
+        y = layer(torch.randn(64, 100, device="cuda", requires_grad=requires_grad))
+        with pytest.raises(RuntimeError, match="invalid gradient"):
+            y.sum().backward()
+    assert layer.weight.grad is None
+    with pytest.raises(hb.HbfpError):
+        layer(torch.randn(64, 90, device="cuda"))
