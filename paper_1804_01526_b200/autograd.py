@@ -27,6 +27,34 @@ import torch
 from . import binding as hb
 
 
+class _HbfpLinearFn(torch.autograd.Function):
+    """The layer's passes as a Python function, for what has to see one (``needs_function`` in ``csrc/host.cpp``)."""
+
+    @staticmethod
+    def forward(ctx, x, weight, bias, layer):
+        ctx.layer = layer
+        ctx.save_for_backward(x)
+        batch = x.shape[0]
+        y = hb.gemm_q(batch, layer.fout, layer.fin, x.contiguous(), layer.views[0], fmtA=layer.fmt_act(0))
+        return y + bias if bias is not None else y
+
+    @staticmethod
+    def backward(ctx, dy):
+        layer = ctx.layer
+        (x,) = ctx.saved_tensors
+        dy = dy.contiguous()
+        batch = x.shape[0]
+        dx = dw = db = None
+        if ctx.needs_input_grad[0]:
+            dx = hb.gemm_q(batch, layer.fin, layer.fout, dy, layer.views[1], fmtA=layer.fmt_act(2))
+        if ctx.needs_input_grad[1]:
+            # contraction over the batch axis: 1-D blocks down the columns of X and dY
+            dw = hb.gemm(1, 0, x.contiguous(), dy, layer.fmt_act(0, batch_axis=True), layer.fmt_act(2, batch_axis=True))
+        if ctx.needs_input_grad[2]:
+            db = dy.sum(dim=0)
+        return dx, dw, db, None
+
+
 class HbfpLinear(torch.nn.Module):
     """``y = x W + b`` with W ``[fin][fout]`` in wide storage; see the module docstring."""
 
@@ -65,8 +93,63 @@ class HbfpLinear(torch.nn.Module):
         self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        return hb.host().linear(x, self.weight, self.bias, self.views[0], self.views[1], self.mant_bits, self.tile, self.batch_block,
-                                self.rounding, self.seed + self.steps, self.stream_id)
+        y = hb.host().linear(x, self.weight, self.bias, self.views[0], self.views[1], self.mant_bits, self.tile, self.batch_block,
+                             self.rounding, self.seed + self.steps, self.stream_id)
+        return y if y is not None else _HbfpLinearFn.apply(x, self.weight, self.bias, self)
+
+
+class _HbfpConv3x3Fn(torch.autograd.Function):
+    """The layer's passes as a Python function, like ``_HbfpLinearFn``."""
+
+    @staticmethod
+    def forward(ctx, x, weight, layer):
+        n, h, w, c = x.shape
+        ctx.layer = layer
+        ctx.save_for_backward(x)
+        x = x.contiguous()
+        px = hb.quantize(x.view(n * h * w, c), 1, layer.fmt_pixels(0))
+        try:
+            # the implicit GEMM reads the taps straight from the packed pixels
+            y = hb.conv_forward(px, layer.views[0], n, h, w, c, 3, 3, 1)
+        except hb.HbfpError as e:
+            if e.code != hb.ERR_UNSUPPORTED:
+                raise
+            # shapes it does not cover: gather the packed operand, then the ordinary GEMM (same product)
+            pa = hb.im2col_packed(px, n, h, w, c, 3, 3, 1)
+            y = hb.gemm_q(n * h * w, layer.fout, 9 * c, pa, layer.views[0])
+        return y.view(n, h, w, layer.fout)
+
+    @staticmethod
+    def backward(ctx, dy):
+        layer = ctx.layer
+        (x,) = ctx.saved_tensors
+        n, h, w, c = x.shape
+        f = layer.fout
+        dy2 = dy.contiguous().view(n * h * w, f)
+        dx = dw = None
+        if ctx.needs_input_grad[0]:
+            try:
+                # the convolution of the packed output gradient with the forward weights regrouped (taps turned by
+                # 180 degrees, feature-map roles swapped) yields dX itself
+                pg = hb.quantize(dy2, 1, layer.fmt_pixels(2))
+                turned = hb.conv_dgrad_filters(layer.views[1], 3, 3, c, f)
+                dx = hb.conv_forward(pg, turned, n, h, w, f, 3, 3, 1).view(n, h, w, c)
+            except hb.HbfpError as e:
+                if e.code != hb.ERR_UNSUPPORTED:
+                    raise
+        if ctx.needs_input_grad[0] and dx is None:
+            # shapes that route does not cover: gradient of the im2col matrix, then its scatter back onto the
+            # pixels (an FP32 operation)
+            dcols = hb.gemm_q(n * h * w, 9 * c, f, dy2, layer.views[1], fmtA=layer.fmt_pixels(2)).view(n, h, w, 3, 3, c)
+            dxp = torch.zeros((n, h + 2, w + 2, c), device=x.device)
+            for i in range(3):
+                for j in range(3):
+                    dxp[:, i:i + h, j:j + w, :] += dcols[:, :, :, i, j, :]
+            dx = dxp[:, 1:h + 1, 1:w + 1, :].contiguous()
+        if ctx.needs_input_grad[1]:
+            pa_t = hb.im2col_packed_t(x.contiguous(), 3, 3, 1, layer.fmt_batch(0))
+            dw = hb.gemm_q(9 * c, f, n * h * w, pa_t, dy2, fmtB=layer.fmt_batch(2))
+        return dx, dw, None
 
 
 class HbfpConv3x3(torch.nn.Module):
@@ -103,4 +186,5 @@ class HbfpConv3x3(torch.nn.Module):
         self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        return hb.host().conv3x3(x, self.weight, self.views[0], self.views[1], self.mant_bits, self.pixel_block, self.c, self.fout)
+        y = hb.host().conv3x3(x, self.weight, self.views[0], self.views[1], self.mant_bits, self.pixel_block, self.c, self.fout)
+        return y if y is not None else _HbfpConv3x3Fn.apply(x, self.weight, self)

@@ -10,6 +10,7 @@
 #include <torch/csrc/autograd/functions/utils.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <torch/csrc/autograd/saved_variable.h>
+#include <torch/csrc/jit/frontend/tracer.h>
 #include <ATen/ATen.h>
 #include <ATen/core/LegacyTypeDispatch.h>
 #include <ATen/cuda/CUDAContext.h>
@@ -434,6 +435,15 @@ at::Tensor product(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const
     ok_or_raise(run_gemm(M, N, K, a, b, out, nullptr, HBFP_GEMM_AUTO, bias), "hbfp_gemm_q");
     return out;
 }
+// Whether a pass runs under something that has to see an autograd.Function to record, transform or refuse it: a trace, a functorch
+// transform, an input with a forward-mode tangent. A node of this file would vanish from the first (what is left of it there is an
+// empty tensor) and drop the tangent; the layer then goes through its Python function (autograd.py).
+bool needs_function(std::initializer_list<at::Tensor> inputs) {
+    if (torch::jit::tracer::isTracing() || c10::impl::tls_is_dispatch_key_included(c10::DispatchKey::FuncTorchDynamicLayerFrontMode)) return true;
+    for (const at::Tensor& t : inputs)
+        if (t.defined() && t._fw_grad(/*level=*/0).defined()) return true;
+    return false;
+}
 // Everything a pass computes lies below autograd; gradients come out as plain tensors.
 struct Below {
     at::AutoDispatchBelowADInplaceOrView below;
@@ -473,12 +483,14 @@ struct LinearNode : public torch::autograd::Node {
     }
 };
 
-// linear(x, weight, bias or None, c0, c1, mant_bits, tile, batch_block, rounding, seed, stream_id) -> y
+// linear(x, weight, bias or None, c0, c1, mant_bits, tile, batch_block, rounding, seed, stream_id) -> y, or None where the pass
+// needs a Python function
 PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!want(n, 11)) return nullptr;
     return layer_call([&]() -> PyObject* {
         const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
         const at::Tensor bias = a[2] != Py_None ? tensor_of(a[2], "bias") : at::Tensor();
+        if (needs_function({x, w, bias})) return same(Py_None);
         const PackedTensor c0 = packed_of(a[3]);
         LinearNode proto;
         proto.mant_bits = (int)as_ll(a[5]); proto.tile = (int)as_ll(a[6]); proto.batch_block = (int)as_ll(a[7]); proto.rounding = (int)as_ll(a[8]);
@@ -589,11 +601,12 @@ struct ConvNode : public torch::autograd::Node {
     }
 };
 
-// conv3x3(x, weight, c0, c1, mant_bits, pixel_block, c, f) -> y
+// conv3x3(x, weight, c0, c1, mant_bits, pixel_block, c, f) -> y, or None where the pass needs a Python function
 PyObject* conv3x3(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!want(n, 8)) return nullptr;
     return layer_call([&]() -> PyObject* {
         const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
+        if (needs_function({x, w})) return same(Py_None);
         if (!(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 4)) value_error("%s must be a float32 CUDA tensor [n][h][w][c]", "x");
         auto node = std::shared_ptr<ConvNode>(new ConvNode(), torch::autograd::deleteNode);
         node->mant_bits = (int)as_ll(a[4]);

@@ -260,3 +260,24 @@ def test_inputs_of_the_wrong_width_do_not_train(env):
     assert layer.weight.grad is None
     with pytest.raises(hb.HbfpError):
         layer(torch.randn(64, 90, device="cuda"))
+
+
+@pytest.mark.parametrize("kind", ["linear", "conv"])
+def test_layers_under_a_trace_forward_mode_and_function_transforms(env, kind):
+    """A trace records the layer (and replays it on other inputs, with gradients), what has no derivative of that kind says so."""
+    torch, hbfp_nn, hb = env
+    import torch.autograd.forward_ad as fwad
+    torch.manual_seed(9)
+    layer, shape = (hbfp_nn.HbfpLinear(96, 48, rounding=0), (64, 96)) if kind == "linear" else (hbfp_nn.HbfpConv3x3(64, 64), (2, 16, 16, 64))
+    x, x2 = torch.randn(shape, device="cuda"), torch.randn(shape, device="cuda").requires_grad_(True)
+    traced = torch.jit.trace(layer, (x,), check_trace=False)
+    want, got = layer(x2), traced(x2)
+    assert torch.equal(want, got)
+    dy = torch.randn_like(want)
+    assert torch.equal(*(torch.autograd.grad(y, x2, dy)[0] for y in (want, got)))
+    with fwad.dual_level(), pytest.raises(NotImplementedError):
+        layer(fwad.make_dual(x, torch.ones_like(x)))
+    for transform in (lambda: torch.func.jvp(layer, (x,), (x,)), lambda: torch.func.grad(lambda v: layer(v).sum())(x), lambda: torch.func.vmap(layer)(x[None])):
+        with pytest.raises(RuntimeError, match="functorch transforms"):
+            transform()
+    assert torch.equal(layer(x2), want)
