@@ -28,7 +28,8 @@ from . import binding as hb
 
 
 class _HbfpLinearFn(torch.autograd.Function):
-    """The layer's passes as a Python function, for what has to see one (``needs_function`` in ``csrc/host.cpp``)."""
+    """The layer's passes as a Python function, for what has to see one (``needs_function`` in ``csrc/host.cpp``) and for a bias that
+    the product cannot add in its store."""
 
     @staticmethod
     def forward(ctx, x, weight, bias, layer):

@@ -491,6 +491,9 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
         const at::Tensor bias = a[2] != Py_None ? tensor_of(a[2], "bias") : at::Tensor();
         if (needs_function({x, w, bias})) return same(Py_None);
+        // a bias of another type, shape or place (a layer cast to half precision, one value for all outputs): the general addition
+        if (bias.defined() && !(bias.device() == x.device() && bias.scalar_type() == at::kFloat && bias.dim() == 1 && bias.size(0) == w.size(1)))
+            return same(Py_None);
         const PackedTensor c0 = packed_of(a[3]);
         LinearNode proto;
         proto.mant_bits = (int)as_ll(a[5]); proto.tile = (int)as_ll(a[6]); proto.batch_block = (int)as_ll(a[7]); proto.rounding = (int)as_ll(a[8]);
@@ -504,7 +507,6 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
             Below guard;
             const at::Tensor xc = x.contiguous();
             const at::Tensor bc = bias.defined() ? bias.contiguous() : bias;
-            if (bc.defined()) TORCH_CHECK_VALUE(bc.is_cuda() && bc.scalar_type() == at::kFloat && bc.numel() == proto.fout, "bias must hold a float32 value per output on the GPU");
             y = product(xc.size(0), proto.fout, proto.fin, fp32_operand(xc, 0, proto.act(0, false)), c0.operand(), xc, bc.defined() ? (const float*)bc.data_ptr() : nullptr);
         }
         if (torch::autograd::compute_requires_grad(x, w, bias)) {

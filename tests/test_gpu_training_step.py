@@ -281,3 +281,30 @@ def test_layers_under_a_trace_forward_mode_and_function_transforms(env, kind):
         with pytest.raises(RuntimeError, match="functorch transforms"):
             transform()
     assert torch.equal(layer(x2), want)
+
+
+@pytest.mark.parametrize("shape,dtype,device", [((48,), "float16", "cuda"), ((48,), "bfloat16", "cuda"), ((1,), "float32", "cuda"), ((), "float32", "cuda"), ((), "float32", "cpu"),
+                                                ((48,), "float64", "cuda")])
+def test_bias_of_another_type_or_shape(env, shape, dtype, device):
+    """Whatever torch adds to a float32 matrix: the sum's type and values, and a gradient like the bias."""
+    torch, hbfp_nn, hb = env
+    torch.manual_seed(3)
+    layer, x, dy = hbfp_nn.HbfpLinear(96, 48, rounding=0), torch.randn(64, 96, device="cuda"), torch.randn(64, 48, device="cuda")
+    with torch.no_grad():
+        plain = layer(x)
+    layer.bias = torch.nn.Parameter(torch.randn(shape, device=device).to(getattr(torch, dtype)))
+    y = layer(x)
+    want = plain + layer.bias
+    assert y.dtype == want.dtype and torch.equal(y, want)
+    if dtype != "float64":                      # the products take float32 gradients
+        y.backward(dy)
+        assert layer.bias.grad.dtype == layer.bias.dtype and layer.bias.grad.shape == layer.bias.shape
+        sums = dy.sum(0) if shape else dy.sum(0).sum()
+        assert torch.allclose(layer.bias.grad.float(), (sums.sum(0, keepdim=True) if shape == (1,) else sums).to(device), rtol=1e-2, atol=1e-2)
+
+
+def test_a_layer_cast_to_half_precision_computes_as_before(env):
+    torch, hbfp_nn, hb = env
+    layer, x = hbfp_nn.HbfpLinear(96, 48, rounding=0).half(), torch.randn(64, 96, device="cuda")
+    layer(x).sum().backward()
+    assert layer(x).dtype == torch.float32 and layer.weight.grad.dtype == layer.bias.grad.dtype == torch.float16
