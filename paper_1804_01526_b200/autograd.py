@@ -27,6 +27,12 @@ import torch
 from . import binding as hb
 
 
+def _own(layer, cls, name: str) -> bool:
+    """Whether ``layer`` uses the method of ``cls`` itself: the compiled passes make these formats themselves, a layer that
+    overrides one takes its Python function."""
+    return getattr(type(layer), name) is getattr(cls, name) and name not in layer.__dict__
+
+
 class _HbfpLinearFn(torch.autograd.Function):
     """The layer's passes as a Python function, for what has to see one (``needs_function`` in ``csrc/host.cpp``) and for a bias that
     the product cannot add in its store."""
@@ -94,8 +100,10 @@ class HbfpLinear(torch.nn.Module):
         self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        y = hb.host().linear(x, self.weight, self.bias, self.views[0], self.views[1], self.mant_bits, self.tile, self.batch_block,
-                             self.rounding, self.seed + self.steps, self.stream_id)
+        y = None
+        if _own(self, HbfpLinear, "fmt_act"):
+            y = hb.host().linear(x, self.weight, self.bias, self.views[0], self.views[1], self.mant_bits, self.tile, self.batch_block,
+                                 self.rounding, self.seed + self.steps, self.stream_id)
         return y if y is not None else _HbfpLinearFn.apply(x, self.weight, self.bias, self)
 
 
@@ -187,5 +195,7 @@ class HbfpConv3x3(torch.nn.Module):
         self.weight.data = hb.wide_update_value(self.wide, delta.contiguous(), self.fmt_weight(), self.views)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
-        y = hb.host().conv3x3(x, self.weight, self.views[0], self.views[1], self.mant_bits, self.pixel_block, self.c, self.fout)
+        y = None
+        if _own(self, HbfpConv3x3, "fmt_pixels") and _own(self, HbfpConv3x3, "fmt_batch"):
+            y = hb.host().conv3x3(x, self.weight, self.views[0], self.views[1], self.mant_bits, self.pixel_block, self.c, self.fout)
         return y if y is not None else _HbfpConv3x3Fn.apply(x, self.weight, self)

@@ -308,3 +308,29 @@ def test_a_layer_cast_to_half_precision_computes_as_before(env):
     layer, x = hbfp_nn.HbfpLinear(96, 48, rounding=0).half(), torch.randn(64, 96, device="cuda")
     layer(x).sum().backward()
     assert layer(x).dtype == torch.float32 and layer.weight.grad.dtype == layer.bias.grad.dtype == torch.float16
+
+
+def test_layers_that_override_their_formats(env):
+    """The format methods are what a subclass (or one layer) changes the conversions by: both passes use what they return."""
+    import dataclasses
+    torch, hbfp_nn, hb = env
+
+    class Literal(hbfp_nn.HbfpLinear):
+        def fmt_act(self, which, batch_axis=False):
+            return dataclasses.replace(super().fmt_act(which, batch_axis), exp_mode=1)
+
+    # powers of two, where the two exponent rules differ (the block's largest value saturates under the literal one)
+    x = torch.exp2(torch.randint(-6, 3, (64, 96), device="cuda").float())
+    dy = torch.exp2(torch.randint(-6, 3, (64, 48), device="cuda").float())
+    torch.manual_seed(1)
+    own = Literal(96, 48, rounding=0)
+    own(x).backward(dy)
+    f = own.fmt_act(0)
+    assert torch.equal(own(x).detach(), hb.gemm_q(64, 48, 96, x, own.views[0], fmtA=f) + own.bias.detach())
+    assert torch.equal(own.weight.grad, hb.gemm(1, 0, x, dy, own.fmt_act(0, True), own.fmt_act(2, True)))
+    assert not torch.equal(own(x), hb.gemm_q(64, 48, 96, x, own.views[0], fmtA=dataclasses.replace(f, exp_mode=0)) + own.bias)
+    conv, xc = hbfp_nn.HbfpConv3x3(64, 64), torch.randn(2, 16, 16, 64, device="cuda")
+    plain = conv(xc)
+    conv.fmt_pixels = lambda which: hb.Format(mant_bits=4, block=64, stream_id=which)
+    px = hb.quantize(xc.view(-1, 64), 1, conv.fmt_pixels(0))
+    assert torch.equal(conv(xc).view(-1, 64), hb.conv_forward(px, conv.views[0], 2, 16, 16, 64, 3, 3, 1)) and not torch.equal(conv(xc), plain)
