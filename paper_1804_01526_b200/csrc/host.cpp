@@ -467,6 +467,9 @@ struct LinearNode : public torch::autograd::Node {
         variable_list out(3);
         if (!grads[0].defined()) return out;
         const at::Tensor x0 = x_.unpack(shared_from_this());
+        // with create_graph the bias gradient can be differentiated further; the products have no second derivative
+        const bool recorded_sum = task_should_compute_output(2) && at::GradMode::is_enabled() && grads[0].requires_grad();
+        if (recorded_sum) out[2] = grads[0].sum(0);
         Below guard;
         const at::Tensor dy = grads[0].contiguous(), x = x0.contiguous();
         check_f32_cpp(dy);
@@ -475,7 +478,7 @@ struct LinearNode : public torch::autograd::Node {
         if (task_should_compute_output(0)) out[0] = product(batch, fin, fout, fp32_operand(dy, 0, act(2, false)), c1.operand(), dy);
         // (of all columns of X: where there are more than the weights have rows, autograd refuses the gradient's shape)
         if (task_should_compute_output(1)) out[1] = product(x.size(1), fout, batch, fp32_operand(x, 1, act(0, true)), fp32_operand(dy, 0, act(2, true)), dy);
-        if (task_should_compute_output(2)) {
+        if (task_should_compute_output(2) && !recorded_sum) {
             out[2] = empty_f32({fout}, dy);
             ok_or_raise(api.column_sums((const float*)dy.data_ptr(), batch, fout, ld_of(dy), (float*)out[2].data_ptr(), cur_stream()), "hbfp_column_sums");
         }

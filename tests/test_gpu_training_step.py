@@ -334,3 +334,14 @@ def test_layers_that_override_their_formats(env):
     conv.fmt_pixels = lambda which: hb.Format(mant_bits=4, block=64, stream_id=which)
     px = hb.quantize(xc.view(-1, 64), 1, conv.fmt_pixels(0))
     assert torch.equal(conv(xc).view(-1, 64), hb.conv_forward(px, conv.views[0], 2, 16, 16, 64, 3, 3, 1)) and not torch.equal(conv(xc), plain)
+
+
+def test_bias_gradient_can_be_differentiated(env):
+    torch, hbfp_nn, hb = env
+    layer, x = hbfp_nn.HbfpLinear(96, 48, rounding=0), torch.randn(64, 96, device="cuda")
+    dy, v = torch.randn(64, 48, device="cuda", requires_grad=True), torch.randn(48, device="cuda")
+    (db,) = torch.autograd.grad(layer(x), layer.bias, dy, create_graph=True)
+    (g,) = torch.autograd.grad(db, dy, v)
+    assert torch.equal(g, v.expand(64, 48))
+    plain = torch.autograd.grad(layer(x), layer.bias, dy.detach())[0]
+    assert torch.allclose(db, plain, rtol=1e-5, atol=1e-5)
