@@ -465,7 +465,7 @@ struct LinearNode : public torch::autograd::Node {
     void release_variables() override { x_.reset_data(); }
     variable_list apply(variable_list&& grads) override {
         variable_list out(3);
-        if (!grads[0].defined()) return out;
+        if (!grads[0].defined()) grads[0] = input_metadata(0).zeros_like();      // as autograd.Function hands it over
         const at::Tensor x0 = x_.unpack(shared_from_this());
         // with create_graph the bias gradient can be differentiated further; the products have no second derivative
         const bool recorded_sum = task_should_compute_output(2) && at::GradMode::is_enabled() && grads[0].requires_grad();
@@ -588,7 +588,7 @@ struct ConvNode : public torch::autograd::Node {
     }
     variable_list apply(variable_list&& grads) override {
         variable_list out(2);
-        if (!grads[0].defined()) return out;
+        if (!grads[0].defined()) grads[0] = input_metadata(0).zeros_like();      // as autograd.Function hands it over
         const at::Tensor x0 = x_.unpack(shared_from_this());
         Below guard;
         const at::Tensor x = x0.contiguous();

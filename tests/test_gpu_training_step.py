@@ -345,3 +345,22 @@ def test_bias_gradient_can_be_differentiated(env):
     assert torch.equal(g, v.expand(64, 48))
     plain = torch.autograd.grad(layer(x), layer.bias, dy.detach())[0]
     assert torch.allclose(db, plain, rtol=1e-5, atol=1e-5)
+
+
+def test_a_gradient_that_never_came_counts_as_zeros(env):
+    torch, hbfp_nn, hb = env
+
+    class Drop(torch.autograd.Function):
+        @staticmethod
+        def forward(ctx, x):
+            return x.clone()
+
+        @staticmethod
+        def backward(ctx, g):
+            return None
+
+    layer, conv = hbfp_nn.HbfpLinear(96, 48, rounding=0), hbfp_nn.HbfpConv3x3(64, 64)
+    for mod, x in ((layer, torch.randn(64, 96, device="cuda", requires_grad=True)), (conv, torch.randn(2, 16, 16, 64, device="cuda", requires_grad=True))):
+        Drop.apply(mod(x)).sum().backward()
+        for t in (x, *mod.parameters()):
+            assert t.grad.shape == t.shape and not t.grad.any()
