@@ -462,8 +462,12 @@ struct LinearNode : public torch::autograd::Node {
     // X (which = 0) or dY (which = 2) in blocks along a feature axis or along the batch axis
     hbfp_format act(int which, bool batch_axis) const { return make_format(mant_bits, batch_axis ? batch_block : tile, rounding, seed, stream_id + which); }
     std::string name() const override { return "HbfpLinearBackward"; }
-    void release_variables() override { x_.reset_data(); }
+    void release_variables() override {
+        std::lock_guard<std::mutex> lock(mutex_);            // backward passes of several threads may meet in a node
+        x_.reset_data();
+    }
     variable_list apply(variable_list&& grads) override {
+        std::lock_guard<std::mutex> lock(mutex_);
         variable_list out(3);
         if (!grads[0].defined()) grads[0] = input_metadata(0).zeros_like();      // as autograd.Function hands it over
         const at::Tensor x0 = x_.unpack(shared_from_this());
@@ -533,7 +537,10 @@ struct ConvNode : public torch::autograd::Node {
     hbfp_format pixels(int which) const { return make_format(mant_bits, (int)c, 0, 0, which); }           // blocks of c channels of a pixel
     hbfp_format batch(int which) const { return make_format(mant_bits, pixel_block, 0, 0, which); }       // blocks of consecutive pixels
     std::string name() const override { return "HbfpConv3x3Backward"; }
-    void release_variables() override { x_.reset_data(); }
+    void release_variables() override {
+        std::lock_guard<std::mutex> lock(mutex_);            // backward passes of several threads may meet in a node
+        x_.reset_data();
+    }
     static PackedTensor convert(const at::Tensor& x2, const hbfp_format& fmt) {
         PackedTensor p = alloc_packed(x2.size(0), x2.size(1), fmt, x2, "hbfp_quantize");
         ok_or_raise(api.quantize((const float*)x2.data_ptr(), x2.size(0), x2.size(1), ld_of(x2), 1, &fmt, p.mant.data_ptr(), (int8_t*)p.exps.data_ptr(), cur_stream()),
@@ -587,6 +594,7 @@ struct ConvNode : public torch::autograd::Node {
         return dxp.slice(1, 1, h + 1).slice(2, 1, w + 1).contiguous();
     }
     variable_list apply(variable_list&& grads) override {
+        std::lock_guard<std::mutex> lock(mutex_);
         variable_list out(2);
         if (!grads[0].defined()) grads[0] = input_metadata(0).zeros_like();      // as autograd.Function hands it over
         const at::Tensor x0 = x_.unpack(shared_from_this());
