@@ -92,6 +92,16 @@ void check_f32_cpp(const at::Tensor& x) {
 }
 int64_t ld_of(const at::Tensor& x) { return x.size(0) > 1 ? x.stride(0) : std::max<int64_t>(x.size(1), 1); }
 
+// The interpreter lock is let go while memory is allocated and kernels are launched, so that other Python threads run when the
+// launch queue is full or the allocator has to wait for the GPU (a call through ctypes lets it go, too). Nothing in there may touch
+// a Python object.
+struct NoGil {
+    PyThreadState* state = PyEval_SaveThread();
+    NoGil() = default;
+    NoGil(const NoGil&) = delete;
+    ~NoGil() { PyEval_RestoreThread(state); }
+};
+
 void* cur_stream() { return at::cuda::getCurrentCUDAStream().stream(); }
 
 at::Tensor empty_f32(at::IntArrayRef sizes, const at::Tensor& like) { return at::empty(sizes, like.options().dtype(at::kFloat).requires_grad(false)); }
@@ -151,6 +161,11 @@ PyObject* python_error_set() {
     return nullptr;
 }
 template <class F>
+auto without_gil(F f) {
+    NoGil free;
+    return f();
+}
+template <class F>
 PyObject* guarded(F f) {
     try {
         at::AutoDispatchBelowADInplaceOrView below;          // plain tensors: nothing here is recorded for autograd
@@ -182,6 +197,25 @@ PyObject* same(PyObject* o) { Py_INCREF(o); return o; }
 
 // ------------------------------------------------------------------------------ calls
 
+// A call's packed result: buffers handed in, or (None) allocated for it.
+struct Buffers {
+    at::Tensor m, e;
+    Buffers(PyObject* mant, PyObject* exps) {
+        if (mant == Py_None) return;
+        m = tensor_of(mant, "mantissas");
+        e = tensor_of(exps, "exponents");
+    }
+    int make(int64_t rows, int64_t k, const hbfp_format& f, const at::Tensor& like) {
+        if (m.defined()) return HBFP_OK;
+        hbfp_layout L;
+        const int rc = api.packed_layout(rows, k, &f, &L);
+        if (rc) return rc;
+        m = empty_i8(L.mant_bytes, like);
+        e = empty_i8(L.exp_bytes, like);
+        return HBFP_OK;
+    }
+};
+
 // quantize(x, axis, fmt, mant or None, exps or None) -> (mant, exps)
 PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!want(n, 5)) return nullptr;
@@ -190,20 +224,13 @@ PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
         check_f32(x, "x");
         const int axis = (int)as_ll(a[1]);
         const hbfp_format f = format_of(a[2]);
-        at::Tensor m, e;
-        if (a[3] == Py_None) {
-            hbfp_layout L;
-            const int rc = axis == 1 ? api.packed_layout(x.size(0), x.size(1), &f, &L) : api.packed_layout(x.size(1), x.size(0), &f, &L);
-            if (rc) return code(rc);
-            m = empty_i8(L.mant_bytes, x);
-            e = empty_i8(L.exp_bytes, x);
-        } else {
-            m = tensor_of(a[3], "mantissas");
-            e = tensor_of(a[4], "exponents");
-        }
-        const int rc = api.quantize((const float*)x.data_ptr(), x.size(0), x.size(1), ld_of(x), axis, &f, m.data_ptr(), (int8_t*)e.data_ptr(), cur_stream());
+        Buffers out(a[3], a[4]);
+        const int rc = without_gil([&] {
+            const int bad = axis == 1 ? out.make(x.size(0), x.size(1), f, x) : out.make(x.size(1), x.size(0), f, x);
+            return bad ? bad : api.quantize((const float*)x.data_ptr(), x.size(0), x.size(1), ld_of(x), axis, &f, out.m.data_ptr(), (int8_t*)out.e.data_ptr(), cur_stream());
+        });
         if (rc) return code(rc);
-        return Py_BuildValue("(NN)", a[3] == Py_None ? THPVariable_Wrap(m) : same(a[3]), a[3] == Py_None ? THPVariable_Wrap(e) : same(a[4]));
+        return Py_BuildValue("(NN)", a[3] == Py_None ? THPVariable_Wrap(out.m) : same(a[3]), a[3] == Py_None ? THPVariable_Wrap(out.e) : same(a[4]));
     });
 }
 
@@ -223,10 +250,14 @@ PyObject* gemm(PyObject*, PyObject* const* a, Py_ssize_t n) {
         oa.data = A.data_ptr(); oa.ld = ld_of(A); oa.trans = (int32_t)as_ll(a[0]); oa.fmt = format_of(a[4]);
         ob.data = B.data_ptr(); ob.ld = ld_of(B); ob.trans = (int32_t)as_ll(a[1]); ob.fmt = format_of(a[5]);
         const bool fresh = a[6] == Py_None;
-        const at::Tensor out = fresh ? empty_f32({M, N}, A) : tensor_of(a[6], "out");
-        at::Tensor ws;
+        at::Tensor out, ws;
+        if (!fresh) out = tensor_of(a[6], "out");
         if (a[7] != Py_None) ws = tensor_of(a[7], "workspace");
-        const int rc = run_gemm(M, N, K, oa, ob, out, ws.defined() ? &ws : nullptr, (uint32_t)as_ll(a[8]));
+        const uint32_t flags = (uint32_t)as_ll(a[8]);
+        const int rc = without_gil([&] {
+            if (fresh) out = empty_f32({M, N}, A);
+            return run_gemm(M, N, K, oa, ob, out, ws.defined() ? &ws : nullptr, flags);
+        });
         if (rc) return code(rc);
         return fresh ? THPVariable_Wrap(out) : same(a[6]);
     });
@@ -239,10 +270,14 @@ PyObject* gemm_q(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const int64_t M = as_ll(a[0]), N = as_ll(a[1]), K = as_ll(a[2]);
         const Operand oa = operand_of(a[3], as_ll(a[5]), a[7]), ob = operand_of(a[4], as_ll(a[6]), a[8]);
         const bool fresh = a[9] == Py_None;
-        const at::Tensor out = fresh ? empty_f32({M, N}, oa.data) : tensor_of(a[9], "out");
-        at::Tensor ws;
+        at::Tensor out, ws;
+        if (!fresh) out = tensor_of(a[9], "out");
         if (a[10] != Py_None) ws = tensor_of(a[10], "workspace");
-        const int rc = run_gemm(M, N, K, oa.o, ob.o, out, ws.defined() ? &ws : nullptr, (uint32_t)as_ll(a[11]));
+        const uint32_t flags = (uint32_t)as_ll(a[11]);
+        const int rc = without_gil([&] {
+            if (fresh) out = empty_f32({M, N}, oa.data);
+            return run_gemm(M, N, K, oa.o, ob.o, out, ws.defined() ? &ws : nullptr, flags);
+        });
         if (rc) return code(rc);
         return fresh ? THPVariable_Wrap(out) : same(a[9]);
     });
@@ -269,9 +304,13 @@ PyObject* wide_update(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const hbfp_format f = format_of(a[3]);
         ViewPtrs v;
         if (a[4] != Py_None) { view_of(a[4], &v.m0, &v.e0); view_of(a[5], &v.m1, &v.e1); }
-        const at::Tensor value = a[6] == Py_True ? empty_f32({m.size(0), m.size(1)}, m) : at::Tensor();
-        const int rc = api.wide_update((int16_t*)m.data_ptr(), (int8_t*)e.data_ptr(), (const float*)d.data_ptr(), m.size(0), m.size(1), ld_of(d), &f,
-                                       v.m0, v.e0, v.m1, v.e1, value.defined() ? (float*)value.data_ptr() : nullptr, m.size(1), cur_stream());
+        const bool wanted = a[6] == Py_True;
+        at::Tensor value;
+        const int rc = without_gil([&] {
+            if (wanted) value = empty_f32({m.size(0), m.size(1)}, m);
+            return api.wide_update((int16_t*)m.data_ptr(), (int8_t*)e.data_ptr(), (const float*)d.data_ptr(), m.size(0), m.size(1), ld_of(d), &f,
+                                   v.m0, v.e0, v.m1, v.e1, wanted ? (float*)value.data_ptr() : nullptr, m.size(1), cur_stream());
+        });
         return !rc && value.defined() ? THPVariable_Wrap(value) : code(rc);
     });
 }
@@ -282,10 +321,16 @@ PyObject* wide_dequantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return guarded([&]() -> PyObject* {
         const at::Tensor m = tensor_of(a[0], "mantissas"), e = tensor_of(a[1], "exponents");
         const bool fresh = a[3] == Py_None;
-        const at::Tensor out = fresh ? empty_f32({m.size(0), m.size(1)}, m) : tensor_of(a[3], "out");
-        check_f32(out, "out");
-        const int rc = api.wide_dequantize((const int16_t*)m.data_ptr(), (const int8_t*)e.data_ptr(), m.size(0), m.size(1), (int32_t)as_ll(a[2]),
-                                           (float*)out.data_ptr(), ld_of(out), cur_stream());
+        const int32_t tile = (int32_t)as_ll(a[2]);
+        at::Tensor out;
+        if (!fresh) {
+            out = tensor_of(a[3], "out");
+            check_f32(out, "out");
+        }
+        const int rc = without_gil([&] {
+            if (fresh) out = empty_f32({m.size(0), m.size(1)}, m);
+            return api.wide_dequantize((const int16_t*)m.data_ptr(), (const int8_t*)e.data_ptr(), m.size(0), m.size(1), tile, (float*)out.data_ptr(), ld_of(out), cur_stream());
+        });
         if (rc) return code(rc);
         return fresh ? THPVariable_Wrap(out) : same(a[3]);
     });
@@ -296,12 +341,18 @@ PyObject* conv_forward(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!want(n, 11)) return nullptr;
     return guarded([&]() -> PyObject* {
         const Operand px = operand_of(a[0], 0, Py_None), fl = operand_of(a[1], 0, Py_None);
-        const int64_t nn = as_ll(a[2]), h = as_ll(a[3]), w = as_ll(a[4]), nf = as_ll(a[9]);
+        const int64_t nn = as_ll(a[2]), h = as_ll(a[3]), w = as_ll(a[4]), c = as_ll(a[5]), nf = as_ll(a[9]);
+        const int kh = (int)as_ll(a[6]), kw = (int)as_ll(a[7]), pad = (int)as_ll(a[8]);
         const bool fresh = a[10] == Py_None;
-        const at::Tensor out = fresh ? empty_f32({nn * h * w, nf}, px.data) : tensor_of(a[10], "out");
-        check_f32(out, "out");
-        const int rc = api.conv_forward(px.o.data, px.o.exps, nn, h, w, as_ll(a[5]), (int)as_ll(a[6]), (int)as_ll(a[7]), (int)as_ll(a[8]), &px.o.fmt, &fl.o,
-                                        nf, (float*)out.data_ptr(), ld_of(out), cur_stream());
+        at::Tensor out;
+        if (!fresh) {
+            out = tensor_of(a[10], "out");
+            check_f32(out, "out");
+        }
+        const int rc = without_gil([&] {
+            if (fresh) out = empty_f32({nn * h * w, nf}, px.data);
+            return api.conv_forward(px.o.data, px.o.exps, nn, h, w, c, kh, kw, pad, &px.o.fmt, &fl.o, nf, (float*)out.data_ptr(), ld_of(out), cur_stream());
+        });
         if (rc) return code(rc);
         return fresh ? THPVariable_Wrap(out) : same(a[10]);
     });
@@ -314,20 +365,13 @@ PyObject* conv_dgrad_filters(PyObject*, PyObject* const* a, Py_ssize_t n) {
         const Operand c1 = operand_of(a[0], 0, Py_None);
         const int kh = (int)as_ll(a[1]), kw = (int)as_ll(a[2]);
         const int64_t ci = as_ll(a[3]), co = as_ll(a[4]);
-        at::Tensor m, e;
-        if (a[5] == Py_None) {
-            hbfp_layout L;
-            const int rc = api.packed_layout(ci, (int64_t)kh * kw * co, &c1.o.fmt, &L);
-            if (rc) return code(rc);
-            m = empty_i8(L.mant_bytes, c1.data);
-            e = empty_i8(L.exp_bytes, c1.data);
-        } else {
-            m = tensor_of(a[5], "mantissas");
-            e = tensor_of(a[6], "exponents");
-        }
-        const int rc = api.conv_dgrad_filters(c1.o.data, c1.o.exps, kh, kw, ci, co, &c1.o.fmt, m.data_ptr(), (int8_t*)e.data_ptr(), cur_stream());
+        Buffers out(a[5], a[6]);
+        const int rc = without_gil([&] {
+            const int bad = out.make(ci, (int64_t)kh * kw * co, c1.o.fmt, c1.data);
+            return bad ? bad : api.conv_dgrad_filters(c1.o.data, c1.o.exps, kh, kw, ci, co, &c1.o.fmt, out.m.data_ptr(), (int8_t*)out.e.data_ptr(), cur_stream());
+        });
         if (rc) return code(rc);
-        return Py_BuildValue("(NN)", THPVariable_Wrap(m), THPVariable_Wrap(e));
+        return Py_BuildValue("(NN)", THPVariable_Wrap(out.m), THPVariable_Wrap(out.e));
     });
 }
 
@@ -339,22 +383,16 @@ PyObject* im2col_packed_t(PyObject*, PyObject* const* a, Py_ssize_t n) {
         if (!(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 4 && x.is_contiguous()))
             value_error("%s must be a contiguous float32 CUDA tensor [n][h][w][c]", "x");
         const int kh = (int)as_ll(a[1]), kw = (int)as_ll(a[2]);
+        const int pad = (int)as_ll(a[3]);
         const hbfp_format f = format_of(a[4]);
-        at::Tensor m, e;
-        if (a[5] == Py_None) {
-            hbfp_layout L;
-            const int rc = api.packed_layout((int64_t)kh * kw * x.size(3), x.size(0) * x.size(1) * x.size(2), &f, &L);
-            if (rc) return code(rc);
-            m = empty_i8(L.mant_bytes, x);
-            e = empty_i8(L.exp_bytes, x);
-        } else {
-            m = tensor_of(a[5], "mantissas");
-            e = tensor_of(a[6], "exponents");
-        }
-        const int rc = api.im2col_packed_t((const float*)x.data_ptr(), x.size(0), x.size(1), x.size(2), x.size(3), kh, kw, (int)as_ll(a[3]), &f, m.data_ptr(),
-                                           (int8_t*)e.data_ptr(), cur_stream());
+        Buffers out(a[5], a[6]);
+        const int rc = without_gil([&] {
+            const int bad = out.make((int64_t)kh * kw * x.size(3), x.size(0) * x.size(1) * x.size(2), f, x);
+            return bad ? bad : api.im2col_packed_t((const float*)x.data_ptr(), x.size(0), x.size(1), x.size(2), x.size(3), kh, kw, pad, &f, out.m.data_ptr(),
+                                                   (int8_t*)out.e.data_ptr(), cur_stream());
+        });
         if (rc) return code(rc);
-        return Py_BuildValue("(NN)", THPVariable_Wrap(m), THPVariable_Wrap(e));
+        return Py_BuildValue("(NN)", THPVariable_Wrap(out.m), THPVariable_Wrap(out.e));
     });
 }
 
@@ -512,6 +550,7 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
         at::Tensor y;
         {
             Below guard;
+            NoGil free;
             const at::Tensor xc = x.contiguous();
             const at::Tensor bc = bias.defined() ? bias.contiguous() : bias;
             y = product(xc.size(0), proto.fout, proto.fin, fp32_operand(xc, 0, proto.act(0, false)), c0.operand(), xc, bc.defined() ? (const float*)bc.data_ptr() : nullptr);
@@ -630,6 +669,7 @@ PyObject* conv3x3(PyObject*, PyObject* const* a, Py_ssize_t n) {
         at::Tensor y;
         {
             Below guard;
+            NoGil free;
             y = node->forward(x.contiguous(), c0);
         }
         if (torch::autograd::compute_requires_grad(x, w)) {

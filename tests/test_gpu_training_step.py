@@ -364,3 +364,34 @@ def test_a_gradient_that_never_came_counts_as_zeros(env):
         Drop.apply(mod(x)).sum().backward()
         for t in (x, *mod.parameters()):
             assert t.grad.shape == t.shape and not t.grad.any()
+
+
+def test_other_threads_run_while_a_call_is_in_the_library(env):
+    """The interpreter lock is let go around the library: with entry points that only sleep (libc's usleep, whose argument is the
+    product's first extent) in place of the product's, another thread counts on meanwhile."""
+    import ctypes
+    import threading
+    torch, hbfp_nn, hb = env
+    native, L = hb.host(), hb.lib()
+    sleep = ctypes.cast(ctypes.CDLL(None).usleep, ctypes.c_void_p).value
+    entry = {n: ctypes.cast(getattr(L, n), ctypes.c_void_p).value for n in hb._HOST_ENTRY_POINTS}
+    p = hb.quantize(torch.randn(32, 32, device="cuda"), 1, hb.Format(8, 32))
+    out, count, stop = torch.empty(32, 32, device="cuda"), [0], threading.Event()
+
+    def counter():
+        while not stop.wait(0.01):
+            count[0] += 1
+
+    native.bind(hb.HbfpError, *({**entry, "hbfp_gemm_q_workspace": sleep, "hbfp_gemm_q_bias": sleep}[n] for n in hb._HOST_ENTRY_POINTS))
+    thread = threading.Thread(target=counter)
+    try:
+        thread.start()
+        before = count[0]
+        native.gemm_q(300000, 32, 32, p, p, 0, 0, None, None, out, None, 0)      # 0.6 s asleep in the library
+        during = count[0] - before
+    finally:
+        native.bind(hb.HbfpError, *(entry[n] for n in hb._HOST_ENTRY_POINTS))
+        stop.set()
+        thread.join()
+    assert during >= 10
+    assert torch.equal(hb.gemm_q(32, 32, 32, p, p), hb.gemm_q(32, 32, 32, p, p, flags=hb.GEMM_FORCE_SIMT))
