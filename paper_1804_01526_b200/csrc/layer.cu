@@ -99,21 +99,23 @@ column_sums_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
 
 template <int V>
 int column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, cudaStream_t st) {
-    const int64_t tiles = (cols + 32 * V - 1) / (32 * V);
-    if (tiles > 65535) return HBFP_ERR_UNSUPPORTED;
+    constexpr int64_t MOST = 65535ll * 32 * V;                    // columns a grid can have
     // a share of at least one round of loads, more CTAs than that only add to the exchange
     int splits = 1;
     while (splits < 8 && rows >= 2 * splits * CS_WARPS * CS_UNR) splits *= 2;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
-    cfg.gridDim = dim3(splits, (unsigned)tiles, 1);
     cfg.blockDim = dim3(32 * CS_WARPS, 1, 1);
     cfg.stream = st;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = splits; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = splits > 1 ? 1 : 0;
-    HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, column_sums_kernel<V>, x, rows, cols, ld, splits, out));
+    for (int64_t c0 = 0; c0 < cols; c0 += MOST) {
+        const int64_t n = cols - c0 < MOST ? cols - c0 : MOST;
+        cfg.gridDim = dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V)), 1);
+        HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, column_sums_kernel<V>, x + c0, rows, n, ld, splits, out + c0));
+    }
     return HBFP_OK;
 }
 

@@ -395,3 +395,15 @@ def test_other_threads_run_while_a_call_is_in_the_library(env):
         thread.join()
     assert during >= 10
     assert torch.equal(hb.gemm_q(32, 32, 32, p, p), hb.gemm_q(32, 32, 32, p, p, flags=hb.GEMM_FORCE_SIMT))
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 2097121), (130, 2097153), (3, 8388484)])
+def test_column_sums_of_more_columns_than_a_grid_has(env, rows, cols):
+    """A layer's bias gradient for any number of outputs (one and four columns per lane; rows + 1 additions at most)."""
+    import ctypes
+    torch, hbfp_nn, hb = env
+    x, out = torch.randn(rows, cols, device="cuda"), torch.full((cols + 1,), 7.0, device="cuda")
+    assert hb.lib().hbfp_column_sums(ctypes.c_void_p(x.data_ptr()), ctypes.c_int64(rows), ctypes.c_int64(cols), ctypes.c_int64(cols), ctypes.c_void_p(out.data_ptr()),
+                                     ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    d = x.double()
+    assert bool(((out[:-1].double() - d.sum(0)).abs() <= (rows + 1) * 2.0 ** -24 * d.abs().sum(0)).all()) and float(out[-1]) == 7.0
