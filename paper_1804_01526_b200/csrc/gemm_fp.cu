@@ -222,6 +222,19 @@ __device__ __forceinline__ bool fp_blocks(uint64_t (&acc2)[FpCfg<FORM, NCOL, BP,
     return true;
 }
 
+// Form S carries the scale in the operands, so that where sA + sB is above 107 single products or part sums can leave binary32
+// although the block's sum, after cancellation, would not. An infinity stays one (or becomes a NaN) through every later addition:
+// one look at the finished accumulators finds it (0 * x + 0 is 0 for finite x only).
+template <int NC>
+__device__ __forceinline__ bool fp_all_finite(const uint64_t (&acc2)[NC / 2]) {
+    uint64_t t[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+    for (int c = 0; c < NC / 2; ++c) t[c & 3] = ffma2(acc2[c], 0ull, t[c & 3]);
+    float lo, hi;
+    unpack2(fadd2(fadd2(t[0], t[1]), fadd2(t[2], t[3])), lo, hi);
+    return lo == 0.f && hi == 0.f;
+}
+
 // Stores the columns [gj0, gj0 + NC) of row gi: whole 32-byte sectors per lane where the pitch allows it.
 template <int NC>
 __device__ __forceinline__ void fp_store_rows(const uint64_t (&acc2)[NC / 2], const FpProblem& p, int gi, int gj0) {
@@ -484,6 +497,7 @@ gemm_fp_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 #pragma unroll
             for (int c = 0; c < NC / 2; ++c) acc2[c] = 0ull;
             const bool ok = fp_blocks<FORM, NCOL, BP, PAIR>(acc2, p, ra, nblk, col0, ring);
+            if (FORM == FORM_S && ok && !fp_all_finite<NC>(acc2)) atomicCAS(p.status, 0, STATUS_EXPONENT_RANGE);
             if constexpr (!PAIR) if (split) {
                 __syncwarp();
                 fp_split_sum<C::NOUT, NC, BIAS>(acc2, p, base, base_ptr, w, rank, quarter * 32 + lane, col0);

@@ -551,3 +551,25 @@ def test_few_rows_kernels_of_different_plans_run_on_two_streams(hb, first, secon
     assert hb.device_status() == 0
     for _, alone, outs, _ in work:
         assert all(torch.equal(o, alone) for o in outs)
+
+
+@pytest.mark.parametrize("M,N,K", [(128, 128, 256), (600, 520, 1700), (2304, 2176, 1760)])
+def test_scaled_operand_form_reports_products_beyond_binary32(hb, M, N, K):
+    """Products of 2^129 that cancel to 2^122 within a block, in one of its MMA steps or across two: the sum is representable, and the
+    kernel leaves it or records the status, on the way from FP32 operands and from packed ones."""
+    import torch
+    fa, fb = hb.Format(8, 32), hb.Format(8, 32, stream_id=1)
+    a, b = torch.zeros(M, K, device="cuda"), torch.zeros(K, N, device="cuda")
+    a[:, :32] = 127.0 * 2.0 ** 57
+    for k in (1, 16):
+        b.zero_()
+        b[0], b[k] = 127.0 * 2.0 ** 58, -126.0 * 2.0 ** 58
+        pa, pb = hb.quantize(a, 1, fa), hb.quantize(b, 0, fb)
+        want = hb.gemm_q(M, N, K, pa, pb, flags=hb.GEMM_FORCE_SIMT)
+        assert bool((want == 127.0 * 2.0 ** 115).all())
+        for call in (lambda: hb.gemm(0, 0, a, b, fa, fb, flags=hb.GEMM_FORCE_TENSOR), lambda: hb.gemm_q(M, N, K, pa, pb, flags=hb.GEMM_FORCE_TENSOR)):
+            got, rc = call(), hb.device_status_rc()[0]
+            assert rc == hb.ERR_EXPONENT_RANGE or (rc == hb.OK and torch.equal(got, want))
+    for scale in (2.0 ** 50, 2.0 ** -60):          # far inside the range nothing is recorded
+        hb.gemm(0, 0, torch.randn_like(a) * scale, torch.randn_like(b), fa, fb, flags=hb.GEMM_FORCE_TENSOR)
+        assert hb.device_status() == 0
