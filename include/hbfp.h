@@ -371,13 +371,16 @@ HBFP_API int hbfp_gemm_block_partials(int64_t M, int64_t N, int64_t K, const hbf
                                       const hbfp_operand* b, int32_t* P, uint32_t impl,
                                       void* stream);
 
-/* Host-only: name of the GEMM kernel that the calling thread's most recent hbfp_gemm, hbfp_gemm_q,
- * hbfp_gemm_static or hbfp_gemm_block_partials call launched ("gemm_tc2_kernel": two SMs per 256 x 256
- * tile; "gemm_tc_kernel": one SM per tile, and the floating-point operand forms; "gemm_simt_kernel"; "conv_fwd_kernel" after hbfp_conv_forward),
- * "" before the first launch. For
- * measurement scripts that must name the kernel they timed (the paper has no counterpart). The
- * string is static storage. */
+/* Host-only: kind of GEMM kernel that the calling thread's most recent hbfp_gemm, hbfp_gemm_q, hbfp_gemm_q_bias,
+ * hbfp_gemm_static or hbfp_gemm_block_partials call launched: "gemm_tc2_kernel" (two SMs per 256 x 256 tile),
+ * "gemm_tc_kernel" (the other tensor-core products, the floating-point operand forms among them), "gemm_skinny_kernel" (a few
+ * rows against packed weights), "gemm_small_kernel" (the smallest products), "gemm_simt_kernel"; "conv_fwd_kernel" after
+ * hbfp_conv_forward; "" before the first launch. hbfp_last_gemm_launch names the kernel itself: where it differs,
+ * "gemm_fp_kernel" (operand forms, one SM per tile), "gemm_fp_kernel/pair" (two SMs per tile), "gemm_fp_kernel/split" (K split
+ * over the SMs of a cluster) and "gemm_small_fused_kernel" (both FP32 operands converted in the product's launch). For
+ * measurement scripts that must name the kernel they timed (the paper has no counterpart). The strings are static storage. */
 HBFP_API const char* hbfp_last_gemm_kernel(void);
+HBFP_API const char* hbfp_last_gemm_launch(void);
 
 /* Synchronises the current device, then writes to *cycles (host) the length, in SM clock cycles, of the
  * most recent launch of the paired-SM GEMM kernel ("gemm_tc2_kernel") on that device: every CTA reads the

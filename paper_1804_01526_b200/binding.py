@@ -29,7 +29,7 @@ EXPORTS = [
     "hbfp_quantize_tiles", "hbfp_unpack", "hbfp_dequantize", "hbfp_gemm_workspace",
     "hbfp_gemm_q_workspace", "hbfp_gemm", "hbfp_gemm_q", "hbfp_gemm_q_bias", "hbfp_column_sums", "hbfp_gemm_block_partials",
     "hbfp_device_status", "hbfp_gemm_static", "hbfp_wide_quantize", "hbfp_wide_update", "hbfp_wide_update_value", "hbfp_wide_narrow",
-    "hbfp_im2col_packed", "hbfp_im2col_packed_t", "hbfp_wide_dequantize", "hbfp_selftest_bounded_wait", "hbfp_last_gemm_kernel", "hbfp_last_gemm_cycles", "hbfp_conv_forward", "hbfp_quantize_conv_weights", "hbfp_conv_dgrad_filters",
+    "hbfp_im2col_packed", "hbfp_im2col_packed_t", "hbfp_wide_dequantize", "hbfp_selftest_bounded_wait", "hbfp_last_gemm_kernel", "hbfp_last_gemm_launch", "hbfp_last_gemm_cycles", "hbfp_conv_forward", "hbfp_quantize_conv_weights", "hbfp_conv_dgrad_filters",
 ]
 
 
@@ -113,10 +113,11 @@ def lib() -> ctypes.CDLL:
         L.hbfp_wide_dequantize.argtypes = [p, p, i64, i64, i32, p, i64, p]
         L.hbfp_selftest_bounded_wait.argtypes = [i64, i32, p, p]
         L.hbfp_last_gemm_cycles.argtypes = [p]
-        L.hbfp_last_gemm_kernel.restype = ctypes.c_char_p
-        L.hbfp_last_gemm_kernel.argtypes = []
+        for fn in (L.hbfp_last_gemm_kernel, L.hbfp_last_gemm_launch):
+            fn.restype = ctypes.c_char_p
+            fn.argtypes = []
         for name in EXPORTS[1:]:
-            if name != "hbfp_last_gemm_kernel":
+            if name not in ("hbfp_last_gemm_kernel", "hbfp_last_gemm_launch"):
                 getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
@@ -468,8 +469,13 @@ def last_gemm_cycles() -> int:
 
 
 def last_gemm_kernel() -> str:
-    """hbfp_last_gemm_kernel: the GEMM kernel this thread's last GEMM call launched."""
+    """hbfp_last_gemm_kernel: the kind of GEMM kernel this thread's last GEMM call launched."""
     return lib().hbfp_last_gemm_kernel().decode()
+
+
+def last_gemm_launch() -> str:
+    """hbfp_last_gemm_launch: that kernel's own name."""
+    return lib().hbfp_last_gemm_launch().decode()
 
 
 def device_status() -> int:

@@ -34,8 +34,14 @@ int read_clear_device_status(cudaStream_t st, int32_t* out) {
 
 namespace {
 
-// Name of the GEMM kernel the calling thread's last hbfp_gemm* call launched (hbfp_last_gemm_kernel).
+// What the calling thread's last hbfp_gemm* call launched: the family's name (hbfp_last_gemm_kernel) and the kernel's own
+// (hbfp_last_gemm_launch).
 thread_local const char* t_last_gemm_kernel = "";
+thread_local const char* t_last_gemm_launch = "";
+void ran(const char* kernel, const char* launch = nullptr) {
+    t_last_gemm_kernel = kernel;
+    t_last_gemm_launch = launch ? launch : kernel;
+}
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -191,7 +197,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         rc = check_fp32(a, true, M, K);
         if (!rc) rc = check_fp32(b, false, N, K);
         if (rc) return rc;
-        t_last_gemm_kernel = "gemm_small_kernel";
+        ran("gemm_small_kernel", "gemm_small_fused_kernel");
         return launch_gemm_small_fused(M, N, K, a, k_contiguous(a, true), b, k_contiguous(b, false), g.la, C, ldc, st);
     }
     if (!P && flags == HBFP_GEMM_AUTO && a->kind == HBFP_OPERAND_FP32 && a->trans == 0 && a->fmt.tile == 0 &&
@@ -200,7 +206,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         if (rc) return rc;
         rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, st);
         if (rc) return rc;
-        t_last_gemm_kernel = "gemm_skinny_kernel";
+        ran("gemm_skinny_kernel");
         *bias_done = true;
         return launch_gemm_skinny(M, N, K, static_cast<const float*>(a->data), a->ld, &a->fmt, pb, bias, C, ldc, st);
     }
@@ -210,7 +216,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         if (rc) return rc;
         rc = resolve_form(b, false, N, K, g, ws, fb, st);
         if (rc) return rc;
-        t_last_gemm_kernel = "gemm_tc_kernel";      // one SM per tile, like its integer sibling
+        ran("gemm_tc_kernel", g.fp.pair ? "gemm_fp_kernel/pair" : g.fp.splits > 1 ? "gemm_fp_kernel/split" : "gemm_fp_kernel");
         *bias_done = true;
         return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, bias, C, ldc, st);
     }
@@ -219,7 +225,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, st);
     if (rc) return rc;
     if (small) {
-        t_last_gemm_kernel = "gemm_small_kernel";
+        ran("gemm_small_kernel");
         return launch_gemm_small(M, N, pa, pb, C, ldc, st);
     }
     const bool quad_rows = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (ldc % 4) == 0;
@@ -232,15 +238,15 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         const bool pair_ok = !P && quad_rows && flags != HBFP_GEMM_FORCE_TENSOR_1SM && pair_gemm_eligible(M, N, pa, pb, g.tp) &&
                              (long_k || flags == HBFP_GEMM_FORCE_TENSOR_2SM);
         if (pair_ok) {
-            t_last_gemm_kernel = "gemm_tc2_kernel";
+            ran("gemm_tc2_kernel");
             return launch_gemm_tensor_pair(M, N, pa, pb, C, ldc, g.tp, ws ? ws + g.off_partial : nullptr, st);
         }
         if (flags == HBFP_GEMM_FORCE_TENSOR_2SM) return HBFP_ERR_UNSUPPORTED;
-        t_last_gemm_kernel = "gemm_tc_kernel";
+        ran("gemm_tc_kernel");
         return launch_gemm_tensor(M, N, K, pa, pb, C, ldc, P, g.tp, ws ? ws + g.off_partial : nullptr, st);
     }
     if (flags >= HBFP_GEMM_FORCE_TENSOR) return HBFP_ERR_UNSUPPORTED;
-    t_last_gemm_kernel = "gemm_simt_kernel";
+    ran("gemm_simt_kernel");
     return launch_gemm_simt(M, N, K, pa, pb, C, ldc, P, st);
 }
 
@@ -265,6 +271,7 @@ using namespace hbfp;
 extern "C" {
 
 const char* hbfp_last_gemm_kernel(void) { return t_last_gemm_kernel; }
+const char* hbfp_last_gemm_launch(void) { return t_last_gemm_launch; }
 
 const char* hbfp_status_string(int status) {
     switch (status) {
@@ -423,7 +430,7 @@ int hbfp_conv_forward(const void* mant_x, const int8_t* exps_x, int64_t n, int64
     pw.exps = static_cast<const int8_t*>(filters_op->exps);
     pw.mant_bits = filters_op->fmt.mant_bits;
     if (n == 0) return HBFP_OK;
-    t_last_gemm_kernel = "conv_fwd_kernel";
+    ran("conv_fwd_kernel");
     return launch_conv_forward(px, pw, n, h, w, c, kh, kw, pad, filters, Y, ldy, static_cast<cudaStream_t>(stream));
 }
 

@@ -411,19 +411,20 @@ def test_last_gemm_cycles_reports_the_paired_kernel_length(hb):
 # The floating-point operand forms (gemm_fp.cu): short blocks of 8-bit mantissas, 9 to 12 bits; one SM or a pair per tile.
 # Edges of tiles in M and N, a last K stage with a single block, padded blocks, an output pitch that TMA cannot store.
 FP_FORM_CASES = [
-    # m, block, M, N, K, law
-    (8, 32, 2304, 2176, 1760, "lognormal"),
-    (8, 24, 2305, 2051, 1751, "lognormal"),
-    (8, 64, 2304, 2310, 1664, "normal"),
-    (6, 48, 2433, 2177, 1700, "lognormal"),
-    (12, 32, 2176, 2050, 1888, "outliers"),
-    (12, 64, 2433, 2303, 1600, "lognormal"),
-    (10, 40, 2177, 2052, 1990, "normal"),
+    # m, block, M, N, K, law, kernel
+    (8, 32, 2304, 2176, 1760, "lognormal", "gemm_fp_kernel"),
+    (8, 24, 2305, 2051, 1751, "lognormal", "gemm_fp_kernel"),
+    (8, 64, 2304, 2310, 1664, "normal", "gemm_fp_kernel"),
+    (8, 64, 2433, 3071, 1602, "lognormal", "gemm_fp_kernel/pair"),
+    (6, 48, 2433, 2177, 1700, "lognormal", "gemm_fp_kernel"),
+    (12, 32, 2176, 2050, 1888, "outliers", "gemm_fp_kernel"),
+    (12, 64, 2433, 2303, 1600, "lognormal", "gemm_fp_kernel/pair"),
+    (10, 40, 2177, 2052, 1990, "normal", "gemm_fp_kernel"),
 ]
 
 
-@pytest.mark.parametrize("m,b,M,N,K,law", FP_FORM_CASES)
-def test_floating_point_operand_forms_are_bit_equal_to_the_sequential_definition(hb, m, b, M, N, K, law):
+@pytest.mark.parametrize("m,b,M,N,K,law,kernel", FP_FORM_CASES)
+def test_floating_point_operand_forms_are_bit_equal_to_the_sequential_definition(hb, m, b, M, N, K, law, kernel):
     """Block sums are exact in every form and blocks are added in ascending order with one rounding each, so without
     split-K the result is the reference kernel's (gemm_simt, itself bit-equal to the oracle's c_seq) bit for bit;
     the largest mantissas everywhere give the largest block sums."""
@@ -436,9 +437,9 @@ def test_floating_point_operand_forms_are_bit_equal_to_the_sequential_definition
         buf = torch.full((M, N + 3), 7.0, device="cuda")
         for out in (None, buf[:, 1:1 + N]):
             got = hb.gemm(0, 0, X, Y, fa, fb, out=out)
-            assert hb.last_gemm_kernel() == "gemm_tc_kernel" and hb.device_status() == 0
+            assert hb.last_gemm_launch() == kernel and hb.device_status() == 0
             assert torch.equal(got, want)
-            assert torch.equal(hb.gemm_q(M, N, K, pa, pb, out=out), want)
+            assert torch.equal(hb.gemm_q(M, N, K, pa, pb, out=out), want) and hb.last_gemm_launch() == kernel
         assert bool((buf[:, 0] == 7).all()) and bool((buf[:, N + 1:] == 7).all())
 
 
@@ -453,6 +454,7 @@ def test_small_products_of_fp32_operands_converted_straight_to_the_form(hb, m, b
     B = to_dev(wl.draw("normal", (N, K) if tB else (K, N), seed=96))
     fa, fb = hb.Format(m, b, rounding=rounding, seed=6), hb.Format(m, b, rounding=rounding, seed=6, stream_id=1)
     C = hb.gemm(tA, tB, A, B, fa, fb, flags=hb.GEMM_FORCE_TENSOR)
+    assert hb.last_gemm_launch() == ("gemm_fp_kernel" if K < 256 else "gemm_fp_kernel/split")
     pa, pb = hb.quantize(A, 0 if tA else 1, fa), hb.quantize(B, 1 if tB else 0, fb)
     da, db = hb.dequantize(pa).double(), hb.dequantize(pb).double()
     assert hb.device_status() == 0
@@ -467,7 +469,7 @@ def test_contraction_split_over_clusters_of_any_size(hb, m, b, M, N, K):
     fa, fb = hb.Format(m, b), hb.Format(m, b, stream_id=1)
     C = hb.gemm(0, 0, A, B, fa, fb)
     da, db = (hb.dequantize(hb.quantize(x, ax, f)).double() for x, ax, f in ((A, 1, fa), (B, 0, fb)))
-    assert hb.device_status() == 0 and hb.last_gemm_kernel() == "gemm_tc_kernel"
+    assert hb.device_status() == 0 and hb.last_gemm_launch() == "gemm_fp_kernel/split"
     assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
 
 
@@ -486,7 +488,7 @@ def test_few_rows_against_packed_weights_in_one_launch(hb, M, N, K, m, t, roundi
     buf = torch.full((M, N + 3), 7.0, device="cuda")
     for out in (None, buf[:, 1:1 + N]):
         got = hb.gemm_q(M, N, K, X, c0, fmtA=fx, out=out)
-        assert hb.last_gemm_kernel() in ("gemm_skinny_kernel", "gemm_small_kernel") and hb.device_status() == 0
+        assert hb.last_gemm_launch() == "gemm_skinny_kernel" and hb.device_status() == 0
         assert bool(((got.double() - want).abs() <= TOL * mag + 1e-30).all())
     assert bool((buf[:, 0] == 7).all()) and bool((buf[:, N + 1:] == 7).all())
 
@@ -524,7 +526,9 @@ def test_small_products_of_fp32_operands_in_one_launch(hb, M, N, K, m, b, roundi
         if not fresh:
             want = hb.gemm_q(M, N, K, hb.quantize(X.contiguous(), 0 if tA else 1, fa), hb.quantize(B, 1 if tB else 0, fb), flags=hb.GEMM_FORCE_SIMT)
         got = hb.gemm(tA, tB, X, B, fa, fb)
-        assert hb.last_gemm_kernel() == "gemm_small_kernel" and hb.device_status() == 0
+        # draws down columns need whole groups of eight lines
+        fused = rounding == 0 or not ((tA and M % 8) or (not tB and N % 8))
+        assert hb.last_gemm_launch() == ("gemm_small_fused_kernel" if fused else "gemm_small_kernel") and hb.device_status() == 0
         assert torch.equal(got, want)
 
 
