@@ -577,3 +577,20 @@ def test_scaled_operand_form_reports_products_beyond_binary32(hb, M, N, K):
     for scale in (2.0 ** 50, 2.0 ** -60):          # far inside the range nothing is recorded
         hb.gemm(0, 0, torch.randn_like(a) * scale, torch.randn_like(b), fa, fb, flags=hb.GEMM_FORCE_TENSOR)
         assert hb.device_status() == 0
+
+
+@pytest.mark.parametrize("M,N,K", [(128, 10, 1024), (1024, 10, 128), (200, 137, 256), (300, 66, 96)])
+@pytest.mark.parametrize("b", [32, 128])
+def test_integer_tensor_core_kernel_writes_outputs_of_any_width(hb, M, N, K, b):
+    """The single-SM integer kernel at pitches that cannot take 16-byte stores (GEMM_FORCE_TENSOR goes to the operand forms where
+    blocks are short, this flag does not)."""
+    import torch
+    A, B = wl.draw("half_normal", (M, K), seed=61), wl.draw("he_weight", (K, N), seed=62, fan_in=K)
+    fd = dict(mant_bits=8, block=b, rounding=0, seed=0)
+    ref = oracle.hbfp_gemm(0, 0, A, B, ofmt(fd), ofmt(fd))
+    buf = torch.full((M, N + 7), -1.0, device="cuda")
+    for out in (None, buf[:, 3:3 + N]):
+        C = hb.gemm(0, 0, to_dev(A), to_dev(B), gfmt(fd), gfmt(fd), out=out, flags=hb.GEMM_FORCE_TENSOR_1SM).cpu().numpy()
+        assert hb.last_gemm_launch() == "gemm_tc_kernel" and hb.device_status() == 0
+        assert (np.abs(C.astype(np.float64) - ref["c_ref"].astype(np.float64)) <= TOL * ref["a_mag"]).all()
+    assert bool((buf[:, :3] == -1).all()) and bool((buf[:, 3 + N:] == -1).all())

@@ -77,13 +77,13 @@ def test_random_gemm_cases(hb, seed):
         fa = dict(mant_bits=m, block=b, rounding=int(rng.integers(0, 2)), seed=int(rng.integers(0, 1000)), stream_id=0)
         fb = dict(fa, stream_id=1)
         ref = oracle.hbfp_gemm(tA, tB, A, B, oracle.Format(**fa), oracle.Format(**fb))
-        for flags in (hb.GEMM_AUTO, hb.GEMM_FORCE_SIMT, hb.GEMM_FORCE_TENSOR, hb.GEMM_FORCE_SMALL):
+        for flags in (hb.GEMM_AUTO, hb.GEMM_FORCE_SIMT, hb.GEMM_FORCE_TENSOR, hb.GEMM_FORCE_TENSOR_1SM, hb.GEMM_FORCE_SMALL):
             try:
                 C = hb.gemm(tA, tB, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), hb.Format(**fa), hb.Format(**fb),
                             flags=flags).cpu().numpy()
             except hb.HbfpError as e:
                 # a forced kernel may not cover the format (two-plane operands on the small-problem kernel, ...)
-                assert e.code == hb.ERR_UNSUPPORTED and flags in (hb.GEMM_FORCE_TENSOR, hb.GEMM_FORCE_SMALL), (M, N, K, m, b, flags)
+                assert e.code == hb.ERR_UNSUPPORTED and flags in (hb.GEMM_FORCE_TENSOR, hb.GEMM_FORCE_TENSOR_1SM, hb.GEMM_FORCE_SMALL), (M, N, K, m, b, flags)
                 continue
             err = np.abs(C.astype(np.float64) - ref["c_ref"].astype(np.float64))
             assert (err <= 1e-6 * ref["a_mag"] + 1e-300).all(), (M, N, K, m, b, tA, tB, flags)
