@@ -778,7 +778,14 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, in
     // 13 / 15, 4096 cube 197 / 329.
     {
         const int64_t nout = w ? f.ncol / 2 : f.ncol, ctas = ((M + 127) / 128) * ((N + nout - 1) / nout) * f.splits;
+        const int64_t per = (nst + f.splits - 1) / f.splits;       // stages of a CTA
         if (ctas < 74 && nst / f.splits > 24) return FpPlan{};
+        // The narrowest tiles in eight splits say the same of shorter contractions: 128 x 200 x 10865 (b = 64) 22 against 18 us,
+        // 64 x 56 x 12416 (12 bits, b = 32) 27 against 20. With 104 CTAs and more the forms keep blocks of 32 (209 x 448 x 14464,
+        // 12 bits, 38 against 43) and lose long ones of 64, whose MMAs wait for operands: 208 x 384 x 52072 71 against 54.
+        if (f.ncol == (w ? 128 : 64) && f.splits == 8 && ((ctas < 104 && per >= 13) || (la.bp == 64 && per >= 28))) return FpPlan{};
+        // the same without a split, where the tiles alone occupy the chip: 1944 x 576 x 10752, b = 64, 96 against 84
+        if (f.ncol == (w ? 128 : 64) && la.bp == 64 && ctas < 148 && per >= 100) return FpPlan{};
     }
     // Blocks of 64 feed the tensor cores twice as fast as blocks of 32, and one SM's shared memory cannot deliver it: a stage
     // costs 48 KB written and 48 KB read (768 cycles) for 512 cycles of MMAs. A pair of SMs stages and reads a third less each

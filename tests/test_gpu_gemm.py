@@ -594,3 +594,14 @@ def test_integer_tensor_core_kernel_writes_outputs_of_any_width(hb, M, N, K, b):
         assert hb.last_gemm_launch() == "gemm_tc_kernel" and hb.device_status() == 0
         assert (np.abs(C.astype(np.float64) - ref["c_ref"].astype(np.float64)) <= TOL * ref["a_mag"]).all()
     assert bool((buf[:, :3] == -1).all()) and bool((buf[:, 3 + N:] == -1).all())
+
+
+@pytest.mark.parametrize("M,N,K,m,b", [(128, 200, 10865, 8, 64), (64, 56, 12416, 12, 32), (208, 384, 52072, 8, 64)])
+def test_few_tiles_with_a_long_contraction_take_the_integer_kernel(hb, M, N, K, m, b):
+    """More parts of K than a cluster has CTAs: split over the whole chip, and faster by a fifth to a third than the operand forms."""
+    A, B = to_dev(wl.draw("normal", (M, K), seed=131)), to_dev(wl.draw("normal", (K, N), seed=132))
+    fa, fb = hb.Format(m, b), hb.Format(m, b, stream_id=1)
+    C = hb.gemm(0, 0, A, B, fa, fb)
+    assert hb.last_gemm_launch() == "gemm_tc_kernel" and hb.device_status() == 0
+    da, db = hb.dequantize(hb.quantize(A, 1, fa)).double(), hb.dequantize(hb.quantize(B, 0, fb)).double()
+    assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
