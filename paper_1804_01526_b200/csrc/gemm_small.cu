@@ -351,6 +351,13 @@ bool small_fused_eligible(const hbfp_operand* a, bool a_contig, const hbfp_opera
     // (512 cube 18.6 against 10.7 us of device time; 512 x 512 x 256, two CTAs per SM, 10.5 against 14.3 as a call).
     const int64_t ctas = ((M + SM_TILE - 1) / SM_TILE) * ((N + SM_TILE - 1) / SM_TILE);
     if (la.nkb * la.bp > 256 && ctas > 148) return false;
+    // Draws are made again in every tile of a row of tiles: with more tiles than SMs or long columns on both sides two launches
+    // win (device time / as a call: 512 x 512 x 256 19.4 against 11.1, 20.7 / 16.3; 384 cube from columns 21.5 / 10.8, 22.7 / 16.5;
+    // 128 x 1792 x 209 18.4 against 12.1).
+    if (a->fmt.rounding || b->fmt.rounding) {
+        if (la.nkb * la.bp > 128 && ctas > 148) return false;
+        if (la.nkb * la.bp > 384 && ctas > 74 && !a_contig && !b_contig) return false;
+    }
     return (a_contig || a->fmt.rounding == 0 || M % 8 == 0) && (b_contig || b->fmt.rounding == 0 || N % 8 == 0);
 }
 

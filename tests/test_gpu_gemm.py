@@ -605,3 +605,15 @@ def test_few_tiles_with_a_long_contraction_take_the_integer_kernel(hb, M, N, K, 
     assert hb.last_gemm_launch() == "gemm_tc_kernel" and hb.device_status() == 0
     da, db = hb.dequantize(hb.quantize(A, 1, fa)).double(), hb.dequantize(hb.quantize(B, 0, fb)).double()
     assert bool(((C.double() - da @ db.t()).abs() <= TOL * (da.abs() @ db.abs().t()) + 1e-30).all())
+
+
+@pytest.mark.parametrize("M,N,K,tA,rounding,fused", [(512, 512, 256, 0, 1, False), (512, 512, 256, 0, 0, True), (512, 512, 128, 0, 1, True), (256, 448, 448, 1, 1, False), (256, 448, 448, 0, 1, True),
+                                                     (256, 256, 448, 1, 1, True), (256, 256, 256, 1, 1, True)])
+def test_small_products_with_draws_in_one_launch_or_three(hb, M, N, K, tA, rounding, fused):
+    """Where tiles repeat the draws too often the operands are converted on their own: the same bits either way."""
+    import torch
+    A, B = to_dev(wl.draw("normal", (K, M) if tA else (M, K), seed=141)), to_dev(wl.draw("normal", (K, N), seed=142))
+    fa, fb = hb.Format(8, 32, rounding=rounding, seed=4), hb.Format(8, 32, rounding=rounding, seed=4, stream_id=1)
+    got = hb.gemm(tA, 0, A, B, fa, fb)
+    assert hb.last_gemm_launch() == ("gemm_small_fused_kernel" if fused else "gemm_small_kernel") and hb.device_status() == 0
+    assert torch.equal(got, hb.gemm_q(M, N, K, hb.quantize(A, 0 if tA else 1, fa), hb.quantize(B, 0, fb), flags=hb.GEMM_FORCE_SIMT))
