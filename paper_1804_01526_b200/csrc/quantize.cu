@@ -88,8 +88,19 @@ quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
             for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
             const int s = given ? (r < rows ? (int)given[r] : -63) : block_exponent(am, p.m, p.exp_mode);
             const uint4 w = wd[i];
-            round_and_store8<SR, PLANES>(e8, s, p, w, mant, r * kst + col, plane_stride, r < rows && col < kst);
-            check_exponent<PLANES>(s, fa);
+            if constexpr (is_form(PLANES)) {
+                round_and_store8<SR, PLANES>(e8, s, p, w, mant, r * kst + col, plane_stride, r < rows && col < kst);
+                check_exponent<PLANES>(s, fa);
+            } else {
+                // written out: with the address formed before the branch, as the call above does, the kernel with draws no longer fits
+                // 80 registers and spills (4096 x 4096, b = 256: 18.8 -> 19.5 us)
+                uint2 hi, lo;
+                quantize_pack8<SR, PLANES>(e8, s, p, w, hi, lo);
+                if (r < rows && col < kst) {
+                    *reinterpret_cast<uint2*>(mant + r * kst + col) = hi;
+                    if (PLANES == 2) *reinterpret_cast<uint2*>(mant + plane_stride + r * kst + col) = lo;
+                }
+            }
             if ((lane % LPB) == 0 && r < rows && col < K)
                 s_exps[span * KB_PER_SPAN + lane / LPB][warp * 4 + i] = (int8_t)s;
         }
