@@ -1530,7 +1530,9 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
 
 // Whole-axis blocks down the columns (one exponent per column of the stored matrix): pass 1 of 2. Each CTA takes
 // 256 columns and a band of rows, reads rows coalesced and folds its band's maxima into one word per column. Bands of 128 rows
-// where that makes four CTAs per SM, otherwise of 32: a thread's loads leave eight at a time.
+// where that makes four CTAs per SM, otherwise of 32: a thread's loads leave eight at a time. Every band adds an atomic per column,
+// and thousands of them on the words of few columns take longer than the loads: 65536 x 64 14.9 us with bands of 128, 19.3 of 32;
+// 65536 x 200 26.9 / 35.3, 16384 x 512 16.7 / 18.6, but 12000 x 300 20.4 / 18.4, 16384 x 1000 26.8 / 24.8, 8192 x 64 12.4 / 10.4.
 constexpr int CMAX_ROWS = 128, CMAX_ROWS_SHORT = 32;
 __global__ void __launch_bounds__(256)
 col_amax_kernel(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int band, uint32_t* __restrict__ amax) {
@@ -1719,7 +1721,8 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         uint32_t* amax = reinterpret_cast<uint32_t*>(mant);
         HBFP_CUDA_OK(cudaMemsetAsync(amax, 0, (size_t)rows * 4, st));
         const int64_t wide = (rows + 255) / 256;
-        const int band = wide * ((K + CMAX_ROWS - 1) / CMAX_ROWS) >= 4 * 148 || K > 65535ll * CMAX_ROWS_SHORT ? CMAX_ROWS : CMAX_ROWS_SHORT;
+        const bool idle = wide * ((K + CMAX_ROWS - 1) / CMAX_ROWS) < 4 * 148;
+        const int band = idle && (K <= 12288 || (K <= 20480 && wide >= 3)) ? CMAX_ROWS_SHORT : CMAX_ROWS;
         col_amax_kernel<<<dim3((unsigned)wide, (unsigned)((K + band - 1) / band)), 256, 0, st>>>(x, K, rows, ld, band, amax);
         col_exps_kernel<<<(unsigned)wide, 256, 0, st>>>(amax, rows, p, exps);
         if (launch_status()) return HBFP_ERR_CUDA;
