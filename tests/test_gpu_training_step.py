@@ -230,23 +230,25 @@ def test_bias_added_by_the_product_and_its_gradient(env, batch, fin, fout, m, t)
 
 def test_out_of_memory_keeps_its_type(env):
     """A caller that catches torch.OutOfMemoryError to shrink a batch finds it out of the calls and the layers (the allocator's limit
-    for this process is lowered; the GPU has room)."""
+    for this process is lowered; the GPU has room). Results of gigabytes from operands of megabytes, so that nothing the allocator
+    still holds from elsewhere could serve them."""
     torch, hbfp_nn, hb = env
-    A, fmt = torch.randn(6000, 6000, device="cuda"), hb.Format(8, 64)
-    layer, x = hbfp_nn.HbfpLinear(64, 6000, rounding=0), torch.randn(60000, 64, device="cuda")
-    conv, xc = hbfp_nn.HbfpConv3x3(64, 64), torch.randn(64, 32, 32, 64, device="cuda")
+    A, fmt = torch.randn(40000, 8, device="cuda"), hb.Format(8, 64)
+    layer, x = hbfp_nn.HbfpLinear(64, 6000, rounding=0), torch.randn(200000, 64, device="cuda")
+    conv, xc = hbfp_nn.HbfpConv3x3(64, 8192), torch.randn(64, 32, 32, 64, device="cuda")
+    long = torch.randn(10000000, 1, device="cuda")
     px = hb.quantize(xc.view(-1, 64), 1, conv.fmt_pixels(0))
     total = torch.cuda.get_device_properties(0).total_memory
     torch.cuda.empty_cache()
     torch.cuda.set_per_process_memory_fraction((torch.cuda.memory_reserved() + (8 << 20)) / total)
     try:
-        for call in (lambda: hb.gemm(0, 0, A, A, fmt, fmt), lambda: hb.quantize(A, 0, hb.Format(12, 64)), lambda: layer(x), lambda: conv(xc),
+        for call in (lambda: hb.gemm(0, 1, A, A, fmt, fmt), lambda: hb.quantize(long, 1, hb.Format(12, 64)), lambda: layer(x), lambda: conv(xc),
                      lambda: hb.conv_forward(px, conv.views[0], 64, 32, 32, 64, 3, 3, 1)):
             with pytest.raises(torch.OutOfMemoryError):
                 call()
     finally:
         torch.cuda.set_per_process_memory_fraction(1.0)
-    assert layer(x).shape == (60000, 6000)
+    assert layer(x[:60000]).shape == (60000, 6000)
 
 
 def test_inputs_of_the_wrong_width_do_not_train(env):
