@@ -2091,7 +2091,7 @@ wide_dequant_kernel(const int16_t* __restrict__ wide, const int8_t* __restrict__
     if (c >= d1) return;
     const int64_t tc = d1 < (1ll << 31) ? (int64_t)((uint32_t)c / (uint32_t)t) : c / t;
     for (int64_t r0 = (int64_t)blockIdx.y * ROWS; r0 < d0; r0 += (int64_t)gridDim.y * ROWS) {
-        const int64_t tr = r0 / t;
+        const int64_t tr = d0 < (1ll << 31) ? (int64_t)((uint32_t)r0 / (uint32_t)t) : r0 / t;
         const int r_in = (int)(r0 - tr * t);
         uint2 q[ROWS] = {};
         int e[ROWS] = {};
@@ -2101,7 +2101,8 @@ wide_dequant_kernel(const int16_t* __restrict__ wide, const int8_t* __restrict__
                 const int16_t* at = wide + (r0 + i) * d1 + c;
                 if (V == 4) q[i] = *reinterpret_cast<const uint2*>(at);
                 else q[i].x = (uint16_t)*at;
-                e[i] = exps[(tr + (uint32_t)(r_in + i) / (uint32_t)t) * tiles1 + tc];
+                // V = 4: tiles of whole groups of four rows, the four have one exponent
+                e[i] = exps[(V == 4 ? tr : tr + (uint32_t)(r_in + i) / (uint32_t)t) * tiles1 + tc];
             }
 #pragma unroll
         for (int i = 0; i < ROWS; ++i)

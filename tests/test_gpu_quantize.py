@@ -115,6 +115,9 @@ COL_WHOLE_AXIS_CASES = [
     ((2048, 1000), "outliers", F(8, 0, exp_mode=1)),                        # several bands of rows per column
     ((384, 72), "grad", F(12, 0, rounding=1, seed=2)),                      # two planes
     ((256, 8), "normal", F(4, 0)),                                          # eight output rows
+    ((12288, 24), "normal", F(8, 0)),                                       # the longest columns that take short bands of rows
+    ((12300, 24), "lognormal", F(8, 0, rounding=1, seed=5)),                # the shortest that do not
+    ((16384, 520), "normal", F(8, 0)),                                      # unless there are many of them
 ]
 
 
