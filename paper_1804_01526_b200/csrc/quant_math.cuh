@@ -271,11 +271,14 @@ __device__ __forceinline__ int quantize_one(float x, int s, const QParams& p, ui
     return round_sr(x, s, p.qmax, draw_of_element(p, L));
 }
 
-// Exponent bytes of the lines beyond the matrix (rows .. rs of every block) are documented as zero: written by the first CTA.
+// Exponent bytes of the lines beyond the matrix (rows .. rs of every block, at most fifteen) are documented as zero: written by all
+// CTAs, sixteen threads per block. (By the first CTA alone a 57 x 52416 operand's 11 000 bytes took 4 us.)
 __device__ __forceinline__ void zero_padding_lines(int8_t* exps, int64_t rows, int64_t rs, int64_t nkb) {
-    if (rs == rows || blockIdx.x != 0) return;
-    const int pad = (int)(rs - rows);
-    for (int64_t i = threadIdx.x; i < nkb * pad; i += blockDim.x) exps[(i / pad) * rs + rows + i % pad] = 0;
+    if (rs == rows) return;
+    const int64_t line = rows + (threadIdx.x & 15);
+    if (line >= rs) return;
+    const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 4);
+    for (int64_t kb = (int64_t)blockIdx.x * (blockDim.x >> 4) + (threadIdx.x >> 4); kb < nkb; kb += step) exps[kb * rs + line] = 0;
 }
 
 QParams make_params(const hbfp_format* f) {

@@ -326,3 +326,18 @@ def test_one_exponent_per_column_of_any_length(hb, K, cols, m, rounding):
         p = hb.quantize(X, 0, gfmt(fd))
         q, s = decode_packed(p, hb.packed_layout(cols, K, p.fmt))
         assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
+
+
+@pytest.mark.parametrize("rows,K,b", [(1, 52416, 32), (57, 52416, 32), (33, 20003, 24), (15, 64, 64), (17, 300, 48)])
+def test_exponents_of_lines_beyond_the_matrix_are_zero(hb, rows, K, b):
+    """Few rows with many blocks: the padding of every block's exponent line (decode_packed looks at each byte), in buffers that
+    held something else."""
+    import torch
+    x = wl.draw("normal", (rows, K), seed=33)
+    p = hb.alloc_packed(rows, K, hb.Format(8, b))
+    p.mant.fill_(77)
+    p.exps.fill_(77)
+    hb.quantize(torch.from_numpy(x).cuda(), 1, hb.Format(8, b), out=p)
+    q, s = decode_packed(p, hb.packed_layout(rows, K, p.fmt))
+    q_ref, s_ref = oracle.quantize(x, 1, oracle.Format(mant_bits=8, block=b))
+    assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
