@@ -3,7 +3,9 @@
 
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
+#include <utility>
 
 namespace hbfp {
 
@@ -49,9 +51,10 @@ struct GemmPlan {
     Layout la, lb;
     size_t off_am, off_ae, off_bm, off_be, off_partial, total;
     TensorPlan tp;
-    // the floating-point operand forms (gemm_fp.cu) lie behind the packed operands: A, then B
+    // A call on the floating-point operand forms (gemm_fp.cu) uses the same memory in another way: the forms of A and B, then a
+    // packed place for an FP32 operand that cannot be converted straight to its form (weight tiles).
     FpPlan fp;
-    size_t off_fa, off_fb, total_fp;
+    size_t off_fa, off_fb, off_fm, off_fe, total_fp;
 };
 
 size_t fp_plane_bytes(const Layout& L) { return align_up(2 * (size_t)(L.rows * L.kst), 1024); }
@@ -98,11 +101,20 @@ int make_plan(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     // operands that need a pass of their own to take the form
     const int passes = (a->kind != HBFP_OPERAND_FP32 || a->fmt.tile != 0) + (b->kind != HBFP_OPERAND_FP32 || b->fmt.tile != 0);
     g->fp = plan_gemm_fp(M, N, g->la, g->lb, passes);
-    g->off_fa = off;
-    if (g->fp.use) off += fp_bytes(g->la, g->fp, false);
-    g->off_fb = off;
-    if (g->fp.use) off += fp_bytes(g->lb, g->fp, true);
-    g->total_fp = off;
+    g->off_fa = g->off_fb = g->off_fm = g->off_fe = g->total_fp = 0;
+    if (g->fp.use) {
+        g->off_fb = fp_bytes(g->la, g->fp, false);
+        g->off_fm = g->off_fb + fp_bytes(g->lb, g->fp, true);
+        // one place: B is packed after A has been expanded
+        size_t mant = 0, exps = 0;
+        for (const auto& x : {std::make_pair(a, &g->la), std::make_pair(b, &g->lb)})
+            if (x.first->kind == HBFP_OPERAND_FP32 && x.first->fmt.tile != 0) {
+                mant = std::max(mant, align_up((size_t)x.second->mant_bytes, 1024));
+                exps = std::max(exps, align_up((size_t)x.second->exp_bytes, 1024));
+            }
+        g->off_fe = g->off_fm + mant;
+        g->total_fp = g->off_fe + exps;
+    }
     return HBFP_OK;
 }
 
@@ -155,12 +167,12 @@ int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, cons
         const int rc = check_fp32(o, is_a, rows, K);
         if (rc) return rc;
         const float* x = static_cast<const float*>(o->data);
-        const int done = k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, f, st)
-                                               : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, f, st);
-        if (done != HBFP_ERR_UNSUPPORTED) return done;
+        if (o->fmt.tile == 0)          // always covered where plan_gemm_fp takes the forms; a packed place is not reserved for these
+            return k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, f, st)
+                                         : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, f, st);
     }
     Packed p;
-    const int rc = is_a ? resolve_operand(o, true, rows, K, g.la, ws, g.off_am, g.off_ae, &p, st) : resolve_operand(o, false, rows, K, g.lb, ws, g.off_bm, g.off_be, &p, st);
+    const int rc = resolve_operand(o, is_a, rows, K, is_a ? g.la : g.lb, ws, g.off_fm, g.off_fe, &p, st);
     if (rc) return rc;
     return launch_expand(p, g.fp, !is_a, f, st);
 }

@@ -745,7 +745,10 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, in
     const bool w = la.planes == 2;
     // blocks of 128: the integer kernels are as fast (8 bits) or faster (12 bits, 4096 cube: 230 against 310 us)
     if (la.bp > 64) return f;
+    // (within what launch_quantize_form covers, so that a conversion straight to the form is never refused)
     if (M > (1ll << 28) || N > (1ll << 28) || la.kst > (1ll << 29)) return f;
+    const int64_t lines = M > N ? M : N;
+    if (lines * (la.kst / 8) >= (1ll << 39) || ((lines + 31) / 32) * la.nkb >= (1ll << 31)) return f;
     // Packed operands cost a pass each to take the form. It pays where every element is used often enough and the product is
     // large (all with both passes): 2048 cube 34 against 51 us (8 bits, b = 32), 27 against 31 (b = 64), 48 against 58 (12 bits,
     // b = 64), 4096 cube 186 / 290, 123 / 159, 261 / 368; but 1024 x 1024 x 2048 20 / 20, 18 / 14 and 24 / 18 us.

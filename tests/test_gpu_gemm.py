@@ -617,3 +617,19 @@ def test_small_products_with_draws_in_one_launch_or_three(hb, M, N, K, tA, round
     got = hb.gemm(tA, 0, A, B, fa, fb)
     assert hb.last_gemm_launch() == ("gemm_small_fused_kernel" if fused else "gemm_small_kernel") and hb.device_status() == 0
     assert torch.equal(got, hb.gemm_q(M, N, K, hb.quantize(A, 0 if tA else 1, fa), hb.quantize(B, 0, fb), flags=hb.GEMM_FORCE_SIMT))
+
+
+@pytest.mark.parametrize("m,b,tiles", [(8, 32, (0, 0)), (8, 64, (0, 1)), (12, 64, (1, 0)), (8, 32, (1, 1)), (12, 32, (1, 1))])
+def test_operand_forms_stay_inside_the_workspace_they_ask_for(hb, m, b, tiles):
+    """Operands converted straight to their form and, with weight tiles, by way of packed copies that share one place: the reference
+    kernel's bits, and the bytes behind the workspace untouched."""
+    import torch
+    M, N, K = 2433, 2177, 1700
+    A, B = to_dev(wl.draw("lognormal", (M, K), seed=151)), to_dev(wl.draw("normal", (K, N), seed=152))
+    fa, fb = (hb.Format(m, b, tile=b * t, rounding=1, seed=2, stream_id=k) for k, t in enumerate(tiles))
+    need = hb.gemm_workspace(0, 0, M, N, K, fa, fb)
+    ws = torch.full((need + 4096,), 55, dtype=torch.int8, device="cuda")
+    got = hb.gemm(0, 0, A, B, fa, fb, workspace=ws[:need])
+    assert hb.last_gemm_launch().startswith("gemm_fp_kernel") and hb.device_status() == 0
+    assert bool((ws[need:] == 55).all())
+    assert torch.equal(got, hb.gemm_q(M, N, K, hb.quantize(A, 1, fa), hb.quantize(B, 0, fb), flags=hb.GEMM_FORCE_SIMT))

@@ -74,3 +74,16 @@ def test_workspace_query_is_host_only_and_monotone(hb):
     assert 0 < w1 <= w2
     with pytest.raises(hb.HbfpError):           # blocks of the operands must coincide
         hb.gemm_workspace(0, 0, 128, 128, 256, hb.Format(8, 32), hb.Format(8, 64))
+
+
+@pytest.mark.parametrize("m,b", [(8, 32), (8, 64), (12, 32), (12, 64)])
+def test_workspace_holds_what_one_route_uses(hb, m, b):
+    """A product on operand forms takes no packed copies beside them: the larger of the two routes' needs and no more (12 bits: one
+    plane of A, two of B, and the scales)."""
+    n = 4096
+    f = hb.Format(m, b)
+    packed = 2 * sum(hb.packed_sizes(n, n, f))
+    forms = (2 + 2 if m <= 8 else 2 + 4) * n * n + (2 * 4 * n * (n // b) if m > 8 else 0)
+    assert hb.gemm_workspace(0, 0, n, n, n, f, f) == max(packed, forms)
+    tiles = hb.Format(m, b, tile=b)                       # weight tiles are packed first
+    assert max(packed, forms) <= hb.gemm_workspace(0, 0, n, n, n, f, tiles) <= forms + sum(hb.packed_sizes(n, n, f)) + 4096
