@@ -1443,7 +1443,11 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
             v[j + 1] = tile[(q * 32 + j + 1) * QC_COLS + n];
             am = max3_abs_bits(am, v[j], v[j + 1]);
         }
-        if (LB < 2) pmax[q * QC_COLS + n] = am;
+        // Blocks of 32 need no exchange of maxima; they are stored all the same, because a thread may reach the barrier only when its
+        // loads of the tile have returned. Without a value that depends on them before it, a warp's loads could still wait in the load
+        // unit's queue while the copy engine, which that queue does not order, filled the stage again: about one product in a
+        // hundred at 1024 x 4096 x 4096 had 32 columns of mantissas from the next tile.
+        pmax[q * QC_COLS + n] = am;
         // the packed tile of the previous iteration must have left shared memory before it is rewritten
         if (tid == 0 && stores_pending) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         __syncthreads();

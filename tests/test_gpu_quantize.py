@@ -341,3 +341,25 @@ def test_exponents_of_lines_beyond_the_matrix_are_zero(hb, rows, K, b):
     q, s = decode_packed(p, hb.packed_layout(rows, K, p.fmt))
     q_ref, s_ref = oracle.quantize(x, 1, oracle.Format(mant_bits=8, block=b))
     assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
+
+
+@pytest.mark.parametrize("b,m", [(32, 8), (32, 12), (64, 8), (128, 8)])
+def test_streaming_column_quantiser_gives_the_same_bytes_every_time(hb, b, m):
+    """Five or six CTAs per SM read their tiles while the copy engine fills others: hundreds of conversions of one matrix, and of
+    products that convert down both operands' columns, bit by bit."""
+    import torch
+    x = torch.randn(4096, 4096, device="cuda")
+    f = hb.Format(m, b)
+    want = hb.quantize(x, 0, f)
+    got = hb.alloc_packed(4096, 4096, f)
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(300):
+        hb.quantize(x, 0, f, out=got)
+        wrong += (got.mant != want.mant).sum() + (got.exps != want.exps).sum()
+    a = x[:, :1024].contiguous()
+    first = hb.gemm(1, 0, a, x, f, f)
+    for _ in range(300):
+        wrong += (hb.gemm(1, 0, a, x, f, f) != first).sum()
+    ref = hb.gemm_q(1024, 4096, 4096, hb.quantize(a, 0, f), want, flags=hb.GEMM_FORCE_SIMT)
+    assert int(wrong) == 0 and hb.device_status() == 0
+    assert bool(((first - ref).abs() <= 2e-5 * ref.abs().max()).all())
