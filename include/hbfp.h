@@ -264,10 +264,11 @@ typedef struct hbfp_operand {
     hbfp_format fmt;    /* FP32: format to quantise to. PACKED: format it was quantised with         */
 } hbfp_operand;
 
-#define HBFP_GEMM_AUTO 0u        /* smallest problems: tiled kernel; else a tensor-core kernel when it supports the case, else SIMT */
+#define HBFP_GEMM_AUTO 0u        /* smallest problems: tiled kernel; a few rows against packed weights: a kernel of their own;
+                                    else a tensor-core kernel when it supports the case, else SIMT */
 #define HBFP_GEMM_FORCE_SIMT 1u  /* plain dp4a kernel (reference path, any format)           */
 #define HBFP_GEMM_FORCE_TENSOR 2u /* tcgen05 kernel or HBFP_ERR_UNSUPPORTED                  */
-#define HBFP_GEMM_FORCE_TENSOR_1SM 3u  /* as FORCE_TENSOR, but never the paired-SM tile kernel */
+#define HBFP_GEMM_FORCE_TENSOR_1SM 3u  /* the single-SM integer kernel: neither pairs of SMs nor the operand forms */
 #define HBFP_GEMM_FORCE_TENSOR_2SM 4u  /* paired-SM tile kernel or HBFP_ERR_UNSUPPORTED        */
 #define HBFP_GEMM_FORCE_SMALL 5u       /* the tiled kernel that HBFP_GEMM_AUTO takes for the smallest problems (contraction
                                           of at most 512 bytes, at most 296 tiles of 32 x 32; one launch, no split-K,
@@ -286,7 +287,10 @@ HBFP_API int hbfp_gemm_q_workspace(int64_t M, int64_t N, int64_t K, const hbfp_o
  * A: FP32 [M][K] (transA = 0) or [K][M] (transA = 1), row stride lda; B: FP32 [K][N] (transB =
  * 0) or [N][K] (transB = 1), row stride ldb; C: FP32 [M][N], row stride ldc, overwritten.
  * Both operands are first quantised along the contraction axis (fmtA, fmtB; their blocks must
- * coincide) into `workspace` (>= hbfp_gemm_workspace bytes, 256-byte aligned).
+ * coincide) into `workspace` (256-byte aligned). hbfp_gemm_workspace bytes let the call take its fastest kernel. Less is
+ * accepted down to the packed copies of the FP32 operands and the split-K parts of the integer kernels
+ * (HBFP_ERR_WORKSPACE below that); the call then takes those kernels, and where they or the operand forms split K the
+ * order of the FP32 additions, hence the last bits of C, differ with the workspace.
  * forward Y = X W is (0,0); backward-data dX = dY W^T is (0,1); backward-weight dW = X^T dY is
  * (1,0). Without split-K the blocks are accumulated in ascending order with one FP32 rounding
  * each; with split-K (chosen for small C and long K) each split does so and the splits are
@@ -295,7 +299,9 @@ HBFP_API int hbfp_gemm_q_workspace(int64_t M, int64_t N, int64_t K, const hbfp_o
  * 2^(sA + sB) into two factors and need more: the paired-SM kernel chooses the split per K-block and
  * 128-row tile and fails only when that tile's row exponents span more than 104 within one block
  * (or the products leave binary32); the single-SM kernel's biased path needs sA <= 103 (|A| < 2^110
- * at 8-bit mantissas; sA <= 96 for 12-bit mantissas). A kernel that meets exponents outside its range does not depart silently: it
+ * at 8-bit mantissas; sA <= 96 for 12-bit mantissas); the operand forms need sA <= 96 at 9 to 12 bits and, up to
+ * 8 bits, no product or part of a block's sum beyond binary32 (sA + sB <= 107 suffices); the kernel for a few rows
+ * against packed weights needs sB <= 104. A kernel that meets exponents outside its range does not depart silently: it
  * records a code in the device status word (hbfp_device_status then returns
  * HBFP_ERR_EXPONENT_RANGE) and the values of C it wrote for that call are unspecified;
  * HBFP_GEMM_FORCE_SIMT computes the same product without the restriction. */
@@ -312,10 +318,10 @@ HBFP_API int hbfp_gemm(int transA, int transB, int64_t M, int64_t N, int64_t K, 
  * program's memory discipline - a plug-in whose host framework has taken the whole device for
  * its own pool, so that a cudaMalloc from the plug-in fails; a serving or real-time loop in which
  * an allocation is forbidden because it may synchronise the device and stall every stream.
- * Same arguments and result as hbfp_gemm, minus the workspace: the packed operands and the split-K
- * partial tiles live in a fixed HBFP_STATIC_WORKSPACE_BYTES array in device memory that belongs to
+ * Same arguments as hbfp_gemm, minus the workspace, and the result of hbfp_gemm with a workspace of the array's size
+ * (see there): the packed operands and the split-K partial tiles live in a fixed HBFP_STATIC_WORKSPACE_BYTES array in device memory that belongs to
  * the library (every GPU that loads the library holds it until the process exits). The call
- * allocates and frees nothing. Problems whose hbfp_gemm_workspace() exceeds the array are
+ * allocates and frees nothing. Problems whose packed operands and split-K parts exceed the array are
  * rejected with HBFP_ERR_STATIC_LIMIT and nothing is launched (at 8-bit mantissas roughly
  * M*K + N*K <= 15 million elements, e.g. every GEMM of the 784-1024-1024-10 MLP at batch 128).
  * The first call on each device looks up the array's device address (cudaGetSymbolAddress, with
@@ -357,8 +363,8 @@ HBFP_API int hbfp_column_sums(const float* x, int64_t rows, int64_t cols, int64_
  * zero mantissas): the packed im2col operand of hbfp_im2col_packed is never formed. The result equals
  * hbfp_gemm_q on that operand bit for bit (taps accumulated in ascending order, one FP32 rounding each).
  * Y: FP32, 16-byte aligned, row stride ldy >= filters, ldy % 4 == 0. Supported: blocks of 64 or 128
- * channels (c itself, or c = 2 to 4 whole blocks, then K-blocks run tap by tap, block by block), mantissas up to 8 bits, w in {16, 32, 64, 128}, h a multiple of 128 / w, up to 256 filters, at most 36 K-blocks; any
- * other case returns HBFP_ERR_UNSUPPORTED and leaves Y untouched (use hbfp_im2col_packed + hbfp_gemm_q).
+ * channels (c itself, or c = 2 to 4 whole blocks, then K-blocks run tap by tap, block by block), mantissas up to 8 bits,
+ * w in {16, 32, 64, 128}, h a multiple of 128 / w, up to 256 filters, at most 36 K-blocks; any other case returns HBFP_ERR_UNSUPPORTED and leaves Y untouched (use hbfp_im2col_packed + hbfp_gemm_q).
  * Exponent range as for the paired-SM GEMM (hbfp_gemm). Asynchronous on `stream`, allocates nothing. */
 HBFP_API int hbfp_conv_forward(const void* mant_x, const int8_t* exps_x, int64_t n, int64_t h, int64_t w, int64_t c,
                                int kh, int kw, int pad, const hbfp_format* fmt_x, const hbfp_operand* filters_op,

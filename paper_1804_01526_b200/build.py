@@ -22,6 +22,7 @@ EXTRA_OBJECTS = [("quantize_tiles_small.o", "quantize.cu", ["-DHBFP_QUANT_PART=2
 # 8.57 M against 8.86 M at the default level, and 12 % / 9 % fewer cycles for blocks of 64 / 32; the other files were
 # measured too and are a toss-up kernel by kernel (single-SM GEMM: 8-bit + 9 %, 12-bit - 6 %), so they keep the default.
 EXTRA_FLAGS = {"gemm_tc2.cu": ["-Xptxas", "-O1"],
+               # 4096 cube, 8 bits: b = 32 260 -> 200 us, b = 64 160 -> 141; 12 bits: b = 64 275 -> 271, b = 32 455 -> 473
                "gemm_fp.cu": ["-Xptxas", "-O1"],
                "gemm_conv.cu": ["-Xptxas", "-O1"]}      # 128-channel forward 16.0 -> 15.0 us, 64-channel unchanged
 
