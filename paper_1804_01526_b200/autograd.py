@@ -27,10 +27,10 @@ import torch
 from . import binding as hb
 
 
-def _own(layer, cls, name: str) -> bool:
-    """Whether ``layer`` uses the method of ``cls`` itself: the compiled passes make these formats themselves, a layer that
-    overrides one takes its Python function."""
-    return getattr(type(layer), name) is getattr(cls, name) and name not in layer.__dict__
+def _own(layer, cls, *names: str) -> bool:
+    """Whether the class of ``layer`` has these methods from ``cls``: the compiled passes make the formats themselves, a layer that
+    overrides one (in its class or on its own) takes its Python function."""
+    return all(getattr(type(layer), name) is getattr(cls, name) for name in names)
 
 
 class _HbfpLinearFn(torch.autograd.Function):
@@ -101,7 +101,7 @@ class HbfpLinear(torch.nn.Module):
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         y = None
-        if _own(self, HbfpLinear, "fmt_act"):
+        if (type(self) is HbfpLinear or _own(self, HbfpLinear, "fmt_act")) and "fmt_act" not in self.__dict__:
             y = hb.host().linear(x, self.weight, self.bias, self.views[0], self.views[1], self.mant_bits, self.tile, self.batch_block,
                                  self.rounding, self.seed + self.steps, self.stream_id)
         return y if y is not None else _HbfpLinearFn.apply(x, self.weight, self.bias, self)
@@ -196,6 +196,6 @@ class HbfpConv3x3(torch.nn.Module):
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
         y = None
-        if _own(self, HbfpConv3x3, "fmt_pixels") and _own(self, HbfpConv3x3, "fmt_batch"):
+        if (type(self) is HbfpConv3x3 or _own(self, HbfpConv3x3, "fmt_pixels", "fmt_batch")) and not {"fmt_pixels", "fmt_batch"} & self.__dict__.keys():
             y = hb.host().conv3x3(x, self.weight, self.views[0], self.views[1], self.mant_bits, self.pixel_block, self.c, self.fout)
         return y if y is not None else _HbfpConv3x3Fn.apply(x, self.weight, self)

@@ -476,11 +476,13 @@ at::Tensor product(int64_t M, int64_t N, int64_t K, const hbfp_operand& a, const
 // Whether a pass runs under something that has to see an autograd.Function to record, transform or refuse it: a trace, a functorch
 // transform, an input with a forward-mode tangent. A node of this file would vanish from the first (what is left of it there is an
 // empty tensor) and drop the tangent; the layer then goes through its Python function (autograd.py).
-bool needs_function(std::initializer_list<at::Tensor> inputs) {
-    if (torch::jit::tracer::isTracing() || c10::impl::tls_is_dispatch_key_included(c10::DispatchKey::FuncTorchDynamicLayerFrontMode)) return true;
-    for (const at::Tensor& t : inputs)
-        if (t.defined() && t._fw_grad(/*level=*/0).defined()) return true;
-    return false;
+bool has_tangent(const at::Tensor& t) {
+    const torch::autograd::AutogradMeta* meta = t.defined() ? torch::autograd::impl::get_autograd_meta(t) : nullptr;
+    return meta && meta->fw_grad_ && t._fw_grad(/*level=*/0).defined();
+}
+bool needs_function(const at::Tensor& x, const at::Tensor& weight, const at::Tensor& bias = at::Tensor()) {
+    return torch::jit::tracer::isTracing() || c10::impl::tls_is_dispatch_key_included(c10::DispatchKey::FuncTorchDynamicLayerFrontMode) ||
+           has_tangent(x) || has_tangent(weight) || has_tangent(bias);
 }
 // Everything a pass computes lies below autograd; gradients come out as plain tensors.
 struct Below {
@@ -535,7 +537,7 @@ PyObject* linear(PyObject*, PyObject* const* a, Py_ssize_t n) {
     return layer_call([&]() -> PyObject* {
         const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
         const at::Tensor bias = a[2] != Py_None ? tensor_of(a[2], "bias") : at::Tensor();
-        if (needs_function({x, w, bias})) return same(Py_None);
+        if (needs_function(x, w, bias)) return same(Py_None);
         // a bias of another type, shape or place (a layer cast to half precision, one value for all outputs): the general addition
         if (bias.defined() && !(bias.device() == x.device() && bias.scalar_type() == at::kFloat && bias.dim() == 1 && bias.size(0) == w.size(1)))
             return same(Py_None);
@@ -658,7 +660,7 @@ PyObject* conv3x3(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!want(n, 8)) return nullptr;
     return layer_call([&]() -> PyObject* {
         const at::Tensor x = tensor_of(a[0], "x"), w = tensor_of(a[1], "weight");
-        if (needs_function({x, w})) return same(Py_None);
+        if (needs_function(x, w)) return same(Py_None);
         if (!(x.is_cuda() && x.scalar_type() == at::kFloat && x.dim() == 4)) value_error("%s must be a float32 CUDA tensor [n][h][w][c]", "x");
         auto node = std::shared_ptr<ConvNode>(new ConvNode(), torch::autograd::deleteNode);
         node->mant_bits = (int)as_ll(a[4]);
