@@ -157,12 +157,8 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // constant operand of the offset step, and the filter exponents (the same for every tile)
+    // constant operand of the offset step
     for (int i = threadIdx.x; i < G::ONES_BYTES / 4; i += CV_THREADS) reinterpret_cast<uint32_t*>(base_ptr + ones_off)[i] = 0xFFFFFFFFu;
-    for (int i = threadIdx.x; i < p.steps * N_TILE; i += CV_THREADS) {
-        const int t = i / N_TILE, j = i - t * N_TILE;
-        wexp[i] = j < p.filters ? p.exps_w[(int64_t)t * p.rs_w + j] : (int8_t)0;
-    }
     // 127 marks a position outside the image (the columns next to the data stay marked for good)
     for (int i = threadIdx.x; i < G::GRID_BYTES / 4; i += CV_THREADS) reinterpret_cast<uint32_t*>(base_ptr + grid_off)[i] = 0x7f7f7f7fu;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -170,10 +166,17 @@ conv_fwd_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    chain_wait();
+    // the filter exponents are the same for every tile
+    for (int i = threadIdx.x; i < p.steps * N_TILE; i += CV_THREADS) {
+        const int t = i / N_TILE, j = i - t * N_TILE;
+        wexp[i] = j < p.filters ? p.exps_w[(int64_t)t * p.rs_w + j] : (int8_t)0;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_next();
 
     if (warp < CV_CONTROL_WARPS) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(CV_REGS_CONTROL));
@@ -494,7 +497,7 @@ int launch_conv_cfg(const CUtensorMap& mX, const CUtensorMap& mW, const ConvProb
         attr_set[dev] = true;
     }
     const int grid = p.super_tiles < sm_count() ? p.super_tiles : sm_count();
-    conv_fwd_kernel<C, N_TILE><<<grid, CV_THREADS, G::SMEM, st>>>(mX, mW, p);
+    launch_chained(conv_fwd_kernel<C, N_TILE>, grid, CV_THREADS, G::SMEM, st, mX, mW, p);
     return launch_status();
 }
 

@@ -389,6 +389,7 @@ gemm_fp_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     if (PAIR) fp_cluster_barrier();            // both CTAs' barriers and tensor memory exist before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_start();
 
     if (warp < FP_CONTROL_WARPS) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(FP_REGS_CONTROL));
@@ -576,7 +577,8 @@ __device__ __forceinline__ uint32_t f16_pair(float a, float b) {        // exact
 // Form S: rows x kst bytes of one-plane mantissas -> bfloat16 q * 2^s, 16 elements per thread.
 __global__ void __launch_bounds__(256)
 expand_s_kernel(const int8_t* __restrict__ q, const int8_t* __restrict__ exps, int64_t rows, int kst, int lg_bp, int nkb, int64_t rs,
-                uint4* __restrict__ out) {
+                uint4* __restrict__ out, int beside) {
+    const Chain chain(beside);
     const int per = kst >> 4;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= rows * per) return;
@@ -599,7 +601,8 @@ expand_s_kernel(const int8_t* __restrict__ q, const int8_t* __restrict__ exps, i
 template <bool IS_B>
 __global__ void __launch_bounds__(256)
 expand_w_kernel(const int8_t* __restrict__ q, int64_t plane_stride, const int8_t* __restrict__ exps, int64_t rows, int kst, int lg_bp, int nkb,
-                int64_t rs, uint4* __restrict__ out, uint4* __restrict__ out_l, float* __restrict__ scales, int32_t* status) {
+                int64_t rs, uint4* __restrict__ out, uint4* __restrict__ out_l, float* __restrict__ scales, int32_t* status, int beside) {
+    const Chain chain(beside);
     const int per = kst >> 3;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= rows * per) return;
@@ -707,19 +710,9 @@ int fp_launch(FpProblem p, const FpOperand& a, const FpOperand& b, cudaStream_t 
         if (rc) return rc;
     }
     const int tiles = p.tiles_m * p.tiles_n;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    const int csize = PAIR ? 2 : p.splits;
-    cfg.gridDim = dim3(PAIR ? 2 * (tiles < clusters ? tiles : clusters) : p.splits > 1 ? tiles * p.splits : (tiles < sm_count() ? tiles : sm_count()), 1, 1);
-    cfg.blockDim = dim3(FP_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = C::SMEM;
-    cfg.stream = st;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = csize > 1 ? 1 : 0;
-    HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, mA, mB, mB1, mSA, mSB, mC, p));
-    return HBFP_OK;
+    const int grid = PAIR ? 2 * (tiles < clusters ? tiles : clusters) : p.splits > 1 ? tiles * p.splits : (tiles < sm_count() ? tiles : sm_count());
+    launch_chained_clusters(gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, PAIR ? 2 : p.splits, grid, FP_THREADS, C::SMEM, st, mA, mB, mB1, mSA, mSB, mC, p);
+    return launch_status();
 }
 
 template <int FORM, int BP, bool BIAS>
@@ -806,20 +799,20 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, in
     return f;
 }
 
-int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const FpOperand& out, cudaStream_t st) {
+int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, bool beside, const FpOperand& out, cudaStream_t st) {
     const Layout& L = x.L;
     const int lg = log2_of(L.bp);
     if (plan.form == FORM_S) {
         const int64_t n = L.rows * (L.kst / 16);
-        expand_s_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0));
+        launch_chained(expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), (int)beside);
         return launch_status();
     }
     int32_t* status = device_status_word();
     if (!status) return HBFP_ERR_CUDA;
     const int64_t n = L.rows * (L.kst / 8);
     const unsigned g = (unsigned)((n + 255) / 256);
-    if (is_b) expand_w_kernel<true><<<g, 256, 0, st>>>(x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status);
-    else expand_w_kernel<false><<<g, 256, 0, st>>>(x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status);
+    if (is_b) launch_chained(expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, (int)beside);
+    else launch_chained(expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, (int)beside);
     return launch_status();
 }
 

@@ -14,6 +14,7 @@ gemm_simt_kernel(int64_t M, int64_t N, int64_t nkb, int64_t bp,
                  const int8_t* __restrict__ mA, int64_t kstA, int64_t psA, const int8_t* __restrict__ eA, int64_t rsA,
                  const int8_t* __restrict__ mB, int64_t kstB, int64_t psB, const int8_t* __restrict__ eB, int64_t rsB,
                  float* __restrict__ C, int64_t ldc, int32_t* __restrict__ P) {
+    chain_start();
     const int64_t j = (int64_t)blockIdx.x * 16 + (threadIdx.x & 15);
     const int64_t i = (int64_t)blockIdx.y * 16 + (threadIdx.x >> 4);
     if (i >= M || j >= N) return;
@@ -58,7 +59,7 @@ int launch_gemm_simt(int64_t M, int64_t N, int64_t K, const Packed& a, const Pac
     dim3 grid((unsigned)((N + 15) / 16), (unsigned)((M + 15) / 16));
     if (grid.y > 65535) return HBFP_ERR_UNSUPPORTED;
 #define HBFP_SIMT(PA, PB)                                                                            \
-    gemm_simt_kernel<PA, PB><<<grid, 256, 0, st>>>(M, N, a.L.nkb, a.L.bp, a.mant, a.L.kst,           \
+    launch_chained(gemm_simt_kernel<PA, PB>, grid, 256, 0, st, M, N, a.L.nkb, a.L.bp, a.mant, a.L.kst,           \
                                                    a.L.plane_stride, a.exps, a.L.rs, b.mant, b.L.kst, \
                                                    b.L.plane_stride, b.exps, b.L.rs, C, ldc, P)
     if (a.L.planes == 1 && b.L.planes == 1) HBFP_SIMT(1, 1);

@@ -81,6 +81,7 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap mapW, const SkinnyProblem
             *abort_flag = 0;
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            chain_wait();
             for (int i = 0; i < nseg; ++i) {
                 mbar_expect_tx(full_bar + 8 * i, SK_NT * SK_SEG);
                 tma_load_2d(base + i * (SK_NT * SK_SEG), &mapW, (seg0 + i) * SK_SEG, n0, full_bar + 8 * i);
@@ -89,7 +90,10 @@ gemm_skinny_kernel(const __grid_constant__ CUtensorMap mapW, const SkinnyProblem
         __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(p.tmem_cols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        chain_wait();
+        chain_next();
     } else {
+        chain_wait();
         // exponents of the weight rows, sixteen at a time (blocks and rows beyond the matrix: 0, their mantissas are 0)
         for (int i = tid; i < nseg * BPS * (SK_NT / 16); i += 32 * SK_CONV_WARPS) {
             const int kb = kb0 + i / (SK_NT / 16), r = n0 + 16 * (i % (SK_NT / 16));
@@ -358,18 +362,8 @@ int sk_launch(const SkinnyProblem& p, const CUtensorMap& mW, size_t smem, dim3 g
         HBFP_CUDA_OK(cudaFuncSetAttribute(gemm_skinny_kernel<ROWS, BP, SR>, cudaFuncAttributeMaxDynamicSharedMemorySize, SK_SMEM_LIMIT));
         ready[dev] = true;
     }
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(SK_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = p.splits; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = p.splits > 1 ? 1 : 0;
-    HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, gemm_skinny_kernel<ROWS, BP, SR>, mW, p));
-    return HBFP_OK;
+    launch_chained_clusters(gemm_skinny_kernel<ROWS, BP, SR>, p.splits, grid, SK_THREADS, smem, st, mW, p);
+    return launch_status();
 }
 template <int ROWS, bool SR>
 int sk_launch_bp(int bp, const SkinnyProblem& p, const CUtensorMap& mW, size_t smem, dim3 grid, cudaStream_t st) {

@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(256)
 gemm_small_kernel(int64_t M, int64_t N, int nkb, int bp, const int8_t* __restrict__ mA, int64_t kstA,
                   const int8_t* __restrict__ eA, int64_t rsA, const int8_t* __restrict__ mB, int64_t kstB,
                   const int8_t* __restrict__ eB, int64_t rsB, float* __restrict__ C, int64_t ldc) {
+    chain_start();
     extern __shared__ __align__(16) unsigned char smem[];
     int8_t* xA = reinterpret_cast<int8_t*>(smem + 2 * SM_BUF);  // [nkb][32]
     int8_t* xB = xA + (size_t)nkb * SM_TILE;                    // [nkb][32]
@@ -252,6 +253,7 @@ __device__ __forceinline__ void sf_convert_cols(const SmallOperand& o, const Sma
 template <bool SR, int PER>
 __global__ void __launch_bounds__(SF_THREADS)
 gemm_small_fused_kernel(const SmallProblem p) {
+    chain_start();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint32_t amax[2][SF_MAX_GROUPS][SM_TILE];
     __shared__ int8_t xA[SF_MAX_GROUPS / 4 * SM_TILE], xB[SF_MAX_GROUPS / 4 * SM_TILE];      // [block][32]
@@ -323,7 +325,7 @@ int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, fl
         attr_set[dev] = true;
     }
     const dim3 grid((unsigned)((N + SM_TILE - 1) / SM_TILE), (unsigned)((M + SM_TILE - 1) / SM_TILE));
-    gemm_small_kernel<<<grid, 256, smem, st>>>(M, N, nkb, (int)a.L.bp, a.mant, a.L.kst, a.exps, a.L.rs, b.mant, b.L.kst,
+    launch_chained(gemm_small_kernel, grid, 256, smem, st, M, N, nkb, (int)a.L.bp, a.mant, a.L.kst, a.exps, a.L.rs, b.mant, b.L.kst,
                                                b.exps, b.L.rs, C, ldc);
     return launch_status();
 }
@@ -338,7 +340,7 @@ int sf_launch(const SmallProblem& p, dim3 grid, cudaStream_t st) {
         HBFP_CUDA_OK(cudaFuncSetAttribute(gemm_small_fused_kernel<SR, PER>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * SM_TILE * (2 * SM_AUTO_BYTES + 64)));
         attr_set[dev] = true;
     }
-    gemm_small_fused_kernel<SR, PER><<<grid, SF_THREADS, 2 * (size_t)SM_TILE * p.pitch, st>>>(p);      // at most 68 KB
+    launch_chained(gemm_small_fused_kernel<SR, PER>, grid, SF_THREADS, 2 * (size_t)SM_TILE * p.pitch, st, p);      // at most 68 KB
     return launch_status();
 }
 }  // namespace

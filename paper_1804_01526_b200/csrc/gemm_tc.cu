@@ -340,6 +340,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    chain_start();
 
     const Shape sh = make_shape(p.bp);
     const int total_work = p.tiles_m * p.tiles_n * p.splits;
@@ -705,6 +706,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // Sums the split-K partial tiles in ascending split order.
 __global__ void splitk_reduce(const float* __restrict__ partial, int splits, int64_t M, int64_t N, int64_t ldp,
                               float* __restrict__ C, int64_t ldc) {
+    chain_start();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M * N) return;
     const int64_t r = i / N, c = i % N, step = M * ldp;
@@ -773,7 +775,7 @@ int launch_cfg(const Problem& p, const Packed& a, const Packed& b, cudaStream_t 
     }
     const int64_t work = (int64_t)p.tiles_m * p.tiles_n * p.splits;
     const int grid = (int)(work < sm_count() ? work : sm_count());
-    gemm_tc_kernel<N_TILE, PLANES, MAGIC, DUMP, TSTORE><<<grid, THREADS, C::SMEM, st>>>(mA0, mA1, mB0, mB1, mEA, mEB, mC, p);
+    launch_chained(gemm_tc_kernel<N_TILE, PLANES, MAGIC, DUMP, TSTORE>, grid, THREADS, C::SMEM, st, mA0, mA1, mB0, mB1, mEA, mEB, mC, p);
     return launch_status();
 }
 
@@ -887,7 +889,7 @@ int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const P
     if (rc) return rc;
     if (p.splits > 1) {
         const int64_t n = M * N;
-        splitk_reduce<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p.partial, p.splits, M, N, p.ldp, Cout, ldc);
+        launch_chained(splitk_reduce, (unsigned)((n + 255) / 256), 256, 0, st, p.partial, p.splits, M, N, p.ldp, Cout, ldc);
         return launch_status();
     }
     return HBFP_OK;

@@ -9,6 +9,7 @@ namespace {
 template <int V>
 __global__ void __launch_bounds__(256)
 add_bias_kernel(float* __restrict__ C, uint32_t N, int64_t ldc, const float* __restrict__ bias, int64_t total) {
+    chain_start();
     const uint32_t per = N / V;
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < total; i += (int64_t)gridDim.x * 256) {
         const int64_t r = i / per;
@@ -30,6 +31,7 @@ constexpr int CS_WARPS = 8, CS_UNR = 8;
 template <int V>
 __global__ void __launch_bounds__(32 * CS_WARPS)
 column_sums_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, int splits, float* __restrict__ out) {
+    chain_start();
     __shared__ __align__(16) float part[CS_WARPS][32 * V];
     __shared__ __align__(16) float total[32 * V];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -103,18 +105,11 @@ int column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* o
     // a share of at least one round of loads, more CTAs than that only add to the exchange
     int splits = 1;
     while (splits < 8 && rows >= 2 * splits * CS_WARPS * CS_UNR) splits *= 2;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    cfg.blockDim = dim3(32 * CS_WARPS, 1, 1);
-    cfg.stream = st;
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = splits; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = splits > 1 ? 1 : 0;
     for (int64_t c0 = 0; c0 < cols; c0 += MOST) {
         const int64_t n = cols - c0 < MOST ? cols - c0 : MOST;
-        cfg.gridDim = dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V)), 1);
-        HBFP_CUDA_OK(cudaLaunchKernelEx(&cfg, column_sums_kernel<V>, x + c0, rows, n, ld, splits, out + c0));
+        launch_chained_clusters(column_sums_kernel<V>, splits, dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V))), 32 * CS_WARPS, 0, st, x + c0, rows, n, ld,
+                                splits, out + c0);
+        if (launch_status()) return HBFP_ERR_CUDA;
     }
     return HBFP_OK;
 }
@@ -126,8 +121,8 @@ int launch_add_bias(float* C, int64_t M, int64_t N, int64_t ldc, const float* bi
     const int64_t total = quad ? M * (N / 4) : M * N;
     const int64_t blocks = (total + 255) / 256, cap = 148 * 32;
     const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
-    if (quad) add_bias_kernel<4><<<grid, 256, 0, st>>>(C, (uint32_t)N, ldc, bias, total);
-    else add_bias_kernel<1><<<grid, 256, 0, st>>>(C, (uint32_t)N, ldc, bias, total);
+    if (quad) launch_chained(add_bias_kernel<4>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
+    else launch_chained(add_bias_kernel<1>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
     return launch_status();
 }
 

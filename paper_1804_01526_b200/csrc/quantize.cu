@@ -39,7 +39,8 @@ template <int LPB, bool SR, int PLANES>
 __global__ void __launch_bounds__(256, SR ? 3 : 4)
 quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-               int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const int8_t* __restrict__ given = nullptr, const FormArgs fa = FormArgs{}) {
+               int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const int8_t* __restrict__ given, const FormArgs fa) {
+    const Chain chain(p.beside);
     // given != nullptr: one exponent per row for the whole axis, computed beforehand (a block longer than the
     // tile); the kernel then only rounds and packs
     constexpr int B = 8 * LPB;
@@ -136,7 +137,8 @@ template <int PLANES, int RQ, bool SR>      // RQ = bp / 4: padded rows per warp
 __global__ void __launch_bounds__(128)
 quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
                 int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa, const int8_t* __restrict__ given = nullptr) {
+                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa, const int8_t* __restrict__ given) {
+    const Chain chain(p.beside);
     // given != nullptr: one exponent per column for the whole axis, computed beforehand; the blocks are then pieces of it
     constexpr int BP = 4 * RQ, BYTE_PLANES = is_form(PLANES) ? 1 : PLANES;
     __shared__ uint32_t pmax[4][COLT];
@@ -342,6 +344,7 @@ template <int MODE, int PLANES, bool FAST>
 __global__ void __launch_bounds__(256)
 tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, int t, int tp, QParams p,
             int16_t* __restrict__ wide, int8_t* __restrict__ grid, int64_t grid_ld, TileViews tv) {
+    chain_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int fp = FAST ? t + 4 : t + 1;                                   // pitch of the FP32 tile
     float* tile = reinterpret_cast<float*>(smem_raw);                      // [t][fp]
@@ -494,6 +497,7 @@ template <int MODE, int PLANES, int TP>
 __global__ void __launch_bounds__(256)
 tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, QParams p,
                  int16_t* __restrict__ wide, int8_t* __restrict__ grid, int64_t grid_ld, TileViews tv) {
+    chain_start();
     constexpr int G = TP / 8;                          // groups of eight per tile row
     constexpr int NITEMS = TP * G;                     // groups per tile
     constexpr int ITEMS = (NITEMS + 255) / 256;        // per thread
@@ -703,6 +707,7 @@ __device__ __forceinline__ float view_at(const float* x, int64_t ld, int axis, i
 // Pass 1a, blocks along rows: one warp per (line, block).
 __global__ void exps_axis1(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int64_t b,
                            int64_t nkb, QParams p, int8_t* __restrict__ exps, int64_t rs) {
+    chain_start();
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -723,6 +728,7 @@ template <int G, bool SR, int PLANES>
 __global__ void __launch_bounds__(256)
 quant_row_whole(const float* __restrict__ x, int64_t ld, int64_t d1, QParams p, int8_t* __restrict__ mant, int64_t kst,
                 int64_t plane_stride, int8_t* __restrict__ exps) {
+    chain_start();
     __shared__ uint32_t part[8];
     const int tid = threadIdx.x;
     const int64_t r = blockIdx.x;
@@ -762,6 +768,7 @@ quant_row_whole(const float* __restrict__ x, int64_t ld, int64_t d1, QParams p, 
 // neighbouring addresses.
 __global__ void exps_axis0(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int64_t b,
                            int64_t nkb, QParams p, int8_t* __restrict__ exps, int64_t rs) {
+    chain_start();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * nkb) return;
     const int64_t kb = i / rows, r = i % rows;
@@ -775,6 +782,7 @@ __global__ void exps_axis0(const float* __restrict__ x, int64_t rows, int64_t K,
 // exponent and repeats it for every line of the view that crosses the tile.
 __global__ void exps_tiles(const float* __restrict__ x, int64_t d0, int64_t d1, int64_t ld, int64_t t,
                            QParams p, int axis, int8_t* __restrict__ exps, int64_t rs, int64_t nu, int64_t nv) {
+    chain_start();
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (warp >= nu * nv) return;
@@ -799,6 +807,7 @@ __global__ void __launch_bounds__(CONVW_THREADS)
 exps_conv_tiles(const float* __restrict__ x, int64_t taps, int64_t c_in, int64_t c_out, int64_t ld, int64_t t, QParams p,
                 int8_t* __restrict__ exps0, int64_t rs0, int8_t* __restrict__ exps1, int64_t rs1, int64_t nu, int64_t nv,
                 int8_t* __restrict__ tile_exps, uint32_t* __restrict__ amax, bool fill) {
+    chain_start();
     __shared__ uint32_t part[CONVW_THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t u = blockIdx.x / nv, v = blockIdx.x % nv;
@@ -841,6 +850,7 @@ __global__ void mant_generic(const float* __restrict__ x, int64_t d1, int64_t ro
                              int axis, int64_t b, int64_t bp, int64_t nkb, QParams p,
                              const int8_t* __restrict__ exps, int64_t rs, int8_t* __restrict__ mant,
                              int64_t kst, int64_t plane_stride) {
+    chain_start();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t per = kst / 4;
     if (i >= rows * per) return;
@@ -879,6 +889,7 @@ im2col_gather(const int8_t* __restrict__ xm, const int8_t* __restrict__ xe, int 
               int h, int w, int ho, int wo, int kh, int kw, int pad, int lg_bp, int planes,
               uint32_t rows_out, int kst_out, int64_t ps_out, int64_t rs_out,
               int8_t* __restrict__ om, int8_t* __restrict__ oe) {
+    chain_start();
     // A CTA takes 64 consecutive output rows, a warp eight of them; the lanes sweep a row 16 bytes at a
     // time. The filter offsets of the taps are tabulated once per CTA, the pixel coordinates once per row
     // (32-bit arithmetic: the host checks the sizes), and the exponents of the 64 rows are collected in
@@ -953,6 +964,7 @@ template <int PLANES, int NPX, bool SR>      // NPX = b / 4 pixels per thread: 4
 __global__ void __launch_bounds__(256)
 im2col_cols(const float* __restrict__ x, int h, int w, int lg_w, int c, int kh, int kw, int pad, QParams p,
             int64_t kst, int64_t plane_stride, int64_t rs, int8_t* __restrict__ mant, int8_t* __restrict__ exps) {
+    chain_start();
     constexpr int B = 4 * NPX;
     constexpr int BP = B <= 32 ? 32 : B <= 64 ? 64 : 128;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1072,6 +1084,7 @@ template <int PLANES, int W, bool SR>
 __global__ void __launch_bounds__(192, cols3_ctas<PLANES, W, SR>())
 im2col_cols3(const float* __restrict__ x, int h, int c, int kh, int pad, QParams p, int64_t kst, int64_t plane_stride, int64_t rs,
              int8_t* __restrict__ mant, int8_t* __restrict__ exps) {
+    chain_start();
     constexpr int B = 64, ROWS = B / W;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const uint16_t* rnd = reinterpret_cast<const uint16_t*>(smem_raw);       // draws of the rows under the filter [ROWS + kh - 1][W][c] (stochastic)
@@ -1153,6 +1166,7 @@ __global__ void __launch_bounds__(256)
 conv_dgrad_filters_kernel(const int8_t* __restrict__ m1, const int8_t* __restrict__ e1, int64_t kst1, int64_t ps1,
                           int64_t rs1, int taps, int64_t c_in, int64_t c_out, int t, int planes,
                           int8_t* __restrict__ mo, int8_t* __restrict__ eo, int64_t ksto, int64_t pso, int64_t rso) {
+    chain_start();
     const int lane = threadIdx.x & 31;
     const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (item >= c_in * taps) return;
@@ -1176,6 +1190,7 @@ conv_dgrad_filters_kernel(const int8_t* __restrict__ m1, const int8_t* __restric
 __global__ void unpack_kernel(const int8_t* __restrict__ mant, const int8_t* __restrict__ exps, int64_t rows,
                               int64_t K, int64_t b, int64_t bp, int64_t nkb, int64_t kst, int64_t plane_stride,
                               int planes, int64_t rs, int16_t* __restrict__ q, int8_t* __restrict__ s) {
+    chain_start();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q && i < rows * K) {
         const int64_t r = i / K, kk = i % K, o = (kk / b) * bp + kk % b;
@@ -1192,6 +1207,7 @@ __global__ void unpack_kernel(const int8_t* __restrict__ mant, const int8_t* __r
 __global__ void dequant_kernel(const int8_t* __restrict__ mant, const int8_t* __restrict__ exps, int64_t rows,
                                int64_t K, int64_t b, int64_t bp, int64_t kst, int64_t plane_stride, int planes,
                                int64_t rs, float* __restrict__ out, int64_t ld) {
+    chain_start();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * K) return;
     const int64_t r = i / K, kk = i % K, kb = kk / b, o = kb * bp + kk % b;
@@ -1215,6 +1231,7 @@ __global__ void __launch_bounds__(256)
 quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                int8_t* __restrict__ exps, int64_t rs, uint32_t gpr, uint32_t total_groups, const FormArgs fa) {
+    const Chain chain(p.beside);
     constexpr int B = 8 * LPB;
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t g0 = blockIdx.x * (256u * ITEMS) + tid;
@@ -1271,7 +1288,7 @@ int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, c
                           int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa) {
     const uint32_t gpr = (uint32_t)(K / 8), total = (uint32_t)(rows * (K / 8));
     const unsigned grid = (total + 256u * ITEMS - 1u) / (256u * ITEMS);
-#define HBFP_QFLAT(SRV, OUT) quant_row_flat<LPB, SRV, OUT, ITEMS><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
+#define HBFP_QFLAT(SRV, OUT) launch_chained(quant_row_flat<LPB, SRV, OUT, ITEMS>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
     if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QFLAT(true, FORM); else HBFP_QFLAT(false, FORM); }
     else if (p.rounding == 1) { if (L.planes == 1) HBFP_QFLAT(true, 1); else HBFP_QFLAT(true, 2); }
     else { if (L.planes == 1) HBFP_QFLAT(false, 1); else HBFP_QFLAT(false, 2); }
@@ -1304,6 +1321,7 @@ __global__ void __launch_bounds__(256)
 quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int b, QParams p,
                  int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                  int8_t* __restrict__ exps, int64_t rs, int64_t nkb, uint32_t ppr, int64_t total, const FormArgs fa) {
+    const Chain chain(p.beside);
     constexpr int ITEMS = 2;
     const int tid = threadIdx.x, lane = tid & 31;
     float e8[ITEMS][8];
@@ -1351,7 +1369,7 @@ int launch_row_ragged(const float* x, int64_t rows, int64_t K, int64_t ld, const
     const uint32_t ppr = (uint32_t)(L.kst / 8);
     const int64_t total = rows * ppr;
     const unsigned grid = (unsigned)((total + 511) / 512);
-#define HBFP_QROW_RAGGED(SRV, PL) quant_row_ragged<LPB, SRV, PL, VEC><<<grid, 256, 0, st>>>(x, rows, K, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, ppr, total, fa)
+#define HBFP_QROW_RAGGED(SRV, PL) launch_chained(quant_row_ragged<LPB, SRV, PL, VEC>, grid, 256, 0, st, x, rows, K, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, ppr, total, fa)
     if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QROW_RAGGED(true, FORM); else HBFP_QROW_RAGGED(false, FORM); }
     else if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_RAGGED(true, 1); else HBFP_QROW_RAGGED(true, 2); }
     else { if (L.planes == 1) HBFP_QROW_RAGGED(false, 1); else HBFP_QROW_RAGGED(false, 2); }
@@ -1383,6 +1401,7 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
               const __grid_constant__ CUtensorMap mapM1, QParams p, int8_t* __restrict__ exps, int64_t rs,
               int64_t nkb, int64_t K, int64_t R, int tiles_n, int total_tiles, int32_t* status,
               const int8_t* __restrict__ given, int8_t* __restrict__ form_out, int64_t kst, int64_t plane_stride) {
+    const Chain chain(p.beside);
     // given != nullptr: one exponent per column for the whole axis, computed beforehand (blocks longer than a
     // tile); the kernel then only rounds and packs
     extern __shared__ unsigned char smem_dyn[];
@@ -1540,6 +1559,7 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
 constexpr int CMAX_ROWS = 128, CMAX_ROWS_SHORT = 32;
 __global__ void __launch_bounds__(256)
 col_amax_kernel(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int band, uint32_t* __restrict__ amax) {
+    chain_start();
     const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (col >= R) return;
     const int64_t k0 = (int64_t)blockIdx.y * band, k1 = min(K, k0 + band);
@@ -1549,6 +1569,7 @@ col_amax_kernel(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
     atomicMax(amax + col, am);
 }
 __global__ void col_exps_kernel(const uint32_t* __restrict__ amax, int64_t R, QParams p, int8_t* __restrict__ exps) {
+    chain_start();
     const int64_t col = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (col < R) exps[col] = (int8_t)block_exponent(amax[col], p.m, p.exp_mode);
 }
@@ -1588,7 +1609,7 @@ int launch_col_tma(const float* x, int64_t K, int64_t rows, int64_t ld, const QP
     const int64_t total = tiles_n * tiles_k;
     const int64_t cap = (int64_t)sm_count() * ctas_per_sm;
     const int grid = (int)(total < cap ? total : cap);
-    quant_col_tma<PLANES, LB, SR><<<grid, QC_THREADS, smem, st>>>(mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
+    launch_chained(quant_col_tma<PLANES, LB, SR>, grid, QC_THREADS, smem, st, mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
                                                               (int)total, status, given, mant, L.kst, L.plane_stride);
     return launch_status();
 }
@@ -1601,11 +1622,11 @@ int launch_row_fast(const float* x, int64_t rows, int64_t K, int64_t ld, const Q
     dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
     // the last column tile must also cover the exponent rows of blocks that start before K
     if (p.rounding == 1) {
-        if (L.planes == 1) quant_row_fast<LPB, true, 1><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb);
-        else quant_row_fast<LPB, true, 2><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb);
+        if (L.planes == 1) launch_chained(quant_row_fast<LPB, true, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        else launch_chained(quant_row_fast<LPB, true, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
     } else {
-        if (L.planes == 1) quant_row_fast<LPB, false, 1><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb);
-        else quant_row_fast<LPB, false, 2><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb);
+        if (L.planes == 1) launch_chained(quant_row_fast<LPB, false, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        else launch_chained(quant_row_fast<LPB, false, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
     }
     return launch_status();
 }
@@ -1628,7 +1649,7 @@ int launch_tile_full_small(int mode, int planes, int t, unsigned gx, unsigned gy
     memcpy(&p, qparams, sizeof(p));
     memcpy(&tv, tileviews, sizeof(tv));
     const dim3 grid_dim(gx, gy);
-#define HBFP_TILE_FULL_SMALL(MODE, PLANES, TP) tile_kernel_full<MODE, PLANES, TP><<<grid_dim, 256, 0, st>>>(src, ld, d0, d1, p, wide, grid, grid_ld, tv)
+#define HBFP_TILE_FULL_SMALL(MODE, PLANES, TP) launch_chained(tile_kernel_full<MODE, PLANES, TP>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv)
 #define HBFP_TILE_FULL_MODE(MODE)                                                                     \
     do {                                                                                              \
         if (planes == 1) { if (t == 32) HBFP_TILE_FULL_SMALL(MODE, 1, 32); else HBFP_TILE_FULL_SMALL(MODE, 1, 64); } \
@@ -1651,13 +1672,15 @@ int launch_tile_full_small(int mode, int planes, int t, unsigned gx, unsigned gy
 // ------------------------------------------------------------------------------ launchers
 
 int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f,
-                    int8_t* mant, int8_t* exps, cudaStream_t st) {
+                    int8_t* mant, int8_t* exps, cudaStream_t st, bool beside) {
     const int64_t K = axis == 1 ? d1 : d0, rows = axis == 1 ? d0 : d1;
     Layout L;
     int rc = make_layout(rows, K, f, &L);
     if (rc) return rc;
     if (rows == 0) return HBFP_OK;
     const QParams p = make_params(f);
+    QParams one = p;                   // a conversion of one launch
+    one.beside = beside;
     if (K == 0) {
         HBFP_CUDA_OK(cudaMemsetAsync(mant, 0, (size_t)L.mant_bytes, st));
         HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
@@ -1670,9 +1693,9 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     if (f->tile == 0 && axis == 1 && aligned && L.b == L.bp && L.b <= 128 && K % L.b == 0 && L.kst % 512 != 0 &&
         rows * (L.kst / 8) < (1ll << 32) - 4096) {
         switch (L.b) {
-            case 32: return launch_row_flat<4>(x, rows, K, ld, p, L, mant, exps, st);
-            case 64: return launch_row_flat<8>(x, rows, K, ld, p, L, mant, exps, st);
-            case 128: return launch_row_flat<16>(x, rows, K, ld, p, L, mant, exps, st);
+            case 32: return launch_row_flat<4>(x, rows, K, ld, one, L, mant, exps, st);
+            case 64: return launch_row_flat<8>(x, rows, K, ld, one, L, mant, exps, st);
+            case 128: return launch_row_flat<16>(x, rows, K, ld, one, L, mant, exps, st);
             default: break;
         }
     }
@@ -1682,7 +1705,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
         // rows of 2048, 4096, 8192 or 16384 elements stay in a CTA's registers: one pass
         if ((K == 2048 || K == 4096 || K == 8192 || K == 16384) && L.kst == K && rows < (1ll << 31)) {
-#define HBFP_QROW_WHOLE2(GV, SRV, PL) quant_row_whole<GV, SRV, PL><<<(unsigned)rows, 256, 0, st>>>(x, ld, d1, p, mant, L.kst, L.plane_stride, exps)
+#define HBFP_QROW_WHOLE2(GV, SRV, PL) launch_chained(quant_row_whole<GV, SRV, PL>, (unsigned)rows, 256, 0, st, x, ld, d1, p, mant, L.kst, L.plane_stride, exps)
 #define HBFP_QROW_WHOLE(GV)                                                                          \
     do {                                                                                             \
         if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_WHOLE2(GV, true, 1); else HBFP_QROW_WHOLE2(GV, true, 2); }   \
@@ -1694,10 +1717,10 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
             return launch_status();
         }
         const int64_t want = (rows * 32 + 255) / 256;
-        exps_axis1<<<(unsigned)(want < 148 * 16 ? want : 148 * 16), 256, 0, st>>>(x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
+        launch_chained(exps_axis1, (unsigned)(want < 148 * 16 ? want : 148 * 16), 256, 0, st, x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
         if (launch_status()) return HBFP_ERR_CUDA;
         dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
-#define HBFP_QROW_GIVEN(SRV, PL) quant_row_fast<16, SRV, PL><<<grid, 256, 0, st>>>(x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, exps)
+#define HBFP_QROW_GIVEN(SRV, PL) launch_chained(quant_row_fast<16, SRV, PL>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, exps, FormArgs{})
         if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_GIVEN(true, 1); else HBFP_QROW_GIVEN(true, 2); }
         else { if (L.planes == 1) HBFP_QROW_GIVEN(false, 1); else HBFP_QROW_GIVEN(false, 2); }
 #undef HBFP_QROW_GIVEN
@@ -1706,10 +1729,10 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     if (f->tile == 0 && axis == 1 && aligned && d1 % 8 == 0 && L.b == L.bp && L.b <= 256 &&
         rows <= 32ll * 65535) {
         switch (L.b) {
-            case 32: return launch_row_fast<4>(x, rows, K, ld, p, L, mant, exps, st);
-            case 64: return launch_row_fast<8>(x, rows, K, ld, p, L, mant, exps, st);
-            case 128: return launch_row_fast<16>(x, rows, K, ld, p, L, mant, exps, st);
-            case 256: return launch_row_fast<32>(x, rows, K, ld, p, L, mant, exps, st);
+            case 32: return launch_row_fast<4>(x, rows, K, ld, one, L, mant, exps, st);
+            case 64: return launch_row_fast<8>(x, rows, K, ld, one, L, mant, exps, st);
+            case 128: return launch_row_fast<16>(x, rows, K, ld, one, L, mant, exps, st);
+            case 256: return launch_row_fast<32>(x, rows, K, ld, one, L, mant, exps, st);
             default: break;
         }
     }
@@ -1727,8 +1750,8 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         const int64_t wide = (rows + 255) / 256;
         const bool idle = wide * ((K + CMAX_ROWS - 1) / CMAX_ROWS) < 4 * 148;
         const int band = idle && (K <= 12288 || (K <= 20480 && wide >= 3)) ? CMAX_ROWS_SHORT : CMAX_ROWS;
-        col_amax_kernel<<<dim3((unsigned)wide, (unsigned)((K + band - 1) / band)), 256, 0, st>>>(x, K, rows, ld, band, amax);
-        col_exps_kernel<<<(unsigned)wide, 256, 0, st>>>(amax, rows, p, exps);
+        launch_chained(col_amax_kernel, dim3((unsigned)wide, (unsigned)((K + band - 1) / band)), 256, 0, st, x, K, rows, ld, band, amax);
+        launch_chained(col_exps_kernel, (unsigned)wide, 256, 0, st, amax, rows, p, exps);
         if (launch_status()) return HBFP_ERR_CUDA;
         if (stream) {
 #define HBFP_QCOL_GIVEN(PL) (p.rounding ? launch_col_tma<PL, 0, true>(x, K, rows, ld, p, L, mant, exps, st, exps) \
@@ -1738,7 +1761,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         }
         const int64_t pieces = L.kst / 128;
         const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * pieces);
-#define HBFP_QCOL_GIVEN(PL, SRV) quant_col_block<PL, 32, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, 128, p, mant, L.kst, L.plane_stride, exps, L.rs, pieces, tiles_n, FormArgs{}, exps)
+#define HBFP_QCOL_GIVEN(PL, SRV) launch_chained(quant_col_block<PL, 32, SRV>, grid, 128, 0, st, x, K, rows, ld, 128, p, mant, L.kst, L.plane_stride, exps, L.rs, pieces, tiles_n, FormArgs{}, exps)
         if (L.planes == 1) { if (p.rounding) HBFP_QCOL_GIVEN(1, true); else HBFP_QCOL_GIVEN(1, false); }
         else { if (p.rounding) HBFP_QCOL_GIVEN(2, true); else HBFP_QCOL_GIVEN(2, false); }
 #undef HBFP_QCOL_GIVEN
@@ -1747,8 +1770,8 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     if (f->tile == 0 && axis == 0 && aligned && L.b == L.bp && L.b <= 128 && (p.rounding == 0 || rows % 8 == 0) &&
         (reinterpret_cast<uintptr_t>(mant) & 127) == 0 && rows < (1ll << 29) && K < (1ll << 31) &&
         ((rows + QC_COLS - 1) / QC_COLS) * (L.kst / QC_ROWS) < (1ll << 31)) {
-#define HBFP_QCOL_TMA(PL, LBV) (p.rounding ? launch_col_tma<PL, LBV, true>(x, K, rows, ld, p, L, mant, exps, st) \
-                                           : launch_col_tma<PL, LBV, false>(x, K, rows, ld, p, L, mant, exps, st))
+#define HBFP_QCOL_TMA(PL, LBV) (p.rounding ? launch_col_tma<PL, LBV, true>(x, K, rows, ld, one, L, mant, exps, st) \
+                                           : launch_col_tma<PL, LBV, false>(x, K, rows, ld, one, L, mant, exps, st))
         const int lb = L.b == 128 ? 0 : L.b == 64 ? 1 : 2;
         if (L.planes == 1) return lb == 0 ? HBFP_QCOL_TMA(1, 0) : lb == 1 ? HBFP_QCOL_TMA(1, 1) : HBFP_QCOL_TMA(1, 2);
         return lb == 0 ? HBFP_QCOL_TMA(2, 0) : lb == 1 ? HBFP_QCOL_TMA(2, 1) : HBFP_QCOL_TMA(2, 2);
@@ -1757,7 +1780,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     // every other block length up to 128, any pitch and alignment
     if (f->tile == 0 && axis == 0 && L.b <= 128 && ((rows + COLT - 1) / COLT) * L.nkb < (1ll << 31)) {
         const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
-#define HBFP_QCOL(PL, RQ, SRV) quant_col_block<PL, RQ, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, tiles_n, FormArgs{})
+#define HBFP_QCOL(PL, RQ, SRV) launch_chained(quant_col_block<PL, RQ, SRV>, grid, 128, 0, st, x, K, rows, ld, (int)L.b, one, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, tiles_n, FormArgs{}, nullptr)
 #define HBFP_QCOL_SR(PL, RQ) do { if (p.rounding) HBFP_QCOL(PL, RQ, true); else HBFP_QCOL(PL, RQ, false); } while (0)
         if (L.planes == 1) { if (L.bp == 32) HBFP_QCOL_SR(1, 8); else if (L.bp == 64) HBFP_QCOL_SR(1, 16); else HBFP_QCOL_SR(1, 32); }
         else { if (L.bp == 32) HBFP_QCOL_SR(2, 8); else if (L.bp == 64) HBFP_QCOL_SR(2, 16); else HBFP_QCOL_SR(2, 32); }
@@ -1767,9 +1790,9 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     }
     if (f->tile == 0 && axis == 1 && L.b <= 128 && K < (1ll << 30) && rows * (L.kst / 8) < (1ll << 39)) {
         const bool vec = aligned && L.b % 4 == 0;          // every piece starts on a 16-byte boundary
-        if (L.bp == 32) return vec ? launch_row_ragged<4, true>(x, rows, K, ld, p, L, mant, exps, st) : launch_row_ragged<4, false>(x, rows, K, ld, p, L, mant, exps, st);
-        if (L.bp == 64) return vec ? launch_row_ragged<8, true>(x, rows, K, ld, p, L, mant, exps, st) : launch_row_ragged<8, false>(x, rows, K, ld, p, L, mant, exps, st);
-        return vec ? launch_row_ragged<16, true>(x, rows, K, ld, p, L, mant, exps, st) : launch_row_ragged<16, false>(x, rows, K, ld, p, L, mant, exps, st);
+        if (L.bp == 32) return vec ? launch_row_ragged<4, true>(x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<4, false>(x, rows, K, ld, one, L, mant, exps, st);
+        if (L.bp == 64) return vec ? launch_row_ragged<8, true>(x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<8, false>(x, rows, K, ld, one, L, mant, exps, st);
+        return vec ? launch_row_ragged<16, true>(x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<16, false>(x, rows, K, ld, one, L, mant, exps, st);
     }
     if (f->tile > 0 && f->tile <= 128) {
         // single view of a tiled weight: the fused tile kernel with the other view switched off
@@ -1784,19 +1807,19 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
             int64_t items = rows * L.nkb;
             int64_t want = (items + 7) / 8;
             unsigned blocks = (unsigned)(want < 148 * 32 ? want : 148 * 32);
-            exps_axis1<<<blocks, 256, 0, st>>>(x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
+            launch_chained(exps_axis1, blocks, 256, 0, st, x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
         } else {
-            exps_axis0<<<blocks_for(rows * L.nkb, 256), 256, 0, st>>>(x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
+            launch_chained(exps_axis0, blocks_for(rows * L.nkb, 256), 256, 0, st, x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
         }
     } else {
         const int64_t t = f->tile, nu = (d0 + t - 1) / t, nv = (d1 + t - 1) / t;
-        exps_tiles<<<blocks_for(nu * nv * 32, 256), 256, 0, st>>>(x, d0, d1, ld, t, p, axis, exps, L.rs, nu, nv);
+        launch_chained(exps_tiles, blocks_for(nu * nv * 32, 256), 256, 0, st, x, d0, d1, ld, t, p, axis, exps, L.rs, nu, nv);
     }
     if (launch_status()) return HBFP_ERR_CUDA;
     if (L.planes == 1)
-        mant_generic<1><<<blocks_for(rows * (L.kst / 4), 256), 256, 0, st>>>(x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
+        launch_chained(mant_generic<1>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     else
-        mant_generic<2><<<blocks_for(rows * (L.kst / 4), 256), 256, 0, st>>>(x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
+        launch_chained(mant_generic<2>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     return launch_status();
 }
 
@@ -1811,7 +1834,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
             return L.b == 32 ? launch_row_flat<4, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_flat<8, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
         if (aligned && d1 % 8 == 0 && L.b == L.bp && rows <= 32ll * 65535) {
             const dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
-#define HBFP_QFAST(LPB, SRV) quant_row_fast<LPB, SRV, FORM><<<grid, 256, 0, st>>>(x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
+#define HBFP_QFAST(LPB, SRV) launch_chained(quant_row_fast<LPB, SRV, FORM>, grid, 256, 0, st, x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
             if (L.b == 32) { if (p.rounding) HBFP_QFAST(4, true); else HBFP_QFAST(4, false); }
             else { if (p.rounding) HBFP_QFAST(8, true); else HBFP_QFAST(8, false); }
 #undef HBFP_QFAST
@@ -1829,7 +1852,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
     }
     if (((rows + COLT - 1) / COLT) * L.nkb >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
     const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
-#define HBFP_QCOL(RQ, SRV) quant_col_block<FORM, RQ, SRV><<<grid, 128, 0, st>>>(x, K, rows, ld, (int)L.b, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, tiles_n, fa)
+#define HBFP_QCOL(RQ, SRV) launch_chained(quant_col_block<FORM, RQ, SRV>, grid, 128, 0, st, x, K, rows, ld, (int)L.b, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, tiles_n, fa, nullptr)
     if (L.bp == 32) { if (p.rounding) HBFP_QCOL(8, true); else HBFP_QCOL(8, false); }
     else { if (p.rounding) HBFP_QCOL(16, true); else HBFP_QCOL(16, false); }
 #undef HBFP_QCOL
@@ -1840,14 +1863,15 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
 
 // Converts an FP32 operand straight to a floating-point operand form: blocks of at most 64, no weight tiles, elements
 // aligned to 32 bytes (HBFP_ERR_UNSUPPORTED otherwise; the caller converts to the packed layout and expands that).
-int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f, int wide, bool is_b, const FpOperand& o,
-                         cudaStream_t st) {
+int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f, int wide, bool is_b, bool beside,
+                         const FpOperand& o, cudaStream_t st) {
     const int64_t K = axis == 1 ? d1 : d0, rows = axis == 1 ? d0 : d1;
     Layout L;
     int rc = make_layout(rows, K, f, &L);
     if (rc) return rc;
     if (f->tile != 0 || L.bp > 64 || rows == 0 || K == 0 || (L.planes == 2) != (wide != 0)) return HBFP_ERR_UNSUPPORTED;
-    const QParams p = make_params(f);
+    QParams p = make_params(f);
+    p.beside = beside;
     const FormArgs fa{device_status_word()};
     if (!fa.status) return HBFP_ERR_CUDA;
     int8_t* out = static_cast<int8_t*>(o.p0);
@@ -1888,7 +1912,7 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     const bool full = fast && t == tp && (d0 % t) == 0 && (d1 % t) == 0 && ((mant_c0 != nullptr) == (mant_c1 != nullptr)) &&
                       (!mant_c0 || (exps_c0 && exps_c1)) && sh_full + (L0.planes == 2 ? 4 : 0) <= 8;
     if (full) {
-#define HBFP_TILE_FULL(PLANES, TP) tile_kernel_full<MODE, PLANES, TP><<<grid_dim, 256, 0, st>>>(src, ld, d0, d1, p, wide, grid, nv, tv)
+#define HBFP_TILE_FULL(PLANES, TP) launch_chained(tile_kernel_full<MODE, PLANES, TP>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, nv, tv)
         if (t != 128)
             return launch_tile_full_small(MODE, (int)L0.planes, t, grid_dim.x, grid_dim.y, src, ld, d0, d1, &p, wide, grid, nv, &tv, st);
         if (L0.planes == 1) HBFP_TILE_FULL(1, 128); else HBFP_TILE_FULL(2, 128);
@@ -1898,7 +1922,7 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
 #define HBFP_TILE_LAUNCH(PLANES, FAST)                                                                                       \
     do {                                                                                                                     \
         HBFP_CUDA_OK(cudaFuncSetAttribute(tile_kernel<MODE, PLANES, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-        tile_kernel<MODE, PLANES, FAST><<<grid_dim, 256, smem, st>>>(src, ld, d0, d1, t, tp, p, wide, grid, nv, tv);         \
+        launch_chained(tile_kernel<MODE, PLANES, FAST>, grid_dim, 256, smem, st, src, ld, d0, d1, t, tp, p, wide, grid, nv, tv);         \
     } while (0)
     if (L0.planes == 1) {
         if (fast) HBFP_TILE_LAUNCH(1, true); else HBFP_TILE_LAUNCH(1, false);
@@ -1949,7 +1973,7 @@ int launch_quantize_conv_weights(const float* w, int64_t taps, int64_t c_in, int
         if (pass == 1 && !amax) break;
         if (pass == 0 && amax) HBFP_CUDA_OK(cudaMemsetAsync(amax, 0, (size_t)(nu * nv * 4), st));
         const dim3 grid((unsigned)(nu * nv), pass == 0 && amax ? (unsigned)splits : 1u);
-        exps_conv_tiles<<<grid, CONVW_THREADS, 0, st>>>(w, taps, c_in, c_out, ld, t, p, mant_c0 ? exps_c0 : nullptr,
+        launch_chained(exps_conv_tiles, grid, CONVW_THREADS, 0, st, w, taps, c_in, c_out, ld, t, p, mant_c0 ? exps_c0 : nullptr,
                                                         mant_c0 ? L[0].rs : 0, mant_c1 ? exps_c1 : nullptr,
                                                         mant_c1 ? L[1].rs : 0, nu, nv, tile_exps, amax, pass == 1);
         if (launch_status()) return HBFP_ERR_CUDA;
@@ -1960,9 +1984,9 @@ int launch_quantize_conv_weights(const float* w, int64_t taps, int64_t c_in, int
         if (!mant) continue;
         const Layout& A = L[axis];
         if (A.planes == 1)
-            mant_generic<1><<<blocks_for(A.rows * (A.kst / 4), 256), 256, 0, st>>>(w, d1, A.rows, A.k, ld, axis, A.b, A.bp, A.nkb, p, exps, A.rs, mant, A.kst, A.plane_stride);
+            launch_chained(mant_generic<1>, blocks_for(A.rows * (A.kst / 4), 256), 256, 0, st, w, d1, A.rows, A.k, ld, axis, A.b, A.bp, A.nkb, p, exps, A.rs, mant, A.kst, A.plane_stride);
         else
-            mant_generic<2><<<blocks_for(A.rows * (A.kst / 4), 256), 256, 0, st>>>(w, d1, A.rows, A.k, ld, axis, A.b, A.bp, A.nkb, p, exps, A.rs, mant, A.kst, A.plane_stride);
+            launch_chained(mant_generic<2>, blocks_for(A.rows * (A.kst / 4), 256), 256, 0, st, w, d1, A.rows, A.k, ld, axis, A.b, A.bp, A.nkb, p, exps, A.rs, mant, A.kst, A.plane_stride);
         if (launch_status()) return HBFP_ERR_CUDA;
     }
     return HBFP_OK;
@@ -1994,7 +2018,7 @@ int launch_im2col_packed(const int8_t* xm, const int8_t* xe, int64_t n, int64_t 
     const int lg_bp = Lo.bp == 32 ? 5 : Lo.bp == 64 ? 6 : 7;
     if (kh * kw > IM2COL_MAX_TAPS || kh > 100 || kw > 100 || pad > 100) return HBFP_ERR_UNSUPPORTED;
     if (Lo.rows >= (1ll << 31) || Lx.rows >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
-    im2col_gather<<<blocks_for(Lo.rows, IM2COL_ROWS), 256, 0, st>>>(xm, xe, (int)Lx.kst, Lx.plane_stride, (int)h, (int)w, (int)ho, (int)wo,
+    launch_chained(im2col_gather, blocks_for(Lo.rows, IM2COL_ROWS), 256, 0, st, xm, xe, (int)Lx.kst, Lx.plane_stride, (int)h, (int)w, (int)ho, (int)wo,
                                                                    kh, kw, pad, lg_bp, (int)Lo.planes, (uint32_t)Lo.rows, (int)Lo.kst,
                                                                    Lo.plane_stride, Lo.rs, om, oe);
     return launch_status();
@@ -2027,7 +2051,7 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
 #define HBFP_COLS3(PL, WV, SRV)                                                                                                      \
     do {                                                                                                                              \
         if (table > 48 * 1024) HBFP_CUDA_OK(cudaFuncSetAttribute(im2col_cols3<PL, WV, SRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)table)); \
-        im2col_cols3<PL, WV, SRV><<<(unsigned)L.nkb, threads, table, st>>>(x, (int)h, (int)c, kh, pad, p, L.kst, L.plane_stride, L.rs, mant, exps); \
+        launch_chained(im2col_cols3<PL, WV, SRV>, (unsigned)L.nkb, threads, table, st, x, (int)h, (int)c, kh, pad, p, L.kst, L.plane_stride, L.rs, mant, exps); \
     } while (0)
 #define HBFP_COLS3_SR(PL, WV) do { if (p.rounding) HBFP_COLS3(PL, WV, true); else HBFP_COLS3(PL, WV, false); } while (0)
 #define HBFP_COLS3_W(PL) do { if (w == 8) HBFP_COLS3_SR(PL, 8); else if (w == 16) HBFP_COLS3_SR(PL, 16); else if (w == 32) HBFP_COLS3_SR(PL, 32); else HBFP_COLS3_SR(PL, 64); } while (0)
@@ -2042,7 +2066,7 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
 #define HBFP_COLS_LAUNCH2(PL, NPX, SRV)                                                                                       \
     do {                                                                                                                       \
         HBFP_CUDA_OK(cudaFuncSetAttribute(im2col_cols<PL, NPX, SRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));   \
-        im2col_cols<PL, NPX, SRV><<<(unsigned)L.nkb, 256, smem, st>>>(x, (int)h, (int)w, lg_w, (int)c, kh, kw, pad, p, L.kst,     \
+        launch_chained(im2col_cols<PL, NPX, SRV>, (unsigned)L.nkb, 256, smem, st, x, (int)h, (int)w, lg_w, (int)c, kh, kw, pad, p, L.kst,     \
                                                                      L.plane_stride, L.rs, mant, exps);                        \
     } while (0)
 #define HBFP_COLS_LAUNCH(PL, NPX)                                                 \
@@ -2065,7 +2089,7 @@ int launch_conv_dgrad_filters(const Packed& c1, int taps, int64_t c_in, int64_t 
     if (c_in == 0) return HBFP_OK;
     if (Lo.rs != c_in) HBFP_CUDA_OK(cudaMemsetAsync(exps_out, 0, (size_t)Lo.exp_bytes, st));   // padding lines are zero
     const int64_t warps = c_in * taps;
-    conv_dgrad_filters_kernel<<<blocks_for(warps * 32, 256), 256, 0, st>>>(c1.mant, c1.exps, c1.L.kst, c1.L.plane_stride, c1.L.rs,
+    launch_chained(conv_dgrad_filters_kernel, blocks_for(warps * 32, 256), 256, 0, st, c1.mant, c1.exps, c1.L.kst, c1.L.plane_stride, c1.L.rs,
                                                                           taps, c_in, c_out, t, (int)c1.L.planes, mant_out, exps_out,
                                                                           Lo.kst, Lo.plane_stride, Lo.rs);
     return launch_status();
@@ -2075,7 +2099,7 @@ int launch_unpack(const Packed& p, int16_t* q, int8_t* s, cudaStream_t st) {
     const Layout& L = p.L;
     int64_t n = L.rows * (L.k > L.nkb ? L.k : L.nkb);
     if (n == 0) return HBFP_OK;
-    unpack_kernel<<<blocks_for(n, 256), 256, 0, st>>>(p.mant, p.exps, L.rows, L.k, L.b, L.bp, L.nkb, L.kst,
+    launch_chained(unpack_kernel, blocks_for(n, 256), 256, 0, st, p.mant, p.exps, L.rows, L.k, L.b, L.bp, L.nkb, L.kst,
                                                      L.plane_stride, (int)L.planes, L.rs, q, s);
     return launch_status();
 }
@@ -2090,6 +2114,7 @@ template <int V>
 __global__ void __launch_bounds__(256)
 wide_dequant_kernel(const int16_t* __restrict__ wide, const int8_t* __restrict__ exps, int64_t d0, int64_t d1, int t,
                     int64_t tiles1, float* __restrict__ out, int64_t ldo) {
+    chain_start();
     constexpr int ROWS = 4;
     const int64_t c = ((int64_t)blockIdx.x * 256 + threadIdx.x) * V;
     if (c >= d1) return;
@@ -2127,15 +2152,15 @@ int launch_wide_dequantize(const int16_t* wide, const int8_t* exps, int64_t d0, 
     const unsigned rows = (unsigned)std::min<int64_t>((d0 + 3) / 4, 65535);
     const bool vec = tile % 4 == 0 && d1 % 4 == 0 && ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(wide) & 7) == 0 &&
                      (reinterpret_cast<uintptr_t>(out) & 15) == 0;
-    if (vec) wide_dequant_kernel<4><<<dim3(blocks_for(d1, 1024), rows), 256, 0, st>>>(wide, exps, d0, d1, tile, tiles1, out, ldo);
-    else wide_dequant_kernel<1><<<dim3(blocks_for(d1, 256), rows), 256, 0, st>>>(wide, exps, d0, d1, tile, tiles1, out, ldo);
+    if (vec) launch_chained(wide_dequant_kernel<4>, dim3(blocks_for(d1, 1024), rows), 256, 0, st, wide, exps, d0, d1, tile, tiles1, out, ldo);
+    else launch_chained(wide_dequant_kernel<1>, dim3(blocks_for(d1, 256), rows), 256, 0, st, wide, exps, d0, d1, tile, tiles1, out, ldo);
     return launch_status();
 }
 
 int launch_dequantize(const Packed& p, float* out, int64_t ld, cudaStream_t st) {
     const Layout& L = p.L;
     if (L.rows * L.k == 0) return HBFP_OK;
-    dequant_kernel<<<blocks_for(L.rows * L.k, 256), 256, 0, st>>>(p.mant, p.exps, L.rows, L.k, L.b, L.bp, L.kst,
+    launch_chained(dequant_kernel, blocks_for(L.rows * L.k, 256), 256, 0, st, p.mant, p.exps, L.rows, L.k, L.b, L.bp, L.kst,
                                                                  L.plane_stride, (int)L.planes, L.rs, out, ld);
     return launch_status();
 }

@@ -633,3 +633,41 @@ def test_operand_forms_stay_inside_the_workspace_they_ask_for(hb, m, b, tiles):
     assert hb.last_gemm_launch().startswith("gemm_fp_kernel") and hb.device_status() == 0
     assert bool((ws[need:] == 55).all())
     assert torch.equal(got, hb.gemm_q(M, N, K, hb.quantize(A, 1, fa), hb.quantize(B, 0, fb), flags=hb.GEMM_FORCE_SIMT))
+
+
+# Kernels of a stream are placed before their predecessors have ended, and the second operand is converted beside the first: calls
+# that follow one another without a pause, over buffers that are rewritten between them, give what each gives alone. Routes: small
+# fused, forms (row and column conversions, split over clusters, pairs), integer kernels with and without split-K, few rows against
+# weights updated just before, whole-axis blocks.
+@pytest.mark.parametrize("M,N,K,m,b,rounding,tA,packed", [
+    (64, 96, 128, 8, 32, 1, 0, False), (1111, 777, 301, 8, 24, 1, 0, False), (512, 512, 4096, 8, 32, 0, 1, False), (2048, 2560, 256, 12, 64, 1, 0, False),
+    (300, 200, 4000, 8, 128, 0, 1, False), (2304, 2304, 1024, 8, 128, 0, 0, False), (130, 70, 1000, 8, 0, 0, 1, False), (512, 300, 24, 8, 24, 1, 0, False),
+    (16, 512, 768, 8, 64, 0, 0, True), (700, 512, 768, 12, 64, 1, 0, True), (700, 512, 768, 8, 128, 0, 0, True)])
+def test_calls_in_a_row_give_what_each_gives_alone(hb, M, N, K, m, b, rounding, tA, packed):
+    import torch
+    fa, fb = hb.Format(mant_bits=m, block=b, rounding=rounding, seed=3), hb.Format(mant_bits=m, block=b, rounding=rounding, seed=3, stream_id=1)
+    fw = hb.Format(mant_bits=m, block=b, tile=b, rounding=rounding, seed=3, stream_id=1)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    new = lambda *shape: torch.randn(*shape, device="cuda", generator=gen)
+    As = [new(K, M) if tA else new(M, K) for _ in range(4)]
+    Bs = [new(K, N) * 0.1 for _ in range(4)]
+
+    def run(pause):
+        A, B = torch.empty_like(As[0]), torch.empty_like(Bs[0])
+        wide, views = hb.wide_quantize(Bs[0], fw) if packed else (None, None)
+        out = []
+        for i in range(12):
+            A.copy_(As[i % 4])
+            B.copy_(Bs[(i + i // 4) % 4])
+            if pause: torch.cuda.synchronize()
+            if packed: hb.wide_update(wide, B, fw, views=views)
+            if pause: torch.cuda.synchronize()
+            for _ in range(2):
+                out.append(hb.gemm_q(M, N, K, A, views[0], fmtA=fa) if packed else hb.gemm(tA, 0, A, B, fa, fb))
+                if pause: torch.cuda.synchronize()
+        return out
+
+    want = run(True)
+    for _ in range(4):
+        assert all(torch.equal(x, y) for x, y in zip(run(False), want))
+    assert hb.device_status() == 0
