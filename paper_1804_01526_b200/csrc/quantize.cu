@@ -14,10 +14,12 @@
 //                    transposed tile with a swizzled TMA store (full lines in both directions).
 //   quant_col_block  blocks down the columns, any b <= 128 and any pitch: one K-block of 32 columns per CTA.
 //   quant_row_ragged blocks along rows, any b <= 128, row length, pitch and alignment, in one pass.
-//   tile_kernel      t x t weight tiles (t <= 128): one pass writes both packed views and
+//   tile_strip_kernel, tile_kernel_full   t x t weight tiles (t <= 128): one pass writes both packed views and
 //                    the tile exponent grid.
 //   exps_* / mant_generic   two-pass path for every other geometry (any b, any alignment).
 #include "quant_math.cuh"
+
+#include <type_traits>
 
 // This file is compiled twice. Part 1 (default) is the library's quantiser; part 2 holds only the launches of the
 // full-tile kernel for tiles of 32 and 64, built with another ptxas level (see build.py): measured on 8192 x 8192,
@@ -255,77 +257,18 @@ __device__ __forceinline__ void store_wide_values(float* dst, const uint32_t h[4
     reinterpret_cast<float4*>(dst)[1] = make_float4(c.x, c.y, d.x, d.y);
 }
 
-// qt rows have a pitch of tp + 2 halfwords, so that the column reads of view c0 spread over the banks.
-// sh: the views take the top bits of the words in qt (an arithmetic shift by sh bits); for wide storage qt
-// holds the stored words, i.e. the mantissas plus half a narrow unit (see tile_kernel); sh = 0 copies.
-template <int PLANES>
-__device__ __forceinline__ void write_tile_views(const int16_t* qt, int tp, int hi, int wj, int64_t i0, int64_t j0,
-                                                 int64_t u, int64_t v, int s, int sh, const TileViews& tv, int tid) {
-    const int qp = tp + 2;
-    const int lg = 31 - __clz(tp >> 2), gmask = (tp >> 2) - 1;       // tp is 32, 64 or 128
-    int8_t* const mant_c0 = tv.mant_c0; int8_t* const mant_c1 = tv.mant_c1;
-    int8_t* const exps_c0 = tv.exps_c0; int8_t* const exps_c1 = tv.exps_c1;
-    const int64_t kst0 = tv.kst0, ps0 = tv.ps0, rs0 = tv.rs0, nkb0 = tv.nkb0;
-    const int64_t kst1 = tv.kst1, ps1 = tv.ps1, rs1 = tv.rs1, nkb1 = tv.nkb1;
-    // view c1: row i0+ii gets bytes [v*tp, v*tp+tp) = qt[ii][0..tp)
-    if (mant_c1) for (int e = tid; e < hi * (tp / 4); e += 256) {
-        const int ii = e >> lg, g = (e & gmask) * 4;
-        uint32_t h = 0, l = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int q = qt[ii * qp + g + j] >> sh;
-            if (PLANES == 1) h |= (uint32_t)(q & 0xff) << (8 * j);
-            else { h |= (uint32_t)((q >> 4) & 0xff) << (8 * j); l |= (uint32_t)(q & 15) << (8 * j); }
-        }
-        int8_t* dst = mant_c1 + (i0 + ii) * kst1 + v * tp + g;
-        *reinterpret_cast<uint32_t*>(dst) = h;
-        if (PLANES == 2) *reinterpret_cast<uint32_t*>(dst + ps1) = l;
-    }
-    // view c0: row j0+jj gets bytes [u*tp, u*tp+tp) = qt[0..tp)[jj]
-    // (neighbouring threads write neighbouring words of one output row)
-    if (mant_c0) for (int e = tid; e < wj * (tp / 4); e += 256) {
-        const int jj = e >> lg, g = (e & gmask) * 4;
-        uint32_t h = 0, l = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int q = qt[(g + j) * qp + jj] >> sh;
-            if (PLANES == 1) h |= (uint32_t)(q & 0xff) << (8 * j);
-            else { h |= (uint32_t)((q >> 4) & 0xff) << (8 * j); l |= (uint32_t)(q & 15) << (8 * j); }
-        }
-        int8_t* dst = mant_c0 + (j0 + jj) * kst0 + u * tp + g;
-        *reinterpret_cast<uint32_t*>(dst) = h;
-        if (PLANES == 2) *reinterpret_cast<uint32_t*>(dst + ps0) = l;
-    }
-    // replicated exponents: exps_c1[v][i0+ii], exps_c0[u][j0+jj]
-    // (lines beyond the matrix, at most 15 after the last tile, are documented as zero)
-    const int pad1 = u == nkb0 - 1 ? (int)(rs1 - i0) : hi, pad0 = v == nkb1 - 1 ? (int)(rs0 - j0) : wj;
-    if (exps_c1) for (int e = tid; e < pad1; e += 256) exps_c1[v * rs1 + i0 + e] = e < hi ? (int8_t)s : (int8_t)0;
-    if (exps_c0) for (int e = tid; e < pad0; e += 256) exps_c0[u * rs0 + j0 + e] = e < wj ? (int8_t)s : (int8_t)0;
-    // row tails beyond the last tile: zero them (last tile column / last tile row only)
-    if (mant_c1 && v == nkb1 - 1)
-        for (int64_t e = tid; e < (int64_t)hi * ((kst1 - nkb1 * tp) / 4); e += 256) {
-            const int64_t per = (kst1 - nkb1 * tp) / 4, ii = e / per, o = nkb1 * tp + (e % per) * 4;
-            *reinterpret_cast<uint32_t*>(mant_c1 + (i0 + ii) * kst1 + o) = 0;
-            if (PLANES == 2) *reinterpret_cast<uint32_t*>(mant_c1 + ps1 + (i0 + ii) * kst1 + o) = 0;
-        }
-    if (mant_c0 && u == nkb0 - 1)
-        for (int64_t e = tid; e < (int64_t)wj * ((kst0 - nkb0 * tp) / 4); e += 256) {
-            const int64_t per = (kst0 - nkb0 * tp) / 4, jj = e / per, o = nkb0 * tp + (e % per) * 4;
-            *reinterpret_cast<uint32_t*>(mant_c0 + (j0 + jj) * kst0 + o) = 0;
-            if (PLANES == 2) *reinterpret_cast<uint32_t*>(mant_c0 + ps0 + (j0 + jj) * kst0 + o) = 0;
-        }
+// Stochastic rounding to 16 bits: floor((floor(y) + r) / 2^16) of y = x * 2^(16-s), which reaches 2^31, in 32 bits: the upper half of
+// floor(y) plus the carry of the lower one. (Saturated at +-2^31 the conversion leaves what the clamp makes of the value itself; a
+// NaN ends at the lower bound, as a conversion to 64 bits has it.)
+__device__ __forceinline__ int floor_wide(float y, uint32_t r) {
+    const int t = __float2int_rd(y);
+    const int q = (t >> 16) + (int)((((uint32_t)t & 0xFFFFu) + r) >> 16);
+    return y != y ? -32767 : clampq(q, 32767);
 }
-
-
-// Stochastic rounding to 16 bits: x * 2^(16-s) reaches 2^31, so the floor form runs in 64 bits.
-__device__ __forceinline__ int round_sr_wide(float x, int s, uint32_t r) {
-    const long long Y = __float2ll_rd(__fmul_rn(x, pow2f(16 - s)));
-    const long long q = (Y + (long long)r) >> 16;
-    return (int)max(-32767ll, min(32767ll, q));
-}
+__device__ __forceinline__ int round_sr_wide(float x, int s, uint32_t r) { return floor_wide(__fmul_rn(x, pow2f(16 - s)), r); }
 
 // Weight matrices with one exponent per t x t tile (Sec. 4.2 "Tiling", t <= 128) and their wide storage
-// (Sec. 4.2 "Wide weight storage"): one CTA per tile of w [d0][d1], 256 threads.
+// (Sec. 4.2 "Wide weight storage"), for every tile geometry, alignment and width that tile_kernel_full does not take.
 //   MODE 3  quantise FP32 weights src (pitch ld) straight to p.m bits (no wide copy)
 //   MODE 0  quantise FP32 weights src to wide storage: int16 mantissas `wide` (row-major, pitch d1) and
 //           one exponent per tile in grid [tiles along d0][tiles along d1]
@@ -338,162 +281,277 @@ __device__ __forceinline__ int round_sr_wide(float x, int s, uint32_t r) {
 //   c1: rows = d0, contraction along d1 (the stored orientation);  c0: rows = d1, contraction along d0
 // with, for the wide modes, the top p.m bits of the stored 16-bit words (the mantissa plus half a narrow
 // unit: rounded to nearest, clamped to the symmetric range) under the exponent s + 16 - p.m.
-// FAST: t, d1 multiples of 8, pitches and bases 16-byte aligned: a thread handles eight consecutive
-// weights of a row at a time (two 128-bit loads, one Philox call, 128-bit store of the int16 mantissas).
-template <int MODE, int PLANES, bool FAST>
-__global__ void __launch_bounds__(256)
-tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, int t, int tp, QParams p,
-            int16_t* __restrict__ wide, int8_t* __restrict__ grid, int64_t grid_ld, TileViews tv) {
+//
+// Bound by HBM in the limit and by instructions and the latency of its phases before it. A CTA takes a strip of 2^lg_rv x cv tiles, up
+// to 64 rows x 32 KC columns (128 x 128 for tiles above 64): with a CTA per tile, 576 weights of a 24 x 24 tile had 256 threads, five
+// barriers and a start of their own. A warp owns whole rows of one tile row, its lanes consecutive columns, so that every load and
+// store of an unaligned matrix is 32 neighbours; the values stay in registers between the maxima and the rounding. The narrow
+// mantissas go to shared memory in padded coordinates (tile columns and rows tp apart, zeros between), from which view c1 leaves as
+// words of whole rows and view c0 as byte-transposed blocks of 4 columns x 16 rows. Draws are made once per eight weights, into a
+// table per warp. What a thread does once has to be little, it holds only 16 to 32 weights: the counts of tiles and the reciprocal of
+// t come from the host (with 64-bit divisions, predicates on every access and a row of view c1 per warp the same strips took 116
+// instructions per weight of a lane instead of 50). Updates, a CTA per tile before / this: 8192 x 8191, t = 64 355 / 169 us, with draws
+// 504 / 240; 2000 x 3001, t = 24, with draws 96 / 28; 6000 x 6000, t = 24, 12 bits, with draws 279 / 159; 500 x 500, t = 32 8.3 / 6.6.
+struct StripShape {
+    int t, tp, lg_tp, cv, lg_rv, rpw;             // cv * t <= 32 KC, cv * tp <= 160, rpw: rows of a warp
+    int recip, recip_per;                         // ceil(2^16 / t), ceil(2^20 / (cv * tp / 8)): exact for the indices of a strip
+    int nu, nv;                                   // tiles along d0 and d1
+};
+
+// NW warps of up to RPW rows, KC columns per lane.
+template <int MODE, int PLANES, int NW, int RPW, int KC, bool SR>
+__global__ void __launch_bounds__(32 * NW, NW == 16 ? 1 : 4)
+tile_strip_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, const StripShape sh, QParams p,
+                  int16_t* __restrict__ wide, int8_t* __restrict__ grid, int64_t grid_ld, TileViews tv) {
     chain_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int fp = FAST ? t + 4 : t + 1;                                   // pitch of the FP32 tile
-    float* tile = reinterpret_cast<float*>(smem_raw);                      // [t][fp]
-    const int qp = tp + 2;
-    int16_t* qt = reinterpret_cast<int16_t*>(tile + (size_t)t * fp);       // [tp][tp + 2], zero padded
-    __shared__ uint32_t s_am[8];
-    __shared__ int s_exp;
-
-    const int tid = threadIdx.x, lane = tid & 31, wrow = tid >> 5;
-    const int64_t u = blockIdx.y, v = blockIdx.x;       // tile row (along d0), tile column (along d1)
-    const int64_t i0 = u * t, j0 = v * t;
-    const int hi = (int)min((int64_t)t, d0 - i0), wj = (int)min((int64_t)t, d1 - j0);
-    const int G = wj >> 3;                              // FAST: groups of eight per tile row
     constexpr bool UPDATE = MODE == 1 || MODE == 4;
-    const int wbits = MODE == 3 ? p.m : 16, wqmax = MODE == 3 ? p.qmax : 32767;
-    // Wide modes: qt holds the stored word the views are cut from: the mantissa plus half a narrow unit,
-    // held inside the range whose top bits stay within +-qmax (so the shift alone rounds to nearest and
-    // saturates symmetrically). MODE 3 copies (sh = 0).
-    const int sh = MODE == 3 ? 0 : 16 - p.m;
-    const int half = sh > 0 ? 1 << (sh - 1) : 0;
-    const int w_hi = ((p.qmax + 1) << sh) - half - 1, w_lo = -(p.qmax << sh) - half;
-    const uint32_t w_hi2 = ((uint32_t)w_hi & 0xFFFFu) * 0x10001u, w_lo2 = ((uint32_t)w_lo & 0xFFFFu) * 0x10001u;
-    const uint32_t half2 = (uint32_t)half * 0x10001u;
-    auto stored_pair = [&](uint32_t h) { return MODE == 3 ? h : __vadd2(__vmaxs2(__vmins2(h, w_hi2), w_lo2), half2); };
-    auto stored_one = [&](int q) { return MODE == 3 ? q : max(w_lo, min(w_hi, q)) + half; };
-    for (int e = tid; e < tp * qp / 2; e += 256) reinterpret_cast<uint32_t*>(qt)[e] = 0;
-    int s;
+    constexpr int GROUPS = 4 * KC + 1, NT = 32 * NW, LG_NW = NW == 16 ? 4 : 3;      // GROUPS: eights of draws that a row's columns touch
+    const int t = sh.t, tp = sh.tp, cv = sh.cv, rv = 1 << sh.lg_rv, lw = LG_NW - sh.lg_rv;      // 2^lw warps per tile row
+    const int qp = cv * tp + 8;                                            // halfword pitch of qt
+    int16_t* qt = reinterpret_cast<int16_t*>(smem_raw);                    // [rv * tp][qp]
+    uint4* rnd = reinterpret_cast<uint4*>(smem_raw + (size_t)rv * tp * qp * 2);               // [NW][RPW][GROUPS] (SR)
+    __shared__ uint32_t pm[NW][32 * KC];
+    __shared__ int s_exp[64];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int u0 = (int)blockIdx.y << sh.lg_rv, v0 = (int)blockIdx.x * cv;
+    const int64_t i00 = (int64_t)u0 * t, j0 = (int64_t)v0 * t;             // first row and column of the strip
+    const int wj = (int)min((int64_t)(cv * t), d1 - j0), tiles = min(cv, sh.nv - v0);          // columns and tile columns of the strip
+    // this warp's rows: nrow from row0 on, in tile row u0 + ur
+    const int ur = warp >> lw, rb = (warp & ((1 << lw) - 1)) * sh.rpw;
+    const int64_t row0 = i00 + ur * t + rb;
+    const int nrow = u0 + ur < sh.nu ? max(0, (int)min((int64_t)min(sh.rpw, t - rb), d0 - row0)) : 0;
+    int tile_of[KC], qcol[KC];
+    bool in[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+        const int c = lane + 32 * k;
+        in[k] = c < wj;
+        tile_of[k] = in[k] ? (c * sh.recip) >> 16 : 0;
+        qcol[k] = in[k] ? tile_of[k] * (tp - t) + c : 0;
+    }
+    const int nsh = MODE == 3 ? 0 : 16 - p.m, half = nsh > 0 ? 1 << (nsh - 1) : 0;
+    // the top bits of the stored word plus half a narrow unit, held inside the symmetric range
+    auto narrow = [&](int q) { return MODE == 3 ? q : clampq((q + half) >> nsh, p.qmax); };
+    const bool views = tv.mant_c0 != nullptr || tv.mant_c1 != nullptr;
+    if (views && (t != tp || wj < cv * t || (int64_t)(u0 + rv) * t > d0))
+        for (int e = tid; e < rv * tp * qp / 8; e += NT) reinterpret_cast<uint4*>(qt)[e] = make_uint4(0u, 0u, 0u, 0u);
+    int16_t* const qrow = qt + (ur * tp + rb) * qp;
+    const float* const srow = src + row0 * ld + j0 + lane;
+    int16_t* const wrow = wide + row0 * d1 + j0 + lane;
     if (MODE == 2) {
-        __syncthreads();
-        s = grid[u * grid_ld + v];
-        if (FAST) {
-            for (int item = tid; item < hi * G; item += 256) {
-                const int ii = item / G, gj = item - ii * G;
-                const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
-                uint32_t* dst = reinterpret_cast<uint32_t*>(qt + ii * qp + 8 * gj);
-                dst[0] = stored_pair(q8.x); dst[1] = stored_pair(q8.y); dst[2] = stored_pair(q8.z); dst[3] = stored_pair(q8.w);
-            }
-        } else {
-            for (int ii = wrow; ii < hi; ii += 8)
-                for (int jj = lane; jj < wj; jj += 32) qt[ii * qp + jj] = (int16_t)stored_one(wide[(i0 + ii) * d1 + j0 + jj]);
+        if (tid < rv * cv) {
+            const int uu = u0 + tid / cv, vv = v0 + tid % cv;
+            s_exp[tid] = uu < sh.nu && vv < sh.nv ? grid[uu * grid_ld + vv] : 0;
         }
+        __syncthreads();                                                   // the zeros are written
+        int w[RPW][KC];
+#pragma unroll
+        for (int r = 0; r < RPW; ++r)
+#pragma unroll
+            for (int k = 0; k < KC; ++k) w[r][k] = r < nrow && in[k] ? wrow[r * d1 + 32 * k] : 0;
+#pragma unroll
+        for (int r = 0; r < RPW; ++r)
+            if (r < nrow)
+#pragma unroll
+                for (int k = 0; k < KC; ++k)
+                    if (in[k]) qrow[r * qp + qcol[k]] = (int16_t)narrow(w[r][k]);
     } else {
-        const float old_scale = UPDATE ? pow2f(grid[u * grid_ld + v]) : 0.f;
-        uint32_t am = 0;
-        if (FAST) {
-            for (int item = tid; item < hi * G; item += 256) {
-                const int ii = item / G, gj = item - ii * G;
-                const float4* sp = reinterpret_cast<const float4*>(src + (i0 + ii) * ld + j0 + 8 * gj);
-                float4 a = __ldcs(sp), b = __ldcs(sp + 1);
-                if (UPDATE) {
-                    const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
-                    a.x = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x & 0xFFFFu), old_scale), a.x);
-                    a.y = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x >> 16), old_scale), a.y);
-                    a.z = __fadd_rn(__fmul_rn((float)(int16_t)(q8.y & 0xFFFFu), old_scale), a.z);
-                    a.w = __fadd_rn(__fmul_rn((float)(int16_t)(q8.y >> 16), old_scale), a.w);
-                    b.x = __fadd_rn(__fmul_rn((float)(int16_t)(q8.z & 0xFFFFu), old_scale), b.x);
-                    b.y = __fadd_rn(__fmul_rn((float)(int16_t)(q8.z >> 16), old_scale), b.y);
-                    b.z = __fadd_rn(__fmul_rn((float)(int16_t)(q8.w & 0xFFFFu), old_scale), b.z);
-                    b.w = __fadd_rn(__fmul_rn((float)(int16_t)(q8.w >> 16), old_scale), b.w);
-                }
-                float4* tp4 = reinterpret_cast<float4*>(tile + ii * fp + 8 * gj);
-                tp4[0] = a; tp4[1] = b;
-                const float e8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                am = max(am, amax8_bits(e8));
-            }
-        } else {
-            for (int ii = wrow; ii < hi; ii += 8)
-                for (int jj = lane; jj < wj; jj += 32) {
-                    float val = src[(i0 + ii) * ld + j0 + jj];
-                    if (UPDATE) val = __fadd_rn(__fmul_rn((float)wide[(i0 + ii) * d1 + j0 + jj], old_scale), val);
-                    tile[ii * fp + jj] = val;
-                    am = max(am, abs_bits(val));
-                }
-        }
-        for (int off = 16; off > 0; off >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
-        if (lane == 0) s_am[wrow] = am;
-        __syncthreads();
-        if (tid == 0) {
-            uint32_t a = 0;
-            for (int i = 0; i < 8; ++i) a = max(a, s_am[i]);
-            s_exp = block_exponent(a, wbits, p.exp_mode);
-            if (grid) grid[u * grid_ld + v] = (int8_t)s_exp;
-        }
-        __syncthreads();
-        s = s_exp;
-        if (FAST) {
-            const uint32_t qm = qmax_pair(wqmax), nqm = neg_qmax_pair(wqmax);
-            for (int item = tid; item < hi * G; item += 256) {
-                const int ii = item / G, gj = item - ii * G;
-                const float4* tp4 = reinterpret_cast<const float4*>(tile + ii * fp + 8 * gj);
-                const float4 a = tp4[0], b = tp4[1];
-                const float e8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-                uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                if (p.rounding == 1) w = draws_of_group(p, (uint64_t)((i0 + ii) * d1 + j0 + 8 * gj) >> 3);
-                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-                uint32_t h[4];
-                if (MODE == 3) {
-                    // at most 12 bits: the packed halfword forms
-                    const float sc = pow2f(p.rounding == 1 ? 16 - s : -s);
+        // FULL: no row or column of the strip is missing, and nothing asks
+        auto convert = [&](auto is_full) {
+            constexpr bool FULL = decltype(is_full)::value;
+            float x[RPW][KC];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        h[j] = p.rounding == 1 ? round_sr_pair(e8[2 * j], e8[2 * j + 1], sc, ww[j], qm, nqm)
-                                               : round_rne_pair(e8[2 * j], e8[2 * j + 1], sc, qm, nqm);
-                } else {
+            for (int r = 0; r < RPW; ++r)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        int q0, q1;
-                        if (p.rounding == 0) {
-                            q0 = round_rne(e8[2 * j], s, 32767);
-                            q1 = round_rne(e8[2 * j + 1], s, 32767);
-                        } else {
-                            q0 = round_sr_wide(e8[2 * j], s, ww[j] & 0xFFFFu);
-                            q1 = round_sr_wide(e8[2 * j + 1], s, ww[j] >> 16);
-                        }
-                        h[j] = ((uint32_t)q0 & 0xFFFFu) | ((uint32_t)q1 << 16);
+                for (int k = 0; k < KC; ++k) x[r][k] = FULL || (r < nrow && in[k]) ? __ldcs(srow + r * ld + 32 * k) : 0.f;
+            uint4* const my_rnd = rnd + warp * (RPW * GROUPS);
+            // while the loads are in flight; rows that all start with an eight of draws touch one less of them
+            auto draw_eights = [&](auto count) {
+                constexpr int N = decltype(count)::value;
+                for (int i = lane; i < nrow * N; i += 32) {
+                    const int r = i / N, g = i - r * N;
+                    const uint64_t L0 = (uint64_t)((row0 + r) * d1 + j0);
+                    if (8 * g < (int)(L0 & 7) + wj) my_rnd[r * GROUPS + g] = draws_of_group(p, (L0 >> 3) + g);
+                }
+            };
+            auto draw = [&]() {
+                if ((((uint32_t)d1 | (uint32_t)j0) & 7) == 0) draw_eights(std::integral_constant<int, GROUPS - 1>{});
+                else draw_eights(std::integral_constant<int, GROUPS>{});
+            };
+            if (UPDATE) {
+                // the wide words of (at most) eighteen weights at a time, requested together
+                constexpr int RW = RPW * KC <= 18 ? RPW : RPW / 2;
+#pragma unroll
+                for (int r0 = 0; r0 < RPW; r0 += RW) {
+                    int w[RW][KC];
+#pragma unroll
+                    for (int r = 0; r < RW; ++r)
+#pragma unroll
+                        for (int k = 0; k < KC; ++k) w[r][k] = FULL || (r0 + r < nrow && in[k]) ? wrow[(r0 + r) * d1 + 32 * k] : 0;
+                    if (SR && r0 == 0) draw();
+#pragma unroll
+                    for (int k = 0; k < KC; ++k) {
+                        const float old_scale = FULL || nrow > 0 ? pow2f(grid[(u0 + ur) * grid_ld + v0 + tile_of[k]]) : 0.f;
+                        // the product is exact: one rounding
+#pragma unroll
+                        for (int r = 0; r < RW; ++r) x[r0 + r][k] = __fmaf_rn((float)w[r][k], old_scale, x[r0 + r][k]);
                     }
                 }
-                uint32_t* dst = reinterpret_cast<uint32_t*>(qt + ii * qp + 8 * gj);
-                dst[0] = stored_pair(h[0]); dst[1] = stored_pair(h[1]); dst[2] = stored_pair(h[2]); dst[3] = stored_pair(h[3]);
-                if (MODE != 3) *reinterpret_cast<uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) = make_uint4(h[0], h[1], h[2], h[3]);
-                if (MODE == 4) store_wide_values(tv.value + (i0 + ii) * tv.ldv + j0 + 8 * gj, h, pow2f_stored(s));
+            } else if (SR) {
+                draw();
             }
-        } else {
-            for (int ii = wrow; ii < hi; ii += 8)
-                for (int jj = lane; jj < wj; jj += 32) {
-                    const float val = tile[ii * fp + jj];
-                    const uint64_t L = (uint64_t)((i0 + ii) * d1 + j0 + jj);
-                    int q;
-                    if (MODE == 3) q = quantize_one(val, s, p, L);
-                    else if (p.rounding == 0) q = round_rne(val, s, 32767);
-                    else q = round_sr_wide(val, s, draw_of_element(p, L));
-                    qt[ii * qp + jj] = (int16_t)stored_one(q);
-                    if (MODE != 3) wide[(i0 + ii) * d1 + j0 + jj] = (int16_t)q;
-                    if (MODE == 4) tv.value[(i0 + ii) * tv.ldv + j0 + jj] = __fmul_rn((float)q, pow2f_stored(s));
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                uint32_t am = 0;
+#pragma unroll
+                for (int r = 0; r < RPW; r += 2) am = max3_abs_bits(am, x[r][k], x[r + 1][k]);
+                pm[warp][lane + 32 * k] = am;
+            }
+            __syncthreads();
+            // a warp per tile
+            for (int i = warp; i < rv * cv; i += NW) {
+                const int uu = i / cv, vv = i - uu * cv;
+                uint32_t am = 0;
+                for (int c = vv * t + lane; c < (vv + 1) * t; c += 32)
+                    for (int w = 0; w < 1 << lw; ++w) am = max(am, pm[(uu << lw) + w][c]);
+                am = __reduce_max_sync(0xffffffffu, am);
+                if (lane == 0) {
+                    const int s = block_exponent(am, MODE == 3 ? p.m : 16, p.exp_mode);
+                    s_exp[i] = s;
+                    if (grid && u0 + uu < sh.nu && vv < tiles) grid[(u0 + uu) * grid_ld + v0 + vv] = (int8_t)s;
                 }
+            }
+            __syncthreads();
+            const uint16_t* drow = reinterpret_cast<const uint16_t*>(my_rnd) + lane;
+            const uint32_t first = SR ? (uint32_t)((uint64_t)(row0 * d1 + j0) & 7) : 0u, row_step = (uint32_t)(d1 & 7);
+            float scale[KC];
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                const int s = s_exp[ur * cv + tile_of[k]];
+                scale[k] = SR ? pow2f(16 - s) : pow2f(-s);
+            }
+#pragma unroll
+            for (int r = 0; r < RPW; ++r)
+                if (FULL || r < nrow) {
+                    const uint16_t* dr = drow + r * (8 * GROUPS) + ((first + r * row_step) & 7);
+#pragma unroll
+                    for (int k = 0; k < KC; ++k) {
+                        const float y = __fmul_rn(x[r][k], scale[k]);
+                        int q;
+                        if (!SR) {
+                            q = clampq(__float2int_rn(y), MODE == 3 ? p.qmax : 32767);
+                        } else if (MODE == 3) {
+                            q = clampq((__float2int_rd(y) + (int)dr[32 * k]) >> 16, p.qmax);
+                        } else {
+                            q = floor_wide(y, dr[32 * k]);
+                        }
+                        if (FULL || in[k]) {
+                            if (MODE != 3) wrow[r * d1 + 32 * k] = (int16_t)q;
+                            if (MODE == 4) tv.value[(row0 + r) * tv.ldv + j0 + lane + 32 * k] = __fmul_rn((float)q, pow2f_stored(s_exp[ur * cv + tile_of[k]]));
+                            qrow[r * qp + qcol[k]] = (int16_t)narrow(q);
+                        }
+                    }
+                }
+        };
+        if (wj == 32 * KC && sh.rpw == RPW && t == RPW << lw && u0 + rv <= sh.nu && i00 + rv * t <= d0) convert(std::true_type{});
+        else convert(std::false_type{});
+    }
+    if (!views) return;
+    __syncthreads();
+    // bytes of a view from pairs of narrow mantissas: plane 0 the upper (or only) eight bits, plane 1 the four below
+    auto upper = [](uint2 q) {
+        return PLANES == 2 ? __byte_perm((q.x >> 4) & 0x00ff00ffu, (q.y >> 4) & 0x00ff00ffu, 0x6420) : __byte_perm(q.x, q.y, 0x6420);
+    };
+    auto lower = [](uint2 q) { return __byte_perm(q.x & 0x000f000fu, q.y & 0x000f000fu, 0x6420); };
+    // view c1: row i gets bytes [v0 tp, (v0 + tiles) tp) in pieces of eight, and zeros beyond the last tile
+    if (tv.mant_c1) {
+        int8_t* const base = tv.mant_c1 + i00 * tv.kst1 + (int64_t)v0 * tp;
+        const int per = cv * tp / 8;
+        for (int e = tid; e < rv * tp * per; e += NT) {
+            const int r = (int)((uint32_t)(e * sh.recip_per) >> 20), w = 8 * (e - r * per), uu = r >> sh.lg_tp, ii = r & (tp - 1), i = uu * t + ii;
+            if (ii >= t || i00 + i >= d0 || w >= tiles * tp) continue;
+            const uint4 q = *reinterpret_cast<const uint4*>(qt + r * qp + w);
+            int8_t* dst = base + i * tv.kst1 + w;
+            *reinterpret_cast<uint2*>(dst) = make_uint2(upper(make_uint2(q.x, q.y)), upper(make_uint2(q.z, q.w)));
+            if (PLANES == 2) *reinterpret_cast<uint2*>(dst + tv.ps1) = make_uint2(lower(make_uint2(q.x, q.y)), lower(make_uint2(q.z, q.w)));
+        }
+        if (v0 + tiles == sh.nv && (int64_t)sh.nv * tp < tv.kst1)
+            for (int i = warp; i < rv * t && i00 + i < d0; i += NW)
+                for (int64_t o = (int64_t)sh.nv * tp + 4 * lane; o < tv.kst1; o += 128) {
+                    *reinterpret_cast<uint32_t*>(tv.mant_c1 + (i00 + i) * tv.kst1 + o) = 0u;
+                    if (PLANES == 2) *reinterpret_cast<uint32_t*>(tv.mant_c1 + tv.ps1 + (i00 + i) * tv.kst1 + o) = 0u;
+                }
+    }
+    // view c0: row j gets bytes [u0 tp, ...): blocks of 4 columns x 16 rows of qt, byte-transposed
+    if (tv.mant_c0) {
+        const int ncol4 = tiles * tp / 4;
+        for (int e = tid; e < ncol4 * (rv * tp / 16); e += NT) {
+            const int g = (int)((uint32_t)e / (uint32_t)ncol4), c = 4 * (e - g * ncol4), vv = c >> sh.lg_tp, jin = c & (tp - 1);
+            if (u0 + ((16 * g) >> sh.lg_tp) >= sh.nu) continue;
+            const int64_t j = j0 + vv * t + jin;
+            const int cols = (int)min((int64_t)(t - jin), d1 - j);         // of the four that exist
+            if (cols <= 0) continue;
+            uint32_t out[PLANES][4][4];
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                uint2 q[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const uint2*>(qt + (16 * g + 4 * b + i) * qp + c);
+#pragma unroll
+                for (int pl = 0; pl < PLANES; ++pl) {
+                    const uint32_t R0 = pl ? lower(q[0]) : upper(q[0]), R1 = pl ? lower(q[1]) : upper(q[1]);
+                    const uint32_t R2 = pl ? lower(q[2]) : upper(q[2]), R3 = pl ? lower(q[3]) : upper(q[3]);
+                    const uint32_t t0 = __byte_perm(R0, R1, 0x5140), t1 = __byte_perm(R2, R3, 0x5140);
+                    const uint32_t t2 = __byte_perm(R0, R1, 0x7362), t3 = __byte_perm(R2, R3, 0x7362);
+                    out[pl][0][b] = __byte_perm(t0, t1, 0x5410);
+                    out[pl][1][b] = __byte_perm(t0, t1, 0x7632);
+                    out[pl][2][b] = __byte_perm(t2, t3, 0x5410);
+                    out[pl][3][b] = __byte_perm(t2, t3, 0x7632);
+                }
+            }
+            int8_t* dst = tv.mant_c0 + j * tv.kst0 + (int64_t)u0 * tp + 16 * g;
+#pragma unroll
+            for (int pl = 0; pl < PLANES; ++pl)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < cols)
+                        *reinterpret_cast<uint4*>(dst + pl * tv.ps0 + i * tv.kst0) = make_uint4(out[pl][i][0], out[pl][i][1], out[pl][i][2], out[pl][i][3]);
+        }
+        if (u0 + rv >= sh.nu && (int64_t)sh.nu * tp < tv.kst0)             // the row tails
+            for (int c = warp; c < wj; c += NW)
+                for (int64_t o = (int64_t)sh.nu * tp + 4 * lane; o < tv.kst0; o += 128) {
+                    *reinterpret_cast<uint32_t*>(tv.mant_c0 + (j0 + c) * tv.kst0 + o) = 0u;
+                    if (PLANES == 2) *reinterpret_cast<uint32_t*>(tv.mant_c0 + tv.ps0 + (j0 + c) * tv.kst0 + o) = 0u;
+                }
+    }
+    // replicated exponents: exps_c1[v][i], exps_c0[u][j] (lines beyond the matrix, at most 15 after the last tile, are documented as zero)
+    for (int i = warp; i < rv * cv; i += NW) {
+        const int uu = i / cv, vv = i - uu * cv;
+        if (u0 + uu >= sh.nu || vv >= tiles) continue;
+        const int8_t se = (int8_t)(s_exp[i] + nsh);
+        const int64_t ia = i00 + uu * t, ja = j0 + vv * t;
+        if (tv.exps_c1) {
+            const int64_t end = u0 + uu == sh.nu - 1 ? tv.rs1 : ia + t;
+            for (int64_t r = ia + lane; r < end; r += 32) tv.exps_c1[(v0 + vv) * tv.rs1 + r] = r < d0 ? se : (int8_t)0;
+        }
+        if (tv.exps_c0) {
+            const int64_t end = v0 + vv == sh.nv - 1 ? tv.rs0 : ja + t;
+            for (int64_t c = ja + lane; c < end; c += 32) tv.exps_c0[(u0 + uu) * tv.rs0 + c] = c < d1 ? se : (int8_t)0;
         }
     }
-    if (tv.mant_c0 == nullptr && tv.mant_c1 == nullptr) return;
-    __syncthreads();
-    write_tile_views<PLANES>(qt, tp, hi, wj, i0, j0, u, v, s + sh, sh, tv, tid);
 }
 
-// Full tiles of 32, 64 or 128 (the tile is its own padded width), aligned rows: the same arithmetic as
-// tile_kernel with far fewer instructions per weight. A thread keeps its groups of eight weights in registers
+// Tiles of 32, 64 or 128 (the tile is its own padded width), aligned rows of whole eights: the same arithmetic as
+// tile_strip_kernel with fewer instructions per weight. A thread keeps its groups of eight weights in registers
 // between the maximum and the rounding pass (no FP32 tile in shared memory); the rounded words go to a 16-bit
 // tile in shared memory once, from which view c1 leaves as 8-byte pieces cut by byte permutes and view c0 as
 // the byte-transposes of 4 x 4 blocks (eight permutes per block) instead of one shared-memory load, shift and
 // mask per byte. ROWS4 = 4 x 4 blocks stacked per thread for view c0 (wider stores per output row).
-template <int MODE, int PLANES, int TP>
+// GENERAL: the last tile of a row or column of tiles is smaller (its missing groups are zeros), or the width is one that is cut early;
+// a parameter, so that whole tiles ask nothing (8192 x 8192, t = 64: 113 us, 115 with the question). Updates, the kernel for any tile
+// before / this: 1111 x 5000, t = 64, draws 20.6 / 14.2 us, 3000 x 3000, t = 128 28.8 / 23.8, 4096 x 4096, t = 64, 4 bits 51.3 / 34.2.
+template <int MODE, int PLANES, int TP, bool GENERAL>
 __global__ void __launch_bounds__(256)
 tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, QParams p,
                  int16_t* __restrict__ wide, int8_t* __restrict__ grid, int64_t grid_ld, TileViews tv) {
@@ -508,6 +566,8 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
     const int tid = threadIdx.x, lane = tid & 31, wrow = tid >> 5;
     const int64_t u = blockIdx.y, v = blockIdx.x;
     const int64_t i0 = u * TP, j0 = v * TP;
+    const int hi = GENERAL ? (int)min((int64_t)TP, d0 - i0) : TP, wj = GENERAL ? (int)min((int64_t)TP, d1 - j0) : TP;
+    auto there = [&](int ii, int gj) { return !GENERAL || (ii < hi && 8 * gj < wj); };
     constexpr bool UPDATE = MODE == 1 || MODE == 4;
     const int wbits = MODE == 3 ? p.m : 16, wqmax = MODE == 3 ? p.qmax : 32767;
     const int sh = MODE == 3 ? 0 : 16 - p.m;
@@ -515,7 +575,13 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
     const int w_hi = ((p.qmax + 1) << sh) - half - 1, w_lo = -(p.qmax << sh) - half;
     const uint32_t w_hi2 = ((uint32_t)w_hi & 0xFFFFu) * 0x10001u, w_lo2 = ((uint32_t)w_lo & 0xFFFFu) * 0x10001u;
     const uint32_t half2 = (uint32_t)half * 0x10001u;
-    auto stored_pair = [&](uint32_t h) { return MODE == 3 ? h : __vadd2(__vmaxs2(__vmins2(h, w_hi2), w_lo2), half2); };
+    // A 32-bit shift may drag the upper halfword's bits into the lower one's byte: widths too narrow for that are shifted here.
+    const bool early = GENERAL && MODE != 3 && sh + (PLANES == 2 ? 4 : 0) > 8;
+    auto stored_pair = [&](uint32_t h) {
+        if (MODE == 3) return h;
+        const uint32_t w = __vadd2(__vmaxs2(__vmins2(h, w_hi2), w_lo2), half2);
+        return early ? __byte_perm((uint32_t)((int)(int16_t)w >> sh), (uint32_t)((int)w >> (16 + sh)), 0x5410) : w;
+    };
     int s;
     if (MODE == 2) {
         s = grid[u * grid_ld + v];
@@ -524,7 +590,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
             const int item = tid + 256 * k;
             if (NITEMS % 256 == 0 || item < NITEMS) {
                 const int ii = item / G, gj = item - ii * G;
-                const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
+                const uint4 q8 = there(ii, gj) ? *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) : make_uint4(0u, 0u, 0u, 0u);
                 *reinterpret_cast<uint4*>(qt + ii * QP + 8 * gj) = make_uint4(stored_pair(q8.x), stored_pair(q8.y), stored_pair(q8.z), stored_pair(q8.w));
             }
         }
@@ -542,8 +608,10 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
             if (NITEMS % 256 == 0 || item < NITEMS) {
                 const int ii = item / G, gj = item - ii * G;
                 const float4* sp = reinterpret_cast<const float4*>(src + (i0 + ii) * ld + j0 + 8 * gj);
-                a[k] = __ldcs(sp);
-                b[k] = __ldcs(sp + 1);
+                if (there(ii, gj)) {
+                    a[k] = __ldcs(sp);
+                    b[k] = __ldcs(sp + 1);
+                }
             }
         }
         if (UPDATE) {
@@ -552,7 +620,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
                 const int item = tid + 256 * k;
                 if (NITEMS % 256 == 0 || item < NITEMS) {
                     const int ii = item / G, gj = item - ii * G;
-                    const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
+                    const uint4 q8 = there(ii, gj) ? *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) : make_uint4(0u, 0u, 0u, 0u);
                     a[k].x = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x & 0xFFFFu), old_scale), a[k].x);
                     a[k].y = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x >> 16), old_scale), a[k].y);
                     a[k].z = __fadd_rn(__fmul_rn((float)(int16_t)(q8.y & 0xFFFFu), old_scale), a[k].z);
@@ -612,8 +680,8 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
                     }
                 }
                 *reinterpret_cast<uint4*>(qt + ii * QP + 8 * gj) = make_uint4(stored_pair(h[0]), stored_pair(h[1]), stored_pair(h[2]), stored_pair(h[3]));
-                if (MODE != 3) *reinterpret_cast<uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) = make_uint4(h[0], h[1], h[2], h[3]);
-                if (MODE == 4) store_wide_values(tv.value + (i0 + ii) * tv.ldv + j0 + 8 * gj, h, pow2f_stored(s));
+                if (MODE != 3 && there(ii, gj)) *reinterpret_cast<uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) = make_uint4(h[0], h[1], h[2], h[3]);
+                if (MODE == 4 && there(ii, gj)) store_wide_values(tv.value + (i0 + ii) * tv.ldv + j0 + 8 * gj, h, pow2f_stored(s));
             }
         }
     }
@@ -621,7 +689,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
     __syncthreads();
     // Bytes of the views from pairs of stored halfwords: plane 0 takes bits [sh + 4 (PLANES - 1), + 8) of each
     // halfword, plane 1 the four bits below; the masks remove what a 32-bit shift drags across the halfwords.
-    const int sh_hi = sh + (PLANES == 2 ? 4 : 0);
+    const int sh_lo = early ? 0 : sh, sh_hi = sh_lo + (PLANES == 2 ? 4 : 0);
     auto bytes4 = [&](uint32_t w0, uint32_t w1, int k, uint32_t mask) {
         return __byte_perm((w0 >> k) & mask, (w1 >> k) & mask, 0x6420);
     };
@@ -632,11 +700,12 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
         const int item = tid + 256 * k;
         if (NITEMS % 256 == 0 || item < NITEMS) {
             const int ii = item / G, gj = item - ii * G;
+            if (GENERAL && ii >= hi) continue;
             const uint4 q8 = *reinterpret_cast<const uint4*>(qt + ii * QP + 8 * gj);
             int8_t* dst = tv.mant_c1 + (i0 + ii) * tv.kst1 + v * TP + 8 * gj;
             *reinterpret_cast<uint2*>(dst) = make_uint2(bytes4(q8.x, q8.y, sh_hi, 0x00ff00ffu), bytes4(q8.z, q8.w, sh_hi, 0x00ff00ffu));
             if (PLANES == 2)
-                *reinterpret_cast<uint2*>(dst + tv.ps1) = make_uint2(bytes4(q8.x, q8.y, sh, 0x000f000fu), bytes4(q8.z, q8.w, sh, 0x000f000fu));
+                *reinterpret_cast<uint2*>(dst + tv.ps1) = make_uint2(bytes4(q8.x, q8.y, sh_lo, 0x000f000fu), bytes4(q8.z, q8.w, sh_lo, 0x000f000fu));
         }
     }
     // view c0: row j0 + jj, bytes [u TP + g, ...): blocks of 4 columns x (4 ROWS4) rows of qt, byte-transposed
@@ -647,6 +716,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
         const int e = tid + 256 * k;
         if (NBLK % 256 == 0 || e < NBLK) {
             const int jj = (e % (TP / 4)) * 4, g = (e / (TP / 4)) * 4 * ROWS4;
+            if (GENERAL && jj >= wj) continue;
             uint32_t out[PLANES][4][ROWS4];
 #pragma unroll
             for (int rb = 0; rb < ROWS4; ++rb) {
@@ -655,7 +725,7 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
                 for (int i = 0; i < 4; ++i) r[i] = *reinterpret_cast<const uint2*>(qt + (g + 4 * rb + i) * QP + jj);
 #pragma unroll
                 for (int pl = 0; pl < PLANES; ++pl) {
-                    const int kk = pl == 0 ? sh_hi : sh;
+                    const int kk = pl == 0 ? sh_hi : sh_lo;
                     const uint32_t mask = pl == 0 ? 0x00ff00ffu : 0x000f000fu;
                     const uint32_t R0 = bytes4(r[0].x, r[0].y, kk, mask), R1 = bytes4(r[1].x, r[1].y, kk, mask);
                     const uint32_t R2 = bytes4(r[2].x, r[2].y, kk, mask), R3 = bytes4(r[3].x, r[3].y, kk, mask);
@@ -679,18 +749,18 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
         }
     }
     // replicated exponents, and the row tails beyond the last tile
-    if (tid < TP) {
-        tv.exps_c1[v * tv.rs1 + i0 + tid] = (int8_t)s_view;
-        tv.exps_c0[u * tv.rs0 + j0 + tid] = (int8_t)s_view;
+    if (tid < TP) {                                                    // lines beyond the matrix are documented as zero
+        if (!GENERAL || i0 + tid < tv.rs1) tv.exps_c1[v * tv.rs1 + i0 + tid] = tid < hi ? (int8_t)s_view : (int8_t)0;
+        if (!GENERAL || j0 + tid < tv.rs0) tv.exps_c0[u * tv.rs0 + j0 + tid] = tid < wj ? (int8_t)s_view : (int8_t)0;
     }
     if (v == tv.nkb1 - 1)
-        for (int64_t e = tid; e < (int64_t)TP * ((tv.kst1 - tv.nkb1 * TP) / 4); e += 256) {
+        for (int64_t e = tid; e < (int64_t)hi * ((tv.kst1 - tv.nkb1 * TP) / 4); e += 256) {
             const int64_t per = (tv.kst1 - tv.nkb1 * TP) / 4, ii = e / per, o = tv.nkb1 * TP + (e % per) * 4;
             *reinterpret_cast<uint32_t*>(tv.mant_c1 + (i0 + ii) * tv.kst1 + o) = 0;
             if (PLANES == 2) *reinterpret_cast<uint32_t*>(tv.mant_c1 + tv.ps1 + (i0 + ii) * tv.kst1 + o) = 0;
         }
     if (u == tv.nkb0 - 1)
-        for (int64_t e = tid; e < (int64_t)TP * ((tv.kst0 - tv.nkb0 * TP) / 4); e += 256) {
+        for (int64_t e = tid; e < (int64_t)wj * ((tv.kst0 - tv.nkb0 * TP) / 4); e += 256) {
             const int64_t per = (tv.kst0 - tv.nkb0 * TP) / 4, jj = e / per, o = tv.nkb0 * TP + (e % per) * 4;
             *reinterpret_cast<uint32_t*>(tv.mant_c0 + (j0 + jj) * tv.kst0 + o) = 0;
             if (PLANES == 2) *reinterpret_cast<uint32_t*>(tv.mant_c0 + tv.ps0 + (j0 + jj) * tv.kst0 + o) = 0;
@@ -1635,13 +1705,13 @@ int launch_row_fast(const float* x, int64_t rows, int64_t K, int64_t ld, const Q
 
 // Launch of the full-tile kernel for tiles of 32 and 64 (defined in part 2 of this file). The parameter blocks are
 // passed as opaque bytes: their types live in this file's unnamed namespace, which every part compiles alike.
-int launch_tile_full_small(int mode, int planes, int t, unsigned gx, unsigned gy, const float* src, int64_t ld, int64_t d0,
+int launch_tile_full_small(int mode, int planes, int t, bool general, unsigned gx, unsigned gy, const float* src, int64_t ld, int64_t d0,
                            int64_t d1, const void* qparams, int16_t* wide, int8_t* grid, int64_t grid_ld,
                            const void* tileviews, cudaStream_t st);
 
 #if HBFP_QUANT_PART == 2
 
-int launch_tile_full_small(int mode, int planes, int t, unsigned gx, unsigned gy, const float* src, int64_t ld, int64_t d0,
+int launch_tile_full_small(int mode, int planes, int t, bool general, unsigned gx, unsigned gy, const float* src, int64_t ld, int64_t d0,
                            int64_t d1, const void* qparams, int16_t* wide, int8_t* grid, int64_t grid_ld,
                            const void* tileviews, cudaStream_t st) {
     QParams p;
@@ -1649,7 +1719,11 @@ int launch_tile_full_small(int mode, int planes, int t, unsigned gx, unsigned gy
     memcpy(&p, qparams, sizeof(p));
     memcpy(&tv, tileviews, sizeof(tv));
     const dim3 grid_dim(gx, gy);
-#define HBFP_TILE_FULL_SMALL(MODE, PLANES, TP) launch_chained(tile_kernel_full<MODE, PLANES, TP>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv)
+#define HBFP_TILE_FULL_SMALL(MODE, PLANES, TP)                                                                                              \
+    do {                                                                                                                                    \
+        if (general) launch_chained(tile_kernel_full<MODE, PLANES, TP, true>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv); \
+        else launch_chained(tile_kernel_full<MODE, PLANES, TP, false>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv);      \
+    } while (0)
 #define HBFP_TILE_FULL_MODE(MODE)                                                                     \
     do {                                                                                              \
         if (planes == 1) { if (t == 32) HBFP_TILE_FULL_SMALL(MODE, 1, 32); else HBFP_TILE_FULL_SMALL(MODE, 1, 64); } \
@@ -1905,31 +1979,44 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
                       (MODE == 2 || ((ld % 4) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0)) &&
                       (MODE == 3 || (reinterpret_cast<uintptr_t>(wide) & 15) == 0) &&
                       (!value || ((ldv % 4) == 0 && (reinterpret_cast<uintptr_t>(value) & 15) == 0));
-    const size_t smem = (size_t)t * (t + 4) * sizeof(float) + (size_t)tp * (tp + 2) * sizeof(int16_t);
     const dim3 grid_dim((unsigned)nv, (unsigned)nu);
-    // full tiles of 32 / 64 / 128, both views or none, narrow bits cut by 32-bit shifts (see tile_kernel_full)
-    const int sh_full = MODE == 3 ? 0 : 16 - p.m;
-    const bool full = fast && t == tp && (d0 % t) == 0 && (d1 % t) == 0 && ((mant_c0 != nullptr) == (mant_c1 != nullptr)) &&
-                      (!mant_c0 || (exps_c0 && exps_c1)) && sh_full + (L0.planes == 2 ? 4 : 0) <= 8;
+    // tiles of 32 / 64 / 128, both views or none
+    const bool full = fast && t == tp && ((mant_c0 != nullptr) == (mant_c1 != nullptr)) &&
+                      (!mant_c0 || (exps_c0 && exps_c1));
     if (full) {
-#define HBFP_TILE_FULL(PLANES, TP) launch_chained(tile_kernel_full<MODE, PLANES, TP>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, nv, tv)
+        // whole tiles, cut by 32-bit shifts
+        const bool general = d0 % t != 0 || d1 % t != 0 || (MODE != 3 && 16 - p.m + (L0.planes == 2 ? 4 : 0) > 8);
+#define HBFP_TILE_FULL(PLANES, RG) launch_chained(tile_kernel_full<MODE, PLANES, 128, RG>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, nv, tv)
         if (t != 128)
-            return launch_tile_full_small(MODE, (int)L0.planes, t, grid_dim.x, grid_dim.y, src, ld, d0, d1, &p, wide, grid, nv, &tv, st);
-        if (L0.planes == 1) HBFP_TILE_FULL(1, 128); else HBFP_TILE_FULL(2, 128);
+            return launch_tile_full_small(MODE, (int)L0.planes, t, general, grid_dim.x, grid_dim.y, src, ld, d0, d1, &p, wide, grid, nv, &tv, st);
+        if (L0.planes == 1) { if (general) HBFP_TILE_FULL(1, true); else HBFP_TILE_FULL(1, false); }
+        else { if (general) HBFP_TILE_FULL(2, true); else HBFP_TILE_FULL(2, false); }
 #undef HBFP_TILE_FULL
         return launch_status();
     }
-#define HBFP_TILE_LAUNCH(PLANES, FAST)                                                                                       \
-    do {                                                                                                                     \
-        HBFP_CUDA_OK(cudaFuncSetAttribute(tile_kernel<MODE, PLANES, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-        launch_chained(tile_kernel<MODE, PLANES, FAST>, grid_dim, 256, smem, st, src, ld, d0, d1, t, tp, p, wide, grid, nv, tv);         \
+    // Strips of 64 or 96 columns (whichever the tiles fill better) and up to 64 rows, 128 x 128 for tiles above 64.
+    StripShape sh{t, tp, tp == 32 ? 5 : tp == 64 ? 6 : 7, 1, t <= 8 ? 3 : t <= 16 ? 2 : t <= 32 ? 1 : 0, 0, (65536 + t - 1) / t, 0, (int)nu, (int)nv};
+    const int warps = t > 64 ? 16 : 8;
+    sh.rpw = (t + (warps >> sh.lg_rv) - 1) / (warps >> sh.lg_rv);
+    const int cv2 = std::min(64 / t, 160 / tp), cv3 = std::min(96 / t, 160 / tp);
+    const int kc = t > 64 ? 4 : sh.rpw <= 6 && 2 * cv3 > 3 * cv2 ? 3 : 2;
+    if (kc < 4) sh.cv = kc == 3 ? cv3 : cv2;
+    const int rv = 1 << sh.lg_rv, rows = kc == 3 ? 6 : 8, per = sh.cv * tp / 8;
+    sh.recip_per = ((1 << 20) + per - 1) / per;
+    if (nv >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
+    const dim3 strips((unsigned)((nv + sh.cv - 1) / sh.cv), (unsigned)((nu + rv - 1) / rv));
+    const size_t smem = (size_t)rv * tp * (sh.cv * tp + 8) * 2 + (p.rounding && MODE != 2 ? (size_t)warps * rows * (4 * kc + 1) * 16 : 0);
+#define HBFP_STRIP(PLANES, NW, RPW, KC, SRV)                                                                                                      \
+    do {                                                                                                                                          \
+        if (smem > 36 * 1024) HBFP_CUDA_OK(cudaFuncSetAttribute(tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        launch_chained(tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>, strips, 32 * NW, smem, st, src, ld, d0, d1, sh, p, wide, grid, nv, tv);  \
     } while (0)
-    if (L0.planes == 1) {
-        if (fast) HBFP_TILE_LAUNCH(1, true); else HBFP_TILE_LAUNCH(1, false);
-    } else {
-        if (fast) HBFP_TILE_LAUNCH(2, true); else HBFP_TILE_LAUNCH(2, false);
-    }
-#undef HBFP_TILE_LAUNCH
+#define HBFP_STRIP_SR(PLANES, NW, RPW, KC) do { if (p.rounding && MODE != 2) HBFP_STRIP(PLANES, NW, RPW, KC, MODE != 2); else HBFP_STRIP(PLANES, NW, RPW, KC, false); } while (0)
+#define HBFP_STRIP_KC(PLANES) do { if (kc == 2) HBFP_STRIP_SR(PLANES, 8, 8, 2); else if (kc == 3) HBFP_STRIP_SR(PLANES, 8, 6, 3); else HBFP_STRIP_SR(PLANES, 16, 8, 4); } while (0)
+    if (L0.planes == 1) HBFP_STRIP_KC(1); else HBFP_STRIP_KC(2);
+#undef HBFP_STRIP_KC
+#undef HBFP_STRIP_SR
+#undef HBFP_STRIP
     return launch_status();
 }
 

@@ -161,3 +161,37 @@ def test_update_also_writes_the_fp32_value(hb, shape, t, rounding):
     exact = np.ldexp(q16.astype(np.float64), s16).astype(np.float32)      # 16-bit mantissas: exact in binary32
     assert np.array_equal(value, exact)
     assert np.array_equal(hb.wide_dequantize(wide).cpu().numpy(), exact)
+
+
+# Tile geometries that are not whole tiles of 32, 64 or 128 (and these in widths cut from the words early): strips of one to eight tile rows, ragged last tiles and strips in both
+# directions, odd row lengths, every view from FP32 weights, from wide words and after an update.
+@pytest.mark.parametrize("d0,d1,t,m,rounding", [
+    (1, 1, 1, 8, 1), (70, 13, 1, 8, 0), (83, 91, 5, 12, 1), (64, 40, 8, 4, 0), (75, 163, 9, 8, 1), (129, 257, 16, 12, 0), (145, 301, 17, 8, 1), (48, 120, 24, 8, 1),
+    (95, 241, 24, 12, 0), (65, 129, 32, 8, 1), (64, 127, 32, 4, 1), (131, 259, 33, 8, 0), (97, 193, 48, 12, 1), (65, 257, 64, 8, 1), (128, 256, 64, 4, 0),
+    (101, 203, 100, 8, 1), (129, 255, 128, 12, 1), (256, 128, 128, 4, 1), (41, 104, 32, 8, 1), (129, 200, 64, 12, 0), (63, 72, 64, 4, 1), (150, 328, 128, 9, 1)])
+def test_weight_tiles_of_any_geometry(hb, d0, d1, t, m, rounding):
+    fd = F(m, t, rounding, seed=11, stream_id=2)
+    w = wl.draw("lognormal", (d0, d1), seed=77)
+    w[0, 0] = 0.0
+    w[:, d1 // 2] = np.float32(2.0) ** np.arange(d0, dtype=np.float32).clip(0, 20)      # tile maxima at powers of two
+    q16, s16 = oracle.wide_quantize(w, ofmt(fd))
+    wide, views = hb.wide_quantize(to_dev(w), gfmt(fd))
+    assert np.array_equal(wide.mant.cpu().numpy(), q16) and np.array_equal(wide.exps.cpu().numpy(), s16[::t, :])
+    check_views(hb, views, *oracle.wide_narrow(q16, s16, m), t)
+    check_views(hb, hb.wide_narrow(wide, gfmt(fd)), *oracle.wide_narrow(q16, s16, m), t)
+    # a pitch longer than the rows; the update with and without the FP32 value
+    delta = (wl.draw("grad", (d0, d1 + 3), seed=78) * 3).astype(np.float32)
+    q16, s16 = oracle.wide_update(q16, s16, np.ascontiguousarray(delta[:, :d1]), ofmt(fd))
+    other = hb.Wide(wide.mant.clone(), wide.exps.clone(), t)
+    value = hb.wide_update_value(other, to_dev(delta)[:, :d1], gfmt(fd), views)
+    check_views(hb, views, *oracle.wide_narrow(q16, s16, m), t)
+    check_views(hb, hb.wide_update(wide, to_dev(delta)[:, :d1], gfmt(fd)), *oracle.wide_narrow(q16, s16, m), t)
+    for x in (wide, other):
+        assert np.array_equal(x.mant.cpu().numpy(), q16) and np.array_equal(x.exps.cpu().numpy(), s16[::t, :])
+    assert np.array_equal(value.cpu().numpy(), hb.wide_dequantize(wide).cpu().numpy())
+    # straight to m bits
+    c0, c1, grid = hb.quantize_tiles(to_dev(w), gfmt(fd))
+    qn, sn = oracle.quantize(w, 1, ofmt(fd))
+    check_views(hb, (c0, c1), qn, sn, t)
+    assert np.array_equal(grid.cpu().numpy(), sn[::t, :])
+    assert hb.device_status() == 0
