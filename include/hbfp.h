@@ -352,6 +352,10 @@ HBFP_API int hbfp_gemm_q_bias(int64_t M, int64_t N, int64_t K, const hbfp_operan
  * depends on the extents alone. */
 HBFP_API int hbfp_column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, void* stream);
 
+/* The gradient cols [n h w][kh kw c] of an im2col matrix (stride 1, pad = (kh - 1) / 2 = (kw - 1) / 2) added back onto the pixels
+ * out [n][h][w][c] in FP32, the taps in ascending order. */
+HBFP_API int hbfp_fold_taps(const float* cols, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw, int pad, float* out, void* stream);
+
 /* Convolution forward pass as one implicit GEMM (Sec. 5.1: convolutions run through the same BFP dot
  * products): Y [n*h*w][filters] = conv(x, filters), stride 1, `pad` zeros around the image, an output as
  * large as the input (2 pad == kh - 1 == kw - 1). x: the activations [n][h][w][c] converted once per

@@ -27,7 +27,7 @@ ROUND_NEAREST_EVEN, ROUND_STOCHASTIC = 0, 1
 EXPORTS = [
     "hbfp_status_string", "hbfp_packed_layout", "hbfp_packed_sizes", "hbfp_quantize",
     "hbfp_quantize_tiles", "hbfp_unpack", "hbfp_dequantize", "hbfp_gemm_workspace",
-    "hbfp_gemm_q_workspace", "hbfp_gemm", "hbfp_gemm_q", "hbfp_gemm_q_bias", "hbfp_column_sums", "hbfp_gemm_block_partials",
+    "hbfp_gemm_q_workspace", "hbfp_gemm", "hbfp_gemm_q", "hbfp_gemm_q_bias", "hbfp_column_sums", "hbfp_fold_taps", "hbfp_gemm_block_partials",
     "hbfp_device_status", "hbfp_gemm_static", "hbfp_wide_quantize", "hbfp_wide_update", "hbfp_wide_update_value", "hbfp_wide_narrow",
     "hbfp_im2col_packed", "hbfp_im2col_packed_t", "hbfp_wide_dequantize", "hbfp_selftest_bounded_wait", "hbfp_last_gemm_kernel", "hbfp_last_gemm_launch", "hbfp_last_gemm_cycles", "hbfp_conv_forward", "hbfp_quantize_conv_weights", "hbfp_conv_dgrad_filters",
 ]
@@ -113,6 +113,7 @@ def lib() -> ctypes.CDLL:
         L.hbfp_wide_dequantize.argtypes = [p, p, i64, i64, i32, p, i64, p]
         L.hbfp_selftest_bounded_wait.argtypes = [i64, i32, p, p]
         L.hbfp_last_gemm_cycles.argtypes = [p]
+        L.hbfp_fold_taps.argtypes = [p, i64, i64, i64, i64, i32, i32, i32, p, p]
         for fn in (L.hbfp_last_gemm_kernel, L.hbfp_last_gemm_launch):
             fn.restype = ctypes.c_char_p
             fn.argtypes = []
@@ -126,7 +127,7 @@ def lib() -> ctypes.CDLL:
 # Entry points that _host calls, in the order it takes them (csrc/host.cpp, struct Api).
 _HOST_ENTRY_POINTS = ("hbfp_packed_layout", "hbfp_quantize", "hbfp_gemm_q_workspace", "hbfp_wide_update_value", "hbfp_wide_dequantize",
                       "hbfp_conv_forward", "hbfp_conv_dgrad_filters", "hbfp_im2col_packed_t", "hbfp_im2col_packed", "hbfp_gemm_q_bias",
-                      "hbfp_column_sums")
+                      "hbfp_column_sums", "hbfp_fold_taps")
 
 
 def host():

@@ -541,6 +541,12 @@ int hbfp_column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, flo
     return launch_column_sums(x, rows, cols, ld, out, static_cast<cudaStream_t>(stream));
 }
 
+int hbfp_fold_taps(const float* cols, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw, int pad, float* out, void* stream) {
+    if (n < 0 || h <= 0 || w <= 0 || c <= 0 || kh <= 0 || kw <= 0 || pad < 0 || 2 * pad != kh - 1 || 2 * pad != kw - 1) return HBFP_ERR_INVALID_ARG;
+    if (n > 0 && (!cols || !out)) return HBFP_ERR_INVALID_ARG;
+    return launch_fold_taps(cols, n, h, w, c, kh, kw, pad, out, static_cast<cudaStream_t>(stream));
+}
+
 int hbfp_gemm(int transA, int transB, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
               const float* B, int64_t ldb, float* C, int64_t ldc, const hbfp_format* fmtA,
               const hbfp_format* fmtB, void* workspace, size_t workspace_bytes, uint32_t flags, void* stream) {

@@ -209,6 +209,7 @@ int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, c
 // FP32 parts of a layer (layer.cu): the bias added to a stored product, the column sums that are its gradient.
 int launch_add_bias(float* C, int64_t M, int64_t N, int64_t ldc, const float* bias, cudaStream_t st);
 int launch_column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, cudaStream_t st);
+int launch_fold_taps(const float* cols, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw, int pad, float* out, cudaStream_t st);
 
 // Convolution forward as an implicit GEMM over the packed pixels (gemm_conv.cu).
 int launch_conv_forward(const Packed& x, const Packed& wt, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw,

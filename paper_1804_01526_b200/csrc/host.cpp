@@ -34,6 +34,7 @@ struct Api {
     decltype(&hbfp_im2col_packed) im2col_packed;
     decltype(&hbfp_gemm_q_bias) gemm_q_bias;
     decltype(&hbfp_column_sums) column_sums;
+    decltype(&hbfp_fold_taps) fold_taps;
 } api;
 
 // ------------------------------------------------------------------------------ arguments
@@ -628,11 +629,10 @@ struct ConvNode : public torch::autograd::Node {
         }
         if (rc != HBFP_ERR_UNSUPPORTED) raise_status(rc, "hbfp_conv_forward");
         // shapes that route does not cover: gradient of the im2col matrix, then its scatter back onto the pixels (FP32)
-        const at::Tensor dcols = product(n * h * w, 9 * c, f, fp32_operand(dy2, 0, pixels(2)), c1.operand(), dy2).view({n, h, w, 3, 3, c});
-        at::Tensor dxp = at::zeros({n, h + 2, w + 2, c}, dy2.options());
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) dxp.slice(1, i, i + h).slice(2, j, j + w).add_(dcols.select(4, j).select(3, i));
-        return dxp.slice(1, 1, h + 1).slice(2, 1, w + 1).contiguous();
+        const at::Tensor dcols = product(n * h * w, 9 * c, f, fp32_operand(dy2, 0, pixels(2)), c1.operand(), dy2);
+        at::Tensor dx = empty_f32({n, h, w, c}, dy2);
+        ok_or_raise(api.fold_taps((const float*)dcols.data_ptr(), n, h, w, c, 3, 3, 1, (float*)dx.data_ptr(), cur_stream()), "hbfp_fold_taps");
+        return dx;
     }
     variable_list apply(variable_list&& grads) override {
         std::lock_guard<std::mutex> lock(mutex_);

@@ -99,6 +99,44 @@ column_sums_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int6
     if (splits > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
+// The scatter of the gradient of an im2col matrix cols [n h w][kh kw c] (stride 1, output as large as the input) back onto the pixels:
+// out[n][y][x] = sum over the taps (i, j), ascending, of cols[n][y - i + pad][x - j + pad][i][j], from +0, taps outside the image left
+// out. V channels and one pixel per thread, the nine loads of a 3 x 3 filter in flight together; bound by reading the matrix once
+// (131072 pixels x 9 x 32: 151 MB). As a padded tensor, nine shifted additions and a copy it moved five times as much.
+template <int V>
+__global__ void __launch_bounds__(256)
+fold_taps_kernel(const float* __restrict__ cols, uint32_t h, uint32_t w, uint32_t cv, int kh, int kw, int pad, float* __restrict__ out) {
+    chain_start();
+    const uint32_t i = blockIdx.y * blockDim.x + threadIdx.x;              // within the image row blockIdx.x
+    if (i >= w * cv) return;
+    const int x = (int)(i / cv), y = (int)(blockIdx.x % h);
+    const uint32_t ch = (i - (uint32_t)x * cv) * V;
+    const int64_t px = (int64_t)blockIdx.x * w + x, c = (int64_t)cv * V, pitch = (int64_t)kh * kw * c;
+    float acc[V];
+#pragma unroll
+    for (int e = 0; e < V; ++e) acc[e] = 0.f;
+    for (int di = 0; di < kh; ++di) {
+        const int sy = y - di + pad;
+        if (sy < 0 || sy >= (int)h) continue;
+#pragma unroll 3
+        for (int dj = 0; dj < kw; ++dj) {
+            const int sx = x - dj + pad;
+            if (sx < 0 || sx >= (int)w) continue;
+            const float* src = cols + (px + (int64_t)(pad - di) * w + (pad - dj)) * pitch + (di * kw + dj) * c + ch;
+            if (V == 4) {
+                const float4 v = __ldcs(reinterpret_cast<const float4*>(src));
+                acc[0] = __fadd_rn(acc[0], v.x); acc[1 % V] = __fadd_rn(acc[1 % V], v.y);
+                acc[2 % V] = __fadd_rn(acc[2 % V], v.z); acc[3 % V] = __fadd_rn(acc[3 % V], v.w);
+            } else {
+                acc[0] = __fadd_rn(acc[0], __ldcs(src));
+            }
+        }
+    }
+    float* dst = out + px * c + ch;
+    if (V == 4) *reinterpret_cast<float4*>(dst) = make_float4(acc[0], acc[1 % V], acc[2 % V], acc[3 % V]);
+    else *dst = acc[0];
+}
+
 template <int V>
 int column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* out, cudaStream_t st) {
     constexpr int64_t MOST = 65535ll * 32 * V;                    // columns a grid can have
@@ -123,6 +161,19 @@ int launch_add_bias(float* C, int64_t M, int64_t N, int64_t ldc, const float* bi
     const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
     if (quad) launch_chained(add_bias_kernel<4>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
     else launch_chained(add_bias_kernel<1>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
+    return launch_status();
+}
+
+int launch_fold_taps(const float* cols, int64_t n, int64_t h, int64_t w, int64_t c, int kh, int kw, int pad, float* out, cudaStream_t st) {
+    if (n == 0) return HBFP_OK;
+    const bool quad = c % 4 == 0 && ((reinterpret_cast<uintptr_t>(cols) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
+    const int64_t cv = quad ? c / 4 : c, row = w * cv;
+    const int threads = row < 256 ? (int)round_up(row, 32) : 256;
+    const int64_t chunks = (row + threads - 1) / threads;
+    if (n * h >= (1ll << 31) || row >= (1ll << 31) || chunks > 65535) return HBFP_ERR_UNSUPPORTED;
+    const dim3 grid((unsigned)(n * h), (unsigned)chunks);
+    if (quad) launch_chained(fold_taps_kernel<4>, grid, threads, 0, st, cols, (uint32_t)h, (uint32_t)w, (uint32_t)cv, kh, kw, pad, out);
+    else launch_chained(fold_taps_kernel<1>, grid, threads, 0, st, cols, (uint32_t)h, (uint32_t)w, (uint32_t)cv, kh, kw, pad, out);
     return launch_status();
 }
 

@@ -342,3 +342,20 @@ def test_backward_weight_operand_for_three_wide_filters(hb, n, h, w, c, kh, m, r
         q_ref, s_ref = oracle.quantize(cols, 0, ofmt(fd))
     q, s = decode_packed(pa, hb.packed_layout(pa.rows, pa.k, pa.fmt))
     assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
+
+
+@pytest.mark.parametrize("n,h,w,c,k", [(1, 1, 1, 1, 3), (2, 3, 5, 7, 3), (3, 8, 8, 32, 3), (1, 17, 33, 12, 5), (2, 4, 300, 96, 3), (0, 4, 4, 4, 3)])
+def test_fold_of_the_im2col_gradient(hb, n, h, w, c, k):
+    """Shifted additions in the order of the taps, bit for bit."""
+    import ctypes
+    import torch
+    pad = k // 2
+    cols = torch.randn(n * h * w, k, k, c, device="cuda")
+    want = torch.zeros(n, h + 2 * pad, w + 2 * pad, c, device="cuda")
+    for i in range(k):
+        for j in range(k):
+            want[:, i:i + h, j:j + w] += cols[:, i, j].view(n, h, w, c)
+    out = torch.full((n, h, w, c), float("nan"), device="cuda")
+    call = lambda p: hb.lib().hbfp_fold_taps(cols.data_ptr(), n, h, w, c, k, k, p, out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert call(pad) == 0 and call(pad + 1) == hb.ERR_INVALID_ARG
+    assert torch.equal(out, want[:, pad:pad + h, pad:pad + w])
