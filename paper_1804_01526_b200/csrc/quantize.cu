@@ -128,67 +128,86 @@ quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld,
 // ------------------------------------------------------------------------------ quant_col_block
 
 // Blocks down the columns of x [K][R] (contract axis 0); output rows are the columns of x. Any block length up to 128, any
-// pitch and alignment (the paper's tile of 24 among them). A CTA takes one K-block of 32 columns: four warps split the
-// block's rows, so that every load is a warp's 128 consecutive bytes of one row and all of a thread's loads are in flight
-// together; the values stay in registers between the maximum and the rounding. Small and ragged matrices are bound by
-// latency, hence one block per CTA (many short CTAs): 128 x 1024, b = 24, stochastic 5.5 -> 2.7 us; 3001 x 777:
-// 26 -> 8.4 us; 16384 x 16384, nearest-even: 677 -> 403 us.
-constexpr int COLT = 32;
+// pitch and alignment (the paper's tile of 24 among them). A lane takes one column and up to NV of a block's rows, so that every load
+// is a warp's 128 consecutive bytes of one row, all of a thread's loads are in flight together, the values stay in registers between
+// the maximum and the rounding, and the packed bytes of a thread are one whole sector of its output row: nothing passes through shared
+// memory but the draws. Blocks of up to 32 belong to one warp and need no barrier, longer ones to two or four. A block's rows over
+// four warps of eight, through shared memory both ways, left a quarter of the threads idle at b = 24 and waited at two barriers.
+// Before / now: 10000 x 10000, b = 24 154 / 93 us (4.3 / 5.4 TB/s with the padding written), with draws 268 / 110; 20000 x 3001, b = 64,
+// with draws 107 / 69; 5001 x 4999, b = 32 33 / 20; the 12-bit form of 2373 x 4352, b = 24 20.6 / 10.2.
+constexpr int COLT = 32, COL_WARPS = 4;
 
-template <int PLANES, int RQ, bool SR>      // RQ = bp / 4: padded rows per warp (8, 16 or 32)
-__global__ void __launch_bounds__(128)
+template <int PLANES, int NV, int WPB, bool SR>      // WPB: warps per block; the padded block length is 32 WPB
+__global__ void __launch_bounds__(32 * COL_WARPS)
 quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
                 int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa, const int8_t* __restrict__ given) {
     const Chain chain(p.beside);
     // given != nullptr: one exponent per column for the whole axis, computed beforehand; the blocks are then pieces of it
-    constexpr int BP = 4 * RQ, BYTE_PLANES = is_form(PLANES) ? 1 : PLANES;
-    __shared__ uint32_t pmax[4][COLT];
-    __shared__ __align__(16) uint4 rnd[SR ? BP : 1][5];          // draws of a row: its 32 columns lie in at most five groups of eight
-    __shared__ __align__(16) unsigned char s_out[BYTE_PLANES][is_form(PLANES) ? 1 : COLT][BP + 16];
-    const int tid = threadIdx.x, c = tid & 31, q = tid >> 5;
-    const int64_t kb = blockIdx.x / tiles_n, c0 = (int64_t)(blockIdx.x - (unsigned)kb * tiles_n) * COLT;
-    const int64_t k0 = kb * b, col = c0 + c;
-    const int rows_here = (int)min((int64_t)b, K - k0);
-    float v[RQ];
-    const float* src = x + (k0 + q * RQ) * ld + col;
+    constexpr int BP = 32 * WPB, BPC = COL_WARPS / WPB;                // BPC: blocks of a CTA
+    __shared__ uint32_t pmax[WPB > 1 ? COL_WARPS : 1][COLT];
+    __shared__ __align__(16) uint4 rnd[SR ? COL_WARPS : 1][SR ? NV : 1][5];      // draws of a row: its 32 columns lie in at most five groups of eight
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned kg = blockIdx.x / tiles_n;
+    const int64_t kb = (int64_t)kg * BPC + warp / WPB, c0 = (int64_t)(blockIdx.x - kg * tiles_n) * COLT, col = c0 + lane;
+    if (WPB == 1 && kb >= nkb) return;
+    const int part = warp % WPB;
+    const int64_t k0 = kb * b + part * 32;
+    const int n = kb < nkb ? max(0, (int)min((int64_t)min(NV, b - part * 32), K - k0)) : 0;     // rows of this warp
+    const float* src = x + k0 * ld + col;
+    const bool full = n == NV && c0 + COLT <= R;
+    float v[NV];
+    if (full) {
 #pragma unroll
-    for (int j = 0; j < RQ; ++j) v[j] = (q * RQ + j < rows_here && col < R) ? __ldcs(src + (int64_t)j * ld) : 0.f;
+        for (int j = 0; j < NV; ++j) v[j] = __ldcs(src + (int64_t)j * ld);
+    } else {
+#pragma unroll
+        for (int j = 0; j < NV; ++j) v[j] = j < n && col < R ? __ldcs(src + (int64_t)j * ld) : 0.f;
+    }
     // the draws do not depend on the data: they are made while the loads are in flight, one Philox call per group of eight
-    // consecutive source elements
+    // consecutive source elements (rows that all start with a group touch four of them)
     if (SR) {
-        for (int i = tid; i < rows_here * 5; i += 128) {
-            const int kk = i / 5, g = i - kk * 5;
-            const uint64_t L0 = (uint64_t)((k0 + kk) * R + c0);
-            if (g < 4 || (L0 & 7)) rnd[kk][g] = draws_of_group(p, (L0 >> 3) + g);
-        }
+        auto draw = [&](auto count) {
+            constexpr int N = decltype(count)::value;
+            for (int i = lane; i < n * N; i += 32) {
+                const int kk = i / N, g = i - kk * N;
+                rnd[warp][kk][g] = draws_of_group(p, ((uint64_t)((k0 + kk) * R + c0) >> 3) + g);
+            }
+            __syncwarp();
+        };
+        if ((R & 7) == 0) draw(std::integral_constant<int, 4>{});
+        else draw(std::integral_constant<int, 5>{});
     }
     uint32_t am = 0;
 #pragma unroll
-    for (int j = 0; j < RQ; j += 2) am = max3_abs_bits(am, v[j], v[j + 1]);
-    pmax[q][c] = am;
-    __syncthreads();
-    am = max(max(pmax[0][c], pmax[1][c]), max(pmax[2][c], pmax[3][c]));
+    for (int j = 0; j < NV; j += 2) am = max3_abs_bits(am, v[j], v[j + 1]);
+    if (WPB > 1) {
+        pmax[warp][lane] = am;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < WPB; ++w) am = max(am, pmax[warp - part + w][lane]);
+        if (kb >= nkb) return;
+    }
     const int s = given ? (col < R ? (int)given[col] : -63) : block_exponent(am, p.m, p.exp_mode);
     check_exponent<PLANES>(s, fa);
-    if constexpr (is_form(PLANES)) { if (q == 0 && col < R) store_exponent<PLANES>(exps, kb * rs + col, s); }
-    else if (!given && q == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
+    if constexpr (is_form(PLANES)) { if (part == 0 && col < R) store_exponent<PLANES>(exps, kb * rs + col, s); }
+    else if (!given && part == 0 && col < rs) exps[kb * rs + col] = col < R ? (int8_t)s : (int8_t)0;      // lines beyond the matrix are documented as zero
     const uint32_t qm = qmax_pair(p.qmax), nqm = neg_qmax_pair(p.qmax);
     const float sc = pow2f(SR ? 16 - s : -s);
-    const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd);
+    const uint16_t* rnd16 = reinterpret_cast<const uint16_t*>(rnd[SR ? warp : 0]) + lane;
     const uint32_t first = SR ? (uint32_t)((uint64_t)(k0 * R + c0) & 7) : 0u, row_step = (uint32_t)(R & 7);
-    uint32_t fo[is_form(PLANES) ? 2 : 1][RQ / 2];               // the form's elements of this thread, pair by pair
+    uint32_t hi[8], lo[8];
+    uint32_t fo[is_form(PLANES) ? 2 : 1][16];
 #pragma unroll
-    for (int w = 0; w < RQ / 4; ++w) {
-        uint32_t h[2], hi, lo;
+    for (int w = 0; w < 8; ++w) {
+        uint32_t h[2] = {0u, 0u};
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int j = 4 * w + 2 * k;
+            if (j >= NV) continue;                                     // the block's padding
             if (SR) {
-                // zeros below the block or the matrix stay zero whatever the draw (their table rows are not read)
-                const int kk = q * RQ + j;
-                const uint32_t r0 = kk < rows_here ? rnd16[kk * 40 + ((first + (uint32_t)kk * row_step) & 7) + c] : 0u;
-                const uint32_t r1 = kk + 1 < rows_here ? rnd16[(kk + 1) * 40 + ((first + (uint32_t)(kk + 1) * row_step) & 7) + c] : 0u;
+                // zeros below the block or the matrix stay zero whatever the draw (their table rows hold anything)
+                const uint32_t r0 = rnd16[j * 40 + ((first + (uint32_t)j * row_step) & 7)], r1 = rnd16[(j + 1) * 40 + ((first + (uint32_t)(j + 1) * row_step) & 7)];
                 h[k] = round_sr_pair2(v[j], v[j + 1], sc, r0, r1, qm, nqm);
             } else {
                 h[k] = round_rne_pair(v[j], v[j + 1], sc, qm, nqm);
@@ -198,38 +217,45 @@ quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, i
             form_pair<PLANES>(h[0], pow2f(s), fo[0][2 * w], fo[1][2 * w]);
             form_pair<PLANES>(h[1], pow2f(s), fo[0][2 * w + 1], fo[1][2 * w + 1]);
         } else {
-            pack4<BYTE_PLANES>(h[0], h[1], hi, lo);
-            *reinterpret_cast<uint32_t*>(&s_out[0][c][q * RQ + 4 * w]) = hi;
-            if (PLANES == 2) *reinterpret_cast<uint32_t*>(&s_out[BYTE_PLANES - 1][c][q * RQ + 4 * w]) = lo;
+            pack4<PLANES>(h[0], h[1], hi[w], lo[w]);
         }
     }
+    if (col >= R) return;
     if constexpr (is_form(PLANES)) {
-        if (col >= R) return;
 #pragma unroll
         for (int pl = 0; pl < (PLANES == FORM_WIDE_B ? 2 : 1); ++pl) {
-            uint4* dst = reinterpret_cast<uint4*>(mant + 2 * (pl * plane_stride + col * kst + kb * BP + q * RQ));
-#pragma unroll
-            for (int i = 0; i < RQ / 8; ++i) dst[i] = make_uint4(fo[pl][4 * i], fo[pl][4 * i + 1], fo[pl][4 * i + 2], fo[pl][4 * i + 3]);
-            if (kb == nkb - 1 && q == 0)                          // the row tail [nkb * bp, kst)
-                for (int64_t o = nkb * BP; o < kst; o += 8) *reinterpret_cast<uint4*>(mant + 2 * (pl * plane_stride + col * kst + o)) = make_uint4(0, 0, 0, 0);
+            int8_t* row = mant + 2 * (pl * plane_stride + col * kst);
+            store_sector(row + 2 * (kb * BP + part * 32), &fo[pl][0]);
+            store_sector(row + 2 * (kb * BP + part * 32) + 32, &fo[pl][8]);
+            if (kb == nkb - 1 && part == 0)                            // the row tail [nkb * bp, kst)
+                for (int64_t o = nkb * BP; o < kst; o += 8) *reinterpret_cast<uint4*>(row + 2 * o) = make_uint4(0, 0, 0, 0);
         }
-        return;
+    } else {
+#pragma unroll
+        for (int pl = 0; pl < PLANES; ++pl) {
+            int8_t* row = mant + pl * plane_stride + col * kst;
+            store_sector(row + kb * BP + part * 32, pl ? lo : hi);
+            if (kb == nkb - 1 && part == 0)
+                for (int64_t o = nkb * BP; o < kst; o += 16) *reinterpret_cast<uint4*>(row + o) = make_uint4(0, 0, 0, 0);
+        }
     }
-    __syncthreads();
-    // neighbouring threads write neighbouring 16-byte pieces of an output row
-    constexpr int PPR = BP / 16;
-#pragma unroll
-    for (int pl = 0; pl < BYTE_PLANES; ++pl)
-        for (int i = tid; i < COLT * PPR; i += 128) {
-            const int r = i / PPR, piece = i - r * PPR;
-            if (c0 + r < R)
-                *reinterpret_cast<uint4*>(mant + pl * plane_stride + (c0 + r) * kst + kb * BP + 16 * piece) =
-                    *reinterpret_cast<const uint4*>(&s_out[pl][r][16 * piece]);
-        }
-    // the row tail [nkb * bp, kst)
-    if (kb == nkb - 1 && q < BYTE_PLANES && col < R)
-        for (int64_t o = nkb * BP; o < kst; o += 16)
-            *reinterpret_cast<uint4*>(mant + q * plane_stride + col * kst + o) = make_uint4(0, 0, 0, 0);
+}
+
+// One launch for blocks of b (padded to bp): OUT is 1 or 2 planes or a form.
+template <int OUT>
+int launch_col_block(const float* x, int64_t K, int64_t rows, int64_t ld, int b, int64_t bp, int64_t nkb, const QParams& p, const Layout& L, int8_t* mant, int8_t* exps,
+                     cudaStream_t st, const FormArgs& fa, const int8_t* given) {
+    const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT);
+    const int64_t per = 128 / bp, grid = (int64_t)tiles_n * ((nkb + per - 1) / per);
+#define HBFP_QCOL(NV, WPB, SRV) launch_chained(quant_col_block<OUT, NV, WPB, SRV>, (unsigned)grid, 32 * COL_WARPS, 0, st, x, K, rows, ld, b, p, mant, L.kst, L.plane_stride, exps, L.rs, nkb, tiles_n, fa, given)
+#define HBFP_QCOL_SR(NV, WPB) do { if (p.rounding) HBFP_QCOL(NV, WPB, true); else HBFP_QCOL(NV, WPB, false); } while (0)
+    if (bp == 32) { if (b <= 24) HBFP_QCOL_SR(24, 1); else HBFP_QCOL_SR(32, 1); }
+    else if (bp == 64) HBFP_QCOL_SR(32, 2);
+    else if constexpr (!is_form(OUT)) HBFP_QCOL_SR(32, 4);
+    else return HBFP_ERR_UNSUPPORTED;
+#undef HBFP_QCOL_SR
+#undef HBFP_QCOL
+    return launch_status();
 }
 
 // ------------------------------------------------------------------------------ weight tiles
@@ -1834,12 +1860,8 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
 #undef HBFP_QCOL_GIVEN
         }
         const int64_t pieces = L.kst / 128;
-        const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * pieces);
-#define HBFP_QCOL_GIVEN(PL, SRV) launch_chained(quant_col_block<PL, 32, SRV>, grid, 128, 0, st, x, K, rows, ld, 128, p, mant, L.kst, L.plane_stride, exps, L.rs, pieces, tiles_n, FormArgs{}, exps)
-        if (L.planes == 1) { if (p.rounding) HBFP_QCOL_GIVEN(1, true); else HBFP_QCOL_GIVEN(1, false); }
-        else { if (p.rounding) HBFP_QCOL_GIVEN(2, true); else HBFP_QCOL_GIVEN(2, false); }
-#undef HBFP_QCOL_GIVEN
-        return launch_status();
+        return L.planes == 1 ? launch_col_block<1>(x, K, rows, ld, 128, 128, pieces, p, L, mant, exps, st, FormArgs{}, exps)
+                             : launch_col_block<2>(x, K, rows, ld, 128, 128, pieces, p, L, mant, exps, st, FormArgs{}, exps);
     }
     if (f->tile == 0 && axis == 0 && aligned && L.b == L.bp && L.b <= 128 && (p.rounding == 0 || rows % 8 == 0) &&
         (reinterpret_cast<uintptr_t>(mant) & 127) == 0 && rows < (1ll << 29) && K < (1ll << 31) &&
@@ -1853,14 +1875,8 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     }
     // every other block length up to 128, any pitch and alignment
     if (f->tile == 0 && axis == 0 && L.b <= 128 && ((rows + COLT - 1) / COLT) * L.nkb < (1ll << 31)) {
-        const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
-#define HBFP_QCOL(PL, RQ, SRV) launch_chained(quant_col_block<PL, RQ, SRV>, grid, 128, 0, st, x, K, rows, ld, (int)L.b, one, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, tiles_n, FormArgs{}, nullptr)
-#define HBFP_QCOL_SR(PL, RQ) do { if (p.rounding) HBFP_QCOL(PL, RQ, true); else HBFP_QCOL(PL, RQ, false); } while (0)
-        if (L.planes == 1) { if (L.bp == 32) HBFP_QCOL_SR(1, 8); else if (L.bp == 64) HBFP_QCOL_SR(1, 16); else HBFP_QCOL_SR(1, 32); }
-        else { if (L.bp == 32) HBFP_QCOL_SR(2, 8); else if (L.bp == 64) HBFP_QCOL_SR(2, 16); else HBFP_QCOL_SR(2, 32); }
-#undef HBFP_QCOL_SR
-#undef HBFP_QCOL
-        return launch_status();
+        return L.planes == 1 ? launch_col_block<1>(x, K, rows, ld, (int)L.b, L.bp, L.nkb, one, L, mant, exps, st, FormArgs{}, nullptr)
+                             : launch_col_block<2>(x, K, rows, ld, (int)L.b, L.bp, L.nkb, one, L, mant, exps, st, FormArgs{}, nullptr);
     }
     if (f->tile == 0 && axis == 1 && L.b <= 128 && K < (1ll << 30) && rows * (L.kst / 8) < (1ll << 39)) {
         const bool vec = aligned && L.b % 4 == 0;          // every piece starts on a 16-byte boundary
@@ -1925,12 +1941,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
         return p.rounding ? launch_col_tma<FORM, 2, true>(x, K, rows, ld, p, L, out, scales, st) : launch_col_tma<FORM, 2, false>(x, K, rows, ld, p, L, out, scales, st);
     }
     if (((rows + COLT - 1) / COLT) * L.nkb >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
-    const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT), grid = (unsigned)(tiles_n * L.nkb);
-#define HBFP_QCOL(RQ, SRV) launch_chained(quant_col_block<FORM, RQ, SRV>, grid, 128, 0, st, x, K, rows, ld, (int)L.b, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, tiles_n, fa, nullptr)
-    if (L.bp == 32) { if (p.rounding) HBFP_QCOL(8, true); else HBFP_QCOL(8, false); }
-    else { if (p.rounding) HBFP_QCOL(16, true); else HBFP_QCOL(16, false); }
-#undef HBFP_QCOL
-    return launch_status();
+    return launch_col_block<FORM>(x, K, rows, ld, (int)L.b, L.bp, L.nkb, p, L, out, scales, st, fa, nullptr);
 }
 
 }  // namespace
