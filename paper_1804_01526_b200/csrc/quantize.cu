@@ -1405,31 +1405,45 @@ int launch_row_flat(const float* x, int64_t rows, int64_t K, int64_t ld, const Q
 
 // ------------------------------------------------------------------------------ quant_row_ragged
 
+// Quotient and remainder by a divisor known to the host (magic = floor((2^32 - 1) / d)), for numerators below 2^32: the estimate is at
+// most one short. A division of 64 bits per piece of eight was half of these kernels' instructions.
+struct Divisor { uint32_t d, magic; };
+inline Divisor divisor(uint32_t d) { return {d, 0xFFFFFFFFu / d}; }
+__device__ __forceinline__ uint32_t divide(uint32_t n, const Divisor& v, uint32_t& rest) {
+    uint32_t q = __umulhi(n, v.magic);
+    rest = n - q * v.d;
+    if (rest >= v.d) { rest -= v.d; ++q; }
+    return q;
+}
+
 // Blocks along rows for every other block length up to 128, row length, pitch and alignment (24 columns per block, odd row
 // lengths). As in quant_row_flat the packed row, padding included, is cut into pieces of eight elements numbered through the
 // whole matrix, LPB = bp / 8 lanes per block; a piece that lies in a block's padding loads nothing. Without alignment a lane
 // fetches its eight floats one by one (the sectors of a warp's pieces stay in L1 between them), and its eight draws may
 // straddle two Philox groups: the second call is made only then. One pass instead of the two of exps_axis1 and
-// mant_generic, which index, divide and draw per element: 1111 x 3001, b = 24, stochastic 53 -> 9.7 us, 16384 x 16384,
-// nearest-even 2627 -> 287 us.
+// mant_generic, which index, divide and draw per element: 16384 x 16384, b = 24, nearest-even 2627 -> 287 us. Matrices beyond 2^32
+// pieces are launched in parts. With a 64-bit division per piece, before / now: 10000 x 10000, b = 24, draws 168 / 152 us, 8320 x 1708,
+// b = 128, draws 24.7 / 20.6, 100 x 16380, b = 24, draws 8.3 / 5.2. (Unaligned rows: a lane per element of 32 neighbours, a warp reduction
+// and a byte store per 32 elements, 20000 x 3001, b = 24 210 us against 75; the three aligned quads around the eight floats 85.)
 template <int LPB, bool SR, int PLANES, bool VEC>
 __global__ void __launch_bounds__(256)
 quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int b, QParams p,
                  int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
-                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, uint32_t ppr, int64_t total, const FormArgs fa) {
+                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const Divisor ppr, int64_t row_first, uint32_t total, const FormArgs fa) {
     const Chain chain(p.beside);
     constexpr int ITEMS = 2;
     const int tid = threadIdx.x, lane = tid & 31;
     float e8[ITEMS][8];
     int64_t row[ITEMS];
-    int cb[ITEMS], kk0[ITEMS];             // block of the row; first element of the piece along the row
+    int cb[ITEMS], kk0[ITEMS], pc[ITEMS];             // block of the row; first element of the piece along the row; piece of the row
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const int64_t g = (int64_t)blockIdx.x * (256 * ITEMS) + i * 256 + tid;
-        row[i] = g / ppr;
-        const int pc = (int)(g - row[i] * ppr);
-        cb[i] = pc / LPB;
-        const int within = 8 * (pc - cb[i] * LPB);
+        const uint32_t g = blockIdx.x * (256u * ITEMS) + i * 256 + tid;
+        uint32_t rest;
+        row[i] = row_first + divide(g, ppr, rest);
+        pc[i] = (int)rest;
+        cb[i] = pc[i] / LPB;
+        const int within = 8 * (pc[i] - cb[i] * LPB);
         kk0[i] = cb[i] * b + within;
         const int n = (g < total && cb[i] < nkb) ? (int)min((int64_t)(b - within), K - kk0[i]) : 0;    // elements of the piece
         const float* src = x + row[i] * ld + kk0[i];
@@ -1444,32 +1458,38 @@ quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t l
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const bool live = (int64_t)blockIdx.x * (256 * ITEMS) + i * 256 + tid < total;
+        const bool live = blockIdx.x * (256u * ITEMS) + i * 256 + tid < total;
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
         if (SR) w = draws_of_eight(p, (uint64_t)(row[i] * K + kk0[i]));          // the matrix is rows x K as passed
         uint32_t am = amax8_bits(e8[i]);
 #pragma unroll
         for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
         const int s = block_exponent(am, p.m, p.exp_mode);
-        const int pc = cb[i] * LPB + (kk0[i] - cb[i] * b) / 8;
-        round_and_store8<SR, PLANES>(e8[i], s, p, w, mant, row[i] * kst + 8 * (int64_t)pc, plane_stride, live);
+        round_and_store8<SR, PLANES>(e8[i], s, p, w, mant, row[i] * kst + 8 * (int64_t)pc[i], plane_stride, live);
         check_exponent<PLANES>(s, fa);
         if (live && (lane % LPB) == 0 && cb[i] < nkb) store_exponent<PLANES>(exps, (int64_t)cb[i] * rs + row[i], s);
     }
-    if (!is_form(PLANES)) zero_padding_lines(exps, rows, rs, nkb);
+    if (!is_form(PLANES) && row_first == 0) zero_padding_lines(exps, rows, rs, nkb);
 }
 
-template <int LPB, bool VEC, int FORM = 0>
-int launch_row_ragged(const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
+// OUT: 1 or 2 planes or a form. vec: pieces of eight start on 16-byte boundaries.
+template <int OUT>
+int launch_row_ragged(bool vec, const float* x, int64_t rows, int64_t K, int64_t ld, const QParams& p, const Layout& L,
                       int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa = FormArgs{}) {
-    const uint32_t ppr = (uint32_t)(L.kst / 8);
-    const int64_t total = rows * ppr;
-    const unsigned grid = (unsigned)((total + 511) / 512);
-#define HBFP_QROW_RAGGED(SRV, PL) launch_chained(quant_row_ragged<LPB, SRV, PL, VEC>, grid, 256, 0, st, x, rows, K, ld, (int)L.b, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, ppr, total, fa)
-    if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QROW_RAGGED(true, FORM); else HBFP_QROW_RAGGED(false, FORM); }
-    else if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_RAGGED(true, 1); else HBFP_QROW_RAGGED(true, 2); }
-    else { if (L.planes == 1) HBFP_QROW_RAGGED(false, 1); else HBFP_QROW_RAGGED(false, 2); }
-#undef HBFP_QROW_RAGGED
+    const int64_t ppr = L.kst / 8, rows_per = std::max<int64_t>(1, ((1ll << 32) - 65536) / ppr);       // pieces of a row; rows of a launch
+    if (ppr >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
+    const Divisor d = divisor((uint32_t)ppr);
+    QParams q = p;
+    for (int64_t r = 0; r < rows; r += rows_per, q.beside = 0) {
+        const int64_t total = std::min(rows - r, rows_per) * ppr;
+#define HBFP_RAGGED(LPB, SRV, VEC) launch_chained(quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 511) / 512), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
+#define HBFP_RAGGED_SR(LPB, VEC) do { if (p.rounding) HBFP_RAGGED(LPB, true, VEC); else HBFP_RAGGED(LPB, false, VEC); } while (0)
+#define HBFP_RAGGED_VEC(LPB) do { if (vec) HBFP_RAGGED_SR(LPB, true); else HBFP_RAGGED_SR(LPB, false); } while (0)
+        if (L.bp == 32) HBFP_RAGGED_VEC(4); else if (L.bp == 64) HBFP_RAGGED_VEC(8); else HBFP_RAGGED_VEC(16);
+#undef HBFP_RAGGED_VEC
+#undef HBFP_RAGGED_SR
+#undef HBFP_RAGGED
+    }
     return launch_status();
 }
 
@@ -1880,9 +1900,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     }
     if (f->tile == 0 && axis == 1 && L.b <= 128 && K < (1ll << 30) && rows * (L.kst / 8) < (1ll << 39)) {
         const bool vec = aligned && L.b % 4 == 0;          // every piece starts on a 16-byte boundary
-        if (L.bp == 32) return vec ? launch_row_ragged<4, true>(x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<4, false>(x, rows, K, ld, one, L, mant, exps, st);
-        if (L.bp == 64) return vec ? launch_row_ragged<8, true>(x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<8, false>(x, rows, K, ld, one, L, mant, exps, st);
-        return vec ? launch_row_ragged<16, true>(x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<16, false>(x, rows, K, ld, one, L, mant, exps, st);
+        return L.planes == 1 ? launch_row_ragged<1>(vec, x, rows, K, ld, one, L, mant, exps, st) : launch_row_ragged<2>(vec, x, rows, K, ld, one, L, mant, exps, st);
     }
     if (f->tile > 0 && f->tile <= 128) {
         // single view of a tiled weight: the fused tile kernel with the other view switched off
@@ -1931,9 +1949,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
             return launch_status();
         }
         if (K >= (1ll << 30) || rows * (L.kst / 8) >= (1ll << 39)) return HBFP_ERR_UNSUPPORTED;
-        const bool vec = aligned && L.b % 4 == 0;
-        if (L.bp == 32) return vec ? launch_row_ragged<4, true, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_ragged<4, false, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
-        return vec ? launch_row_ragged<8, true, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_ragged<8, false, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
+        return launch_row_ragged<FORM>(aligned && L.b % 4 == 0, x, rows, K, ld, p, L, out, scales, st, fa);
     }
     if (aligned && L.b == L.bp && (p.rounding == 0 || rows % 8 == 0) && rows < (1ll << 29) && K < (1ll << 31) &&
         ((rows + QC_COLS - 1) / QC_COLS) * (L.kst / QC_ROWS) < (1ll << 31)) {
