@@ -47,7 +47,7 @@ constexpr int RESCALE_WARPS = 8;                   // two per sub-partition
 constexpr int COL_GROUPS = RESCALE_WARPS / 4;      // warps sharing a lane quarter split the columns
 // The control warps take the lowest warp ids: the issue logic favours them over the rescale
 // warps of the same sub-partition, and a starved MMA issuer stalls the whole pipeline.
-constexpr int CONTROL_WARPS = 4;      // one warpgroup: producer, MMA issuer, table builder, one spare
+constexpr int CONTROL_WARPS = 4;      // one warpgroup: producer, MMA issuer, two table builders
 constexpr int PRODUCER_WARP = 0;
 constexpr int MMA_WARP = 1;
 constexpr int TABLE_WARP = 2;
@@ -309,7 +309,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     const uint32_t bar_off = table_off + C::TABLE_BYTES;
     const uint32_t bars = base + bar_off;
     const uint32_t full_bar = bars;                          // stage landed (mantissa tiles and exponent slices)
-    const uint32_t empty_bar = bars + 8 * STAGES;            // stage consumed (MMA commit + table warp)
+    const uint32_t empty_bar = bars + 8 * STAGES;            // stage consumed (MMA commit + table warps)
     const uint32_t tfull_bar = bars + 16 * STAGES;           // block sums complete (MMA commit) and scale table written
     const uint32_t tempty_bar = tfull_bar + 8 * GROUPS;      // group read (and re-armed) by every rescale warp
     const uint32_t done_bar = tempty_bar + 8 * GROUPS;
@@ -318,10 +318,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    // a second table builder where there are blocks enough to share (few and long ones: 2048 cube, one block per row, 13.8 us with one,
+    // 14.3 with two; one block of 64 per tile, 131072 x 576 x 64, 54.4 against 55.9)
+    const bool two_builders = !TSTORE && p.bp <= STAGE_K;
+
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(full_bar + 8 * s, 1);
-            mbar_init(empty_bar + 8 * s, 2);                 // MMA commit + table warp
+            mbar_init(empty_bar + 8 * s, two_builders ? 3 : 2);      // MMA commit + the table warps
         }
         for (int g = 0; g < GROUPS; ++g) {
             mbar_init(tfull_bar + 8 * g, 2);                 // MMA commit + table warp
@@ -396,13 +400,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 else if (sh.spb == 2) mma_issue_loop<N_TILE, PLANES, MAGIC, false, 2, TSTORE>(p, sh, ma);
                 else mma_issue_loop<N_TILE, PLANES, MAGIC, false, 1, TSTORE>(p, sh, ma);
             }
-        } else if (warp == TABLE_WARP) {
-            // -------------------------------------------------------------- scale-table builder
+        } else if (warp == TABLE_WARP || two_builders) {
+            // -------------------------------------------------------------- scale-table builders (warps 2 and 3)
+            // Warp 2 builds the tables of the even blocks (counted over all tiles), warp 3 those of the odd ones: one builder set the pace
+            // of narrow tiles, and its sleeping waits woke late. Packed operands, before / with prompt waits / with two builders:
+            // 936 x 748 x 1287, b = 24 18.2 / 16.7 / 15.3 us, 576 x 64 x 131072, b = 64 32.7 / 31.1 / 29.0, 400 x 4000 x 4000, b = 128
+            // 28.7 / 26.3 / 24.8, 2000 cube, b = 128 20.5 / 19.2 / 18.4.
             // The table of block b goes to slot b % (2 GROUPS) and its arrival counts on tfull[b % GROUPS].
             // It is written once the previous phase of that barrier (block b - GROUPS) is complete: the
             // MMAs of that block were issued only after every rescale warp had finished block
             // b - 2 GROUPS, the last reader of the slot, and the barrier is back in the phase that the
             // arrival for b belongs to.
+            static_assert(GROUPS % 2 == 0, "a builder keeps its groups");
+            const uint32_t me = (uint32_t)(warp - TABLE_WARP);
             uint32_t s = 0, ph = 0, g = 0, gph = 0, slot = 0, it = 0, blk = 0;
             bool ok = true, out_of_range = false;
             for (int wi = blockIdx.x; ok && wi < total_work; wi += gridDim.x) {
@@ -410,11 +420,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                 const int nst = stages_of(sh, w.nblk);
                 int left = w.nblk, sib = 0;
                 for (int si = 0; ok && si < nst; ++si, ++it) {
-                    if (!mbar_wait_warp(full_bar + 8 * s, ph, abort_flag, p.status, 401)) { ok = false; break; }
+                    if (!mbar_wait_warp_fast(full_bar + 8 * s, ph, abort_flag, p.status, 401)) { ok = false; break; }
                     const unsigned char* eA = base_ptr + (exp_base - base) + s * C::EXP_STAGE;
                     const unsigned char* eB = eA + C::EXP_A;
                     const int nb = sh.lng ? (sib == 0 ? 1 : 0) : min(sh.bps, left);   // blocks that start in this stage
                     for (int jb = 0; jb < nb; ++jb) {
+                        if (two_builders && (blk & 1u) != me) {
+                            ring_next<GROUPS>(g, gph);
+                            if (++slot == (uint32_t)TSLOTS) slot = 0;
+                            ++blk;
+                            continue;
+                        }
                         // this lane's N_TILE / 32 column exponents and 4 row exponents of the block
                         constexpr int CPL = N_TILE / 32;      // 8, 4 or 2 column bytes per lane
                         uint32_t cw[2] = {0u, 0u};
@@ -432,7 +448,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                         uint4 r0;
                         r0.x = exp_to_field(ra, 0, 127); r0.y = exp_to_field(ra, 1, 127);
                         r0.z = exp_to_field(ra, 2, 127); r0.w = exp_to_field(ra, 3, 127);
-                        if (!mbar_wait_warp(tfull_bar + 8 * g, gph ^ 1, abort_flag, p.status, 402)) { ok = false; break; }
+                        if (!mbar_wait_warp_fast(tfull_bar + 8 * g, gph ^ 1, abort_flag, p.status, 402)) { ok = false; break; }
                         uint32_t* tb = tables + slot * C::TABLE_SLOT_WORDS;
                         if (CPL == 8) {
                             *reinterpret_cast<uint4*>(tb + 8 * lane) = make_uint4(cs[0], cs[1], cs[2], cs[3]);
@@ -444,7 +460,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                         }
                         *reinterpret_cast<uint4*>(tb + N_TILE + 4 * lane) = r0;
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(tfull_bar + 8 * g);
+                        mbar_arrive_elect(tfull_bar + 8 * g);
                         ring_next<GROUPS>(g, gph);
                         if (++slot == (uint32_t)TSLOTS) slot = 0;
                         ++blk;
@@ -452,7 +468,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
                     if (sh.lng) { if (++sib == sh.spk) sib = 0; }
                     left -= nb;
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(empty_bar + 8 * s);      // the exponent slices are consumed
+                    mbar_arrive_elect(empty_bar + 8 * s);      // the exponent slices are consumed
                     ring_next<STAGES>(s, ph);
                 }
             }
@@ -500,7 +516,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
             for (int c = 0; c < COLS_PER_WARP / 2; ++c) acc2[c] = 0ull;
             for (int kb = w.kb0; kb < w.kb0 + w.nblk; ++kb, ++blk) {
                 // one wait per block: the block sums are complete and the scale table is written
-                if (!__all_sync(0xffffffffu, mbar_wait_quick(tfull_bar + 8 * g, gph, abort_flag, p.status, 302))) { ok = false; break; }
+                if (!mbar_wait_warp_fast(tfull_bar + 8 * g, gph, abort_flag, p.status, 302)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t taddr = lane_addr + g * PARTS * N_TILE;
                 const uint32_t* tab = tables + slot * C::TABLE_SLOT_WORDS + col0;
