@@ -239,7 +239,8 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     if (rc) return rc;
     if (small) {
         ran("gemm_small_kernel");
-        return launch_gemm_small(M, N, pa, pb, C, ldc, st);
+        *bias_done = true;
+        return launch_gemm_small(M, N, pa, pb, bias, C, ldc, st);
     }
     const bool quad_rows = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && (ldc % 4) == 0;
     const bool want_tensor = flags != HBFP_GEMM_FORCE_SIMT && g.tp.supported &&
@@ -256,7 +257,8 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         }
         if (flags == HBFP_GEMM_FORCE_TENSOR_2SM) return HBFP_ERR_UNSUPPORTED;
         ran("gemm_tc_kernel");
-        return launch_gemm_tensor(M, N, K, pa, pb, C, ldc, P, g.tp, ws ? ws + g.off_partial : nullptr, st);
+        *bias_done = !P && g.tp.splits > 1;
+        return launch_gemm_tensor(M, N, K, pa, pb, bias, C, ldc, P, g.tp, ws ? ws + g.off_partial : nullptr, st);
     }
     if (flags >= HBFP_GEMM_FORCE_TENSOR) return HBFP_ERR_UNSUPPORTED;
     ran("gemm_simt_kernel");

@@ -153,7 +153,7 @@ int launch_gemm_simt(int64_t M, int64_t N, int64_t K, const Packed& a, const Pac
 
 // Tiled dp4a kernel for small problems (gemm_small.cu): one-plane operands, one launch, no split-K.
 bool small_gemm_eligible(int64_t M, int64_t N, const Packed& a, const Packed& b, bool any_size);
-int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, float* C, int64_t ldc, cudaStream_t st);
+int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, const float* bias, float* C, int64_t ldc, cudaStream_t st);
 // The same from FP32 operands, conversion included (contig: K is contiguous).
 bool small_fused_eligible(const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, int64_t M, int64_t N, const Layout& la);
 int launch_gemm_small_fused(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, const Layout& la,
@@ -177,7 +177,8 @@ struct TensorPlan {
 };
 TensorPlan plan_gemm_tensor(int64_t M, int64_t N, int64_t K, const Layout& la, const Layout& lb,
                             int mant_bits_a, int mant_bits_b);
-int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const Packed& b, float* C,
+// bias: added by the sum of the parts, only where K is split (plan.splits > 1).
+int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const Packed& b, const float* bias, float* C,
                        int64_t ldc, int32_t* P, const TensorPlan& plan, void* partial,
                        cudaStream_t st);
 

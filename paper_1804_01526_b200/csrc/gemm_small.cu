@@ -35,7 +35,7 @@ __device__ __forceinline__ void copy16_async(void* dst_shared, const void* src_g
 __global__ void __launch_bounds__(256)
 gemm_small_kernel(int64_t M, int64_t N, int nkb, int bp, const int8_t* __restrict__ mA, int64_t kstA,
                   const int8_t* __restrict__ eA, int64_t rsA, const int8_t* __restrict__ mB, int64_t kstB,
-                  const int8_t* __restrict__ eB, int64_t rsB, float* __restrict__ C, int64_t ldc) {
+                  const int8_t* __restrict__ eB, int64_t rsB, const float* __restrict__ bias, float* __restrict__ C, int64_t ldc) {
     chain_start();
     extern __shared__ __align__(16) unsigned char smem[];
     int8_t* xA = reinterpret_cast<int8_t*>(smem + 2 * SM_BUF);  // [nkb][32]
@@ -125,7 +125,7 @@ gemm_small_kernel(int64_t M, int64_t N, int nkb, int bp, const int8_t* __restric
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
             const int64_t i = i0 + cr0 + 8 * a, j = j0 + cc0 + b;
-            if (i < M && j < N) C[i * ldc + j] = acc[2 * a + b];
+            if (i < M && j < N) C[i * ldc + j] = bias ? __fadd_rn(acc[2 * a + b], __ldg(bias + j)) : acc[2 * a + b];
         }
 }
 
@@ -313,7 +313,7 @@ bool small_gemm_eligible(int64_t M, int64_t N, const Packed& a, const Packed& b,
     return any_size || (a.L.nkb * a.L.bp <= SM_AUTO_BYTES && ctas <= SM_AUTO_CTAS);
 }
 
-int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, float* C, int64_t ldc, cudaStream_t st) {
+int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, const float* bias, float* C, int64_t ldc, cudaStream_t st) {
     const int nkb = (int)a.L.nkb;
     const size_t smem = 2 * SM_BUF + 2 * (size_t)nkb * SM_TILE;          // at most 132 KB
     // the attribute belongs to the device: set once per device (same value from any thread)
@@ -326,7 +326,7 @@ int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, fl
     }
     const dim3 grid((unsigned)((N + SM_TILE - 1) / SM_TILE), (unsigned)((M + SM_TILE - 1) / SM_TILE));
     launch_chained(gemm_small_kernel, grid, 256, smem, st, M, N, nkb, (int)a.L.bp, a.mant, a.L.kst, a.exps, a.L.rs, b.mant, b.L.kst,
-                                               b.exps, b.L.rs, C, ldc);
+                                               b.exps, b.L.rs, bias, C, ldc);
     return launch_status();
 }
 

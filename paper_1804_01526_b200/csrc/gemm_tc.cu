@@ -719,9 +719,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     }
 }
 
-// Sums the split-K partial tiles in ascending split order.
+// Sums the split-K partial tiles in ascending split order, then adds the bias (may be null) of the column.
 __global__ void splitk_reduce(const float* __restrict__ partial, int splits, int64_t M, int64_t N, int64_t ldp,
-                              float* __restrict__ C, int64_t ldc) {
+                              const float* __restrict__ bias, float* __restrict__ C, int64_t ldc) {
     chain_start();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= M * N) return;
@@ -737,7 +737,7 @@ __global__ void splitk_reduce(const float* __restrict__ partial, int splits, int
         for (int k = 0; k < 8; ++k)
             if (s + k < splits) acc = s + k == 0 ? v[0] : __fadd_rn(acc, v[k]);
     }
-    C[r * ldc + c] = acc;
+    C[r * ldc + c] = bias ? __fadd_rn(acc, __ldg(bias + c)) : acc;
 }
 
 // ------------------------------------------------------------------------------ host side
@@ -863,7 +863,7 @@ TensorPlan plan_gemm_tensor(int64_t M, int64_t N, int64_t K, const Layout& la, c
     return t;
 }
 
-int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const Packed& b, float* Cout, int64_t ldc,
+int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const Packed& b, const float* bias, float* Cout, int64_t ldc,
                        int32_t* P, const TensorPlan& plan, void* partial, cudaStream_t st) {
     (void)K;
     if (!plan.supported) return HBFP_ERR_UNSUPPORTED;
@@ -905,7 +905,7 @@ int launch_gemm_tensor(int64_t M, int64_t N, int64_t K, const Packed& a, const P
     if (rc) return rc;
     if (p.splits > 1) {
         const int64_t n = M * N;
-        launch_chained(splitk_reduce, (unsigned)((n + 255) / 256), 256, 0, st, p.partial, p.splits, M, N, p.ldp, Cout, ldc);
+        launch_chained(splitk_reduce, (unsigned)((n + 255) / 256), 256, 0, st, p.partial, p.splits, M, N, p.ldp, bias, Cout, ldc);
         return launch_status();
     }
     return HBFP_OK;

@@ -409,3 +409,16 @@ def test_column_sums_of_more_columns_than_a_grid_has(env, rows, cols):
                                      ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
     d = x.double()
     assert bool(((out[:-1].double() - d.sum(0)).abs() <= (rows + 1) * 2.0 ** -24 * d.abs().sum(0)).all()) and float(out[-1]) == 7.0
+
+
+@pytest.mark.parametrize("batch,fin,fout,tile", [(300, 296, 92, 32), (520, 64, 33, 24), (936, 1287, 200, 24), (130, 4000, 70, 64), (700, 640, 640, 64), (16, 256, 130, 32)])
+def test_bias_added_by_whichever_kernel_ends_the_product(env, batch, fin, fout, tile):
+    """The smallest products, sums of split-K parts, unsplit tiles and a few rows: the value of adding it afterwards, bit for bit."""
+    torch, hbfp_nn, hb = env
+    layer = hbfp_nn.HbfpLinear(fin, fout, tile=tile, rounding=0)
+    x = torch.randn(batch, fin, device="cuda")
+    with torch.no_grad():
+        plain = layer(x)
+        layer.bias.normal_()
+        assert torch.equal(layer(x), plain + layer.bias)
+    assert hb.device_status() == 0
