@@ -217,6 +217,21 @@ struct Buffers {
     }
 };
 
+// packed_layout(rows, k, fmt) -> the members of hbfp_layout by name
+PyObject* packed_layout(PyObject*, PyObject* const* a, Py_ssize_t n) {
+    if (!want(n, 3)) return nullptr;
+    return guarded([&]() -> PyObject* {
+        const int64_t rows = as_ll(a[0]), k = as_ll(a[1]);
+        const hbfp_format f = format_of(a[2]);
+        hbfp_layout L;
+        const int rc = api.packed_layout(rows, k, &f, &L);
+        if (rc) return code(rc);
+        return Py_BuildValue("{sLsLsLsLsLsLsLsLsLsLsL}", "rows", (long long)L.rows, "k", (long long)L.k, "b", (long long)L.b, "bp", (long long)L.bp, "nkb", (long long)L.nkb,
+                             "kst", (long long)L.kst, "planes", (long long)L.planes, "plane_stride", (long long)L.plane_stride, "rs", (long long)L.rs,
+                             "mant_bytes", (long long)L.mant_bytes, "exp_bytes", (long long)L.exp_bytes);
+    });
+}
+
 // quantize(x, axis, fmt, mant or None, exps or None) -> (mant, exps)
 PyObject* quantize(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (!want(n, 5)) return nullptr;
@@ -705,7 +720,7 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 #define HBFP_METHOD(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
-PyMethodDef methods[] = {HBFP_METHOD(bind), HBFP_METHOD(quantize), HBFP_METHOD(gemm), HBFP_METHOD(gemm_q), HBFP_METHOD(wide_update),
+PyMethodDef methods[] = {HBFP_METHOD(bind), HBFP_METHOD(packed_layout), HBFP_METHOD(quantize), HBFP_METHOD(gemm), HBFP_METHOD(gemm_q), HBFP_METHOD(wide_update),
                          HBFP_METHOD(wide_dequantize), HBFP_METHOD(conv_forward), HBFP_METHOD(conv_dgrad_filters),
                          HBFP_METHOD(im2col_packed_t), HBFP_METHOD(linear), HBFP_METHOD(conv3x3),
                          {nullptr, nullptr, 0, nullptr}};
