@@ -1425,27 +1425,37 @@ __device__ __forceinline__ uint32_t divide(uint32_t n, const Divisor& v, uint32_
 // pieces are launched in parts. With a 64-bit division per piece, before / now: 10000 x 10000, b = 24, draws 168 / 152 us, 8320 x 1708,
 // b = 128, draws 24.7 / 20.6, 100 x 16380, b = 24, draws 8.3 / 5.2. (Unaligned rows: a lane per element of 32 neighbours, a warp reduction
 // and a byte store per 32 elements, 20000 x 3001, b = 24 210 us against 75; the three aligned quads around the eight floats 85.)
+// Pieces of a warp. On unaligned rows with draws, as many whole blocks as 64 Philox groups serve: their elements are consecutive, so two
+// calls per lane into a table per warp do for what took two per piece (5001 columns, b = 32, 4999 rows 45.2 -> 39.6 us, 1111 x 3001,
+// b = 24 9.7 -> 8.0). Aligned rows mostly start at a group and need one call per piece; the lanes that the table leaves idle cost them
+// more (10000 x 10000, b = 24 152 -> 177, 8320 x 1708, b = 128 20.6 -> 25.9).
+template <int LPB, bool TABLE>
+__host__ __device__ constexpr int ragged_pieces() { return TABLE ? 64 - LPB : 64; }
+
 template <int LPB, bool SR, int PLANES, bool VEC>
 __global__ void __launch_bounds__(256)
 quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int b, QParams p,
                  int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                  int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const Divisor ppr, int64_t row_first, uint32_t total, const FormArgs fa) {
     const Chain chain(p.beside);
-    constexpr int ITEMS = 2;
-    const int tid = threadIdx.x, lane = tid & 31;
+    constexpr bool TABLE = SR && !VEC;
+    constexpr int ITEMS = 2, PIECES = ragged_pieces<LPB, TABLE>();
+    __shared__ __align__(16) uint4 rnd[TABLE ? 8 : 1][TABLE ? 65 : 1];         // (the word after the last group is read and not used)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t g0 = (blockIdx.x * 8 + warp) * PIECES;
     float e8[ITEMS][8];
     int64_t row[ITEMS];
     int cb[ITEMS], kk0[ITEMS], pc[ITEMS];             // block of the row; first element of the piece along the row; piece of the row
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const uint32_t g = blockIdx.x * (256u * ITEMS) + i * 256 + tid;
+        const uint32_t g = g0 + i * 32 + lane;
         uint32_t rest;
         row[i] = row_first + divide(g, ppr, rest);
         pc[i] = (int)rest;
         cb[i] = pc[i] / LPB;
         const int within = 8 * (pc[i] - cb[i] * LPB);
         kk0[i] = cb[i] * b + within;
-        const int n = (g < total && cb[i] < nkb) ? (int)min((int64_t)(b - within), K - kk0[i]) : 0;    // elements of the piece
+        const int n = (g < total && i * 32 + lane < PIECES && cb[i] < nkb) ? (int)min((int64_t)(b - within), K - kk0[i]) : 0;    // elements of the piece
         const float* src = x + row[i] * ld + kk0[i];
         if (VEC && n >= 8) {
             const float4 u = __ldcs(reinterpret_cast<const float4*>(src)), w = __ldcs(reinterpret_cast<const float4*>(src) + 1);
@@ -1456,11 +1466,26 @@ quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t l
             for (int j = 0; j < 8; ++j) e8[i][j] = j < n ? __ldg(src + j) : 0.f;
         }
     }
+    // the draws do not depend on the data: they are made while the loads are in flight (the matrix is rows x K as passed)
+    uint64_t first = 0;
+    if (TABLE) {
+        first = __shfl_sync(0xffffffffu, (unsigned long long)(row[0] * K + min((int64_t)kk0[0], K)), 0) >> 3;
+        rnd[TABLE ? warp : 0][TABLE ? lane : 0] = draws_of_group(p, first + lane);
+        rnd[TABLE ? warp : 0][TABLE ? lane + 32 : 0] = draws_of_group(p, first + lane + 32);
+        __syncwarp();
+    }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
-        const bool live = blockIdx.x * (256u * ITEMS) + i * 256 + tid < total;
+        const bool live = g0 + i * 32 + lane < total && i * 32 + lane < PIECES;
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (SR) w = draws_of_eight(p, (uint64_t)(row[i] * K + kk0[i]));          // the matrix is rows x K as passed
+        if (SR && VEC) w = draws_of_eight(p, (uint64_t)(row[i] * K + kk0[i]));
+        if (TABLE) {
+            const int at = live && cb[i] < nkb ? (int)((uint64_t)(row[i] * K + min((int64_t)kk0[i], K)) - 8 * first) : 0;     // halfword of the table
+            const uint32_t* word = reinterpret_cast<const uint32_t*>(rnd[TABLE ? warp : 0]) + (at >> 1);
+            const uint32_t t[5] = {word[0], word[1], word[2], word[3], word[4]};
+            w = at & 1 ? make_uint4(__funnelshift_r(t[0], t[1], 16), __funnelshift_r(t[1], t[2], 16), __funnelshift_r(t[2], t[3], 16), __funnelshift_r(t[3], t[4], 16))
+                       : make_uint4(t[0], t[1], t[2], t[3]);
+        }
         uint32_t am = amax8_bits(e8[i]);
 #pragma unroll
         for (int off = 1; off < LPB; off <<= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
@@ -1482,7 +1507,7 @@ int launch_row_ragged(bool vec, const float* x, int64_t rows, int64_t K, int64_t
     QParams q = p;
     for (int64_t r = 0; r < rows; r += rows_per, q.beside = 0) {
         const int64_t total = std::min(rows - r, rows_per) * ppr;
-#define HBFP_RAGGED(LPB, SRV, VEC) launch_chained(quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 511) / 512), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
+#define HBFP_RAGGED(LPB, SRV, VEC) launch_chained(quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 8 * ragged_pieces<LPB, SRV && !VEC>() - 1) / (8 * ragged_pieces<LPB, SRV && !VEC>())), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
 #define HBFP_RAGGED_SR(LPB, VEC) do { if (p.rounding) HBFP_RAGGED(LPB, true, VEC); else HBFP_RAGGED(LPB, false, VEC); } while (0)
 #define HBFP_RAGGED_VEC(LPB) do { if (vec) HBFP_RAGGED_SR(LPB, true); else HBFP_RAGGED_SR(LPB, false); } while (0)
         if (L.bp == 32) HBFP_RAGGED_VEC(4); else if (L.bp == 64) HBFP_RAGGED_VEC(8); else HBFP_RAGGED_VEC(16);

@@ -363,3 +363,19 @@ def test_streaming_column_quantiser_gives_the_same_bytes_every_time(hb, b, m):
     ref = hb.gemm_q(1024, 4096, 4096, hb.quantize(a, 0, f), want, flags=hb.GEMM_FORCE_SIMT)
     assert int(wrong) == 0 and hb.device_status() == 0
     assert bool(((first - ref).abs() <= 2e-5 * ref.abs().max()).all())
+
+
+# The ragged kernels where their units end: one element, one block less or more than a warp's, blocks of one, two and four warps, rows that
+# start at every alignment, draws that straddle groups, a table of draws that ends inside a row.
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("lines,K,b,m,rounding", [
+    (1, 1, 24, 8, 1), (33, 23, 24, 8, 1), (31, 25, 24, 12, 0), (65, 120, 24, 8, 0), (7, 361, 24, 8, 1), (40, 97, 32, 8, 1), (37, 515, 32, 4, 1), (29, 127, 48, 12, 1),
+    (64, 129, 64, 8, 0), (35, 449, 64, 8, 1), (3, 255, 100, 8, 1), (33, 385, 128, 8, 1), (130, 257, 128, 12, 0), (5, 4000, 20, 8, 1)])
+def test_ragged_row_and_column_kernels_at_their_edges(hb, axis, lines, K, b, m, rounding):
+    fd = dict(mant_bits=m, block=b, rounding=rounding, seed=21, stream_id=3)
+    x = wl.draw("lognormal", (lines, K) if axis == 1 else (K, lines), seed=5)
+    p = hb.quantize(to_dev(x), axis, gfmt(fd))
+    q, s = decode_packed(p, hb.packed_layout(p.rows, p.k, p.fmt))
+    q_ref, s_ref = oracle.quantize(x, axis, ofmt(fd))
+    assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
+    assert hb.device_status() == 0
