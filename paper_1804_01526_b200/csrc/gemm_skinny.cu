@@ -362,7 +362,7 @@ int sk_launch(const SkinnyProblem& p, const CUtensorMap& mW, size_t smem, dim3 g
         HBFP_CUDA_OK(cudaFuncSetAttribute(gemm_skinny_kernel<ROWS, BP, SR>, cudaFuncAttributeMaxDynamicSharedMemorySize, SK_SMEM_LIMIT));
         ready[dev] = true;
     }
-    launch_chained_clusters(gemm_skinny_kernel<ROWS, BP, SR>, p.splits, grid, SK_THREADS, smem, st, mW, p);
+    launch_chained_clusters(gemm_skinny_kernel<ROWS, BP, SR>, p.splits, grid, SK_THREADS, smem, st, true, mW, p);
     return launch_status();
 }
 template <int ROWS, bool SR>

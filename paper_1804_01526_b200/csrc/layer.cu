@@ -145,7 +145,7 @@ int column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* o
     while (splits < 8 && rows >= 2 * splits * CS_WARPS * CS_UNR) splits *= 2;
     for (int64_t c0 = 0; c0 < cols; c0 += MOST) {
         const int64_t n = cols - c0 < MOST ? cols - c0 : MOST;
-        launch_chained_clusters(column_sums_kernel<V>, splits, dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V))), 32 * CS_WARPS, 0, st, x + c0, rows, n, ld,
+        launch_chained_clusters(column_sums_kernel<V>, splits, dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V))), 32 * CS_WARPS, 0, st, true, x + c0, rows, n, ld,
                                 splits, out + c0);
         if (launch_status()) return HBFP_ERR_CUDA;
     }
