@@ -137,9 +137,9 @@ int check_fp32(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K) {
     return o->ld < (k_contiguous(o, is_a) ? K : rows) ? HBFP_ERR_INVALID_ARG : HBFP_OK;
 }
 
-// Quantises an FP32 operand into the workspace (or takes a packed one as is). beside: next to the conversion launched before.
+// Quantises an FP32 operand into the workspace (or takes a packed one as is).
 int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const Layout& L,
-                    char* ws, size_t off_m, size_t off_e, Packed* out, bool beside, cudaStream_t st) {
+                    char* ws, size_t off_m, size_t off_e, Packed* out, int place, cudaStream_t st) {
     out->L = L;
     out->mant_bits = o->fmt.mant_bits;
     if (o->kind == HBFP_OPERAND_PACKED) {
@@ -157,25 +157,24 @@ int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, c
     out->mant = m;
     out->exps = e;
     const float* x = static_cast<const float*>(o->data);
-    return k_contiguous(o, is_a) ? launch_quantize(x, rows, K, o->ld, 1, &o->fmt, m, e, st, beside) : launch_quantize(x, K, rows, o->ld, 0, &o->fmt, m, e, st, beside);
+    return k_contiguous(o, is_a) ? launch_quantize(x, rows, K, o->ld, 1, &o->fmt, m, e, st, place) : launch_quantize(x, K, rows, o->ld, 0, &o->fmt, m, e, st, place);
 }
 
 // An operand in the floating-point form at `f`: converted straight to it where it is an FP32 matrix without weight tiles,
-// otherwise packed (or taken packed) and expanded. B is converted beside A (which always has a launch), except through the packed
-// place, which both may use.
-int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const GemmPlan& g, char* ws, const FpOperand& f, cudaStream_t st) {
+// otherwise packed (or taken packed) and expanded; the place is that of the last launch. The packed place is one for both operands.
+int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const GemmPlan& g, char* ws, const FpOperand& f, int place, cudaStream_t st) {
     if (o->kind == HBFP_OPERAND_FP32) {
         const int rc = check_fp32(o, is_a, rows, K);
         if (rc) return rc;
         const float* x = static_cast<const float*>(o->data);
         if (o->fmt.tile == 0)          // always covered where plan_gemm_fp takes the forms; a packed place is not reserved for these
-            return k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, !is_a, f, st)
-                                         : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, !is_a, f, st);
+            return k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, place, f, st)
+                                         : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, place, f, st);
     }
     Packed p;
-    const int rc = resolve_operand(o, is_a, rows, K, is_a ? g.la : g.lb, ws, g.off_fm, g.off_fe, &p, false, st);
+    const int rc = resolve_operand(o, is_a, rows, K, is_a ? g.la : g.lb, ws, g.off_fm, g.off_fe, &p, CHAINED, st);
     if (rc) return rc;
-    return launch_expand(p, g.fp, !is_a, !is_a && o->kind == HBFP_OPERAND_PACKED, f, st);
+    return launch_expand(p, g.fp, !is_a, place, f, st);
 }
 
 // bias (may be null) is added in the kernel's own store where it can; *bias_done says so, otherwise the caller adds it.
@@ -217,7 +216,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         b->kind == HBFP_OPERAND_PACKED && skinny_gemm_eligible(M, N, g.la, g.lb, a->fmt.mant_bits, b->fmt.mant_bits)) {
         rc = check_fp32(a, true, M, K);
         if (rc) return rc;
-        rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, false, st);
+        rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, CHAINED, st);
         if (rc) return rc;
         ran("gemm_skinny_kernel");
         *bias_done = true;
@@ -225,17 +224,20 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     }
     if (use_fp && !small) {
         const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
-        rc = resolve_form(a, true, M, K, g, ws, fa, st);
+        const bool beside = b->kind == HBFP_OPERAND_PACKED || b->fmt.tile == 0;       // B in one launch
+        rc = resolve_form(a, true, M, K, g, ws, fa, beside ? LEAD : CHAINED, st);
         if (rc) return rc;
-        rc = resolve_form(b, false, N, K, g, ws, fb, st);
+        rc = resolve_form(b, false, N, K, g, ws, fb, beside ? BESIDE : CHAINED, st);
         if (rc) return rc;
         ran("gemm_tc_kernel", g.fp.pair ? "gemm_fp_kernel/pair" : g.fp.splits > 1 ? "gemm_fp_kernel/split" : "gemm_fp_kernel");
         *bias_done = true;
         return launch_gemm_fp(M, N, g.la, g.fp, fa, fb, bias, C, ldc, st);
     }
-    rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, false, st);
+    // two conversions of one launch each (longer blocks and weight tiles may take several, or another kernel)
+    const bool beside = a->kind == HBFP_OPERAND_FP32 && b->kind == HBFP_OPERAND_FP32 && a->fmt.tile == 0 && b->fmt.tile == 0 && K > 0 && g.la.b <= 256;
+    rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, beside ? LEAD : CHAINED, st);
     if (rc) return rc;
-    rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, a->kind == HBFP_OPERAND_FP32 && K > 0, st);
+    rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, beside ? BESIDE : CHAINED, st);
     if (rc) return rc;
     if (small) {
         ran("gemm_small_kernel");

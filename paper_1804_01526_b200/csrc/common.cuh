@@ -69,12 +69,23 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 
 __device__ __forceinline__ void chain_start() { chain_wait(); chain_next(); }
 
-// The conversion of a product's second operand depends on nothing that the conversion of the first one does: it runs beside it
-// (`beside`) and waits only when it is through. What both depend on has ended by then, because the first conversion says
-// chain_next after its own wait; what follows waits for the second one and with it for both.
+// How a launch follows the one before it on its stream.
+//   CHAINED  as above
+//   LEAD     not before that kernel has ended, as any launch; the next one may run beside it
+//   BESIDE   next to the launch before it, which is a LEAD (or the last of a conversion that has one): the conversion of a product's
+//            second operand, which reads and writes nothing that the conversion of the first one writes. It waits when it is through,
+//            and what follows waits for it and with it for both.
+// What a BESIDE kernel reads without waiting has to be visible to it by other means than chain_wait, which gives the waiting grid the
+// writes of the kernel before it and no other grid anything: the weights that a chained update has just written reach a conversion
+// two launches later only because a whole kernel boundary lies between. The LEAD is that boundary: it is launched when everything
+// before it has ended and been flushed, and nothing that the BESIDE kernel reads is written from then on.
+// Back to back, all three launches chained / with LEAD and BESIDE (with a chained conversion in place of the LEAD, which has no such
+// boundary): 1111 x 777 x 3001 (b = 24, with draws) 36.3 / 34.8 us (33.7), 1024 x 4096 x 4096 (b = 32) 71.2 / 69.0 (67.9), 4096 cube,
+// 12 bits 329.7 / 328.1 (326.3).
+enum Place : int { CHAINED = 0, LEAD = 1, BESIDE = 2 };
 struct Chain {
     bool beside;
-    __device__ __forceinline__ explicit Chain(int b) : beside(b != 0) {
+    __device__ __forceinline__ explicit Chain(int place) : beside(place == BESIDE) {
         if (!beside) chain_wait();
         chain_next();
     }
@@ -82,7 +93,7 @@ struct Chain {
 };
 
 template <class... Params, class... Args>
-inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+inline void launch_placed(int place, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.gridDim = grid;
@@ -92,8 +103,12 @@ inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = place == LEAD ? 0 : 1;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);      // launch_status() has the verdict
+}
+template <class... Params, class... Args>
+inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    launch_placed(CHAINED, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 // The same with clusters of `cluster` CTAs along x; not chained where the kernel's tiles want the order of an empty chip (gemm_fp.cu).
 template <class... Params, class... Args>
@@ -127,9 +142,10 @@ struct Packed {
 };
 
 // Quantiser launchers (quantize.cu).
-// beside: the kernel launched before on the stream is a conversion that shares no memory with this one (see Chain).
+// place: LEAD or BESIDE for the first and the second of two conversions that share no memory; a conversion of several launches is
+// CHAINED in place of BESIDE.
 int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int contract_axis,
-                    const hbfp_format* f, int8_t* mant, int8_t* exps, cudaStream_t st, bool beside = false);
+                    const hbfp_format* f, int8_t* mant, int8_t* exps, cudaStream_t st, int place = CHAINED);
 int launch_quantize_tiles(const float* w, int64_t d0, int64_t d1, int64_t ld, const hbfp_format* f,
                           int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1,
                           int8_t* tile_exps, cudaStream_t st);
@@ -205,10 +221,10 @@ struct FpPlan {
     int form, pair, ncol, splits, kb_per_split, planes_b;
 };
 FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, int passes);
-int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, bool beside, const FpOperand& out, cudaStream_t st);
+int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, int place, const FpOperand& out, cudaStream_t st);
 // Converts an FP32 operand straight to a form (quantize.cu); HBFP_ERR_UNSUPPORTED for weight tiles.
 int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int contract_axis, const hbfp_format* f, int wide, bool is_b,
-                         bool beside, const FpOperand& out, cudaStream_t st);
+                         int place, const FpOperand& out, cudaStream_t st);
 int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, const float* bias, float* C,
                    int64_t ldc, cudaStream_t st);
 

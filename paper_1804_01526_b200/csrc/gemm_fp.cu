@@ -577,8 +577,8 @@ __device__ __forceinline__ uint32_t f16_pair(float a, float b) {        // exact
 // Form S: rows x kst bytes of one-plane mantissas -> bfloat16 q * 2^s, 16 elements per thread.
 __global__ void __launch_bounds__(256)
 expand_s_kernel(const int8_t* __restrict__ q, const int8_t* __restrict__ exps, int64_t rows, int kst, int lg_bp, int nkb, int64_t rs,
-                uint4* __restrict__ out, int beside) {
-    const Chain chain(beside);
+                uint4* __restrict__ out, int place) {
+    const Chain chain(place);
     const int per = kst >> 4;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= rows * per) return;
@@ -601,8 +601,8 @@ expand_s_kernel(const int8_t* __restrict__ q, const int8_t* __restrict__ exps, i
 template <bool IS_B>
 __global__ void __launch_bounds__(256)
 expand_w_kernel(const int8_t* __restrict__ q, int64_t plane_stride, const int8_t* __restrict__ exps, int64_t rows, int kst, int lg_bp, int nkb,
-                int64_t rs, uint4* __restrict__ out, uint4* __restrict__ out_l, float* __restrict__ scales, int32_t* status, int beside) {
-    const Chain chain(beside);
+                int64_t rs, uint4* __restrict__ out, uint4* __restrict__ out_l, float* __restrict__ scales, int32_t* status, int place) {
+    const Chain chain(place);
     const int per = kst >> 3;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= rows * per) return;
@@ -803,20 +803,20 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, in
     return f;
 }
 
-int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, bool beside, const FpOperand& out, cudaStream_t st) {
+int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, int place, const FpOperand& out, cudaStream_t st) {
     const Layout& L = x.L;
     const int lg = log2_of(L.bp);
     if (plan.form == FORM_S) {
         const int64_t n = L.rows * (L.kst / 16);
-        launch_chained(expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), (int)beside);
+        launch_placed(place, expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), place);
         return launch_status();
     }
     int32_t* status = device_status_word();
     if (!status) return HBFP_ERR_CUDA;
     const int64_t n = L.rows * (L.kst / 8);
     const unsigned g = (unsigned)((n + 255) / 256);
-    if (is_b) launch_chained(expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, (int)beside);
-    else launch_chained(expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, (int)beside);
+    if (is_b) launch_placed(place, expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, place);
+    else launch_placed(place, expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, place);
     return launch_status();
 }
 

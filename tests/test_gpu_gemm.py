@@ -671,3 +671,89 @@ def test_calls_in_a_row_give_what_each_gives_alone(hb, M, N, K, m, b, rounding, 
     for _ in range(4):
         assert all(torch.equal(x, y) for x, y in zip(run(False), want))
     assert hb.device_status() == 0
+
+
+def edges_in_order(graph) -> list:
+    """The kinds of the edges of a captured chain of nodes, from its first node on: 0 the whole of the node before, 1 programmatic."""
+    import ctypes
+    driver, raw, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert driver.cuGraphGetEdges_v2(raw, None, None, None, ctypes.byref(n)) == 0
+    source, target, data = (ctypes.c_uint64 * n.value)(), (ctypes.c_uint64 * n.value)(), (ctypes.c_uint8 * 8 * n.value)()
+    assert driver.cuGraphGetEdges_v2(raw, source, target, data, ctypes.byref(n)) == 0
+    step = {a: (b, d[2]) for a, b, d in zip(source, target, data)}         # third byte of CUgraphEdgeData: the type
+    assert len(step) == n.value                                 # one way through
+    (at,) = set(step) - {b for b, _ in step.values()}
+    kinds = []
+    while at in step:
+        at, kind = step[at]
+        kinds.append(kind)
+    return kinds
+
+
+# The conversion that runs beside another one reads before it has waited for anything: what a chained kernel wrote is visible to it only
+# past a whole kernel boundary, which the first conversion has to be.
+@pytest.mark.parametrize("m,b,tA,packed", [(8, 32, 1, None), (8, 24, 0, None), (12, 64, 0, None), (8, 128, 1, None), (8, 32, 0, "B"), (12, 32, 0, "B"), (12, 64, 0, "AB")])
+def test_second_conversion_comes_after_a_whole_kernel_boundary(hb, m, b, tA, packed):
+    import torch
+    M, N, K = 2048, 2304, 2048
+    fa, fb = hb.Format(mant_bits=m, block=b), hb.Format(mant_bits=m, block=b, stream_id=1)
+    fw = hb.Format(mant_bits=m, block=b, tile=b, stream_id=1)
+    A, W = torch.randn(K if tA else M, M if tA else K, device="cuda"), torch.randn(K, N, device="cuda") * 0.05
+    wide, views = hb.wide_quantize(W, fw)
+    delta = W * 0.01
+    a = hb.quantize(A, 1, fa) if packed == "AB" else A
+    C, ws = torch.empty(M, N, device="cuda"), torch.empty(1 << 27, dtype=torch.int8, device="cuda")
+
+    def step():
+        if packed:
+            hb.wide_update(wide, delta, fw, views=views)
+            hb.gemm_q(M, N, K, a, views[0], fmtA=fa, out=C, workspace=ws)
+        else:
+            hb.wide_dequantize(wide, W)
+            hb.gemm(tA, 0, A, W, fa, fb, C, ws)
+
+    step()                                                # sets the kernels' attributes once
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        step()
+    kinds = edges_in_order(graph)
+    # the kernel that writes the second operand, the first conversion, the second one, the product
+    assert len(kinds) == 3 and kinds[:2] == [0, 1]
+
+
+# Routes in which the second operand is converted beside the first, on an operand that the kernel before has just written: packed
+# weights of an update in place, the FP32 value of wide weights.
+@pytest.mark.parametrize("m,b", [(8, 32), (8, 64), (12, 64), (12, 32)])
+@pytest.mark.parametrize("kind", ["packed weights", "both packed", "fp32"])
+def test_products_of_operands_that_the_kernel_before_has_written(hb, m, b, kind):
+    import torch
+    M, N, K = 2048, 2304, 2048
+    fa, fb = hb.Format(mant_bits=m, block=b), hb.Format(mant_bits=m, block=b, stream_id=1)
+    fw = hb.Format(mant_bits=m, block=b, tile=b, stream_id=1)
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    A = torch.randn(M, K, device="cuda", generator=gen)
+    w0 = torch.randn(K, N, device="cuda", generator=gen) * 0.05
+    deltas = [torch.randn(K, N, device="cuda", generator=gen) * 0.05 for _ in range(3)]
+    pa = hb.quantize(A, 1, fa) if kind == "both packed" else A
+
+    def run(pause):
+        wide, views = hb.wide_quantize(w0, fw)
+        W = torch.empty(K, N, device="cuda")
+        out = []
+        for i in range(12):
+            if kind == "fp32":
+                hb.wide_update(wide, deltas[i % 3], fw, want_views=False)
+                hb.wide_dequantize(wide, W)
+            else:
+                hb.wide_update(wide, deltas[i % 3], fw, views=views)
+            if pause: torch.cuda.synchronize()
+            out.append(hb.gemm(0, 0, A, W, fa, fb) if kind == "fp32" else hb.gemm_q(M, N, K, pa, views[0], fmtA=fa))
+            if pause: torch.cuda.synchronize()
+        return out
+
+    want = run(True)
+    assert hb.last_gemm_launch().startswith("gemm_fp_kernel")
+    for _ in range(4):
+        assert all(torch.equal(x, y) for x, y in zip(run(False), want))
+    assert hb.device_status() == 0
