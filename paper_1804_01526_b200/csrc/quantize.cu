@@ -14,7 +14,7 @@
 //                    transposed tile with a swizzled TMA store (full lines in both directions).
 //   quant_col_block  blocks down the columns, any b <= 128 and any pitch: one K-block of 32 columns per CTA.
 //   quant_row_ragged blocks along rows, any b <= 128, row length, pitch and alignment, in one pass.
-//   tile_strip_kernel, tile_kernel_full   t x t weight tiles (t <= 128): one pass writes both packed views and
+//   tile_strip_kernel, tile_kernel, tile_kernel_full   t x t weight tiles (t <= 128): one pass writes both packed views and
 //                    the tile exponent grid.
 //   exps_* / mant_generic   two-pass path for every other geometry (any b, any alignment).
 #include "quant_math.cuh"
@@ -293,8 +293,222 @@ __device__ __forceinline__ int floor_wide(float y, uint32_t r) {
 }
 __device__ __forceinline__ int round_sr_wide(float x, int s, uint32_t r) { return floor_wide(__fmul_rn(x, pow2f(16 - s)), r); }
 
+// qt rows have a pitch of tp + 2 halfwords, so that the column reads of view c0 spread over the banks.
+// sh: the views take the top bits of the words in qt (an arithmetic shift by sh bits); for wide storage qt
+// holds the stored words, i.e. the mantissas plus half a narrow unit (see tile_kernel); sh = 0 copies.
+template <int PLANES>
+__device__ __forceinline__ void write_tile_views(const int16_t* qt, int tp, int hi, int wj, int64_t i0, int64_t j0,
+                                                 int64_t u, int64_t v, int s, int sh, const TileViews& tv, int tid) {
+    const int qp = tp + 2;
+    const int lg = 31 - __clz(tp >> 2), gmask = (tp >> 2) - 1;       // tp is 32, 64 or 128
+    int8_t* const mant_c0 = tv.mant_c0; int8_t* const mant_c1 = tv.mant_c1;
+    int8_t* const exps_c0 = tv.exps_c0; int8_t* const exps_c1 = tv.exps_c1;
+    const int64_t kst0 = tv.kst0, ps0 = tv.ps0, rs0 = tv.rs0, nkb0 = tv.nkb0;
+    const int64_t kst1 = tv.kst1, ps1 = tv.ps1, rs1 = tv.rs1, nkb1 = tv.nkb1;
+    // view c1: row i0+ii gets bytes [v*tp, v*tp+tp) = qt[ii][0..tp)
+    if (mant_c1) for (int e = tid; e < hi * (tp / 4); e += 256) {
+        const int ii = e >> lg, g = (e & gmask) * 4;
+        uint32_t h = 0, l = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = qt[ii * qp + g + j] >> sh;
+            if (PLANES == 1) h |= (uint32_t)(q & 0xff) << (8 * j);
+            else { h |= (uint32_t)((q >> 4) & 0xff) << (8 * j); l |= (uint32_t)(q & 15) << (8 * j); }
+        }
+        int8_t* dst = mant_c1 + (i0 + ii) * kst1 + v * tp + g;
+        *reinterpret_cast<uint32_t*>(dst) = h;
+        if (PLANES == 2) *reinterpret_cast<uint32_t*>(dst + ps1) = l;
+    }
+    // view c0: row j0+jj gets bytes [u*tp, u*tp+tp) = qt[0..tp)[jj]
+    // (neighbouring threads write neighbouring words of one output row)
+    if (mant_c0) for (int e = tid; e < wj * (tp / 4); e += 256) {
+        const int jj = e >> lg, g = (e & gmask) * 4;
+        uint32_t h = 0, l = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int q = qt[(g + j) * qp + jj] >> sh;
+            if (PLANES == 1) h |= (uint32_t)(q & 0xff) << (8 * j);
+            else { h |= (uint32_t)((q >> 4) & 0xff) << (8 * j); l |= (uint32_t)(q & 15) << (8 * j); }
+        }
+        int8_t* dst = mant_c0 + (j0 + jj) * kst0 + u * tp + g;
+        *reinterpret_cast<uint32_t*>(dst) = h;
+        if (PLANES == 2) *reinterpret_cast<uint32_t*>(dst + ps0) = l;
+    }
+    // replicated exponents: exps_c1[v][i0+ii], exps_c0[u][j0+jj]
+    // (lines beyond the matrix, at most 15 after the last tile, are documented as zero)
+    const int pad1 = u == nkb0 - 1 ? (int)(rs1 - i0) : hi, pad0 = v == nkb1 - 1 ? (int)(rs0 - j0) : wj;
+    if (exps_c1) for (int e = tid; e < pad1; e += 256) exps_c1[v * rs1 + i0 + e] = e < hi ? (int8_t)s : (int8_t)0;
+    if (exps_c0) for (int e = tid; e < pad0; e += 256) exps_c0[u * rs0 + j0 + e] = e < wj ? (int8_t)s : (int8_t)0;
+    // row tails beyond the last tile: zero them (last tile column / last tile row only)
+    if (mant_c1 && v == nkb1 - 1)
+        for (int64_t e = tid; e < (int64_t)hi * ((kst1 - nkb1 * tp) / 4); e += 256) {
+            const int64_t per = (kst1 - nkb1 * tp) / 4, ii = e / per, o = nkb1 * tp + (e % per) * 4;
+            *reinterpret_cast<uint32_t*>(mant_c1 + (i0 + ii) * kst1 + o) = 0;
+            if (PLANES == 2) *reinterpret_cast<uint32_t*>(mant_c1 + ps1 + (i0 + ii) * kst1 + o) = 0;
+        }
+    if (mant_c0 && u == nkb0 - 1)
+        for (int64_t e = tid; e < (int64_t)wj * ((kst0 - nkb0 * tp) / 4); e += 256) {
+            const int64_t per = (kst0 - nkb0 * tp) / 4, jj = e / per, o = nkb0 * tp + (e % per) * 4;
+            *reinterpret_cast<uint32_t*>(mant_c0 + (j0 + jj) * kst0 + o) = 0;
+            if (PLANES == 2) *reinterpret_cast<uint32_t*>(mant_c0 + ps0 + (j0 + jj) * kst0 + o) = 0;
+        }
+}
+
+// The same (modes below) with one CTA of 256 threads per tile, the FP32 tile and the words in shared memory: the tile_strip_kernel's strips
+// leave most of the chip idle where the tiles are few, and its 32-bit accesses cost more than this kernel's sixteen bytes on tiles of
+// whole eights that its strips are wide for one of (rule and both sides measured in launch_tiles).
+// FAST: t, d1 multiples of 8, pitches and bases 16-byte aligned: a thread handles eight consecutive
+// weights of a row at a time (two 128-bit loads, one Philox call, 128-bit store of the int16 mantissas).
+template <int MODE, int PLANES, bool FAST>
+__global__ void __launch_bounds__(256)
+tile_kernel(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t d1, int t, int tp, QParams p,
+            int16_t* __restrict__ wide, int8_t* __restrict__ grid, int64_t grid_ld, TileViews tv) {
+    chain_start();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int fp = FAST ? t + 4 : t + 1;                                   // pitch of the FP32 tile
+    float* tile = reinterpret_cast<float*>(smem_raw);                      // [t][fp]
+    const int qp = tp + 2;
+    int16_t* qt = reinterpret_cast<int16_t*>(tile + (size_t)t * fp);       // [tp][tp + 2], zero padded
+    __shared__ uint32_t s_am[8];
+    __shared__ int s_exp;
+
+    const int tid = threadIdx.x, lane = tid & 31, wrow = tid >> 5;
+    const int64_t u = blockIdx.y, v = blockIdx.x;       // tile row (along d0), tile column (along d1)
+    const int64_t i0 = u * t, j0 = v * t;
+    const int hi = (int)min((int64_t)t, d0 - i0), wj = (int)min((int64_t)t, d1 - j0);
+    const int G = wj >> 3;                              // FAST: groups of eight per tile row
+    constexpr bool UPDATE = MODE == 1 || MODE == 4;
+    const int wbits = MODE == 3 ? p.m : 16, wqmax = MODE == 3 ? p.qmax : 32767;
+    // Wide modes: qt holds the stored word the views are cut from: the mantissa plus half a narrow unit,
+    // held inside the range whose top bits stay within +-qmax (so the shift alone rounds to nearest and
+    // saturates symmetrically). MODE 3 copies (sh = 0).
+    const int sh = MODE == 3 ? 0 : 16 - p.m;
+    const int half = sh > 0 ? 1 << (sh - 1) : 0;
+    const int w_hi = ((p.qmax + 1) << sh) - half - 1, w_lo = -(p.qmax << sh) - half;
+    const uint32_t w_hi2 = ((uint32_t)w_hi & 0xFFFFu) * 0x10001u, w_lo2 = ((uint32_t)w_lo & 0xFFFFu) * 0x10001u;
+    const uint32_t half2 = (uint32_t)half * 0x10001u;
+    auto stored_pair = [&](uint32_t h) { return MODE == 3 ? h : __vadd2(__vmaxs2(__vmins2(h, w_hi2), w_lo2), half2); };
+    auto stored_one = [&](int q) { return MODE == 3 ? q : max(w_lo, min(w_hi, q)) + half; };
+    for (int e = tid; e < tp * qp / 2; e += 256) reinterpret_cast<uint32_t*>(qt)[e] = 0;
+    int s;
+    if (MODE == 2) {
+        __syncthreads();
+        s = grid[u * grid_ld + v];
+        if (FAST) {
+            for (int item = tid; item < hi * G; item += 256) {
+                const int ii = item / G, gj = item - ii * G;
+                const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
+                uint32_t* dst = reinterpret_cast<uint32_t*>(qt + ii * qp + 8 * gj);
+                dst[0] = stored_pair(q8.x); dst[1] = stored_pair(q8.y); dst[2] = stored_pair(q8.z); dst[3] = stored_pair(q8.w);
+            }
+        } else {
+            for (int ii = wrow; ii < hi; ii += 8)
+                for (int jj = lane; jj < wj; jj += 32) qt[ii * qp + jj] = (int16_t)stored_one(wide[(i0 + ii) * d1 + j0 + jj]);
+        }
+    } else {
+        const float old_scale = UPDATE ? pow2f(grid[u * grid_ld + v]) : 0.f;
+        uint32_t am = 0;
+        if (FAST) {
+            for (int item = tid; item < hi * G; item += 256) {
+                const int ii = item / G, gj = item - ii * G;
+                const float4* sp = reinterpret_cast<const float4*>(src + (i0 + ii) * ld + j0 + 8 * gj);
+                float4 a = __ldcs(sp), b = __ldcs(sp + 1);
+                if (UPDATE) {
+                    const uint4 q8 = *reinterpret_cast<const uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj);
+                    a.x = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x & 0xFFFFu), old_scale), a.x);
+                    a.y = __fadd_rn(__fmul_rn((float)(int16_t)(q8.x >> 16), old_scale), a.y);
+                    a.z = __fadd_rn(__fmul_rn((float)(int16_t)(q8.y & 0xFFFFu), old_scale), a.z);
+                    a.w = __fadd_rn(__fmul_rn((float)(int16_t)(q8.y >> 16), old_scale), a.w);
+                    b.x = __fadd_rn(__fmul_rn((float)(int16_t)(q8.z & 0xFFFFu), old_scale), b.x);
+                    b.y = __fadd_rn(__fmul_rn((float)(int16_t)(q8.z >> 16), old_scale), b.y);
+                    b.z = __fadd_rn(__fmul_rn((float)(int16_t)(q8.w & 0xFFFFu), old_scale), b.z);
+                    b.w = __fadd_rn(__fmul_rn((float)(int16_t)(q8.w >> 16), old_scale), b.w);
+                }
+                float4* tp4 = reinterpret_cast<float4*>(tile + ii * fp + 8 * gj);
+                tp4[0] = a; tp4[1] = b;
+                const float e8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                am = max(am, amax8_bits(e8));
+            }
+        } else {
+            for (int ii = wrow; ii < hi; ii += 8)
+                for (int jj = lane; jj < wj; jj += 32) {
+                    float val = src[(i0 + ii) * ld + j0 + jj];
+                    if (UPDATE) val = __fadd_rn(__fmul_rn((float)wide[(i0 + ii) * d1 + j0 + jj], old_scale), val);
+                    tile[ii * fp + jj] = val;
+                    am = max(am, abs_bits(val));
+                }
+        }
+        for (int off = 16; off > 0; off >>= 1) am = max(am, __shfl_xor_sync(0xffffffffu, am, off));
+        if (lane == 0) s_am[wrow] = am;
+        __syncthreads();
+        if (tid == 0) {
+            uint32_t a = 0;
+            for (int i = 0; i < 8; ++i) a = max(a, s_am[i]);
+            s_exp = block_exponent(a, wbits, p.exp_mode);
+            if (grid) grid[u * grid_ld + v] = (int8_t)s_exp;
+        }
+        __syncthreads();
+        s = s_exp;
+        if (FAST) {
+            const uint32_t qm = qmax_pair(wqmax), nqm = neg_qmax_pair(wqmax);
+            for (int item = tid; item < hi * G; item += 256) {
+                const int ii = item / G, gj = item - ii * G;
+                const float4* tp4 = reinterpret_cast<const float4*>(tile + ii * fp + 8 * gj);
+                const float4 a = tp4[0], b = tp4[1];
+                const float e8[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+                uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                if (p.rounding == 1) w = draws_of_group(p, (uint64_t)((i0 + ii) * d1 + j0 + 8 * gj) >> 3);
+                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+                uint32_t h[4];
+                if (MODE == 3) {
+                    // at most 12 bits: the packed halfword forms
+                    const float sc = pow2f(p.rounding == 1 ? 16 - s : -s);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        h[j] = p.rounding == 1 ? round_sr_pair(e8[2 * j], e8[2 * j + 1], sc, ww[j], qm, nqm)
+                                               : round_rne_pair(e8[2 * j], e8[2 * j + 1], sc, qm, nqm);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        int q0, q1;
+                        if (p.rounding == 0) {
+                            q0 = round_rne(e8[2 * j], s, 32767);
+                            q1 = round_rne(e8[2 * j + 1], s, 32767);
+                        } else {
+                            q0 = round_sr_wide(e8[2 * j], s, ww[j] & 0xFFFFu);
+                            q1 = round_sr_wide(e8[2 * j + 1], s, ww[j] >> 16);
+                        }
+                        h[j] = ((uint32_t)q0 & 0xFFFFu) | ((uint32_t)q1 << 16);
+                    }
+                }
+                uint32_t* dst = reinterpret_cast<uint32_t*>(qt + ii * qp + 8 * gj);
+                dst[0] = stored_pair(h[0]); dst[1] = stored_pair(h[1]); dst[2] = stored_pair(h[2]); dst[3] = stored_pair(h[3]);
+                if (MODE != 3) *reinterpret_cast<uint4*>(wide + (i0 + ii) * d1 + j0 + 8 * gj) = make_uint4(h[0], h[1], h[2], h[3]);
+                if (MODE == 4) store_wide_values(tv.value + (i0 + ii) * tv.ldv + j0 + 8 * gj, h, pow2f_stored(s));
+            }
+        } else {
+            for (int ii = wrow; ii < hi; ii += 8)
+                for (int jj = lane; jj < wj; jj += 32) {
+                    const float val = tile[ii * fp + jj];
+                    const uint64_t L = (uint64_t)((i0 + ii) * d1 + j0 + jj);
+                    int q;
+                    if (MODE == 3) q = quantize_one(val, s, p, L);
+                    else if (p.rounding == 0) q = round_rne(val, s, 32767);
+                    else q = round_sr_wide(val, s, draw_of_element(p, L));
+                    qt[ii * qp + jj] = (int16_t)stored_one(q);
+                    if (MODE != 3) wide[(i0 + ii) * d1 + j0 + jj] = (int16_t)q;
+                    if (MODE == 4) tv.value[(i0 + ii) * tv.ldv + j0 + jj] = __fmul_rn((float)q, pow2f_stored(s));
+                }
+        }
+    }
+    if (tv.mant_c0 == nullptr && tv.mant_c1 == nullptr) return;
+    __syncthreads();
+    write_tile_views<PLANES>(qt, tp, hi, wj, i0, j0, u, v, s + sh, sh, tv, tid);
+}
+
 // Weight matrices with one exponent per t x t tile (Sec. 4.2 "Tiling", t <= 128) and their wide storage
-// (Sec. 4.2 "Wide weight storage"), for every tile geometry, alignment and width that tile_kernel_full does not take.
+// (Sec. 4.2 "Wide weight storage"), for every tile geometry, alignment and width
+// that neither tile_kernel_full nor tile_kernel takes.
 //   MODE 3  quantise FP32 weights src (pitch ld) straight to p.m bits (no wide copy)
 //   MODE 0  quantise FP32 weights src to wide storage: int16 mantissas `wide` (row-major, pitch d1) and
 //           one exponent per tile in grid [tiles along d0][tiles along d1]
@@ -2047,13 +2261,52 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
 #undef HBFP_TILE_FULL
         return launch_status();
     }
+    // A CTA per tile or strips of tiles (148 SMs; a wave of the one are 148 to 1184 CTAs, by the tile; us, the one / the other).
+    //   Few small tiles: strips leave SMs idle, even cut down as below (100 x 100, t = 8, update 7.4 / 8.3, cut down, and 14.4 as they were;
+    //   512 x 512, t = 24 8.7 / 9.7 and 11.5). What reads the wide words gains for longer (1000 x 1000, t = 24 12.8 / 14.5, from FP32 11.3 /
+    //   11.3), without vectors for shorter.
+    //   Aligned tiles above 32: sixteen bytes per access against four (4096 x 4096, t = 72, update 69 / 182, t = 120 58 / 100, t = 40 66 / 77).
+    //   48 is the one length whose strips have no idle lane: many of those are faster in strips where no word is read (51 / 40).
+    //   Others above 64: a strip is one tile, with 44 % of its lanes idle at t = 72 and one CTA per SM (2000 x 3001, t = 72, update 35 / 66, from
+    //   FP32 27 / 44); the draws, made per element there and from a table here, take most of that back (86 / 100, t = 84 even; from FP32 even at 72).
+    constexpr bool FROM_WORDS = MODE != 0 && MODE != 3, UPDATE = MODE == 1 || MODE == 4;
+    const int64_t tiles = nu * nv;
+    const bool draws = p.rounding && MODE != 2;
+    bool per_tile;
+    if (fast && t <= 32) per_tile = tiles <= (t == tp ? 592 : FROM_WORDS && t >= 16 ? 1776 : 1184);
+    else if (fast && t == tp) per_tile = t == 64 && tiles <= 592;
+    else if (fast) per_tile = FROM_WORDS || t != 48 || tiles <= 1184;
+    else if (t <= 64) per_tile = t <= (FROM_WORDS ? 32 : 24) && tiles <= 592;
+    else per_tile = draws ? UPDATE && t <= 76 && tiles > 592 : t <= (FROM_WORDS ? 96 : 88) && tiles > 148;
+    if (per_tile) {
+        const size_t smem = (size_t)t * (t + 4) * sizeof(float) + (size_t)tp * (tp + 2) * sizeof(int16_t);
+#define HBFP_TILE(PLANES, FAST)                                                                                               \
+    do {                                                                                                                      \
+        rc = allow_shared<tile_kernel<MODE, PLANES, FAST>>(128 * 132 * sizeof(float) + 128 * 130 * sizeof(int16_t));          \
+        if (rc) return rc;                                                                                                    \
+        launch_chained(tile_kernel<MODE, PLANES, FAST>, grid_dim, 256, smem, st, src, ld, d0, d1, t, tp, p, wide, grid, nv, tv); \
+    } while (0)
+        if (L0.planes == 1) { if (fast) HBFP_TILE(1, true); else HBFP_TILE(1, false); }
+        else { if (fast) HBFP_TILE(2, true); else HBFP_TILE(2, false); }
+#undef HBFP_TILE
+        return launch_status();
+    }
     // Strips of 64 or 96 columns (whichever the tiles fill better) and up to 64 rows, 128 x 128 for tiles above 64.
     StripShape sh{t, tp, tp == 32 ? 5 : tp == 64 ? 6 : 7, 1, t <= 8 ? 3 : t <= 16 ? 2 : t <= 32 ? 1 : 0, 0, (65536 + t - 1) / t, 0, (int)nu, (int)nv};
     const int warps = t > 64 ? 16 : 8;
-    sh.rpw = (t + (warps >> sh.lg_rv) - 1) / (warps >> sh.lg_rv);
-    const int cv2 = std::min(64 / t, 160 / tp), cv3 = std::min(96 / t, 160 / tp);
-    const int kc = t > 64 ? 4 : sh.rpw <= 6 && 2 * cv3 > 3 * cv2 ? 3 : 2;
-    if (kc < 4) sh.cv = kc == 3 ? cv3 : cv2;
+    auto warp_rows = [&]() { return (t + (warps >> sh.lg_rv) - 1) / (warps >> sh.lg_rv); };
+    if (t <= 64) {
+        const int cv2 = std::min(64 / t, 160 / tp), cv3 = std::min(96 / t, 160 / tp);
+        sh.cv = warp_rows() <= 6 && 2 * cv3 > 3 * cv2 ? cv3 : cv2;
+        // smaller ones where these leave SMs idle
+        auto strips = [&]() { return ((nu + (1 << sh.lg_rv) - 1) >> sh.lg_rv) * ((nv + sh.cv - 1) / sh.cv); };
+        while (strips() < 148 && (sh.lg_rv > 0 || sh.cv > 1)) {
+            if (sh.lg_rv > 0 && ((1 << sh.lg_rv) >= sh.cv || sh.cv == 1)) --sh.lg_rv;
+            else sh.cv = (sh.cv + 1) / 2;
+        }
+    }
+    sh.rpw = warp_rows();
+    const int kc = t > 64 ? 4 : sh.cv * t > 64 ? 3 : 2;
     const int rv = 1 << sh.lg_rv, rows = kc == 3 ? 6 : 8, per = sh.cv * tp / 8;
     sh.recip_per = ((1 << 20) + per - 1) / per;
     if (nv >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;

@@ -3,6 +3,8 @@
 // matrix descriptors, tensor-map creation.
 #pragma once
 
+#include <atomic>
+
 #include <cuda.h>
 #include <stdint.h>
 
@@ -287,6 +289,19 @@ int current_device() {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return -1;
     return dev;
+}
+// Allows a kernel up to `bytes` of dynamic shared memory, once per device. The limit belongs to the kernel, not to a call: always the
+// most that any call needs, or one thread would lower it between another's attribute and its launch.
+template <auto KERNEL>
+int allow_shared(int bytes) {
+    static std::atomic<bool> done[MAX_DEVICES];
+    const int dev = current_device();
+    if (dev < 0) return HBFP_ERR_CUDA;
+    if (!done[dev].load(std::memory_order_acquire)) {
+        HBFP_CUDA_OK(cudaFuncSetAttribute(KERNEL, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        done[dev].store(true, std::memory_order_release);
+    }
+    return HBFP_OK;
 }
 
 int sm_count() {

@@ -195,3 +195,51 @@ def test_weight_tiles_of_any_geometry(hb, d0, d1, t, m, rounding):
     check_views(hb, (c0, c1), qn, sn, t)
     assert np.array_equal(grid.cpu().numpy(), sn[::t, :])
     assert hb.device_status() == 0
+
+
+# The same on both sides of every line between a CTA per tile and strips, with strips cut down and whole, and a view by itself: small and
+# middling tiles, aligned and not, with and without draws.
+@pytest.mark.parametrize("d0,d1,t,m,rounding", [
+    (58, 111, 2, 8, 1), (101, 101, 4, 12, 0), (130, 262, 5, 8, 1), (192, 400, 8, 8, 1), (201, 411, 8, 4, 0), (300, 290, 12, 12, 1), (272, 1120, 16, 8, 0),
+    (480, 928, 16, 8, 1), (500, 501, 20, 8, 1), (601, 597, 24, 8, 0), (600, 1160, 24, 12, 1), (864, 1224, 24, 8, 1), (1008, 1032, 24, 4, 0), (420, 1100, 28, 8, 0),
+    (780, 797, 32, 8, 1), (400, 520, 40, 8, 1), (1648, 1728, 48, 8, 0), (1632, 1736, 48, 8, 1), (800, 993, 65, 8, 0), (1600, 1699, 65, 8, 1), (216, 360, 72, 12, 1),
+    (1000, 1003, 88, 8, 0), (1250, 1251, 96, 8, 0), (224, 560, 112, 8, 1), (1344, 1512, 112, 8, 0)])
+def test_weight_tiles_on_both_sides_of_the_kernels_rule(hb, d0, d1, t, m, rounding):
+    test_weight_tiles_of_any_geometry(hb, d0, d1, t, m, rounding)
+    # a view by itself
+    fd = F(m, t, rounding, seed=11, stream_id=2)
+    w = wl.draw("lognormal", (d0, d1), seed=78)
+    for axis in (0, 1):
+        p = hb.quantize(to_dev(w), axis, gfmt(fd))
+        q, s = decode_packed(p, hb.packed_layout(p.rows, p.k, p.fmt))
+        q_ref, s_ref = oracle.quantize(w, axis, ofmt(fd))
+        assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
+
+
+@pytest.mark.parametrize("d0,d1,t,rounding,per_tile", [
+    (64, 64, 8, 0, True), (100, 100, 5, 1, True), (256, 300, 24, 0, True), (1000, 1000, 24, 1, True), (2048, 2048, 40, 0, True), (1000, 1000, 72, 1, True),
+    (4096, 4096, 80, 0, True), (2048, 2048, 120, 1, True), (1001, 1003, 72, 0, True), (2000, 3001, 72, 1, True), (256, 300, 8, 0, False), (784, 1024, 8, 1, False),
+    (1111, 5001, 24, 0, False), (1000, 1500, 32, 1, False), (2000, 3001, 100, 1, False)])
+def test_launches_of_weight_updates(hb, d0, d1, t, rounding, per_tile):
+    """A CTA per tile, or strips of which there are enough for every SM where the tiles are."""
+    import ctypes
+    import torch
+
+    class Params(ctypes.Structure):                       # CUDA_KERNEL_NODE_PARAMS_v2
+        _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint), ("rest", ctypes.c_void_p * 4)]
+
+    f = hb.Format(mant_bits=8, block=t, tile=t, rounding=rounding)
+    wide, views = hb.wide_quantize(torch.randn(d0, d1, device="cuda"), f)
+    delta = torch.zeros(d0, d1, device="cuda")
+    hb.wide_update(wide, delta, f, views=views)           # sets the kernels' attributes
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        hb.wide_update(wide, delta, f, views=views)
+    driver, node, n, p = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_size_t(1), Params()
+    assert driver.cuGraphGetNodes(ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.byref(node), ctypes.byref(n)) == 0 and n.value == 1
+    assert driver.cuGraphKernelNodeGetParams_v2(node, ctypes.byref(p)) == 0
+    nu, nv = -(-d0 // t), -(-d1 // t)
+    ctas = p.grid[0] * p.grid[1]
+    assert (tuple(p.grid) == (nv, nu, 1) and p.block[0] == 256) == per_tile
+    assert min(148, nu * nv) <= ctas <= nu * nv
