@@ -894,29 +894,31 @@ tile_kernel_full(const float* __restrict__ src, int64_t ld, int64_t d0, int64_t 
             const int item = tid + 256 * k;
             if (NITEMS % 256 == 0 || item < NITEMS) {
                 const int ii = item / G, gj = item - ii * G;
-                const float e8[8] = {a[k].x, a[k].y, a[k].z, a[k].w, b[k].x, b[k].y, b[k].z, b[k].w};
-                uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                if (p.rounding == 1) w = draws_of_group(p, (uint64_t)((i0 + ii) * d1 + j0 + 8 * gj) >> 3);
-                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-                uint32_t h[4];
-                if (MODE == 3) {
-                    const float sc = pow2f(p.rounding == 1 ? 16 - s : -s);
+                uint32_t h[4] = {0u, 0u, 0u, 0u};
+                if (there(ii, gj)) {                                   // (a missing group of eight is zero whatever its draws)
+                    const float e8[8] = {a[k].x, a[k].y, a[k].z, a[k].w, b[k].x, b[k].y, b[k].z, b[k].w};
+                    uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                    if (p.rounding == 1) w = draws_of_group(p, (uint64_t)((i0 + ii) * d1 + j0 + 8 * gj) >> 3);
+                    const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
+                    if (MODE == 3) {
+                        const float sc = pow2f(p.rounding == 1 ? 16 - s : -s);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        h[j] = p.rounding == 1 ? round_sr_pair(e8[2 * j], e8[2 * j + 1], sc, ww[j], qm, nqm)
-                                               : round_rne_pair(e8[2 * j], e8[2 * j + 1], sc, qm, nqm);
-                } else {
+                        for (int j = 0; j < 4; ++j)
+                            h[j] = p.rounding == 1 ? round_sr_pair(e8[2 * j], e8[2 * j + 1], sc, ww[j], qm, nqm)
+                                                   : round_rne_pair(e8[2 * j], e8[2 * j + 1], sc, qm, nqm);
+                    } else {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        int q0, q1;
-                        if (p.rounding == 0) {
-                            q0 = round_rne(e8[2 * j], s, 32767);
-                            q1 = round_rne(e8[2 * j + 1], s, 32767);
-                        } else {
-                            q0 = round_sr_wide(e8[2 * j], s, ww[j] & 0xFFFFu);
-                            q1 = round_sr_wide(e8[2 * j + 1], s, ww[j] >> 16);
+                        for (int j = 0; j < 4; ++j) {
+                            int q0, q1;
+                            if (p.rounding == 0) {
+                                q0 = round_rne(e8[2 * j], s, 32767);
+                                q1 = round_rne(e8[2 * j + 1], s, 32767);
+                            } else {
+                                q0 = round_sr_wide(e8[2 * j], s, ww[j] & 0xFFFFu);
+                                q1 = round_sr_wide(e8[2 * j + 1], s, ww[j] >> 16);
+                            }
+                            h[j] = ((uint32_t)q0 & 0xFFFFu) | ((uint32_t)q1 << 16);
                         }
-                        h[j] = ((uint32_t)q0 & 0xFFFFu) | ((uint32_t)q1 << 16);
                     }
                 }
                 *reinterpret_cast<uint4*>(qt + ii * QP + 8 * gj) = make_uint4(stored_pair(h[0]), stored_pair(h[1]), stored_pair(h[2]), stored_pair(h[3]));
