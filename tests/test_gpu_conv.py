@@ -344,7 +344,7 @@ def test_backward_weight_operand_for_three_wide_filters(hb, n, h, w, c, kh, m, r
     assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
 
 
-@pytest.mark.parametrize("n,h,w,c,k", [(1, 1, 1, 1, 3), (2, 3, 5, 7, 3), (3, 8, 8, 32, 3), (1, 17, 33, 12, 5), (2, 4, 300, 96, 3), (0, 4, 4, 4, 3)])
+@pytest.mark.parametrize("n,h,w,c,k", [(1, 1, 1, 1, 3), (2, 3, 5, 7, 3), (3, 8, 8, 32, 3), (1, 17, 33, 12, 5), (2, 4, 300, 96, 3), (0, 4, 4, 4, 3), (1, 1, 5600001, 3, 3)])
 def test_fold_of_the_im2col_gradient(hb, n, h, w, c, k):
     """Shifted additions in the order of the taps, bit for bit."""
     import ctypes
