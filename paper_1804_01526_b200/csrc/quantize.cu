@@ -2316,7 +2316,8 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     const size_t smem = (size_t)rv * tp * (sh.cv * tp + 8) * 2 + (p.rounding && MODE != 2 ? (size_t)warps * rows * (4 * kc + 1) * 16 : 0);
 #define HBFP_STRIP(PLANES, NW, RPW, KC, SRV)                                                                                                      \
     do {                                                                                                                                          \
-        if (smem > 36 * 1024) HBFP_CUDA_OK(cudaFuncSetAttribute(tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        rc = allow_shared<tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>>(96 * 1024);       /* eight tile rows of five tiles of 8 with draws: 93 KB */     \
+        if (rc) return rc;                                                                                                                        \
         launch_chained(tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>, strips, 32 * NW, smem, st, src, ld, d0, d1, sh, p, wide, grid, nv, tv);  \
     } while (0)
 #define HBFP_STRIP_SR(PLANES, NW, RPW, KC) do { if (p.rounding && MODE != 2) HBFP_STRIP(PLANES, NW, RPW, KC, MODE != 2); else HBFP_STRIP(PLANES, NW, RPW, KC, false); } while (0)
@@ -2436,7 +2437,8 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
     if (n == 0) return HBFP_OK;
     if (h > 32768 || c > 4096 || L.nkb >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
     const size_t smem = (size_t)(b / w + kh - 1) * w * c * sizeof(float);
-    if (smem > 200 * 1024) return HBFP_ERR_UNSUPPORTED;
+    constexpr int IM2COL_SMEM_MAX = 200 * 1024;
+    if (smem > IM2COL_SMEM_MAX) return HBFP_ERR_UNSUPPORTED;
     const QParams p = make_params(f);
     if (L.rs != L.rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
     if (L.kst != L.nkb * L.bp) HBFP_CUDA_OK(cudaMemsetAsync(mant, 0, (size_t)L.mant_bytes, st));     // row tails
@@ -2445,7 +2447,8 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
         const size_t table = p.rounding ? (size_t)(b / w + kh - 1) * w * c * 2 : 0;
 #define HBFP_COLS3(PL, WV, SRV)                                                                                                      \
     do {                                                                                                                              \
-        if (table > 48 * 1024) HBFP_CUDA_OK(cudaFuncSetAttribute(im2col_cols3<PL, WV, SRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)table)); \
+        rc = allow_shared<im2col_cols3<PL, WV, SRV>>(IM2COL_SMEM_MAX / 2);          /* two bytes of draws for every four of values */    \
+        if (rc) return rc;                                                                                                            \
         launch_chained(im2col_cols3<PL, WV, SRV>, (unsigned)L.nkb, threads, table, st, x, (int)h, (int)c, kh, pad, p, L.kst, L.plane_stride, L.rs, mant, exps); \
     } while (0)
 #define HBFP_COLS3_SR(PL, WV) do { if (p.rounding) HBFP_COLS3(PL, WV, true); else HBFP_COLS3(PL, WV, false); } while (0)
@@ -2460,7 +2463,8 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
     while ((1 << lg_w) < w) ++lg_w;
 #define HBFP_COLS_LAUNCH2(PL, NPX, SRV)                                                                                       \
     do {                                                                                                                       \
-        HBFP_CUDA_OK(cudaFuncSetAttribute(im2col_cols<PL, NPX, SRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));   \
+        rc = allow_shared<im2col_cols<PL, NPX, SRV>>(IM2COL_SMEM_MAX);                                                          \
+        if (rc) return rc;                                                                                                     \
         launch_chained(im2col_cols<PL, NPX, SRV>, (unsigned)L.nkb, 256, smem, st, x, (int)h, (int)w, lg_w, (int)c, kh, kw, pad, p, L.kst,     \
                                                                      L.plane_stride, L.rs, mant, exps);                        \
     } while (0)

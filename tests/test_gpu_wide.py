@@ -243,3 +243,29 @@ def test_launches_of_weight_updates(hb, d0, d1, t, rounding, per_tile):
     ctas = p.grid[0] * p.grid[1]
     assert (tuple(p.grid) == (nv, nu, 1) and p.block[0] == 256) == per_tile
     assert min(148, nu * nv) <= ctas <= nu * nv
+
+
+def test_tiles_of_different_lengths_from_two_threads(hb):
+    """One kernel serves several tile lengths, each with its own need of shared memory: a thread that launches the one must not take
+    from another what it launches the other with."""
+    import threading
+    import torch
+    failed = []
+
+    def work(t):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            f = hb.Format(mant_bits=8, block=t, tile=t, rounding=1, seed=2)
+            w = torch.randn(1000, 1000, device="cuda")
+            wide, views = hb.wide_quantize(w, f)
+            try:
+                for _ in range(4000):
+                    hb.wide_update(wide, w, f, views=views)
+            except hb.HbfpError as e:
+                failed.append((t, str(e)))
+            stream.synchronize()
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in (8, 16)]
+    for x in threads: x.start()
+    for x in threads: x.join()
+    assert not failed and hb.device_status() == 0
