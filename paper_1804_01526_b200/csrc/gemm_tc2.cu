@@ -409,6 +409,7 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long cycles_start = clock64();
     const uint32_t rank = cluster_ctarank();                 // 0 = leader
     const int cluster = (int)cluster_id_x(), nclusters = (int)cluster_count_x();
     const int total_work = p.tiles_m * p.tiles_n * p.splits;
@@ -440,7 +441,6 @@ gemm_tc2_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     chain_next();
-    const long long cycles_start = clock64();
 
     if (warp < CONTROL_WARPS) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_CONTROL));

@@ -408,6 +408,19 @@ def test_last_gemm_cycles_reports_the_paired_kernel_length(hb):
     assert hb.device_status() == 0
 
 
+def test_last_gemm_cycles_counts_from_the_kernels_start(hb):
+    """A launch of one K-block and one tile per cluster: 5900 cycles, 2600 of them before the work begins (barriers, tensor memory, both
+    SMs of each pair ready); without those it would be 3300."""
+    import torch
+    f = hb.Format(8, 128)
+    a, b = hb.quantize(torch.randn(9472, 128, device="cuda"), 1, f), hb.quantize(torch.randn(512, 128, device="cuda"), 1, f)
+    cycles = []
+    for _ in range(9):
+        hb.gemm_q(9472, 512, 128, a, b, flags=hb.GEMM_FORCE_TENSOR_2SM)
+        cycles.append(hb.last_gemm_cycles())
+    assert 4600 < sorted(cycles)[4] < 12000
+
+
 # The floating-point operand forms (gemm_fp.cu): short blocks of 8-bit mantissas, 9 to 12 bits; one SM or a pair per tile.
 # Edges of tiles in M and N, a last K stage with a single block, padded blocks, an output pitch that TMA cannot store.
 FP_FORM_CASES = [
