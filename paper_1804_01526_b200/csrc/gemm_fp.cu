@@ -711,10 +711,16 @@ int fp_launch(FpProblem p, const FpOperand& a, const FpOperand& b, cudaStream_t 
     }
     const int tiles = p.tiles_m * p.tiles_n;
     const int grid = PAIR ? 2 * (tiles < clusters ? tiles : clusters) : p.splits > 1 ? tiles * p.splits : (tiles < sm_count() ? tiles : sm_count());
-    // A long persistent launch is not chained: placed on SMs as they fall free its CTAs share panels in L2 less well, which costs more
-    // than the launch's start (4096 cube, 12 bits, with conversions: 332 us before any chaining, 334 chained, 325 against 328 not).
+    // A long launch of the 12-bit form is not chained: its three operand planes are the heaviest traffic there is, and CTAs placed as SMs
+    // fall free share panels in L2 less well than CTAs placed on an empty chip, which costs a long launch more than its start. Chained /
+    // not, with conversions, in order of K-blocks x tiles of a CTA: 2048 cube, b = 64 (128) 59.3 / 61.5 us; 4096 x 4096 x 1024, b = 32 (224)
+    // 144.3 / 144.6; 1024 x 4096 x 4096, b = 24 (342) 208.6 / 209.6; 3072 cube, b = 32 (384) 220.5 / 221.1; from there on 4096 cube, b = 64
+    // (448) 301.9 / 301.7; 8192 x 8192 x 512, b = 32 (448) 295.0 / 289.0; 3072 cube, b = 24 (512) 285.0 / 284.5; 4096 cube, b = 32 (896)
+    // 486.5 / 484.0; 4096 cube, b = 24 (1197) 640.2 / 633.5. The 8-bit form gains by it at every size: 2048 cube, b = 32 (128) 40.1 / 42.8,
+    // 4096 cube, b = 64 (256) 149.9 / 153.0, b = 32 (512) 205.0 / 207.5, b = 24 (684) 325.7 / 328.3, 4096 x 4096 x 8192, b = 32 (1024) 484.4 /
+    // 486.6.
     const int ctas = PAIR ? grid / 2 : grid;
-    const bool chained = p.splits > 1 || (int64_t)((tiles + ctas - 1) / ctas) * p.nkb < 400;
+    const bool chained = FORM == FORM_S || p.splits > 1 || (int64_t)((tiles + ctas - 1) / ctas) * p.nkb < 400;
     launch_chained_clusters(gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, PAIR ? 2 : p.splits, grid, FP_THREADS, C::SMEM, st, chained, mA, mB, mB1, mSA, mSB, mC, p);
     return launch_status();
 }

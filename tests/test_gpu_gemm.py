@@ -735,6 +735,21 @@ def test_second_conversion_comes_after_a_whole_kernel_boundary(hb, m, b, tA, pac
     assert len(kinds) == 3 and kinds[:2] == [0, 1]
 
 
+# The product itself is placed early too, but for long launches of the 12-bit form.
+@pytest.mark.parametrize("n,m,b,chained", [(2048, 8, 32, 1), (4096, 8, 32, 1), (4096, 8, 24, 1), (4096, 8, 64, 1), (2048, 12, 64, 1), (4096, 12, 64, 0), (4096, 12, 24, 0)])
+def test_products_of_operand_forms_are_placed_early(hb, n, m, b, chained):
+    import torch
+    f = hb.Format(mant_bits=m, block=b)
+    A, C, ws = torch.randn(n, n, device="cuda"), torch.empty(n, n, device="cuda"), torch.empty(1 << 28, dtype=torch.int8, device="cuda")
+    hb.gemm(0, 0, A, A, f, f, C, ws)
+    assert hb.last_gemm_launch().startswith("gemm_fp_kernel")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        hb.gemm(0, 0, A, A, f, f, C, ws)
+    assert edges_in_order(graph) == [1, chained]
+
+
 # Routes in which the second operand is converted beside the first, on an operand that the kernel before has just written: packed
 # weights of an update in place, the FP32 value of wide weights.
 @pytest.mark.parametrize("m,b", [(8, 32), (8, 64), (12, 64), (12, 32)])
