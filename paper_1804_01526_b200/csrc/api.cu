@@ -24,6 +24,35 @@ int32_t* device_status_word() {
     return p;
 }
 
+// Words through which one conversion passes on to the next what it has waited for (see Placing), taken in turn.
+constexpr unsigned long long TURN_WORDS = 4096;
+__device__ unsigned long long g_turn_words[TURN_WORDS];
+
+unsigned long long* turn_words() {
+    static std::atomic<unsigned long long*> known[64];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    unsigned long long* p = known[dev].load(std::memory_order_acquire);
+    if (!p) {
+        if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_turn_words) != cudaSuccess) return nullptr;
+        known[dev].store(p, std::memory_order_release);
+    }
+    return p;
+}
+
+// The places of two conversions, the second beside the first or (where it may not be) after it.
+struct PlacedPair {
+    Placing first, second;
+    explicit PlacedPair(bool beside) {
+        static std::atomic<unsigned long long> turns{0};
+        unsigned long long* const words = beside ? turn_words() : nullptr;
+        if (!words) return;
+        const unsigned long long turn = ++turns;
+        first = {LEAD, words + turn % TURN_WORDS, turn};
+        second = {BESIDE, words + turn % TURN_WORDS, turn};
+    }
+};
+
 int read_clear_device_status(cudaStream_t st, int32_t* out) {
     HBFP_CUDA_OK(cudaStreamSynchronize(st));
     int32_t v = 0, zero = 0;
@@ -139,7 +168,7 @@ int check_fp32(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K) {
 
 // Quantises an FP32 operand into the workspace (or takes a packed one as is).
 int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const Layout& L,
-                    char* ws, size_t off_m, size_t off_e, Packed* out, int place, cudaStream_t st) {
+                    char* ws, size_t off_m, size_t off_e, Packed* out, const Placing& at, cudaStream_t st) {
     out->L = L;
     out->mant_bits = o->fmt.mant_bits;
     if (o->kind == HBFP_OPERAND_PACKED) {
@@ -157,24 +186,24 @@ int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, c
     out->mant = m;
     out->exps = e;
     const float* x = static_cast<const float*>(o->data);
-    return k_contiguous(o, is_a) ? launch_quantize(x, rows, K, o->ld, 1, &o->fmt, m, e, st, place) : launch_quantize(x, K, rows, o->ld, 0, &o->fmt, m, e, st, place);
+    return k_contiguous(o, is_a) ? launch_quantize(x, rows, K, o->ld, 1, &o->fmt, m, e, st, at) : launch_quantize(x, K, rows, o->ld, 0, &o->fmt, m, e, st, at);
 }
 
 // An operand in the floating-point form at `f`: converted straight to it where it is an FP32 matrix without weight tiles,
 // otherwise packed (or taken packed) and expanded; the place is that of the last launch. The packed place is one for both operands.
-int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const GemmPlan& g, char* ws, const FpOperand& f, int place, cudaStream_t st) {
+int resolve_form(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const GemmPlan& g, char* ws, const FpOperand& f, const Placing& at, cudaStream_t st) {
     if (o->kind == HBFP_OPERAND_FP32) {
         const int rc = check_fp32(o, is_a, rows, K);
         if (rc) return rc;
         const float* x = static_cast<const float*>(o->data);
         if (o->fmt.tile == 0)          // always covered where plan_gemm_fp takes the forms; a packed place is not reserved for these
-            return k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, place, f, st)
-                                         : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, place, f, st);
+            return k_contiguous(o, is_a) ? launch_quantize_form(x, rows, K, o->ld, 1, &o->fmt, g.fp.form, !is_a, at, f, st)
+                                         : launch_quantize_form(x, K, rows, o->ld, 0, &o->fmt, g.fp.form, !is_a, at, f, st);
     }
     Packed p;
-    const int rc = resolve_operand(o, is_a, rows, K, is_a ? g.la : g.lb, ws, g.off_fm, g.off_fe, &p, CHAINED, st);
+    const int rc = resolve_operand(o, is_a, rows, K, is_a ? g.la : g.lb, ws, g.off_fm, g.off_fe, &p, Placing{}, st);
     if (rc) return rc;
-    return launch_expand(p, g.fp, !is_a, place, f, st);
+    return launch_expand(p, g.fp, !is_a, at, f, st);
 }
 
 // bias (may be null) is added in the kernel's own store where it can; *bias_done says so, otherwise the caller adds it.
@@ -216,7 +245,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
         b->kind == HBFP_OPERAND_PACKED && skinny_gemm_eligible(M, N, g.la, g.lb, a->fmt.mant_bits, b->fmt.mant_bits)) {
         rc = check_fp32(a, true, M, K);
         if (rc) return rc;
-        rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, CHAINED, st);
+        rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, Placing{}, st);
         if (rc) return rc;
         ran("gemm_skinny_kernel");
         *bias_done = true;
@@ -225,9 +254,10 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     if (use_fp && !small) {
         const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
         const bool beside = b->kind == HBFP_OPERAND_PACKED || b->fmt.tile == 0;       // B in one launch
-        rc = resolve_form(a, true, M, K, g, ws, fa, beside ? LEAD : CHAINED, st);
+        const PlacedPair at(beside);
+        rc = resolve_form(a, true, M, K, g, ws, fa, at.first, st);
         if (rc) return rc;
-        rc = resolve_form(b, false, N, K, g, ws, fb, beside ? BESIDE : CHAINED, st);
+        rc = resolve_form(b, false, N, K, g, ws, fb, at.second, st);
         if (rc) return rc;
         ran("gemm_tc_kernel", g.fp.pair ? "gemm_fp_kernel/pair" : g.fp.splits > 1 ? "gemm_fp_kernel/split" : "gemm_fp_kernel");
         *bias_done = true;
@@ -235,9 +265,10 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     }
     // two conversions of one launch each (longer blocks and weight tiles may take several, or another kernel)
     const bool beside = a->kind == HBFP_OPERAND_FP32 && b->kind == HBFP_OPERAND_FP32 && a->fmt.tile == 0 && b->fmt.tile == 0 && K > 0 && g.la.b <= 256;
-    rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, beside ? LEAD : CHAINED, st);
+    const PlacedPair at(beside);
+    rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, at.first, st);
     if (rc) return rc;
-    rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, beside ? BESIDE : CHAINED, st);
+    rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, at.second, st);
     if (rc) return rc;
     if (small) {
         ran("gemm_small_kernel");

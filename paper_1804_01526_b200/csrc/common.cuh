@@ -69,31 +69,48 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 
 __device__ __forceinline__ void chain_start() { chain_wait(); chain_next(); }
 
-// How a launch follows the one before it on its stream.
+// How a conversion follows the launch before it on its stream.
 //   CHAINED  as above
-//   LEAD     not before that kernel has ended, as any launch; the next one may run beside it
-//   BESIDE   next to the launch before it, which is a LEAD (or the last of a conversion that has one): the conversion of a product's
-//            second operand, which reads and writes nothing that the conversion of the first one writes. It waits when it is through,
-//            and what follows waits for it and with it for both.
-// What a BESIDE kernel reads without waiting has to be visible to it by other means than chain_wait, which gives the waiting grid the
-// writes of the kernel before it and no other grid anything: the weights that a chained update has just written reach a conversion
-// two launches later only because a whole kernel boundary lies between. The LEAD is that boundary: it is launched when everything
-// before it has ended and been flushed, and nothing that the BESIDE kernel reads is written from then on.
-// Back to back, all three launches chained / with LEAD and BESIDE (with a chained conversion in place of the LEAD, which has no such
-// boundary): 1111 x 777 x 3001 (b = 24, with draws) 36.3 / 34.8 us (33.7), 1024 x 4096 x 4096 (b = 32) 71.2 / 69.0 (67.9), 4096 cube,
-// 12 bits 329.7 / 328.1 (326.3).
+//   LEAD     chained, and the launch after it may be BESIDE
+//   BESIDE   next to the LEAD before it: the conversion of a product's second operand, which reads and writes nothing that the conversion
+//            of the first one writes. It waits when it is through, and what follows waits for it and with it for both.
+// What a BESIDE kernel reads, a chained kernel before the LEAD may have written (weights updated just before). The LEAD's wait gives
+// those writes to the LEAD alone, and that the LEAD's CTAs have said chain_next orders no memory. So the LEAD passes them on: past its
+// wait its first thread releases a word of memory, to a value that no other pair of launches has, and every CTA of the BESIDE kernel
+// acquires that word before it reads anything: release and acquire at the scope of the GPU are cumulative. A CTA that does not find the
+// value waits for the whole LEAD (a word taken over by a later call, a CTA that starts after the word was given back), which is slower
+// and as right. The first CTA gives the word back, so that a replayed graph starts without it. Loads of a BESIDE kernel are not .nc.
+// Back to back, all three launches chained / so / with a plain launch as the LEAD, which is a kernel boundary by itself (and before the
+// word, when nothing passed the writes on): 1111 x 777 x 3001, b = 24, draws 36.3 / 34.2 / 34.8 us (33.7); 1024 x 4096 x 4096, b = 32
+// 71.2 / 67.8 / 68.2 (67.0); 512 cube, b = 64 11.0 / 10.4 / 12.4 (9.9). A call by itself: 512 cube 13.6 / 12.5 / 12.1 (12.1).
 enum Place : int { CHAINED = 0, LEAD = 1, BESIDE = 2 };
+struct Placing {
+    int place = CHAINED;
+    unsigned long long* word = nullptr;
+    unsigned long long turn = 0;
+};
 struct Chain {
-    bool beside;
-    __device__ __forceinline__ explicit Chain(int place) : beside(place == BESIDE) {
-        if (!beside) chain_wait();
+    const Placing at;
+    __device__ __forceinline__ explicit Chain(const Placing& a) : at(a) {
+        if (at.place == BESIDE) {
+            unsigned long long seen = at.turn;
+            if (threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(at.word) : "memory");
+            if (__syncthreads_or(seen != at.turn)) chain_wait();
+        } else {
+            chain_wait();
+            if (at.place == LEAD && (blockIdx.x | blockIdx.y | threadIdx.x) == 0) asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(at.word), "l"(at.turn) : "memory");
+        }
         chain_next();
     }
-    __device__ __forceinline__ ~Chain() { if (beside) chain_wait(); }
+    __device__ __forceinline__ ~Chain() {
+        if (at.place != BESIDE) return;
+        chain_wait();
+        if ((blockIdx.x | blockIdx.y | threadIdx.x) == 0) asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at.word), "l"(0ull) : "memory");
+    }
 };
 
 template <class... Params, class... Args>
-inline void launch_placed(int place, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.gridDim = grid;
@@ -103,12 +120,8 @@ inline void launch_placed(int place, void (*kernel)(Params...), dim3 grid, dim3 
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = place == LEAD ? 0 : 1;
+    cfg.numAttrs = 1;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);      // launch_status() has the verdict
-}
-template <class... Params, class... Args>
-inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-    launch_placed(CHAINED, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 // The same with clusters of `cluster` CTAs along x; not chained where the kernel's tiles want the order of an empty chip (gemm_fp.cu).
 template <class... Params, class... Args>
@@ -145,7 +158,7 @@ struct Packed {
 // place: LEAD or BESIDE for the first and the second of two conversions that share no memory; a conversion of several launches is
 // CHAINED in place of BESIDE.
 int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int contract_axis,
-                    const hbfp_format* f, int8_t* mant, int8_t* exps, cudaStream_t st, int place = CHAINED);
+                    const hbfp_format* f, int8_t* mant, int8_t* exps, cudaStream_t st, const Placing& at = Placing{});
 int launch_quantize_tiles(const float* w, int64_t d0, int64_t d1, int64_t ld, const hbfp_format* f,
                           int8_t* mant_c0, int8_t* exps_c0, int8_t* mant_c1, int8_t* exps_c1,
                           int8_t* tile_exps, cudaStream_t st);
@@ -221,10 +234,10 @@ struct FpPlan {
     int form, pair, ncol, splits, kb_per_split, planes_b;
 };
 FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, int passes);
-int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, int place, const FpOperand& out, cudaStream_t st);
+int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const Placing& at, const FpOperand& out, cudaStream_t st);
 // Converts an FP32 operand straight to a form (quantize.cu); HBFP_ERR_UNSUPPORTED for weight tiles.
 int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int contract_axis, const hbfp_format* f, int wide, bool is_b,
-                         int place, const FpOperand& out, cudaStream_t st);
+                         const Placing& at, const FpOperand& out, cudaStream_t st);
 int launch_gemm_fp(int64_t M, int64_t N, const Layout& la, const FpPlan& plan, const FpOperand& a, const FpOperand& b, const float* bias, float* C,
                    int64_t ldc, cudaStream_t st);
 

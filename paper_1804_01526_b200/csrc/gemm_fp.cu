@@ -577,15 +577,15 @@ __device__ __forceinline__ uint32_t f16_pair(float a, float b) {        // exact
 // Form S: rows x kst bytes of one-plane mantissas -> bfloat16 q * 2^s, 16 elements per thread.
 __global__ void __launch_bounds__(256)
 expand_s_kernel(const int8_t* __restrict__ q, const int8_t* __restrict__ exps, int64_t rows, int kst, int lg_bp, int nkb, int64_t rs,
-                uint4* __restrict__ out, int place) {
-    const Chain chain(place);
+                uint4* __restrict__ out, const Placing at) {
+    const Chain chain(at);
     const int per = kst >> 4;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= rows * per) return;
     const int64_t r = i / per;
     const int o = (int)(i - r * per) << 4, kb = o >> lg_bp;
-    const uint4 b = *reinterpret_cast<const uint4*>(q + r * kst + o);
-    const int s = kb < nkb ? (int)exps[(int64_t)kb * rs + r] : 0;
+    const uint4 b = __ldcs(reinterpret_cast<const uint4*>(q + r * kst + o));
+    const int s = kb < nkb ? (int)__ldca(reinterpret_cast<const signed char*>(exps) + (int64_t)kb * rs + r) : 0;
     const float sc = __uint_as_float((uint32_t)(s + 127) << 23);
     float f[8], h[8];
     bytes_to_floats(make_uint2(b.x, b.y), f);
@@ -601,19 +601,19 @@ expand_s_kernel(const int8_t* __restrict__ q, const int8_t* __restrict__ exps, i
 template <bool IS_B>
 __global__ void __launch_bounds__(256)
 expand_w_kernel(const int8_t* __restrict__ q, int64_t plane_stride, const int8_t* __restrict__ exps, int64_t rows, int kst, int lg_bp, int nkb,
-                int64_t rs, uint4* __restrict__ out, uint4* __restrict__ out_l, float* __restrict__ scales, int32_t* status, int place) {
-    const Chain chain(place);
+                int64_t rs, uint4* __restrict__ out, uint4* __restrict__ out_l, float* __restrict__ scales, int32_t* status, const Placing at) {
+    const Chain chain(at);
     const int per = kst >> 3;
     const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= rows * per) return;
     const int64_t r = i / per;
     const int o = (int)(i - r * per) << 3, kb = o >> lg_bp;
-    const uint2 bh = *reinterpret_cast<const uint2*>(q + r * kst + o), bl = *reinterpret_cast<const uint2*>(q + plane_stride + r * kst + o);
+    const uint2 bh = __ldcs(reinterpret_cast<const uint2*>(q + r * kst + o)), bl = __ldcs(reinterpret_cast<const uint2*>(q + plane_stride + r * kst + o));
     float fh[8], fl[8];
     bytes_to_floats(bh, fh);
     bytes_to_floats(bl, fl);
     if ((o & ((1 << lg_bp) - 1)) == 0 && kb < nkb) {
-        const int s = exps[(int64_t)kb * rs + r];
+        const int s = __ldca(reinterpret_cast<const signed char*>(exps) + (int64_t)kb * rs + r);
         scales[(int64_t)kb * rs + r] = __uint_as_float((uint32_t)(s + 127) << 23);
         // the kernel forms P * 2^sA with |P| below 2^30: finite up to here, reported beyond
         if (!IS_B && s > 96) atomicCAS(status, 0, STATUS_EXPONENT_RANGE);
@@ -809,20 +809,20 @@ FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, in
     return f;
 }
 
-int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, int place, const FpOperand& out, cudaStream_t st) {
+int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const Placing& at, const FpOperand& out, cudaStream_t st) {
     const Layout& L = x.L;
     const int lg = log2_of(L.bp);
     if (plan.form == FORM_S) {
         const int64_t n = L.rows * (L.kst / 16);
-        launch_placed(place, expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), place);
+        launch_chained(expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), at);
         return launch_status();
     }
     int32_t* status = device_status_word();
     if (!status) return HBFP_ERR_CUDA;
     const int64_t n = L.rows * (L.kst / 8);
     const unsigned g = (unsigned)((n + 255) / 256);
-    if (is_b) launch_placed(place, expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, place);
-    else launch_placed(place, expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, place);
+    if (is_b) launch_chained(expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, at);
+    else launch_chained(expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, at);
     return launch_status();
 }
 

@@ -16,7 +16,7 @@ struct QParams {
     int exp_mode;
     int rounding;
     uint32_t key0, key1, stream_id;
-    int place;      // of the launch (see Place)
+    Placing at;     // of the launch
 };
 
 __device__ __forceinline__ uint32_t abs_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
@@ -291,7 +291,7 @@ QParams make_params(const hbfp_format* f) {
     p.key0 = (uint32_t)f->seed;
     p.key1 = (uint32_t)(f->seed >> 32);
     p.stream_id = f->stream_id;
-    p.place = CHAINED;
+    p.at = Placing{};
     return p;
 }
 

@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(256, SR ? 3 : 4)
 quant_row_fast(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const int8_t* __restrict__ given, const FormArgs fa) {
-    const Chain chain(p.place);
+    const Chain chain(p.at);
     // given != nullptr: one exponent per row for the whole axis, computed beforehand (a block longer than the
     // tile); the kernel then only rounds and packs
     constexpr int B = 8 * LPB;
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(32 * COL_WARPS)
 quant_col_block(const float* __restrict__ x, int64_t K, int64_t R, int64_t ld, int b, QParams p,
                 int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                 int8_t* __restrict__ exps, int64_t rs, int64_t nkb, unsigned tiles_n, const FormArgs fa, const int8_t* __restrict__ given) {
-    const Chain chain(p.place);
+    const Chain chain(p.at);
     // given != nullptr: one exponent per column for the whole axis, computed beforehand; the blocks are then pieces of it
     constexpr int BP = 32 * WPB, BPC = COL_WARPS / WPB;                // BPC: blocks of a CTA
     __shared__ uint32_t pmax[WPB > 1 ? COL_WARPS : 1][COLT];
@@ -247,7 +247,7 @@ int launch_col_block(const float* x, int64_t K, int64_t rows, int64_t ld, int b,
                      cudaStream_t st, const FormArgs& fa, const int8_t* given) {
     const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT);
     const int64_t per = 128 / bp, grid = (int64_t)tiles_n * ((nkb + per - 1) / per);
-#define HBFP_QCOL(NV, WPB, SRV) launch_placed(p.place, quant_col_block<OUT, NV, WPB, SRV>, (unsigned)grid, 32 * COL_WARPS, 0, st, x, K, rows, ld, b, p, mant, L.kst, L.plane_stride, exps, L.rs, nkb, tiles_n, fa, given)
+#define HBFP_QCOL(NV, WPB, SRV) launch_chained(quant_col_block<OUT, NV, WPB, SRV>, (unsigned)grid, 32 * COL_WARPS, 0, st, x, K, rows, ld, b, p, mant, L.kst, L.plane_stride, exps, L.rs, nkb, tiles_n, fa, given)
 #define HBFP_QCOL_SR(NV, WPB) do { if (p.rounding) HBFP_QCOL(NV, WPB, true); else HBFP_QCOL(NV, WPB, false); } while (0)
     if (bp == 32) { if (b <= 24) HBFP_QCOL_SR(24, 1); else HBFP_QCOL_SR(32, 1); }
     else if (bp == 64) HBFP_QCOL_SR(32, 2);
@@ -1543,7 +1543,7 @@ __global__ void __launch_bounds__(256)
 quant_row_flat(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, QParams p,
                int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                int8_t* __restrict__ exps, int64_t rs, uint32_t gpr, uint32_t total_groups, const FormArgs fa) {
-    const Chain chain(p.place);
+    const Chain chain(p.at);
     constexpr int B = 8 * LPB;
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t g0 = blockIdx.x * (256u * ITEMS) + tid;
@@ -1600,7 +1600,7 @@ int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, c
                           int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa) {
     const uint32_t gpr = (uint32_t)(K / 8), total = (uint32_t)(rows * (K / 8));
     const unsigned grid = (total + 256u * ITEMS - 1u) / (256u * ITEMS);
-#define HBFP_QFLAT(SRV, OUT) launch_placed(p.place, quant_row_flat<LPB, SRV, OUT, ITEMS>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
+#define HBFP_QFLAT(SRV, OUT) launch_chained(quant_row_flat<LPB, SRV, OUT, ITEMS>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
     if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QFLAT(true, FORM); else HBFP_QFLAT(false, FORM); }
     else if (p.rounding == 1) { if (L.planes == 1) HBFP_QFLAT(true, 1); else HBFP_QFLAT(true, 2); }
     else { if (L.planes == 1) HBFP_QFLAT(false, 1); else HBFP_QFLAT(false, 2); }
@@ -1653,7 +1653,7 @@ __global__ void __launch_bounds__(256)
 quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t ld, int b, QParams p,
                  int8_t* __restrict__ mant, int64_t kst, int64_t plane_stride,
                  int8_t* __restrict__ exps, int64_t rs, int64_t nkb, const Divisor ppr, int64_t row_first, uint32_t total, const FormArgs fa) {
-    const Chain chain(p.place);
+    const Chain chain(p.at);
     constexpr bool TABLE = SR && !VEC;
     constexpr int ITEMS = 2, PIECES = ragged_pieces<LPB, TABLE>();
     __shared__ __align__(16) uint4 rnd[TABLE ? 8 : 1][TABLE ? 65 : 1];         // (the word after the last group is read and not used)
@@ -1679,7 +1679,7 @@ quant_row_ragged(const float* __restrict__ x, int64_t rows, int64_t K, int64_t l
             e8[i][4] = w.x; e8[i][5] = w.y; e8[i][6] = w.z; e8[i][7] = w.w;
         } else {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) e8[i][j] = j < n ? __ldg(src + j) : 0.f;
+            for (int j = 0; j < 8; ++j) e8[i][j] = j < n ? __ldca(src + j) : 0.f;
         }
     }
     // the draws do not depend on the data: they are made while the loads are in flight (the matrix is rows x K as passed)
@@ -1721,9 +1721,9 @@ int launch_row_ragged(bool vec, const float* x, int64_t rows, int64_t K, int64_t
     if (ppr >= (1ll << 31)) return HBFP_ERR_UNSUPPORTED;
     const Divisor d = divisor((uint32_t)ppr);
     QParams q = p;
-    for (int64_t r = 0; r < rows; r += rows_per, q.place = CHAINED) {
+    for (int64_t r = 0; r < rows; r += rows_per, q.at = Placing{}) {
         const int64_t total = std::min(rows - r, rows_per) * ppr;
-#define HBFP_RAGGED(LPB, SRV, VEC) launch_placed(q.place, quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 8 * ragged_pieces<LPB, SRV && !VEC>() - 1) / (8 * ragged_pieces<LPB, SRV && !VEC>())), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
+#define HBFP_RAGGED(LPB, SRV, VEC) launch_chained(quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 8 * ragged_pieces<LPB, SRV && !VEC>() - 1) / (8 * ragged_pieces<LPB, SRV && !VEC>())), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
 #define HBFP_RAGGED_SR(LPB, VEC) do { if (p.rounding) HBFP_RAGGED(LPB, true, VEC); else HBFP_RAGGED(LPB, false, VEC); } while (0)
 #define HBFP_RAGGED_VEC(LPB) do { if (vec) HBFP_RAGGED_SR(LPB, true); else HBFP_RAGGED_SR(LPB, false); } while (0)
         if (L.bp == 32) HBFP_RAGGED_VEC(4); else if (L.bp == 64) HBFP_RAGGED_VEC(8); else HBFP_RAGGED_VEC(16);
@@ -1758,7 +1758,7 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
               const __grid_constant__ CUtensorMap mapM1, QParams p, int8_t* __restrict__ exps, int64_t rs,
               int64_t nkb, int64_t K, int64_t R, int tiles_n, int total_tiles, int32_t* status,
               const int8_t* __restrict__ given, int8_t* __restrict__ form_out, int64_t kst, int64_t plane_stride) {
-    const Chain chain(p.place);
+    const Chain chain(p.at);
     // given != nullptr: one exponent per column for the whole axis, computed beforehand (blocks longer than a
     // tile); the kernel then only rounds and packs
     extern __shared__ unsigned char smem_dyn[];
@@ -1786,6 +1786,7 @@ quant_col_tma(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ 
     __syncthreads();
     const int first = blockIdx.x, step = gridDim.x;
     if (tid == 0) {
+        if (p.at.place == BESIDE) asm volatile("fence.proxy.async.global;" ::: "memory");      // what was acquired is read by the copy engine
         for (int s = 0; s < QC_STAGES; ++s) {
             const int t = first + s * step;
             if (t < total_tiles) {
@@ -1966,7 +1967,7 @@ int launch_col_tma(const float* x, int64_t K, int64_t rows, int64_t ld, const QP
     const int64_t total = tiles_n * tiles_k;
     const int64_t cap = (int64_t)sm_count() * ctas_per_sm;
     const int grid = (int)(total < cap ? total : cap);
-    launch_placed(p.place, quant_col_tma<PLANES, LB, SR>, grid, QC_THREADS, smem, st, mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
+    launch_chained(quant_col_tma<PLANES, LB, SR>, grid, QC_THREADS, smem, st, mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
                                                               (int)total, status, given, mant, L.kst, L.plane_stride);
     return launch_status();
 }
@@ -1979,11 +1980,11 @@ int launch_row_fast(const float* x, int64_t rows, int64_t K, int64_t ld, const Q
     dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
     // the last column tile must also cover the exponent rows of blocks that start before K
     if (p.rounding == 1) {
-        if (L.planes == 1) launch_placed(p.place, quant_row_fast<LPB, true, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
-        else launch_placed(p.place, quant_row_fast<LPB, true, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        if (L.planes == 1) launch_chained(quant_row_fast<LPB, true, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        else launch_chained(quant_row_fast<LPB, true, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
     } else {
-        if (L.planes == 1) launch_placed(p.place, quant_row_fast<LPB, false, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
-        else launch_placed(p.place, quant_row_fast<LPB, false, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        if (L.planes == 1) launch_chained(quant_row_fast<LPB, false, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        else launch_chained(quant_row_fast<LPB, false, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
     }
     return launch_status();
 }
@@ -2033,7 +2034,7 @@ int launch_tile_full_small(int mode, int planes, int t, bool general, unsigned g
 // ------------------------------------------------------------------------------ launchers
 
 int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f,
-                    int8_t* mant, int8_t* exps, cudaStream_t st, int place) {
+                    int8_t* mant, int8_t* exps, cudaStream_t st, const Placing& at) {
     const int64_t K = axis == 1 ? d1 : d0, rows = axis == 1 ? d0 : d1;
     Layout L;
     int rc = make_layout(rows, K, f, &L);
@@ -2041,8 +2042,8 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     if (rows == 0) return HBFP_OK;
     const QParams p = make_params(f);
     QParams one = p, last = p;         // the only launch of a conversion, the last of several
-    one.place = place;
-    last.place = place == LEAD ? LEAD : CHAINED;
+    one.at = at;
+    if (at.place == LEAD) last.at = at;
     if (K == 0) {
         HBFP_CUDA_OK(cudaMemsetAsync(mant, 0, (size_t)L.mant_bytes, st));
         HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
@@ -2067,7 +2068,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
         // rows of 2048, 4096, 8192 or 16384 elements stay in a CTA's registers: one pass
         if ((K == 2048 || K == 4096 || K == 8192 || K == 16384) && L.kst == K && rows < (1ll << 31)) {
-#define HBFP_QROW_WHOLE2(GV, SRV, PL) launch_placed(last.place, quant_row_whole<GV, SRV, PL>, (unsigned)rows, 256, 0, st, x, ld, d1, p, mant, L.kst, L.plane_stride, exps)
+#define HBFP_QROW_WHOLE2(GV, SRV, PL) launch_chained(quant_row_whole<GV, SRV, PL>, (unsigned)rows, 256, 0, st, x, ld, d1, p, mant, L.kst, L.plane_stride, exps)
 #define HBFP_QROW_WHOLE(GV)                                                                          \
     do {                                                                                             \
         if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_WHOLE2(GV, true, 1); else HBFP_QROW_WHOLE2(GV, true, 2); }   \
@@ -2082,7 +2083,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         launch_chained(exps_axis1, (unsigned)(want < 148 * 16 ? want : 148 * 16), 256, 0, st, x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
         if (launch_status()) return HBFP_ERR_CUDA;
         dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
-#define HBFP_QROW_GIVEN(SRV, PL) launch_placed(last.place, quant_row_fast<16, SRV, PL>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, exps, FormArgs{})
+#define HBFP_QROW_GIVEN(SRV, PL) launch_chained(quant_row_fast<16, SRV, PL>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, exps, FormArgs{})
         if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_GIVEN(true, 1); else HBFP_QROW_GIVEN(true, 2); }
         else { if (L.planes == 1) HBFP_QROW_GIVEN(false, 1); else HBFP_QROW_GIVEN(false, 2); }
 #undef HBFP_QROW_GIVEN
@@ -2167,9 +2168,9 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     }
     if (launch_status()) return HBFP_ERR_CUDA;
     if (L.planes == 1)
-        launch_placed(last.place, mant_generic<1>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
+        launch_chained(mant_generic<1>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     else
-        launch_placed(last.place, mant_generic<2>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
+        launch_chained(mant_generic<2>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     return launch_status();
 }
 
@@ -2184,7 +2185,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
             return L.b == 32 ? launch_row_flat<4, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_flat<8, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
         if (aligned && d1 % 8 == 0 && L.b == L.bp && rows <= 32ll * 65535) {
             const dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
-#define HBFP_QFAST(LPB, SRV) launch_placed(p.place, quant_row_fast<LPB, SRV, FORM>, grid, 256, 0, st, x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
+#define HBFP_QFAST(LPB, SRV) launch_chained(quant_row_fast<LPB, SRV, FORM>, grid, 256, 0, st, x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
             if (L.b == 32) { if (p.rounding) HBFP_QFAST(4, true); else HBFP_QFAST(4, false); }
             else { if (p.rounding) HBFP_QFAST(8, true); else HBFP_QFAST(8, false); }
 #undef HBFP_QFAST
@@ -2206,7 +2207,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
 
 // Converts an FP32 operand straight to a floating-point operand form: blocks of at most 64, no weight tiles, elements
 // aligned to 32 bytes (HBFP_ERR_UNSUPPORTED otherwise; the caller converts to the packed layout and expands that).
-int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f, int wide, bool is_b, int place,
+int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis, const hbfp_format* f, int wide, bool is_b, const Placing& at,
                          const FpOperand& o, cudaStream_t st) {
     const int64_t K = axis == 1 ? d1 : d0, rows = axis == 1 ? d0 : d1;
     Layout L;
@@ -2214,7 +2215,7 @@ int launch_quantize_form(const float* x, int64_t d0, int64_t d1, int64_t ld, int
     if (rc) return rc;
     if (f->tile != 0 || L.bp > 64 || rows == 0 || K == 0 || (L.planes == 2) != (wide != 0)) return HBFP_ERR_UNSUPPORTED;
     QParams p = make_params(f);
-    p.place = place;
+    p.at = at;
     const FormArgs fa{device_status_word()};
     if (!fa.status) return HBFP_ERR_CUDA;
     int8_t* out = static_cast<int8_t*>(o.p0);

@@ -703,39 +703,7 @@ def edges_in_order(graph) -> list:
     return kinds
 
 
-# The conversion that runs beside another one reads before it has waited for anything: what a chained kernel wrote is visible to it only
-# past a whole kernel boundary, which the first conversion has to be.
-@pytest.mark.parametrize("m,b,tA,packed", [(8, 32, 1, None), (8, 24, 0, None), (12, 64, 0, None), (8, 128, 1, None), (8, 32, 0, "B"), (12, 32, 0, "B"), (12, 64, 0, "AB")])
-def test_second_conversion_comes_after_a_whole_kernel_boundary(hb, m, b, tA, packed):
-    import torch
-    M, N, K = 2048, 2304, 2048
-    fa, fb = hb.Format(mant_bits=m, block=b), hb.Format(mant_bits=m, block=b, stream_id=1)
-    fw = hb.Format(mant_bits=m, block=b, tile=b, stream_id=1)
-    A, W = torch.randn(K if tA else M, M if tA else K, device="cuda"), torch.randn(K, N, device="cuda") * 0.05
-    wide, views = hb.wide_quantize(W, fw)
-    delta = W * 0.01
-    a = hb.quantize(A, 1, fa) if packed == "AB" else A
-    C, ws = torch.empty(M, N, device="cuda"), torch.empty(1 << 27, dtype=torch.int8, device="cuda")
-
-    def step():
-        if packed:
-            hb.wide_update(wide, delta, fw, views=views)
-            hb.gemm_q(M, N, K, a, views[0], fmtA=fa, out=C, workspace=ws)
-        else:
-            hb.wide_dequantize(wide, W)
-            hb.gemm(tA, 0, A, W, fa, fb, C, ws)
-
-    step()                                                # sets the kernels' attributes once
-    torch.cuda.synchronize()
-    graph = torch.cuda.CUDAGraph(keep_graph=True)
-    with torch.cuda.graph(graph):
-        step()
-    kinds = edges_in_order(graph)
-    # the kernel that writes the second operand, the first conversion, the second one, the product
-    assert len(kinds) == 3 and kinds[:2] == [0, 1]
-
-
-# The product itself is placed early too, but for long launches of the 12-bit form.
+# The second conversion runs beside the first, the product is placed early, but for long launches of the 12-bit form.
 @pytest.mark.parametrize("n,m,b,chained", [(2048, 8, 32, 1), (4096, 8, 32, 1), (4096, 8, 24, 1), (4096, 8, 64, 1), (2048, 12, 64, 1), (4096, 12, 64, 0), (4096, 12, 24, 0)])
 def test_products_of_operand_forms_are_placed_early(hb, n, m, b, chained):
     import torch
@@ -752,11 +720,12 @@ def test_products_of_operand_forms_are_placed_early(hb, n, m, b, chained):
 
 # Routes in which the second operand is converted beside the first, on an operand that the kernel before has just written: packed
 # weights of an update in place, the FP32 value of wide weights.
-@pytest.mark.parametrize("m,b", [(8, 32), (8, 64), (12, 64), (12, 32)])
+# Replayed too: the word through which the first conversion passes on what it has waited for starts every replay anew.
+@pytest.mark.parametrize("m,b,N", [(8, 32, 2304), (8, 64, 2304), (12, 64, 2304), (12, 32, 2304), (8, 24, 2307), (12, 24, 2307)])
 @pytest.mark.parametrize("kind", ["packed weights", "both packed", "fp32"])
-def test_products_of_operands_that_the_kernel_before_has_written(hb, m, b, kind):
+def test_products_of_operands_that_the_kernel_before_has_written(hb, m, b, N, kind):
     import torch
-    M, N, K = 2048, 2304, 2048
+    M, K = 2048, 2048
     fa, fb = hb.Format(mant_bits=m, block=b), hb.Format(mant_bits=m, block=b, stream_id=1)
     fw = hb.Format(mant_bits=m, block=b, tile=b, stream_id=1)
     gen = torch.Generator(device="cuda").manual_seed(9)
@@ -784,4 +753,22 @@ def test_products_of_operands_that_the_kernel_before_has_written(hb, m, b, kind)
     assert hb.last_gemm_launch().startswith("gemm_fp_kernel")
     for _ in range(4):
         assert all(torch.equal(x, y) for x, y in zip(run(False), want))
+    wide, views = hb.wide_quantize(w0, fw)
+    W, C, ws, delta = torch.empty(K, N, device="cuda"), torch.empty(M, N, device="cuda"), torch.empty(1 << 27, dtype=torch.int8, device="cuda"), deltas[0].clone()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        if kind == "fp32":
+            hb.wide_update(wide, delta, fw, want_views=False)
+            hb.wide_dequantize(wide, W)
+            hb.gemm(0, 0, A, W, fa, fb, C, ws)
+        else:
+            hb.wide_update(wide, delta, fw, views=views)
+            hb.gemm_q(M, N, K, pa, views[0], fmtA=fa, out=C, workspace=ws)
+    got = []
+    for i in range(12):
+        delta.copy_(deltas[i % 3])
+        graph.replay()
+        got.append(C.clone())
+    assert all(torch.equal(x, y) for x, y in zip(got, want))
     assert hb.device_status() == 0
