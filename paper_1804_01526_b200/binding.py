@@ -46,6 +46,12 @@ class _CFormat(ctypes.Structure):
                 ("reserved", ctypes.c_uint32), ("seed", ctypes.c_uint64)]
 
 
+class _CLayout(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int64) for n in
+                ("rows", "k", "b", "bp", "nkb", "kst", "planes", "plane_stride", "rs",
+                 "mant_bytes", "exp_bytes")]
+
+
 class _COperand(ctypes.Structure):
     _fields_ = [("struct_size", ctypes.c_uint32), ("kind", ctypes.c_int32),
                 ("data", ctypes.c_void_p), ("exps", ctypes.c_void_p), ("ld", ctypes.c_int64),
@@ -163,7 +169,12 @@ def _dptr(t: Optional[torch.Tensor]) -> ctypes.c_void_p:
 
 
 def packed_layout(rows: int, k: int, fmt: Format) -> dict:
-    return _got((_native or host()).packed_layout(rows, k, fmt), "hbfp_packed_layout")
+    if type(fmt) is Format:
+        return _got((_native or host()).packed_layout(rows, k, fmt), "hbfp_packed_layout")
+    # another class says in its c() what it stands for, here as in packed_sizes
+    out, cf = _CLayout(), fmt.c()
+    _check(lib().hbfp_packed_layout(rows, k, ctypes.byref(cf), ctypes.byref(out)), "hbfp_packed_layout")
+    return {n: getattr(out, n) for n, _ in _CLayout._fields_}
 
 
 def packed_sizes(rows: int, k: int, fmt: Format) -> Tuple[int, int]:

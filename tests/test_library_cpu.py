@@ -55,6 +55,16 @@ def test_packed_layout(hb, rows, k, m, b, exp):
     assert hb.packed_sizes(rows, k, hb.Format(m, b)) == (lay["mant_bytes"], lay["exp_bytes"])
 
 
+def test_a_format_that_makes_its_own_descriptor_is_read_alike_everywhere(hb):
+    class Wider(hb.Format):
+        def c(self):
+            return hb.Format(self.mant_bits, 4 * self.block).c()
+
+    lay = hb.packed_layout(9, 300, Wider(8, 24))
+    assert lay == hb.packed_layout(9, 300, hb.Format(8, 96)) and lay["b"] == 96
+    assert hb.packed_sizes(9, 300, Wider(8, 24)) == (lay["mant_bytes"], lay["exp_bytes"])
+
+
 def test_bad_formats_are_rejected(hb):
     for f in (hb.Format(1, 32), hb.Format(13, 32), hb.Format(8, -1), hb.Format(8, 32, tile=16),
               hb.Format(8, 32, rounding=2), hb.Format(8, 32, exp_mode=3)):
