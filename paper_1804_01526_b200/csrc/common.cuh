@@ -89,21 +89,27 @@ struct Placing {
     unsigned long long* word = nullptr;
     unsigned long long turn = 0;
 };
+// (The usual place first: with the others in the way rows of 1024 x 1024, b = 32, took 3.3 us instead of 3.1.)
 struct Chain {
-    const Placing at;
+    const Placing& at;
     __device__ __forceinline__ explicit Chain(const Placing& a) : at(a) {
+        if (__builtin_expect(at.place == CHAINED, 1)) {
+            chain_wait();
+            chain_next();
+            return;
+        }
         if (at.place == BESIDE) {
             unsigned long long seen = at.turn;
             if (threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(at.word) : "memory");
             if (__syncthreads_or(seen != at.turn)) chain_wait();
         } else {
             chain_wait();
-            if (at.place == LEAD && (blockIdx.x | blockIdx.y | threadIdx.x) == 0) asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(at.word), "l"(at.turn) : "memory");
+            if ((blockIdx.x | blockIdx.y | threadIdx.x) == 0) asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(at.word), "l"(at.turn) : "memory");
         }
         chain_next();
     }
     __device__ __forceinline__ ~Chain() {
-        if (at.place != BESIDE) return;
+        if (__builtin_expect(at.place != BESIDE, 1)) return;
         chain_wait();
         if ((blockIdx.x | blockIdx.y | threadIdx.x) == 0) asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at.word), "l"(0ull) : "memory");
     }
