@@ -43,13 +43,14 @@ unsigned long long* turn_words() {
 // The places of two conversions, the second beside the first or (where it may not be) after it.
 struct PlacedPair {
     Placing first, second;
-    explicit PlacedPair(bool beside) {
+    // second_bytes: loaded by the second conversion
+    PlacedPair(bool beside, int64_t second_bytes) {
         static std::atomic<unsigned long long> turns{0};
         unsigned long long* const words = beside ? turn_words() : nullptr;
         if (!words) return;
         const unsigned long long turn = ++turns;
-        first = {LEAD, words + turn % TURN_WORDS, turn};
-        second = {BESIDE, words + turn % TURN_WORDS, turn};
+        first = {LEAD, words + turn % TURN_WORDS, turn, second_bytes};
+        second = {BESIDE, words + turn % TURN_WORDS, turn, 0};
     }
 };
 
@@ -166,6 +167,12 @@ int check_fp32(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K) {
     return o->ld < (k_contiguous(o, is_a) ? K : rows) ? HBFP_ERR_INVALID_ARG : HBFP_OK;
 }
 
+// Bytes that the conversion of B loads through L1: none where it loads by the copy engine (whole blocks down aligned columns).
+int64_t streamed_bytes(const hbfp_operand* b, int64_t N, int64_t K, const Layout& L) {
+    if (b->kind == HBFP_OPERAND_PACKED) return L.planes * N * K;
+    return !k_contiguous(b, false) && L.b == L.bp && L.b <= 128 && b->ld % 4 == 0 ? 0 : 4 * N * K;
+}
+
 // Quantises an FP32 operand into the workspace (or takes a packed one as is).
 int resolve_operand(const hbfp_operand* o, bool is_a, int64_t rows, int64_t K, const Layout& L,
                     char* ws, size_t off_m, size_t off_e, Packed* out, const Placing& at, cudaStream_t st) {
@@ -254,7 +261,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     if (use_fp && !small) {
         const FpOperand fa = fp_operand(g.la, g.fp, false, ws + g.off_fa), fb = fp_operand(g.lb, g.fp, true, ws + g.off_fb);
         const bool beside = b->kind == HBFP_OPERAND_PACKED || b->fmt.tile == 0;       // B in one launch
-        const PlacedPair at(beside);
+        const PlacedPair at(beside, streamed_bytes(b, N, K, g.lb));
         rc = resolve_form(a, true, M, K, g, ws, fa, at.first, st);
         if (rc) return rc;
         rc = resolve_form(b, false, N, K, g, ws, fb, at.second, st);
@@ -265,7 +272,7 @@ int gemm_impl(int64_t M, int64_t N, int64_t K, const hbfp_operand* a, const hbfp
     }
     // two conversions of one launch each (longer blocks and weight tiles may take several, or another kernel)
     const bool beside = a->kind == HBFP_OPERAND_FP32 && b->kind == HBFP_OPERAND_FP32 && a->fmt.tile == 0 && b->fmt.tile == 0 && K > 0 && g.la.b <= 256;
-    const PlacedPair at(beside);
+    const PlacedPair at(beside, streamed_bytes(b, N, K, g.lb));
     rc = resolve_operand(a, true, M, K, g.la, ws, g.off_am, g.off_ae, &pa, at.first, st);
     if (rc) return rc;
     rc = resolve_operand(b, false, N, K, g.lb, ws, g.off_bm, g.off_be, &pb, at.second, st);

@@ -88,6 +88,7 @@ struct Placing {
     int place = CHAINED;
     unsigned long long* word = nullptr;
     unsigned long long turn = 0;
+    int64_t more = 0;             // of a LEAD: bytes that the BESIDE launch loads
 };
 // (The usual place first: with the others in the way rows of 1024 x 1024, b = 32, took 3.3 us instead of 3.1.)
 struct Chain {
@@ -115,8 +116,28 @@ struct Chain {
     }
 };
 
+// Two kinds of kernels are not chained behind a product, that is where this thread has launched one on the stream since its last launch
+// that was not chained (times behind a product, chained / not):
+// - Those that load 50 MB and more. The products take most of an SM's memory as shared memory, and an SM keeps its split between that and
+//   L1 until it has been idle. A kernel that is placed behind a product never lets it be: it runs with the little L1 that the product had
+//   left, which is what its loads in flight are held in. Update of 8192 x 8192, t = 64 156 / 113 us, with its FP32 value 215 / 154, rows of
+//   8192 x 8192 converted, b = 32 68 / 56; 4096 x 4096, t = 64 40 / 32, b = 32 17.3 / 14.8, its column sums 18 / 13; 2048 x 4096, t = 64 18.4 /
+//   16.9, b = 32 8.4 / 8.6; 2048 x 2048, t = 64 8.8 / 10.7. Kernels that load through the copy engine keep their data in shared memory and
+//   are always chained.
+// - A few long CTAs (at most two per SM, of thousands of elements): placed as SMs fall free, they crowd on the first of them. Update of
+//   1024 x 1024, t = 24, with draws 15.6 / 12.7 us, t = 128 with its FP32 value 11.6 / 8.6.
+// Behind other kernels they are chained (rows of 8192 x 8192 back to back 51.2 / 53.1, updates of 1024 x 1024, t = 24 10.7 / 12.5).
+constexpr int64_t STREAMED_BYTES = 50 * 1000 * 1000;
+constexpr unsigned FEW_CTAS = 2 * 148;
+struct LastProduct {
+    cudaStream_t st = nullptr;
+    bool holds = false;
+};
+inline thread_local LastProduct t_last_product;
+inline void note_product(cudaStream_t st) { t_last_product = {st, true}; }
+
 template <class... Params, class... Args>
-inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+inline void launch_one(bool chained, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.gridDim = grid;
@@ -126,8 +147,32 @@ inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, siz
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = chained;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);      // launch_status() has the verdict
+}
+template <class... Params, class... Args>
+inline void launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    launch_one(true, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+}
+// Whether a kernel that loads so many bytes is chained.
+inline bool chain_streamed(int64_t bytes, cudaStream_t st) {
+    const bool chained = bytes < STREAMED_BYTES || !t_last_product.holds || t_last_product.st != st;
+    if (!chained) t_last_product.holds = false;
+    return chained;
+}
+template <class... Params, class... Args>
+inline void launch_streamed(int64_t bytes, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    launch_one(chain_streamed(bytes, st), kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+}
+// A conversion. A BESIDE launch is always chained, a LEAD counts for both.
+template <class... Params, class... Args>
+inline void launch_placed(const Placing& at, int64_t bytes, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    launch_one(at.place == BESIDE || chain_streamed(bytes + at.more, st), kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+}
+// The same as launch_streamed for long CTAs.
+template <class... Params, class... Args>
+inline void launch_streamed_long(int64_t bytes, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    launch_one(chain_streamed(grid.x * grid.y <= FEW_CTAS ? STREAMED_BYTES : bytes, st), kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 // The same with clusters of `cluster` CTAs along x; not chained where the kernel's tiles want the order of an empty chip (gemm_fp.cu).
 template <class... Params, class... Args>

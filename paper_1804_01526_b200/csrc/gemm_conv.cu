@@ -498,6 +498,7 @@ int launch_conv_cfg(const CUtensorMap& mX, const CUtensorMap& mW, const ConvProb
     }
     const int grid = p.super_tiles < sm_count() ? p.super_tiles : sm_count();
     launch_chained(conv_fwd_kernel<C, N_TILE>, grid, CV_THREADS, G::SMEM, st, mX, mW, p);
+    note_product(st);
     return launch_status();
 }
 

@@ -722,6 +722,7 @@ int fp_launch(FpProblem p, const FpOperand& a, const FpOperand& b, cudaStream_t 
     const int ctas = PAIR ? grid / 2 : grid;
     const bool chained = FORM == FORM_S || p.splits > 1 || (int64_t)((tiles + ctas - 1) / ctas) * p.nkb < 400;
     launch_chained_clusters(gemm_fp_kernel<FORM, NCOL, BP, PAIR, BIAS>, PAIR ? 2 : p.splits, grid, FP_THREADS, C::SMEM, st, chained, mA, mB, mB1, mSA, mSB, mC, p);
+    note_product(st);
     return launch_status();
 }
 
@@ -814,15 +815,15 @@ int launch_expand(const Packed& x, const FpPlan& plan, bool is_b, const Placing&
     const int lg = log2_of(L.bp);
     if (plan.form == FORM_S) {
         const int64_t n = L.rows * (L.kst / 16);
-        launch_chained(expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), at);
+        launch_placed(at, L.rows * L.kst, expand_s_kernel, (unsigned)((n + 255) / 256), 256, 0, st, x.mant, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), at);
         return launch_status();
     }
     int32_t* status = device_status_word();
     if (!status) return HBFP_ERR_CUDA;
     const int64_t n = L.rows * (L.kst / 8);
     const unsigned g = (unsigned)((n + 255) / 256);
-    if (is_b) launch_chained(expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, at);
-    else launch_chained(expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, at);
+    if (is_b) launch_placed(at, L.rows * L.kst * 2, expand_w_kernel<true>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), static_cast<uint4*>(out.p1), out.scales, status, at);
+    else launch_placed(at, L.rows * L.kst * 2, expand_w_kernel<false>, g, 256, 0, st, x.mant, L.plane_stride, x.exps, L.rows, (int)L.kst, lg, (int)L.nkb, L.rs, static_cast<uint4*>(out.p0), nullptr, out.scales, status, at);
     return launch_status();
 }
 

@@ -363,6 +363,7 @@ int sk_launch(const SkinnyProblem& p, const CUtensorMap& mW, size_t smem, dim3 g
         ready[dev] = true;
     }
     launch_chained_clusters(gemm_skinny_kernel<ROWS, BP, SR>, p.splits, grid, SK_THREADS, smem, st, true, mW, p);
+    note_product(st);
     return launch_status();
 }
 template <int ROWS, bool SR>

@@ -327,6 +327,7 @@ int launch_gemm_small(int64_t M, int64_t N, const Packed& a, const Packed& b, co
     const dim3 grid((unsigned)((N + SM_TILE - 1) / SM_TILE), (unsigned)((M + SM_TILE - 1) / SM_TILE));
     launch_chained(gemm_small_kernel, grid, 256, smem, st, M, N, nkb, (int)a.L.bp, a.mant, a.L.kst, a.exps, a.L.rs, b.mant, b.L.kst,
                                                b.exps, b.L.rs, bias, C, ldc);
+    note_product(st);
     return launch_status();
 }
 
@@ -341,6 +342,7 @@ int sf_launch(const SmallProblem& p, dim3 grid, cudaStream_t st) {
         attr_set[dev] = true;
     }
     launch_chained(gemm_small_fused_kernel<SR, PER>, grid, SF_THREADS, 2 * (size_t)SM_TILE * p.pitch, st, p);      // at most 68 KB
+    note_product(st);
     return launch_status();
 }
 }  // namespace

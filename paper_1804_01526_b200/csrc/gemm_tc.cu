@@ -792,6 +792,7 @@ int launch_cfg(const Problem& p, const Packed& a, const Packed& b, cudaStream_t 
     const int64_t work = (int64_t)p.tiles_m * p.tiles_n * p.splits;
     const int grid = (int)(work < sm_count() ? work : sm_count());
     launch_chained(gemm_tc_kernel<N_TILE, PLANES, MAGIC, DUMP, TSTORE>, grid, THREADS, C::SMEM, st, mA0, mA1, mB0, mB1, mEA, mEB, mC, p);
+    note_product(st);
     return launch_status();
 }
 

@@ -733,6 +733,7 @@ int launch_gemm_tensor_pair(int64_t M, int64_t N, const Packed& a, const Packed&
     if (p.bp == 128) gemm_tc2_kernel<0><<<2 * clusters, THREADS, SMEM, st>>>(mA, mB, mEA, mEB, p);
     else if (p.bp == 64) gemm_tc2_kernel<1><<<2 * clusters, THREADS, SMEM, st>>>(mA, mB, mEA, mEB, p);
     else gemm_tc2_kernel<2><<<2 * clusters, THREADS, SMEM, st>>>(mA, mB, mEA, mEB, p);
+    note_product(st);
     return launch_status();
 }
 

@@ -145,7 +145,7 @@ int column_sums(const float* x, int64_t rows, int64_t cols, int64_t ld, float* o
     while (splits < 8 && rows >= 2 * splits * CS_WARPS * CS_UNR) splits *= 2;
     for (int64_t c0 = 0; c0 < cols; c0 += MOST) {
         const int64_t n = cols - c0 < MOST ? cols - c0 : MOST;
-        launch_chained_clusters(column_sums_kernel<V>, splits, dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V))), 32 * CS_WARPS, 0, st, true, x + c0, rows, n, ld,
+        launch_chained_clusters(column_sums_kernel<V>, splits, dim3(splits, (unsigned)((n + 32 * V - 1) / (32 * V))), 32 * CS_WARPS, 0, st, chain_streamed(4 * rows * n, st), x + c0, rows, n, ld,
                                 splits, out + c0);
         if (launch_status()) return HBFP_ERR_CUDA;
     }
@@ -159,8 +159,8 @@ int launch_add_bias(float* C, int64_t M, int64_t N, int64_t ldc, const float* bi
     const int64_t total = quad ? M * (N / 4) : M * N;
     const int64_t blocks = (total + 255) / 256, cap = 148 * 32;
     const unsigned grid = (unsigned)(blocks < cap ? blocks : cap);
-    if (quad) launch_chained(add_bias_kernel<4>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
-    else launch_chained(add_bias_kernel<1>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
+    if (quad) launch_streamed(4 * M * N, add_bias_kernel<4>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
+    else launch_streamed(4 * M * N, add_bias_kernel<1>, grid, 256, 0, st, C, (uint32_t)N, ldc, bias, total);
     return launch_status();
 }
 
@@ -175,8 +175,8 @@ int launch_fold_taps(const float* cols, int64_t n, int64_t h, int64_t w, int64_t
     for (int64_t x0 = 0; x0 < w; x0 += most) {
         const uint32_t part = (uint32_t)(w - x0 < most ? w - x0 : most);
         const dim3 grid((unsigned)(n * h), (unsigned)((part * cv + threads - 1) / threads));
-        if (quad) launch_chained(fold_taps_kernel<4>, grid, threads, 0, st, cols, (uint32_t)h, (uint32_t)w, (uint32_t)x0, part, (uint32_t)cv, kh, kw, pad, out);
-        else launch_chained(fold_taps_kernel<1>, grid, threads, 0, st, cols, (uint32_t)h, (uint32_t)w, (uint32_t)x0, part, (uint32_t)cv, kh, kw, pad, out);
+        if (quad) launch_streamed(4 * n * h * part * c * kh * kw, fold_taps_kernel<4>, grid, threads, 0, st, cols, (uint32_t)h, (uint32_t)w, (uint32_t)x0, part, (uint32_t)cv, kh, kw, pad, out);
+        else launch_streamed(4 * n * h * part * c * kh * kw, fold_taps_kernel<1>, grid, threads, 0, st, cols, (uint32_t)h, (uint32_t)w, (uint32_t)x0, part, (uint32_t)cv, kh, kw, pad, out);
         if (launch_status()) return HBFP_ERR_CUDA;
     }
     return HBFP_OK;

@@ -247,7 +247,7 @@ int launch_col_block(const float* x, int64_t K, int64_t rows, int64_t ld, int b,
                      cudaStream_t st, const FormArgs& fa, const int8_t* given) {
     const unsigned tiles_n = (unsigned)((rows + COLT - 1) / COLT);
     const int64_t per = 128 / bp, grid = (int64_t)tiles_n * ((nkb + per - 1) / per);
-#define HBFP_QCOL(NV, WPB, SRV) launch_chained(quant_col_block<OUT, NV, WPB, SRV>, (unsigned)grid, 32 * COL_WARPS, 0, st, x, K, rows, ld, b, p, mant, L.kst, L.plane_stride, exps, L.rs, nkb, tiles_n, fa, given)
+#define HBFP_QCOL(NV, WPB, SRV) launch_placed(p.at, 4 * K * rows, quant_col_block<OUT, NV, WPB, SRV>, (unsigned)grid, 32 * COL_WARPS, 0, st, x, K, rows, ld, b, p, mant, L.kst, L.plane_stride, exps, L.rs, nkb, tiles_n, fa, given)
 #define HBFP_QCOL_SR(NV, WPB) do { if (p.rounding) HBFP_QCOL(NV, WPB, true); else HBFP_QCOL(NV, WPB, false); } while (0)
     if (bp == 32) { if (b <= 24) HBFP_QCOL_SR(24, 1); else HBFP_QCOL_SR(32, 1); }
     else if (bp == 64) HBFP_QCOL_SR(32, 2);
@@ -268,6 +268,10 @@ struct TileViews {
     int8_t* mant_c1; int64_t kst1, ps1; int8_t* exps_c1; int64_t rs1, nkb1;
     float* value; int64_t ldv;      // FP32 value of the wide words (modes that write them), or null
 };
+
+// Bytes that the modes below load: FP32 and words.
+template <int MODE>
+constexpr int64_t tile_bytes(int64_t d0, int64_t d1) { return d0 * d1 * (MODE == 1 || MODE == 4 ? 6 : MODE == 2 ? 2 : 4); }
 
 // 2^e for every stored exponent: below -126 the power itself is subnormal, and its product with a mantissa is exact.
 __device__ __forceinline__ float pow2f_stored(int e) {
@@ -1600,7 +1604,7 @@ int launch_row_flat_items(const float* x, int64_t rows, int64_t K, int64_t ld, c
                           int8_t* mant, int8_t* exps, cudaStream_t st, const FormArgs& fa) {
     const uint32_t gpr = (uint32_t)(K / 8), total = (uint32_t)(rows * (K / 8));
     const unsigned grid = (total + 256u * ITEMS - 1u) / (256u * ITEMS);
-#define HBFP_QFLAT(SRV, OUT) launch_chained(quant_row_flat<LPB, SRV, OUT, ITEMS>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
+#define HBFP_QFLAT(SRV, OUT) launch_placed(p.at, 4 * rows * K, quant_row_flat<LPB, SRV, OUT, ITEMS>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, gpr, total, fa)
     if constexpr (FORM != 0) { if (p.rounding == 1) HBFP_QFLAT(true, FORM); else HBFP_QFLAT(false, FORM); }
     else if (p.rounding == 1) { if (L.planes == 1) HBFP_QFLAT(true, 1); else HBFP_QFLAT(true, 2); }
     else { if (L.planes == 1) HBFP_QFLAT(false, 1); else HBFP_QFLAT(false, 2); }
@@ -1723,7 +1727,7 @@ int launch_row_ragged(bool vec, const float* x, int64_t rows, int64_t K, int64_t
     QParams q = p;
     for (int64_t r = 0; r < rows; r += rows_per, q.at = Placing{}) {
         const int64_t total = std::min(rows - r, rows_per) * ppr;
-#define HBFP_RAGGED(LPB, SRV, VEC) launch_chained(quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 8 * ragged_pieces<LPB, SRV && !VEC>() - 1) / (8 * ragged_pieces<LPB, SRV && !VEC>())), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
+#define HBFP_RAGGED(LPB, SRV, VEC) launch_placed(q.at, 4 * rows * K, quant_row_ragged<LPB, SRV, OUT, VEC>, (unsigned)((total + 8 * ragged_pieces<LPB, SRV && !VEC>() - 1) / (8 * ragged_pieces<LPB, SRV && !VEC>())), 256, 0, st, x, rows, K, ld, (int)L.b, q, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, d, r, (uint32_t)total, fa)
 #define HBFP_RAGGED_SR(LPB, VEC) do { if (p.rounding) HBFP_RAGGED(LPB, true, VEC); else HBFP_RAGGED(LPB, false, VEC); } while (0)
 #define HBFP_RAGGED_VEC(LPB) do { if (vec) HBFP_RAGGED_SR(LPB, true); else HBFP_RAGGED_SR(LPB, false); } while (0)
         if (L.bp == 32) HBFP_RAGGED_VEC(4); else if (L.bp == 64) HBFP_RAGGED_VEC(8); else HBFP_RAGGED_VEC(16);
@@ -1967,7 +1971,7 @@ int launch_col_tma(const float* x, int64_t K, int64_t rows, int64_t ld, const QP
     const int64_t total = tiles_n * tiles_k;
     const int64_t cap = (int64_t)sm_count() * ctas_per_sm;
     const int grid = (int)(total < cap ? total : cap);
-    launch_chained(quant_col_tma<PLANES, LB, SR>, grid, QC_THREADS, smem, st, mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
+    launch_placed(p.at, 0, quant_col_tma<PLANES, LB, SR>, grid, QC_THREADS, smem, st, mX, mM0, mM1, p, exps, L.rs, L.nkb, K, rows, (int)tiles_n,
                                                               (int)total, status, given, mant, L.kst, L.plane_stride);
     return launch_status();
 }
@@ -1980,11 +1984,11 @@ int launch_row_fast(const float* x, int64_t rows, int64_t K, int64_t ld, const Q
     dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
     // the last column tile must also cover the exponent rows of blocks that start before K
     if (p.rounding == 1) {
-        if (L.planes == 1) launch_chained(quant_row_fast<LPB, true, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
-        else launch_chained(quant_row_fast<LPB, true, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        if (L.planes == 1) launch_placed(p.at, 4 * rows * K, quant_row_fast<LPB, true, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        else launch_placed(p.at, 4 * rows * K, quant_row_fast<LPB, true, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
     } else {
-        if (L.planes == 1) launch_chained(quant_row_fast<LPB, false, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
-        else launch_chained(quant_row_fast<LPB, false, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        if (L.planes == 1) launch_placed(p.at, 4 * rows * K, quant_row_fast<LPB, false, 1>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
+        else launch_placed(p.at, 4 * rows * K, quant_row_fast<LPB, false, 2>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, nullptr, FormArgs{});
     }
     return launch_status();
 }
@@ -2009,8 +2013,8 @@ int launch_tile_full_small(int mode, int planes, int t, bool general, unsigned g
     const dim3 grid_dim(gx, gy);
 #define HBFP_TILE_FULL_SMALL(MODE, PLANES, TP)                                                                                              \
     do {                                                                                                                                    \
-        if (general) launch_chained(tile_kernel_full<MODE, PLANES, TP, true>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv); \
-        else launch_chained(tile_kernel_full<MODE, PLANES, TP, false>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv);      \
+        if (general) launch_streamed(tile_bytes<MODE>(d0, d1), tile_kernel_full<MODE, PLANES, TP, true>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv); \
+        else launch_streamed(tile_bytes<MODE>(d0, d1), tile_kernel_full<MODE, PLANES, TP, false>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, grid_ld, tv);      \
     } while (0)
 #define HBFP_TILE_FULL_MODE(MODE)                                                                     \
     do {                                                                                              \
@@ -2068,7 +2072,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         if (L.rs != rows) HBFP_CUDA_OK(cudaMemsetAsync(exps, 0, (size_t)L.exp_bytes, st));
         // rows of 2048, 4096, 8192 or 16384 elements stay in a CTA's registers: one pass
         if ((K == 2048 || K == 4096 || K == 8192 || K == 16384) && L.kst == K && rows < (1ll << 31)) {
-#define HBFP_QROW_WHOLE2(GV, SRV, PL) launch_chained(quant_row_whole<GV, SRV, PL>, (unsigned)rows, 256, 0, st, x, ld, d1, p, mant, L.kst, L.plane_stride, exps)
+#define HBFP_QROW_WHOLE2(GV, SRV, PL) launch_placed(last.at, 4 * rows * K, quant_row_whole<GV, SRV, PL>, (unsigned)rows, 256, 0, st, x, ld, d1, p, mant, L.kst, L.plane_stride, exps)
 #define HBFP_QROW_WHOLE(GV)                                                                          \
     do {                                                                                             \
         if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_WHOLE2(GV, true, 1); else HBFP_QROW_WHOLE2(GV, true, 2); }   \
@@ -2083,7 +2087,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         launch_chained(exps_axis1, (unsigned)(want < 148 * 16 ? want : 148 * 16), 256, 0, st, x, rows, K, ld, L.b, L.nkb, p, exps, L.rs);
         if (launch_status()) return HBFP_ERR_CUDA;
         dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
-#define HBFP_QROW_GIVEN(SRV, PL) launch_chained(quant_row_fast<16, SRV, PL>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, exps, FormArgs{})
+#define HBFP_QROW_GIVEN(SRV, PL) launch_placed(last.at, 4 * rows * K, quant_row_fast<16, SRV, PL>, grid, 256, 0, st, x, rows, K, ld, p, mant, L.kst, L.plane_stride, exps, L.rs, L.nkb, exps, FormArgs{})
         if (p.rounding == 1) { if (L.planes == 1) HBFP_QROW_GIVEN(true, 1); else HBFP_QROW_GIVEN(true, 2); }
         else { if (L.planes == 1) HBFP_QROW_GIVEN(false, 1); else HBFP_QROW_GIVEN(false, 2); }
 #undef HBFP_QROW_GIVEN
@@ -2113,7 +2117,7 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
         const int64_t wide = (rows + 255) / 256;
         const bool idle = wide * ((K + CMAX_ROWS - 1) / CMAX_ROWS) < 4 * 148;
         const int band = idle && (K <= 12288 || (K <= 20480 && wide >= 3)) ? CMAX_ROWS_SHORT : CMAX_ROWS;
-        launch_chained(col_amax_kernel, dim3((unsigned)wide, (unsigned)((K + band - 1) / band)), 256, 0, st, x, K, rows, ld, band, amax);
+        launch_streamed(4 * rows * K, col_amax_kernel, dim3((unsigned)wide, (unsigned)((K + band - 1) / band)), 256, 0, st, x, K, rows, ld, band, amax);
         launch_chained(col_exps_kernel, (unsigned)wide, 256, 0, st, amax, rows, p, exps);
         if (launch_status()) return HBFP_ERR_CUDA;
         if (stream) {
@@ -2168,9 +2172,9 @@ int launch_quantize(const float* x, int64_t d0, int64_t d1, int64_t ld, int axis
     }
     if (launch_status()) return HBFP_ERR_CUDA;
     if (L.planes == 1)
-        launch_chained(mant_generic<1>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
+        launch_placed(last.at, 4 * rows * K, mant_generic<1>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     else
-        launch_chained(mant_generic<2>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
+        launch_placed(last.at, 4 * rows * K, mant_generic<2>, blocks_for(rows * (L.kst / 4), 256), 256, 0, st, x, d1, rows, K, ld, axis, L.b, L.bp, L.nkb, p, exps, L.rs, mant, L.kst, L.plane_stride);
     return launch_status();
 }
 
@@ -2185,7 +2189,7 @@ int quantize_form(const float* x, int64_t d1, int64_t ld, int axis, int64_t rows
             return L.b == 32 ? launch_row_flat<4, FORM>(x, rows, K, ld, p, L, out, scales, st, fa) : launch_row_flat<8, FORM>(x, rows, K, ld, p, L, out, scales, st, fa);
         if (aligned && d1 % 8 == 0 && L.b == L.bp && rows <= 32ll * 65535) {
             const dim3 grid((unsigned)((L.kst + 511) / 512), (unsigned)((rows + 31) / 32));
-#define HBFP_QFAST(LPB, SRV) launch_chained(quant_row_fast<LPB, SRV, FORM>, grid, 256, 0, st, x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
+#define HBFP_QFAST(LPB, SRV) launch_placed(p.at, 4 * rows * K, quant_row_fast<LPB, SRV, FORM>, grid, 256, 0, st, x, rows, K, ld, p, out, L.kst, L.plane_stride, scales, L.rs, L.nkb, nullptr, fa)
             if (L.b == 32) { if (p.rounding) HBFP_QFAST(4, true); else HBFP_QFAST(4, false); }
             else { if (p.rounding) HBFP_QFAST(8, true); else HBFP_QFAST(8, false); }
 #undef HBFP_QFAST
@@ -2256,7 +2260,7 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     if (full) {
         // whole tiles, cut by 32-bit shifts
         const bool general = d0 % t != 0 || d1 % t != 0 || (MODE != 3 && 16 - p.m + (L0.planes == 2 ? 4 : 0) > 8);
-#define HBFP_TILE_FULL(PLANES, RG) launch_chained(tile_kernel_full<MODE, PLANES, 128, RG>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, nv, tv)
+#define HBFP_TILE_FULL(PLANES, RG) launch_streamed_long(tile_bytes<MODE>(d0, d1), tile_kernel_full<MODE, PLANES, 128, RG>, grid_dim, 256, 0, st, src, ld, d0, d1, p, wide, grid, nv, tv)
         if (t != 128)
             return launch_tile_full_small(MODE, (int)L0.planes, t, general, grid_dim.x, grid_dim.y, src, ld, d0, d1, &p, wide, grid, nv, &tv, st);
         if (L0.planes == 1) { if (general) HBFP_TILE_FULL(1, true); else HBFP_TILE_FULL(1, false); }
@@ -2287,7 +2291,7 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     do {                                                                                                                      \
         rc = allow_shared<tile_kernel<MODE, PLANES, FAST>>(128 * 132 * sizeof(float) + 128 * 130 * sizeof(int16_t));          \
         if (rc) return rc;                                                                                                    \
-        launch_chained(tile_kernel<MODE, PLANES, FAST>, grid_dim, 256, smem, st, src, ld, d0, d1, t, tp, p, wide, grid, nv, tv); \
+        launch_streamed(tile_bytes<MODE>(d0, d1), tile_kernel<MODE, PLANES, FAST>, grid_dim, 256, smem, st, src, ld, d0, d1, t, tp, p, wide, grid, nv, tv); \
     } while (0)
         if (L0.planes == 1) { if (fast) HBFP_TILE(1, true); else HBFP_TILE(1, false); }
         else { if (fast) HBFP_TILE(2, true); else HBFP_TILE(2, false); }
@@ -2319,7 +2323,7 @@ int launch_tiles(const float* src, int64_t ld, int64_t d0, int64_t d1, const hbf
     do {                                                                                                                                          \
         rc = allow_shared<tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>>(96 * 1024);       /* eight tile rows of five tiles of 8 with draws: 93 KB */     \
         if (rc) return rc;                                                                                                                        \
-        launch_chained(tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>, strips, 32 * NW, smem, st, src, ld, d0, d1, sh, p, wide, grid, nv, tv);  \
+        launch_streamed_long(tile_bytes<MODE>(d0, d1), tile_strip_kernel<MODE, PLANES, NW, RPW, KC, SRV>, strips, 32 * NW, smem, st, src, ld, d0, d1, sh, p, wide, grid, nv, tv);  \
     } while (0)
 #define HBFP_STRIP_SR(PLANES, NW, RPW, KC) do { if (p.rounding && MODE != 2) HBFP_STRIP(PLANES, NW, RPW, KC, MODE != 2); else HBFP_STRIP(PLANES, NW, RPW, KC, false); } while (0)
 #define HBFP_STRIP_KC(PLANES) do { if (kc == 2) HBFP_STRIP_SR(PLANES, 8, 8, 2); else if (kc == 3) HBFP_STRIP_SR(PLANES, 8, 6, 3); else HBFP_STRIP_SR(PLANES, 16, 8, 4); } while (0)
@@ -2450,7 +2454,7 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
     do {                                                                                                                              \
         rc = allow_shared<im2col_cols3<PL, WV, SRV>>(IM2COL_SMEM_MAX / 2);          /* two bytes of draws for every four of values */    \
         if (rc) return rc;                                                                                                            \
-        launch_chained(im2col_cols3<PL, WV, SRV>, (unsigned)L.nkb, threads, table, st, x, (int)h, (int)c, kh, pad, p, L.kst, L.plane_stride, L.rs, mant, exps); \
+        launch_streamed(4 * n * h * w * c, im2col_cols3<PL, WV, SRV>, (unsigned)L.nkb, threads, table, st, x, (int)h, (int)c, kh, pad, p, L.kst, L.plane_stride, L.rs, mant, exps); \
     } while (0)
 #define HBFP_COLS3_SR(PL, WV) do { if (p.rounding) HBFP_COLS3(PL, WV, true); else HBFP_COLS3(PL, WV, false); } while (0)
 #define HBFP_COLS3_W(PL) do { if (w == 8) HBFP_COLS3_SR(PL, 8); else if (w == 16) HBFP_COLS3_SR(PL, 16); else if (w == 32) HBFP_COLS3_SR(PL, 32); else HBFP_COLS3_SR(PL, 64); } while (0)
@@ -2466,7 +2470,7 @@ int launch_im2col_cols(const float* x, int64_t n, int64_t h, int64_t w, int64_t 
     do {                                                                                                                       \
         rc = allow_shared<im2col_cols<PL, NPX, SRV>>(IM2COL_SMEM_MAX);                                                          \
         if (rc) return rc;                                                                                                     \
-        launch_chained(im2col_cols<PL, NPX, SRV>, (unsigned)L.nkb, 256, smem, st, x, (int)h, (int)w, lg_w, (int)c, kh, kw, pad, p, L.kst,     \
+        launch_streamed(4 * n * h * w * c, im2col_cols<PL, NPX, SRV>, (unsigned)L.nkb, 256, smem, st, x, (int)h, (int)w, lg_w, (int)c, kh, kw, pad, p, L.kst,     \
                                                                      L.plane_stride, L.rs, mant, exps);                        \
     } while (0)
 #define HBFP_COLS_LAUNCH(PL, NPX)                                                 \
@@ -2552,15 +2556,15 @@ int launch_wide_dequantize(const int16_t* wide, const int8_t* exps, int64_t d0, 
     const unsigned rows = (unsigned)std::min<int64_t>((d0 + 3) / 4, 65535);
     const bool vec = tile % 4 == 0 && d1 % 4 == 0 && ldo % 4 == 0 && (reinterpret_cast<uintptr_t>(wide) & 7) == 0 &&
                      (reinterpret_cast<uintptr_t>(out) & 15) == 0;
-    if (vec) launch_chained(wide_dequant_kernel<4>, dim3(blocks_for(d1, 1024), rows), 256, 0, st, wide, exps, d0, d1, tile, tiles1, out, ldo);
-    else launch_chained(wide_dequant_kernel<1>, dim3(blocks_for(d1, 256), rows), 256, 0, st, wide, exps, d0, d1, tile, tiles1, out, ldo);
+    if (vec) launch_streamed(2 * d0 * d1, wide_dequant_kernel<4>, dim3(blocks_for(d1, 1024), rows), 256, 0, st, wide, exps, d0, d1, tile, tiles1, out, ldo);
+    else launch_streamed(2 * d0 * d1, wide_dequant_kernel<1>, dim3(blocks_for(d1, 256), rows), 256, 0, st, wide, exps, d0, d1, tile, tiles1, out, ldo);
     return launch_status();
 }
 
 int launch_dequantize(const Packed& p, float* out, int64_t ld, cudaStream_t st) {
     const Layout& L = p.L;
     if (L.rows * L.k == 0) return HBFP_OK;
-    launch_chained(dequant_kernel, blocks_for(L.rows * L.k, 256), 256, 0, st, p.mant, p.exps, L.rows, L.k, L.b, L.bp, L.kst,
+    launch_streamed(L.planes * L.rows * L.k, dequant_kernel, blocks_for(L.rows * L.k, 256), 256, 0, st, p.mant, p.exps, L.rows, L.k, L.b, L.bp, L.kst,
                                                                  L.plane_stride, (int)L.planes, L.rs, out, ld);
     return launch_status();
 }

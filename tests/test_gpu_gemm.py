@@ -718,6 +718,38 @@ def test_products_of_operand_forms_are_placed_early(hb, n, m, b, chained):
     assert edges_in_order(graph) == [1, chained]
 
 
+# Kernels that load much through L1 are not placed behind a product, which leaves them little of it, nor are a few long CTAs; others are,
+# and those behind others.
+@pytest.mark.parametrize("rows,op,chained", [(1024, "rows", 1), (8192, "rows", 0), (1024, "columns", 1), (8192, "columns", 0), (1024, "update", 1), (4096, "update", 0), (512, "long update", 0), (8192, "value", 0)])
+def test_long_kernels_and_long_ctas_are_not_placed_behind_a_product(hb, rows, op, chained):
+    import torch
+    t = 128 if op == "long update" else 64
+    f, fw = hb.Format(block=24 if op == "columns" else 64), hb.Format(block=t, tile=t)
+    pa, pb = hb.quantize(torch.randn(512, 256, device="cuda"), 1, f), hb.quantize(torch.randn(512, 256, device="cuda"), 1, f)
+    x, C, ws = torch.randn(rows, 4096, device="cuda"), torch.empty(512, 512, device="cuda"), torch.empty(1 << 24, dtype=torch.int8, device="cuda")
+    out = hb.quantize(x, 0 if op == "columns" else 1, f)
+    wide, views = hb.wide_quantize(x, fw)
+    other = torch.empty_like(x)
+
+    def kernel():
+        if op == "rows": hb.quantize(x, 1, f, out)
+        elif op == "columns": hb.quantize(x, 0, f, out)
+        elif op.endswith("update"): hb.wide_update(wide, x, fw, views=views)
+        else: hb.wide_dequantize(wide, other)
+
+    def steps():
+        hb.gemm_q(512, 512, 256, pa, pb, out=C, workspace=ws)
+        kernel()
+        kernel()
+
+    steps()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        steps()
+    assert edges_in_order(graph)[-2:] == [chained, 1]
+
+
 # Routes in which the second operand is converted beside the first, on an operand that the kernel before has just written: packed
 # weights of an update in place, the FP32 value of wide weights.
 # Replayed too: the word through which the first conversion passes on what it has waited for starts every replay anew.
