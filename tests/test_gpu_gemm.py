@@ -570,6 +570,31 @@ def test_few_rows_kernels_of_different_plans_run_on_two_streams(hb, first, secon
         assert all(torch.equal(o, alone) for o in outs)
 
 
+# Calls of several launches each, placed early behind one another, on two streams at once: both conversions beside each other, forms
+# (split, in pairs), integer kernels with and without split-K, the smallest products.
+@pytest.mark.parametrize("first,second", [
+    ((1111, 777, 3001, 8, 24), (512, 512, 4096, 8, 32)), ((2048, 2304, 512, 12, 64), (2304, 2304, 1024, 8, 128)), ((300, 200, 4000, 8, 128), (2048, 2304, 512, 8, 64)),
+    ((64, 96, 128, 8, 32), (1024, 1024, 1024, 8, 32))])
+def test_products_of_fp32_operands_on_two_streams(hb, first, second):
+    import torch
+    work = []
+    for k, (M, N, K, m, b) in enumerate((first, second)):
+        A, B = to_dev(wl.draw("normal", (M, K), seed=130 + k)), to_dev(wl.draw("outliers", (K, N), seed=140 + k))
+        fa, fb = hb.Format(m, b, rounding=1, seed=4), hb.Format(m, b, rounding=1, seed=4, stream_id=1)
+        alone = hb.gemm(0, 0, A, B, fa, fb)
+        ws = torch.empty(max(hb.gemm_workspace(0, 0, M, N, K, fa, fb), 1), dtype=torch.int8, device="cuda")
+        work.append((torch.cuda.Stream(), alone, [torch.empty_like(alone) for _ in range(48)], lambda o, a=(0, 0, A, B, fa, fb), w=ws: hb.gemm(*a, out=o, workspace=w)))
+    torch.cuda.synchronize()
+    for i in range(48):
+        for stream, _, outs, call in work:
+            with torch.cuda.stream(stream):
+                call(outs[i])
+    torch.cuda.synchronize()
+    assert hb.device_status() == 0
+    for _, alone, outs, _ in work:
+        assert all(torch.equal(o, alone) for o in outs)
+
+
 @pytest.mark.parametrize("M,N,K", [(128, 128, 256), (600, 520, 1700), (2304, 2176, 1760)])
 def test_scaled_operand_form_reports_products_beyond_binary32(hb, M, N, K):
     """Products of 2^129 that cancel to 2^122 within a block, in one of its MMA steps or across two: the sum is representable, and the

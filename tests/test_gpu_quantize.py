@@ -379,3 +379,23 @@ def test_ragged_row_and_column_kernels_at_their_edges(hb, axis, lines, K, b, m, 
     q_ref, s_ref = oracle.quantize(x, axis, ofmt(fd))
     assert np.array_equal(q, q_ref) and np.array_equal(s, s_ref)
     assert hb.device_status() == 0
+
+
+@pytest.mark.parametrize("rounding", [0, 1])
+def test_ragged_rows_of_more_pieces_than_one_launch_numbers(hb, rounding):
+    """2^32 pieces of eight and a few: rows of one element, padded to 128. The last rows of the first launch and all of the second."""
+    import torch
+    rows = ((1 << 32) - 65536) // 16 + 5003
+    fd = dict(mant_bits=8, block=24, rounding=rounding, seed=3, stream_id=2)
+    x = torch.randn(rows, 1, device="cuda", generator=torch.Generator(device="cuda").manual_seed(8))
+    p = hb.quantize(x, 1, gfmt(fd))
+    lay = hb.packed_layout(rows, 1, p.fmt)
+    assert lay["kst"] == 128 and lay["nkb"] == 1
+    for r0, n in ((0, 3000), (rows - 8000, 8000)):
+        q_ref, s_ref = oracle.quantize_indexed(x[r0:r0 + n].cpu().numpy(), 1, ofmt(fd), np.arange(r0, r0 + n, dtype=np.int64)[:, None])
+        mant = p.mant[r0 * 128:(r0 + n) * 128].view(n, 128)
+        assert np.array_equal(mant[:, :1].cpu().numpy(), q_ref) and not bool(mant[:, 1:].any())
+        assert np.array_equal(p.exps[r0:r0 + n].cpu().numpy()[:, None], s_ref)
+    assert not bool(p.exps[rows:lay["rs"]].any()) and hb.device_status() == 0
+    del x, p, mant
+    torch.cuda.empty_cache()

@@ -422,3 +422,42 @@ def test_bias_added_by_whichever_kernel_ends_the_product(env, batch, fin, fout, 
         layer.bias.normal_()
         assert torch.equal(layer(x), plain + layer.bias)
     assert hb.device_status() == 0
+
+
+@pytest.mark.parametrize("kind", ["linear", "linear12", "conv"])
+def test_layer_step_captured_in_a_cuda_graph(env, kind):
+    """Forward, both gradients and the update of the weights in one graph: replays train on as the same steps outside one do."""
+    torch, hbfp_nn, hb = env
+
+    def make():
+        torch.manual_seed(5)
+        if kind == "conv":
+            return hbfp_nn.HbfpConv3x3(64, 64)
+        return hbfp_nn.HbfpLinear(600, 712, mant_bits=12 if kind == "linear12" else 8, tile=64 if kind == "linear12" else 24, rounding=0)
+
+    x = torch.randn((8, 16, 16, 64) if kind == "conv" else (2100, 600), device="cuda", requires_grad=True)
+    dy = torch.randn((8, 16, 16, 64) if kind == "conv" else (2100, 712), device="cuda")
+
+    def step(layer, grads):
+        got = torch.autograd.grad(layer(x), [x, layer.weight], dy)
+        for out, g in zip(grads, got):
+            out.copy_(g)
+        layer.apply_update(got[1] * -1e-2)
+
+    eager, captured = make(), make()
+    want, got = ([torch.empty_like(x), torch.empty_like(eager.weight)] for _ in range(2))
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        step(make(), got)                                 # sets the kernels' attributes
+    torch.cuda.current_stream().wait_stream(side)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step(captured, got)
+    for _ in range(4):
+        step(eager, want)
+        graph.replay()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+        assert torch.equal(captured.wide.mant, eager.wide.mant) and torch.equal(captured.wide.exps, eager.wide.exps)
+        assert torch.equal(captured.weight.data, eager.weight.data)
+    assert hb.device_status() == 0
