@@ -104,6 +104,8 @@ def lib() -> ctypes.CDLL:
         L.hbfp_gemm_q_workspace.argtypes = [i64, i64, i64, p, p, p]
         L.hbfp_gemm.argtypes = [i32, i32, i64, i64, i64, p, i64, p, i64, p, i64, p, p, p, sz, u32, p]
         L.hbfp_gemm_q.argtypes = [i64, i64, i64, p, p, p, i64, p, sz, u32, p]
+        L.hbfp_gemm_q_bias.argtypes = [i64, i64, i64, p, p, p, p, i64, p, sz, u32, p]
+        L.hbfp_column_sums.argtypes = [p, i64, i64, i64, p, p]
         L.hbfp_gemm_static.argtypes = [i32, i32, i64, i64, i64, p, i64, p, i64, p, i64, p, p, u32, p]
         L.hbfp_gemm_block_partials.argtypes = [i64, i64, i64, p, p, p, u32, p]
         L.hbfp_device_status.argtypes = [p, p]
