@@ -56,12 +56,15 @@ inline int make_layout(int64_t rows, int64_t k, const hbfp_format* f, Layout* L)
 inline int launch_status() { return cudaGetLastError() == cudaSuccess ? HBFP_OK : HBFP_ERR_CUDA; }
 
 // Chained launches. A call is a chain of kernels of 2 to 20 us each, and between two of them in a stream lie the end of the one,
-// the launch of the other and its start. Every kernel is launched so that its CTAs may be placed as soon as all CTAs of the kernel
-// before it have started and an SM has room (programmatic stream serialization); it sets up its barriers and tensor memory there
-// and then waits for that kernel to end (chain_wait) before it touches global memory. The wait covers the whole stream: the
-// kernel before it had waited in its turn. Every kernel launched by launch_chained has to wait, in at least one thread.
-// Back to back with conversions, before / after: 256 cube 8.2 / 6.4 us, 1111 x 777 x 3001 (b = 24, with draws) 45.9 / 37.7,
-// 1024 x 4096 x 4096 (b = 32) 75.0 / 65.5, 2048 cube (b = 64) 39.3 / 31, 16 rows against 4096 x 4096 packed weights 11.6 / 9.1.
+// the launch of the other and its start. Kernels are launched so that their CTAs may be placed as soon as all CTAs of the kernel
+// before have started and an SM has room (programmatic stream serialization); they set up their barriers and tensor memory there
+// and then wait for that kernel to end (chain_wait) before they touch global memory. The wait covers the whole stream: the
+// kernel before had waited in its turn. Every kernel launched by launch_chained has to wait, in at least one thread. Launched plainly
+// are the paired-SM integer GEMM, long launches of the 12-bit operand forms (gemm_fp.cu), long kernels and a few long CTAs behind a
+// product (below) and the wait probe.
+// It is the gap between launches that shrinks: calls back to back with their conversions, without chains / with them: 256 cube 8.2 / 6.4
+// us, 1111 x 777 x 3001 (b = 24, with draws) 46.3 / 34.1, 1024 x 4096 x 4096 (b = 32) 77 / 67.6, 2048 cube (b = 64) 39.3 / 30.1, 16 rows against
+// 4096 x 4096 packed weights 11.6 / 8.9. A call of one launch takes by itself what it took.
 // A kernel says that its successor may be placed (chain_next) only after it has itself waited and, where it uses tensor memory, has
 // allocated it: a successor that took the columns first would wait for a kernel that waits for the columns.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

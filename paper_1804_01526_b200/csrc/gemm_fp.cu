@@ -743,6 +743,7 @@ inline int log2_of(int64_t v) { int l = 0; while ((1ll << l) < v) ++l; return l;
 
 }  // namespace
 
+// (The times below are both sides' before launches were chained: what each launch adds has since become less on either side.)
 FpPlan plan_gemm_fp(int64_t M, int64_t N, const Layout& la, const Layout& lb, int passes) {
     FpPlan f{};
     if (M <= 0 || N <= 0 || la.nkb <= 0 || la.planes != lb.planes || la.bp != lb.bp || la.nkb != lb.nkb || la.b != lb.b) return f;

@@ -351,6 +351,7 @@ int sf_launch(const SmallProblem& p, dim3 grid, cudaStream_t st) {
 bool small_fused_eligible(const hbfp_operand* a, bool a_contig, const hbfp_operand* b, bool b_contig, int64_t M, int64_t N, const Layout& la) {
     if (a->kind != HBFP_OPERAND_FP32 || b->kind != HBFP_OPERAND_FP32 || a->fmt.tile != 0 || b->fmt.tile != 0) return false;
     if (la.bp > 128 || la.nkb * la.bp > SM_AUTO_BYTES || la.nkb <= 0) return false;
+    // (Times of both sides before launches were chained.)
     // A CTA's registers fill an SM when a column conversion holds 512 K; a second round of tiles then costs more than two launches
     // (512 cube 18.6 against 10.7 us of device time; 512 x 512 x 256, two CTAs per SM, 10.5 against 14.3 as a call).
     const int64_t ctas = ((M + SM_TILE - 1) / SM_TILE) * ((N + SM_TILE - 1) / SM_TILE);

@@ -6,7 +6,8 @@
 // warp ids, and a starved MMA issuer stalls everything):
 //   warp 0     TMA producer: mantissa tiles (128B-swizzled, K-major) and exponent slices
 //   warp 1     MMA issuer (one thread) and owner of the tensor-memory allocation
-//   warp 2     scale-table builder: turns the int8 exponent slices of each block into 2^sA / 2^sB
+//   warps 2, 3 scale-table builders: turn the int8 exponent slices of each block into 2^sA / 2^sB (warp 3 takes every other block where
+//              there are blocks enough to share)
 //   warps 4-11 rescale: tcgen05.ld the int32 block sums, scale by 2^(sA+sB), accumulate in FP32
 //              registers (128 rows x N_TILE columns per tile), store C
 // A stage is 128 bytes of K for every row of the A (128 rows) and B (N_TILE rows) tiles, i.e. four

@@ -12,7 +12,8 @@
 //   quant_col_tma    blocks down the columns, b in {32,64,128}, 16-byte aligned pitch: persistent
 //                    CTAs stream 128 x 64 FP32 tiles through a TMA pipeline and write the packed,
 //                    transposed tile with a swizzled TMA store (full lines in both directions).
-//   quant_col_block  blocks down the columns, any b <= 128 and any pitch: one K-block of 32 columns per CTA.
+//   quant_col_block  blocks down the columns, any b <= 128 and any pitch: 32 columns of four, two or one K-blocks (by their length)
+//                    per CTA, a lane per column.
 //   quant_row_ragged blocks along rows, any b <= 128, row length, pitch and alignment, in one pass.
 //   tile_strip_kernel, tile_kernel, tile_kernel_full   t x t weight tiles (t <= 128): one pass writes both packed views and
 //                    the tile exponent grid.
