@@ -85,7 +85,8 @@ __device__ __forceinline__ void chain_start() { chain_wait(); chain_next(); }
 // and as right. The first CTA gives the word back, so that a replayed graph starts without it. Loads of a BESIDE kernel are not .nc.
 // Back to back, all three launches chained / so / with a plain launch as the LEAD, which is a kernel boundary by itself (and before the
 // word, when nothing passed the writes on): 1111 x 777 x 3001, b = 24, draws 36.3 / 34.2 / 34.8 us (33.7); 1024 x 4096 x 4096, b = 32
-// 71.2 / 67.8 / 68.2 (67.0); 512 cube, b = 64 11.0 / 10.4 / 12.4 (9.9). A call by itself: 512 cube 13.6 / 12.5 / 12.1 (12.1).
+// 71.2 / 67.8 / 68.2 (67.0); 512 cube, b = 64 11.0 / 10.4 / 12.4 (9.9). By itself a 512 cube takes 1.13 / 1.02 / 1.00 of what it took,
+// over 36 formats and orders.
 enum Place : int { CHAINED = 0, LEAD = 1, BESIDE = 2 };
 struct Placing {
     int place = CHAINED;
